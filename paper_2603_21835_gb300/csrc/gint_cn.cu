@@ -3,9 +3,9 @@
 // coefficients, (S + i dt/2 H) psi(t + dt) = (S - i dt/2 H) psi(t) (paper Sec. 2: the density matrix
 // and the time propagation of the coefficients with the overlap matrix), and the energy-density
 // matrix E = (S^{-1} H D + D H S^{-1}) / 2.  All in float64 on this library's own kernels
-// (gint_la.cu: tiled GEMM, blocked L D L^T and its solves); the density matrix also has a
-// tensor-core build (float16 three-term split, gint_dm.cu).  A context holds every buffer, so the
-// compute calls allocate nothing.
+// (gint_sg.cu: float64 products from exact digit products on the tensor cores; gint_la.cu: blocked
+// L D L^T and its solves); the density matrix also has a mixed-precision build (float16 three-term split,
+// gint_dm.cu).  A context holds every buffer, so the compute calls allocate nothing.
 //
 // The step solves A X = S psi with A = S + i dt/2 H and returns 2 X - psi, which equals
 // A^{-1} (S - i dt/2 H) psi since S - i dt/2 H = 2 S - A: a real-by-complex product replaces the
@@ -51,7 +51,8 @@ unsigned blocks_for(long long n) { return (unsigned)std::min<long long>((n + 255
 struct gint_cn {
   int n = 0, nocc = 0, device = 0;
   double2 *A = nullptr;        // n x n: the factor (complex), or two real n x n matrices (gint_edm)
-  double2 *work = nullptr;     // n x 64: the factorisation's panel workspace
+  double2 *work = nullptr;     // the factorisation's panel workspace (gla::ldl_work)
+  gla::SgWork sg{};            // scratch of the float64 products
   int *info = nullptr;
   void *dmw = nullptr;         // tensor-core density-matrix build: packed operands and scales
   unsigned *status = nullptr;  // its device error word
@@ -64,6 +65,7 @@ int gint_cn_destroy(gint_cn *c) {
   cudaSetDevice(c->device);
   cudaFree(c->A);
   cudaFree(c->work);
+  cudaFree(c->sg.buf);
   cudaFree(c->info);
   cudaFree(c->dmw);
   cudaFree(c->status);
@@ -79,8 +81,14 @@ int gint_cn_create(int n, int nocc, gint_cn **out) {
   c->nocc = nocc;
   cudaGetDevice(&c->device);
   const size_t nn = (size_t)n * n;
-  if (cudaMalloc(&c->A, nn * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc(&c->work, (size_t)n * 64 * sizeof(double2)) != cudaSuccess ||
+  // panels of the step (complex, nocc right-hand sides) and of the energy-density matrix (real, n)
+  const size_t work = std::max(gla::ldl_work<double2>(n, nocc) * sizeof(double2), gla::ldl_work<double>(n, n) * sizeof(double));
+  // products: S psi and H D (right rows: 2 nocc or n), the density matrix (contraction 2 nocc), the panels
+  c->sg.bytes = std::max({gla::sg_bytes(n + std::max((long long)n, 2LL * nocc), n), gla::sg_bytes(2LL * n, 2LL * nocc),
+                          gla::sg_bytes(gla::ldl_rows<double2>(n, nocc), 64), gla::sg_bytes(gla::ldl_rows<double>(n, n), 64)});
+  if (cudaDeviceGetAttribute(&c->sg.num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
+      cudaMalloc(&c->A, nn * sizeof(double2)) != cudaSuccess || cudaMalloc(&c->work, work) != cudaSuccess ||
+      cudaMalloc(&c->sg.buf, c->sg.bytes) != cudaSuccess ||
       cudaMalloc(&c->info, sizeof(int)) != cudaSuccess || cudaMalloc(&c->dmw, gint_dm_tc_bytes(n, nocc)) != cudaSuccess ||
       cudaMalloc(&c->status, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(c->info, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->status, 0, sizeof(unsigned)) != cudaSuccess) {
@@ -88,6 +96,7 @@ int gint_cn_create(int n, int nocc, gint_cn **out) {
     gint_cn_destroy(c);
     return GINT_ENOMEM;
   }
+  c->sg.status = c->status;
   *out = c;
   return GINT_OK;
 }
@@ -102,15 +111,20 @@ int gint_cn_step(gint_cn *c, const double *S, const double *H, double dt, const 
   if (cudaMemsetAsync(c->info, 0, sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
   k_cn_mat<<<blocks_for(nn), 256, 0, st>>>(nn, S, H, 0.5 * dt, c->A);
   if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA;
-  // X = S psi: real and imaginary parts (strided real views of the interleaved complex arrays)
-  for (int part = 0; part < 2; ++part) {
-    const int rc = gla::gemm<double>(0, n, k, n, 1.0, gla::view<double>(S, 1, n),
-                                     gla::view<double>(psi + part, 2LL * n, 2), 0.0, psi_out + part, 2, 2LL * n, st);
-    if (rc) return rc;
-  }
-  int rc = gla::ldl_factor<double2>(n, c->A, n, c->work, c->info, false, st);
+  // X = S psi as one real product: column 2 c + part of the interleaved complex arrays
+  gla::SgProduct p{};
+  p.M = p.K = n;
+  p.N = 2 * k;
+  p.A = gla::sg_real(S, 1, n);
+  p.B = gla::SgView{psi, 2LL * n, 1, 4, 2, 0, nullptr};
+  p.C = psi_out;
+  p.crh = 4;
+  p.crl = 2;
+  p.cch = 2LL * n;
+  p.ccl = 1;
+  int rc = gla::sg_gemm(&p, 1, c->sg, st);
   if (rc) return rc;
-  if ((rc = gla::ldl_solve<double2>(n, k, c->A, n, X, n, st))) return rc;
+  if ((rc = gla::ldl_factor_solve<double2>(n, c->A, n, k, X, n, c->work, c->info, false, c->sg, st))) return rc;
   k_cn_finish<<<blocks_for((long long)n * k), 256, 0, st>>>((long long)n * k, reinterpret_cast<const double2 *>(psi), X);
   return cudaGetLastError() == cudaSuccess ? GINT_OK : GINT_ECUDA;
 }
@@ -120,8 +134,18 @@ int gint_dm_build(gint_cn *c, const double *psi, const double *f, double *D, voi
   const int n = c->n;
   // D = A B^T over k = 2 s + (real, imaginary part): A_ik = f_s psi_is, B_ik = psi_is (real views);
   // the lower triangle is computed and mirrored, so D is symmetric bit for bit
-  const gla::View<double> Av{psi, 2, 2LL * n, 1, f}, Bv{psi, 2, 2LL * n, 1, nullptr};
-  return gla::gemm<double>(2, n, n, 2 * c->nocc, 1.0, Av, Bv, 0.0, D, 1, n, (cudaStream_t)stream);
+  gla::SgProduct p{};
+  p.M = p.N = n;
+  p.K = 2 * c->nocc;
+  p.mode = 2;
+  p.A = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f};
+  p.B = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, nullptr};
+  p.C = D;
+  p.crh = 2;
+  p.crl = 1;
+  p.cch = 2LL * n;
+  p.ccl = n;
+  return gla::sg_gemm(&p, 1, c->sg, (cudaStream_t)stream);
 }
 
 int gint_dm_build_f16x3(gint_cn *c, const double *psi, const double *f, double *D, void *stream) {
@@ -139,10 +163,19 @@ int gint_edm(gint_cn *c, const double *S, const double *H, const double *D, doub
       cudaMemcpyAsync(F, S, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return GINT_ECUDA;
   // X = H D, then X <- S^{-1} X (S = L D L^T), E = (X + X^T) / 2
-  int rc = gla::gemm<double>(0, n, n, n, 1.0, gla::view<double>(H, 1, n), gla::view<double>(D, n, 1), 0.0, X, 1, n, st);
+  gla::SgProduct p{};
+  p.M = p.N = p.K = n;
+  p.A = gla::sg_real(H, 1, n);
+  p.B = gla::sg_real(D, n, 1);
+  p.C = X;
+  p.crh = 2;
+  p.crl = 1;
+  p.cch = 2LL * n;
+  p.ccl = n;
+  int rc = gla::sg_gemm(&p, 1, c->sg, st);
   if (rc) return rc;
-  if ((rc = gla::ldl_factor<double>(n, F, n, reinterpret_cast<double *>(c->work), c->info, true, st))) return rc;
-  if ((rc = gla::ldl_solve<double>(n, n, F, n, X, n, st))) return rc;
+  if ((rc = gla::ldl_factor_solve<double>(n, F, n, n, X, n, reinterpret_cast<double *>(c->work), c->info, true, c->sg, st)))
+    return rc;
   k_sym_half<<<blocks_for((long long)n * n), 256, 0, st>>>(n, X, E);
   return cudaGetLastError() == cudaSuccess ? GINT_OK : GINT_ECUDA;
 }

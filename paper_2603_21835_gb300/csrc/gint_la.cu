@@ -1,18 +1,22 @@
 // gint_la.cu -- float64 dense linear algebra of the propagation steps around the grid passes (the
-// Crank-Nicolson step and the density and energy-density matrices of paper Sec. 2): a tiled GEMM and
-// the blocked L D L^T factorisation without pivoting with its triangular solves, real and complex.
+// Crank-Nicolson step and the energy-density matrix of paper Sec. 2): a blocked L D L^T factorisation
+// without pivoting with its triangular solves, real and complex.
 //
-// The GB300 runs float64 on its CUDA cores only, at about 2 fused multiply-adds per clock per SM, so
-// every kernel here is bound by the float64 pipe: a 64 x 64 output tile per CTA keeps 16 independent
-// accumulators per thread, far more than the pipe's latency needs, and operand traffic (a few bytes
-// per thousand multiply-adds) is immaterial.  Latency-bound pieces (the 64 x 64 diagonal blocks, the
-// 64-wide panel and right-hand-side substitutions) are small next to the GEMM updates.
+// The products (trailing updates, and the updates of the solve) run on the tensor cores (gint_sg.cu).
+// What is left on the CUDA cores' float64 pipe (2 fused multiply-adds per clock per SM: a warp-wide
+// float64 instruction occupies it for 16 clocks, a dependent chain sees its latency at every step) are
+// the NB x NB diagonal blocks and the NB-wide substitutions: both grow with NB, the number of launches
+// falls with it; NB = 32 complex or 64 real keeps the two of similar size for n of a few hundred and more.
 //
 // L D L^T without pivoting: the Crank-Nicolson matrix S + i dt/2 H is complex symmetric with a
 // positive definite Hermitian part S, so its leading blocks are nonsingular and elimination without
 // pivoting is stable for small dt (the growth stays of order 1 + dt^2 |H S^-1 H| / 4); the overlap
 // S of the energy-density matrix is symmetric positive definite.  Symmetry halves the flops of a
 // general LU.
+//
+// The right-hand sides ride along with the factorisation as further rows of the matrix ([A; B^T]): a
+// panel step turns their block into W = (L^-1 B)^T and leaves D^-1 L^-1 B in B, so the forward
+// substitution costs no launches of its own and only the backward one follows.
 #include <algorithm>
 
 #include "gint.h"
@@ -27,29 +31,19 @@ struct Ar;
 template <>
 struct Ar<double> {
   static __device__ __forceinline__ double zero() { return 0.0; }
-  static __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }  // c + a b
   static __device__ __forceinline__ double fms(double a, double b, double c) { return ::fma(-a, b, c); }  // c - a b
   static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
-  static __device__ __forceinline__ double scale(double a, double s) { return a * s; }
-  static __device__ __forceinline__ double axpby(double a, double x, double b, double y) { return a * x + b * y; }
   static __device__ __forceinline__ double inv(double d) { return 1.0 / d; }
   static __device__ __forceinline__ bool bad_pivot(double d, bool spd) { return spd ? !(d > 0.0) : !(d != 0.0 && isfinite(d)); }
 };
 template <>
 struct Ar<double2> {
   static __device__ __forceinline__ double2 zero() { return make_double2(0.0, 0.0); }
-  static __device__ __forceinline__ double2 fma(double2 a, double2 b, double2 c) {
-    return make_double2(::fma(-a.y, b.y, ::fma(a.x, b.x, c.x)), ::fma(a.y, b.x, ::fma(a.x, b.y, c.y)));
-  }
   static __device__ __forceinline__ double2 fms(double2 a, double2 b, double2 c) {
     return make_double2(::fma(a.y, b.y, ::fma(-a.x, b.x, c.x)), ::fma(-a.y, b.x, ::fma(-a.x, b.y, c.y)));
   }
   static __device__ __forceinline__ double2 mul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-  }
-  static __device__ __forceinline__ double2 scale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
-  static __device__ __forceinline__ double2 axpby(double a, double2 x, double b, double2 y) {
-    return make_double2(a * x.x + b * y.x, a * x.y + b * y.y);
   }
   // 1 / d = conj(d) / |d|^2
   static __device__ __forceinline__ double2 inv(double2 d) {
@@ -62,196 +56,128 @@ struct Ar<double2> {
   }
 };
 
-template <typename T>
-__device__ __forceinline__ T vat(const View<T> &v, int r, int k) {
-  T x = v.p[(long long)r * v.sr + (long long)(k >> 1) * v.skh + (long long)(k & 1) * v.skl];
-  if (v.ks) x = Ar<T>::scale(x, v.ks[k >> 1]);
-  return x;
-}
-
-// ---------------------------------------------------------------------------------------- GEMM
-constexpr int kBM = 64, kGT = 256;
-template <typename T>
-struct GemmK {
-  static constexpr int BK = 16;
-};
-template <>
-struct GemmK<double2> {
-  static constexpr int BK = 8;
-};
-
-// One CTA per 64 x 64 tile of C; thread (tx, ty) of 16 x 16 owns rows tx + 16 a and columns
-// ty + 16 b (a, b < 4), so a warp reads 16 consecutive elements of each shared operand row.  The
-// next K slab is loaded into registers while the current one is multiplied.
-template <typename T, int MODE>
-__global__ void __launch_bounds__(kGT, 2) k_gemm(int M, int N, int K, double alpha, View<T> A, View<T> B, double beta,
-                                              T *__restrict__ C, long long cr, long long cc) {
-  constexpr int BK = GemmK<T>::BK, NL = BK * kBM / kGT;
-  const int tm = blockIdx.x, tn = blockIdx.y;
-  if (MODE != 0 && tm < tn) return;
-  __shared__ T As[BK][kBM], Bs[BK][kBM];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = tm * kBM, n0 = tn * kBM;
-  T acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = Ar<T>::zero();
-  T ra[NL], rb[NL];
-  auto load = [&](int k0) {
-#pragma unroll
-    for (int q = 0; q < NL; ++q) {
-      const int e = tid + kGT * q, r = e & (kBM - 1), k = k0 + e / kBM;
-      ra[q] = (m0 + r < M && k < K) ? vat(A, m0 + r, k) : Ar<T>::zero();
-      rb[q] = (n0 + r < N && k < K) ? vat(B, n0 + r, k) : Ar<T>::zero();
-    }
-  };
-  load(0);
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    __syncthreads();  // the previous slab's reads are done
-#pragma unroll
-    for (int q = 0; q < NL; ++q) {
-      const int e = tid + kGT * q;
-      As[e / kBM][e & (kBM - 1)] = ra[q];
-      Bs[e / kBM][e & (kBM - 1)] = rb[q];
-    }
-    __syncthreads();
-    if (k0 + BK < K) load(k0 + BK);
-#pragma unroll
-    for (int k = 0; k < BK; ++k) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = As[k][tx + 16 * i];
-        b[i] = Bs[k][ty + 16 * i];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = Ar<T>::fma(a[i], b[j], acc[i][j]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gm = m0 + tx + 16 * i, gn = n0 + ty + 16 * j;
-      if (gm >= M || gn >= N || (MODE != 0 && gm < gn)) continue;
-      T *c = C + (long long)gm * cr + (long long)gn * cc;
-      const T v = beta == 0.0 ? Ar<T>::scale(acc[i][j], alpha) : Ar<T>::axpby(alpha, acc[i][j], beta, *c);
-      *c = v;
-      if (MODE == 2 && gm != gn) C[(long long)gn * cr + (long long)gm * cc] = v;
-    }
-}
-
 // ------------------------------------------------------------------------ L D L^T, diagonal block
-constexpr int kNB = 64;  // block width of the factorisation and of the solves
+constexpr int kDT = 256;
 
-// One CTA factors the nb x nb diagonal block in shared memory (column-major, leading dimension
-// nb + 1), right-looking: at step j, l_kj = a_kj / d_j, then a_ik -= a_ij l_kj for i >= k > j.
+// One CTA factors the nb x nb diagonal block, right-looking: at step j, l_kj = a_kj / d_j, then
+// a_ik -= a_ij l_kj for i >= k > j.  The elements stay in the registers of their threads (column-major
+// triangular order, so a thread's elements finish early); the column of the next step is published in
+// shared memory.  Warp 0 alone forms 1 / d_j and the scaled column: a float64 division is some forty
+// dependent instructions, and every further warp that repeats it takes the pipe from the others (the
+// former kernel, all eight warps dividing: 170 us for a complex block of 64; this one 22 us for one of 32).
 template <typename T>
-__global__ void __launch_bounds__(kGT) k_ldl_diag(int nb, T *__restrict__ A, long long lda, int j0, int spd,
-                                                  int *__restrict__ info) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T *s = reinterpret_cast<T *>(smem_raw);
-  const int LS = nb + 1;
-  T *lcol = s + nb * LS;
+__global__ void __launch_bounds__(kDT) k_ldl_diag(int nb, T *__restrict__ A, long long lda, int j0, int spd,
+                                                  int *__restrict__ info, T *__restrict__ dinv) {
+  constexpr int NB = LdlBlock<T>::NB, NE = NB * (NB + 1) / 2, PER = (NE + kDT - 1) / kDT;
+  __shared__ T col[2][NB], lcol[NB];
   const int tid = threadIdx.x;
-  for (int e = tid; e < nb * nb; e += kGT) {
-    const int i = e % nb, j = e / nb;
-    if (i >= j) s[i + j * LS] = A[i + j * lda];
+  T a[PER];
+  int ei[PER], ek[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    int e = tid + kDT * q, k = 0;
+    ei[q] = ek[q] = -1;
+    a[q] = Ar<T>::zero();
+    if (e < NE) {
+      // column k starts at k NB - k (k - 1) / 2
+      k = (int)((2 * NB + 1 - sqrtf((float)((2 * NB + 1) * (2 * NB + 1) - 8 * e))) * 0.5f);
+      while (k > 0 && k * NB - k * (k - 1) / 2 > e) --k;
+      while ((k + 1) * NB - (k + 1) * k / 2 <= e) ++k;
+      const int i = k + (e - (k * NB - k * (k - 1) / 2));
+      if (i < nb && k < nb) {
+        ei[q] = i;
+        ek[q] = k;
+        a[q] = A[i + k * lda];
+        if (k == 0) col[0][i] = a[q];
+      }
+    }
   }
   bool bad = false;
   for (int j = 0; j < nb; ++j) {
-    __syncthreads();
-    const T d = s[j + j * LS];
-    if (tid == 0 && !bad && Ar<T>::bad_pivot(d, spd)) {
-      bad = true;
-      atomicCAS(info, 0, j0 + j + 1);
+    const T *c = col[j & 1];
+    __syncthreads();  // column j is published
+    if (tid < 32) {
+      const T d = c[j], di = Ar<T>::inv(d);
+      if (tid == 0) {
+        if (!bad && Ar<T>::bad_pivot(d, spd)) {
+          bad = true;
+          atomicCAS(info, 0, j0 + j + 1);
+        }
+        dinv[j] = di;
+        A[j + j * lda] = d;
+      }
+      for (int k = j + 1 + tid; k < nb; k += 32) {
+        const T l = Ar<T>::mul(c[k], di);
+        lcol[k] = l;
+        A[k + j * lda] = l;
+      }
     }
-    const T dinv = Ar<T>::inv(d);
-    for (int k = j + 1 + tid; k < nb; k += kGT) lcol[k] = Ar<T>::mul(s[k + j * LS], dinv);
     __syncthreads();
-    const int m = nb - 1 - j;
-    for (int e = tid; e < m * m; e += kGT) {
-      const int i = j + 1 + e % m, k = j + 1 + e / m;
-      if (i >= k) s[i + k * LS] = Ar<T>::fms(s[i + j * LS], lcol[k], s[i + k * LS]);
-    }
-    __syncthreads();
-    for (int k = j + 1 + tid; k < nb; k += kGT) s[k + j * LS] = lcol[k];
-  }
-  __syncthreads();
-  for (int e = tid; e < nb * nb; e += kGT) {
-    const int i = e % nb, j = e / nb;
-    if (i >= j) A[i + j * lda] = s[i + j * LS];
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      if (ek[q] > j) {
+        a[q] = Ar<T>::fms(c[ei[q]], lcol[ek[q]], a[q]);
+        if (ek[q] == j + 1) col[(j + 1) & 1][ei[q]] = a[q];
+      }
   }
 }
 
 // ------------------------------------------------------------- unit-triangular multi-vector solves
-// Vectors v < nv, element j < nb at X[v vs + j es]; the nb x nb block L (element (i, j) at
+// Vectors v < nv, element i < nb at X[v vs + i es]; the nb x nb block L (element (i, j) at
 // L[i + j ldl]) in shared memory:
 //   TRANS = false: L y = x (unit lower; forward), TRANS = true: L^T y = x (backward).
-// PANEL (forward only): the panel of the factorisation, W = y (work, element (v, j) at W[v + j ldw])
-// and x = y / d_j (d_j = the factor's diagonal, L[j + j ldl]).
-// A CTA takes kSV vectors with one thread per (element, vector) and eliminates column by column (at
-// step j, y_j is final and every later element subtracts its multiple): the float64 work of a block
-// is spread over many CTAs and all four schedulers of an SM, where one thread per vector would leave
-// most of the GPU's float64 units idle (a float64 warp instruction occupies a scheduler's unit for
-// many cycles).
-constexpr int kSV = 8;                 // vectors per CTA
-constexpr int kSVT = kSV * 64;         // threads: (element < 64) x (vector < kSV)
-template <typename T, bool TRANS, bool PANEL>
-__global__ void __launch_bounds__(kSVT) k_trsv(int nb, const T *__restrict__ L, long long ldl, int nv, T *__restrict__ X,
-                                               long long vs, long long es, T *__restrict__ W, long long ldw) {
+// PANEL (forward only): the panel of the factorisation, W = y (element (v, j) at W[v + j ldw]) and
+// x = y / d_j.  Vectors nv .. nv + nv2 - 1 are those of a second array (the right-hand sides).
+// A CTA takes SV vectors with one thread per (element, vector), vectors fastest, and eliminates column by
+// column (at step j, y_j is final and every later element subtracts its multiple): a warp holds 32 / SV
+// elements, so warps whose elements are final drop out and the float64 pipe does little more than the
+// triangle's own multiply-adds.
+template <typename T>
+struct Vecs {
+  T *X;
+  long long vs, es;
+};
+template <typename T, int NB, int SV, bool TRANS, bool PANEL>
+__global__ void __launch_bounds__(NB * SV) k_trsv(int nb, const T *__restrict__ L, long long ldl, int nv, Vecs<T> X,
+                                                  int nv2, Vecs<T> X2, T *__restrict__ W, long long ldw,
+                                                  const T *__restrict__ dinv) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T *Ls = reinterpret_cast<T *>(smem_raw);  // nb x nb: Ls[i + j nb] = L(i, j), or L(j, i) for TRANS
-  T *xs = Ls + nb * nb;                     // [vector][element]
-  const int tid = threadIdx.x, i = tid & 63, vl = tid >> 6, v = blockIdx.x * kSV + vl;
-  for (int e = tid; e < nb * nb; e += kSVT) {
-    const int r = e % nb, c = e / nb;
-    Ls[e] = TRANS ? L[c + (long long)r * ldl] : L[r + (long long)c * ldl];
+  T *Ls = reinterpret_cast<T *>(smem_raw);  // Ls[i + j NB] = L(i, j), or L(j, i) for TRANS
+  T *xs = Ls + NB * NB;                     // [element][vector]
+  const int tid = threadIdx.x, vl = tid % SV, i = tid / SV, v = blockIdx.x * SV + vl;
+  for (int e = tid; e < NB * NB; e += NB * SV) {
+    const int r = e % NB, c = e / NB;
+    if (r < nb && c < nb && (TRANS ? r < c : r > c)) Ls[e] = TRANS ? L[c + (long long)r * ldl] : L[r + (long long)c * ldl];
   }
-  const bool act = v < nv && i < nb;
-  T *x = X + (long long)(v < nv ? v : 0) * vs;
-  T xi = act ? x[(long long)i * es] : Ar<T>::zero();
-  xs[vl * 64 + i] = xi;
-  // step j reads element j (final after the previous step's barrier) and writes elements != j only
+  const bool act = v < nv + nv2 && i < nb;
+  T *x = nullptr;
+  if (act) x = v < nv ? X.X + v * X.vs + i * X.es : X2.X + (v - nv) * X2.vs + i * X2.es;
+  T xi = act ? *x : Ar<T>::zero();
+  if (i == (TRANS ? nb - 1 : 0)) xs[tid] = xi;
+  // step j reads element j (final and published after step j - 1) and changes later elements only
   if (!TRANS) {
     for (int j = 0; j + 1 < nb; ++j) {
       __syncthreads();
-      const T yj = xs[vl * 64 + j];
       if (i > j && i < nb) {
-        xi = Ar<T>::fms(Ls[i + j * nb], yj, xi);
-        xs[vl * 64 + i] = xi;
+        xi = Ar<T>::fms(Ls[i + j * NB], xs[j * SV + vl], xi);
+        if (i == j + 1) xs[tid] = xi;
       }
     }
   } else {
     for (int j = nb - 1; j > 0; --j) {
       __syncthreads();
-      const T yj = xs[vl * 64 + j];
       if (i < j) {
-        xi = Ar<T>::fms(Ls[i + j * nb], yj, xi);
-        xs[vl * 64 + i] = xi;
+        xi = Ar<T>::fms(Ls[i + j * NB], xs[j * SV + vl], xi);
+        if (i == j - 1) xs[tid] = xi;
       }
     }
   }
   if (!act) return;
   if (PANEL) {
     W[v + (long long)i * ldw] = xi;
-    x[(long long)i * es] = Ar<T>::mul(xi, Ar<T>::inv(Ls[i + i * nb]));
+    *x = Ar<T>::mul(xi, dinv[i]);
   } else {
-    x[(long long)i * es] = xi;
-  }
-}
-
-// B[i, c] /= d_i (the factor's diagonal)
-template <typename T>
-__global__ void k_dscale(int n, int nrhs, const T *__restrict__ A, long long lda, T *__restrict__ B, long long ldb) {
-  const long long tot = (long long)n * nrhs;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e % n);
-    const long long c = e / n;
-    B[i + c * ldb] = Ar<T>::mul(B[i + c * ldb], Ar<T>::inv(A[i + (long long)i * lda]));
+    *x = xi;
   }
 }
 
@@ -267,97 +193,87 @@ int set_smem(F *f, size_t bytes) {
     if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA; \
   } while (0)
 
+// Operand views and C strides of real and complex column-major blocks.
+inline SgView left(const double *p, long long sr, long long sk) { return sg_real(p, sr, sk); }
+inline SgView left(const double2 *p, long long sr, long long sk) { return sg_cplx_left(p, sr, sk); }
+inline SgView right(const double *p, long long sr, long long sk) { return sg_real(p, sr, sk); }
+inline SgView right(const double2 *p, long long sr, long long sk) { return sg_cplx_right(p, sr, sk); }
+// C (M x N, column-major, leading dimension ldc) -= A B with contraction K (all in elements of T)
+template <typename T>
+SgProduct update(int mode, int M, int N, int K, SgView A, SgView B, T *C, long long ldc) {
+  constexpr int c = sizeof(T) == 16 ? 1 : 0, u = 1 + c;  // reals per element
+  SgProduct p{};
+  p.M = u * M;
+  p.N = N;
+  p.K = u * K;
+  p.mode = mode;
+  p.cs = c;
+  p.neg = 1;
+  p.beta = 1;
+  p.A = A;
+  p.B = B;
+  p.C = reinterpret_cast<double *>(C);
+  p.crh = 2;
+  p.crl = 1;
+  p.cch = 2 * u * ldc;
+  p.ccl = u * ldc;
+  return p;
+}
+
+template <typename T, int SV, bool TRANS, bool PANEL>
+int trsv(int nb, const T *L, long long ldl, int nv, Vecs<T> X, int nv2, Vecs<T> X2, T *W, long long ldw, const T *dinv,
+         cudaStream_t st) {
+  constexpr int NB = LdlBlock<T>::NB;
+  const size_t smem = (size_t)(NB * NB + NB * SV) * sizeof(T);
+  if (set_smem(k_trsv<T, NB, SV, TRANS, PANEL>, smem) != GINT_OK) return GINT_ECUDA;
+  k_trsv<T, NB, SV, TRANS, PANEL><<<(unsigned)((nv + nv2 + SV - 1) / SV), NB * SV, smem, st>>>(nb, L, ldl, nv, X, nv2, X2,
+                                                                                               W, ldw, dinv);
+  LA_CHECK();
+  return GINT_OK;
+}
+
 }  // namespace
 
 template <typename T>
-int gemm(int mode, int M, int N, int K, double alpha, View<T> A, View<T> B, double beta, T *C, long long cr,
-         long long cc, cudaStream_t st) {
-  if (M <= 0 || N <= 0) return GINT_OK;
-  const dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + kBM - 1) / kBM));
-  if (grid.y > 65535u) return GINT_EINVAL;
-  if (mode == 0)
-    k_gemm<T, 0><<<grid, kGT, 0, st>>>(M, N, K, alpha, A, B, beta, C, cr, cc);
-  else if (mode == 1)
-    k_gemm<T, 1><<<grid, kGT, 0, st>>>(M, N, K, alpha, A, B, beta, C, cr, cc);
-  else
-    k_gemm<T, 2><<<grid, kGT, 0, st>>>(M, N, K, alpha, A, B, beta, C, cr, cc);
-  LA_CHECK();
-  return GINT_OK;
-}
-
-template <typename T>
-int ldl_factor(int n, T *A, long long lda, T *work, int *info, bool spd, cudaStream_t st) {
-  const size_t diag_smem = (size_t)(kNB * (kNB + 1) + kNB) * sizeof(T);
-  const size_t trsv_smem = (size_t)(kNB * kNB + 64 * kSV) * sizeof(T);
+int ldl_factor_solve(int n, T *A, long long lda, int nrhs, T *B, long long ldb, T *work, int *info, bool spd,
+                     const SgWork &ws, cudaStream_t st) {
+  constexpr int NB = LdlBlock<T>::NB;
   int rc;
-  if ((rc = set_smem(k_ldl_diag<T>, diag_smem)) || (rc = set_smem(k_trsv<T, false, true>, trsv_smem))) return rc;
-  for (int j0 = 0; j0 < n; j0 += kNB) {
-    const int nb = std::min(kNB, n - j0);
-    T *A11 = A + j0 + (long long)j0 * lda;
-    k_ldl_diag<T><<<1, kGT, (size_t)(nb * (nb + 1) + nb) * sizeof(T), st>>>(nb, A11, lda, j0, spd ? 1 : 0, info);
+  const long long ldw = (long long)n + nrhs;
+  T *W = work, *dinv = work + ldw * NB;
+  for (int j0 = 0; j0 < n; j0 += NB) {
+    const int nb = std::min(NB, n - j0), m = n - j0 - nb;
+    T *A11 = A + j0 + (long long)j0 * lda, *A21 = A11 + nb, *B1 = B + j0;
+    k_ldl_diag<T><<<1, kDT, 0, st>>>(nb, A11, lda, j0, spd ? 1 : 0, info, dinv + j0);
     LA_CHECK();
-    const int m = n - j0 - nb;
-    if (m == 0) break;
-    T *A21 = A11 + nb;
-    // panel: W21 = A21 L11^-T, L21 = W21 D1^-1 (rows of A21 are the vectors)
-    k_trsv<T, false, true><<<(unsigned)((m + kSV - 1) / kSV), kSVT, (size_t)(nb * nb + 64 * kSV) * sizeof(T), st>>>(
-        nb, A11, lda, m, A21, 1, lda, work, n);
-    LA_CHECK();
-    // trailing update of the lower triangle: A22 -= W21 L21^T
-    rc = gemm<T>(1, m, m, nb, -1.0, view<T>(work, 1, n), view<T>(A21, 1, lda), 1.0, A21 + (long long)nb * lda, 1, lda,
-                 st);
-    if (rc) return rc;
-  }
-  return GINT_OK;
-}
-
-template <typename T>
-int ldl_solve(int n, int nrhs, const T *A, long long lda, T *B, long long ldb, cudaStream_t st) {
-  if (n <= 0 || nrhs <= 0) return GINT_OK;
-  const size_t trsv_smem = (size_t)(kNB * kNB + 64 * kSV) * sizeof(T);
-  int rc;
-  if ((rc = set_smem(k_trsv<T, false, false>, trsv_smem)) || (rc = set_smem(k_trsv<T, true, false>, trsv_smem)))
-    return rc;
-  const unsigned nvb = (unsigned)((nrhs + kSV - 1) / kSV);
-  // L Y = B, block by block: the diagonal block's substitution, then the rows below
-  for (int k0 = 0; k0 < n; k0 += kNB) {
-    const int nb = std::min(kNB, n - k0);
-    const T *Lkk = A + k0 + (long long)k0 * lda;
-    k_trsv<T, false, false><<<nvb, kSVT, (size_t)(nb * nb + 64 * kSV) * sizeof(T), st>>>(nb, Lkk, lda, nrhs, B + k0,
-                                                                                        ldb, 1, nullptr, 0);
-    LA_CHECK();
-    const int m = n - k0 - nb;
-    if (m > 0 &&
-        (rc = gemm<T>(0, m, nrhs, nb, -1.0, view<T>(Lkk + nb, 1, lda), view<T>(B + k0, ldb, 1), 1.0, B + k0 + nb, 1, ldb,
-                      st)))
+    // panel rows: W = A21 L11^-T, L21 = W D1^-1, and the same for the right-hand sides
+    if (m + nrhs > 0 && (rc = trsv<T, 8, false, true>(nb, A11, lda, m, Vecs<T>{A21, 1, lda}, nrhs, Vecs<T>{B1, ldb, 1}, W,
+                                                      ldw, dinv + j0, st)))
       return rc;
+    if (m == 0) continue;
+    // A22 -= W21 L21^T (lower triangle), B2 -= L21 W_B^T
+    const SgProduct pr[2] = {
+        update<T>(1, m, m, nb, left(W, 1, ldw), right(A21, 1, lda), A21 + (long long)nb * lda, lda),
+        update<T>(0, m, nrhs, nb, left(A21, 1, lda), right(W + m, 1, ldw), B1 + nb, ldb)};
+    if ((rc = sg_gemm(pr, nrhs > 0 ? 2 : 1, ws, st))) return rc;
   }
-  // Y <- D^{-1} Y
-  k_dscale<T><<<(unsigned)std::min<long long>(((long long)n * nrhs + 255) / 256, 4096), 256, 0, st>>>(n, nrhs, A, lda,
-                                                                                                     B, ldb);
-  LA_CHECK();
   // L^T X = Y, last block first, then the rows above
-  for (int k0 = ((n - 1) / kNB) * kNB; k0 >= 0; k0 -= kNB) {
-    const int nb = std::min(kNB, n - k0);
+  for (int k0 = ((n - 1) / NB) * NB; k0 >= 0 && nrhs > 0; k0 -= NB) {
+    const int nb = std::min(NB, n - k0);
     const T *Lkk = A + k0 + (long long)k0 * lda;
-    k_trsv<T, true, false><<<nvb, kSVT, (size_t)(nb * nb + 64 * kSV) * sizeof(T), st>>>(nb, Lkk, lda, nrhs, B + k0, ldb,
-                                                                                       1, nullptr, 0);
-    LA_CHECK();
-    // rows i < k0: B_i -= sum_k L[k0 + k, i] X[k0 + k]
-    if (k0 > 0 && (rc = gemm<T>(0, k0, nrhs, nb, -1.0, view<T>(A + k0, lda, 1), view<T>(B + k0, ldb, 1), 1.0, B, 1,
-                                ldb, st)))
+    if ((rc = trsv<T, 8, true, false>(nb, Lkk, lda, nrhs, Vecs<T>{B + k0, ldb, 1}, 0, Vecs<T>{}, nullptr, 0, nullptr, st)))
       return rc;
+    if (k0 == 0) continue;
+    // rows i < k0: B_i -= sum_k L[k0 + k, i] X[k0 + k]
+    const SgProduct pr = update<T>(0, k0, nrhs, nb, left(A + k0, lda, 1), right(B + k0, ldb, 1), B, ldb);
+    if ((rc = sg_gemm(&pr, 1, ws, st))) return rc;
   }
   return GINT_OK;
 }
 
-template int gemm<double>(int, int, int, int, double, View<double>, View<double>, double, double *, long long,
-                          long long, cudaStream_t);
-template int gemm<double2>(int, int, int, int, double, View<double2>, View<double2>, double, double2 *, long long,
-                           long long, cudaStream_t);
-template int ldl_factor<double>(int, double *, long long, double *, int *, bool, cudaStream_t);
-template int ldl_factor<double2>(int, double2 *, long long, double2 *, int *, bool, cudaStream_t);
-template int ldl_solve<double>(int, int, const double *, long long, double *, long long, cudaStream_t);
-template int ldl_solve<double2>(int, int, const double2 *, long long, double2 *, long long, cudaStream_t);
+template int ldl_factor_solve<double>(int, double *, long long, int, double *, long long, double *, int *, bool,
+                                      const SgWork &, cudaStream_t);
+template int ldl_factor_solve<double2>(int, double2 *, long long, int, double2 *, long long, double2 *, int *, bool,
+                                       const SgWork &, cudaStream_t);
 
 }  // namespace gla

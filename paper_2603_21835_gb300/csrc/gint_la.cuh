@@ -1,43 +1,35 @@
-// gint_la.cuh -- float64 dense linear algebra of the propagation steps (gint_la.cu): a tiled GEMM
-// on strided operand views, and the blocked L D L^T factorisation (no pivoting) with its solve, for
-// real symmetric and complex symmetric (A^T = A, no conjugation) matrices.
+// gint_la.cuh -- float64 dense linear algebra of the propagation steps (gint_la.cu): the blocked
+// L D L^T factorisation (no pivoting) with its solve, for real symmetric and complex symmetric
+// (A^T = A, no conjugation) matrices.  Its products are those of gint_sg.cuh.
 #pragma once
 #include <cuda_runtime.h>
 
+#include "gint_sg.cuh"
+
 namespace gla {
 
-// Operand view of a GEMM: element (r, k) -- r the output row (A) or column (B) index, k the
-// contraction index -- is p[r sr + (k >> 1) skh + (k & 1) skl], times ks[k >> 1] when ks is not
-// null.  An ordinary strided matrix has skh = 2 sk, skl = sk; the real view of interleaved complex
-// data (k = 2 s + real / imaginary part) has skh = the complex stride in doubles, skl = 1.
+// Block width of the factorisation: a 64-wide real contraction either way.
 template <typename T>
-struct View {
-  const T *p;
-  long long sr, skh, skl;
-  const double *ks;
+struct LdlBlock {
+  static constexpr int NB = sizeof(T) == 16 ? 32 : 64;
 };
+// Elements of T that ldl_solve_factor needs as workspace for n x n with nrhs right-hand sides.
 template <typename T>
-inline View<T> view(const T *p, long long sr, long long sk, const double *ks = nullptr) {
-  return View<T>{p, sr, 2 * sk, sk, ks};
+inline size_t ldl_work(long long n, long long nrhs) {
+  return (size_t)(n + nrhs) * LdlBlock<T>::NB + (size_t)n;
+}
+// Operand rows of its largest launch of products (for sg_bytes, contraction 64).
+template <typename T>
+inline long long ldl_rows(long long n, long long nrhs) {
+  return (sizeof(T) == 16 ? 5 : 3) * n + nrhs + 1024;
 }
 
-// C (element (i, j) at C[i cr + j cc]) = alpha A B + beta C, M x N, contraction K; T = double or
-// double2 (complex).  mode 0: every element; mode 1: lower triangle only (i >= j; tiles above the
-// diagonal are skipped); mode 2: the lower triangle, each value also written to (j, i) (C symmetric
-// bit for bit).  beta = 0 does not read C.
+// Solves A X = B in place (B: nrhs columns of n, leading dimension ldb) by A = L D L^T of the n x n matrix
+// A (column-major, leading dimension lda; only the lower triangle is read and it is overwritten).
+// *info (device) = first j + 1 whose pivot d_j is zero or not finite (spd: not positive), else unchanged
+// (the caller zeroes it).
 template <typename T>
-int gemm(int mode, int M, int N, int K, double alpha, View<T> A, View<T> B, double beta, T *C, long long cr,
-         long long cc, cudaStream_t st);
-
-// In-place A = L D L^T of the n x n matrix A (column-major, leading dimension lda; only the lower
-// triangle is read): L unit lower (strictly lower part of A), D on the diagonal.  work: n x 64
-// elements.  *info (device) = first j + 1 whose pivot d_j is zero or not finite (spd: not positive),
-// else unchanged (the caller zeroes it).
-template <typename T>
-int ldl_factor(int n, T *A, long long lda, T *work, int *info, bool spd, cudaStream_t st);
-
-// B <- (L D L^T)^{-1} B for the factor of ldl_factor; B n x nrhs column-major (leading dimension ldb).
-template <typename T>
-int ldl_solve(int n, int nrhs, const T *A, long long lda, T *B, long long ldb, cudaStream_t st);
+int ldl_factor_solve(int n, T *A, long long lda, int nrhs, T *B, long long ldb, T *work, int *info, bool spd,
+                     const SgWork &ws, cudaStream_t st);
 
 }  // namespace gla

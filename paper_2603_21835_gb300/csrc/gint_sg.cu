@@ -1,0 +1,608 @@
+// gint_sg.cu -- float64 matrix products on the tcgen05 tensor cores (gint_sg.cuh).
+//
+// The GB300 multiplies float64 on its CUDA cores at 2 fused multiply-adds per clock per SM (1.25 TFLOP/s)
+// and float16 on its tensor cores some 1500 times faster, so a float64 product is cheaper as many exact
+// float16 ones: the error-free splitting of Ozaki, Ogita, Oishi and Rump ("Error-free transformations of
+// matrix multiplication by using fast routines of matrix multiplication", 2012), here with integer digits.
+//
+//   x_rk = q_rk 2^(e_r - 62), q an integer of at most 62 bits (e_r: the exponent of row r's largest
+//   magnitude, so the rounding of q is 2^-63 of that maximum and values within 2^9 of it are exact);
+//   q = sum_s d_s 256^(7 - s), s = 0..7, d_s in [-128, 127] (balanced digits: the bytes of q + 0x80..80
+//   less 128), exact in float16;
+//   sum_k x_ik y_jk = 2^(..) sum_{l = s + t} 256^(14 - l) sum_k d_s d_t, levels l = 0..7 kept (the
+//   dropped ones are below 2^-60 of the largest products: float64 rounding of one product is 2^-53).
+//
+// The MMAs of level l add at most 8 x 128 products of magnitude 2^14 per accumulator in a range of 128 k:
+// at most 2^24, so every float32 partial sum is an exact integer whatever the tensor core's rounding.
+// After each range the eight levels are drained into two 64-bit integers per element (levels 0-3 and
+// 4-7), and the element is converted to float64 once at the end of the contraction (one rounding; the
+// CUDA cores' float64 chain has one per multiply-add).
+//
+// k_sg_max / k_sg_pack: row exponents and digit blocks.  Block (row tile of TR = 128 left / 64 right rows,
+//   chunk of 16 k): [digit 8][row group TR / 8][k group 2][8 rows][8 k] float16, K-major core matrices
+//   (LBO 128, SBO 256), so a right block is one operand of 512 rows (digit, column).
+// k_sg_mma: persistent, one CTA of 18 warps per SM.  Warp 17 streams the two blocks of a chunk (48 KB) by
+//   bulk copies into a 4-stage ring; warp 16 issues 12 MMAs per chunk, digit s of the left times a run of
+//   digits of the right as ONE operand of up to 4 x 64 rows, which land in the accumulator columns
+//   64 (s + t) .. of level s + t: 512 columns of tensor memory hold all eight levels of a 128 x 64 tile.
+//   Warps 0-15 drain and store a tile while the next one's MMAs run.
+// Bound: 36 digit products, 1152 tensor cycles a chunk (1210 measured).
+#include <cuda_fp16.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "gint.h"
+#include "gint_ptx.cuh"
+#include "gint_sg.cuh"
+
+namespace gla {
+namespace {
+using namespace gptx;
+
+constexpr int kDig = 8;                  // digits of an operand, and levels kept
+constexpr int kTM = 128, kTN = 64;       // output tile
+constexpr int kCK = 16;                  // k of a chunk (one MMA K step)
+constexpr int kRangeChunks = 8;          // chunks per exact accumulation range (128 k)
+constexpr int kSgK = 1024;               // longest contraction packed at once
+constexpr uint32_t kABytes = kDig * kTM * kCK * 2, kBBytes = kDig * kTN * kCK * 2;
+constexpr uint32_t kStage = kABytes + kBBytes;
+constexpr int kStages = 4;
+constexpr uint32_t kSgSmem = kStages * kStage;
+constexpr int kDrainWarps = 16, kMmaWarp = 16, kLoadWarp = 17, kSgThreads = 32 * (kDrainWarps + 2);
+constexpr long long kWaitNs = 2000000000LL;  // bounded waits: 2 s
+constexpr unsigned kErrTimeout = 1u, kErrInflight = 2u;
+constexpr int kNonFinite = 2047;         // row exponent field of a row with an infinity or a NaN
+static_assert(kDig * kTN == 512, "the levels fill the tensor memory");
+
+__device__ __forceinline__ double sg_at(const SgView &v, int r, int k) {
+  if (v.rot) {
+    const double x = v.p[(long long)(r >> 1) * v.rh + (long long)(k >> 1) * v.kh + ((r ^ k) & 1)];
+    return (!(r & 1) && (k & 1)) ? -x : x;
+  }
+  const double x = v.p[(long long)(r >> 1) * v.rh + (long long)(r & 1) * v.rl + (long long)(k >> 1) * v.kh +
+                       (long long)(k & 1) * v.kl];
+  return v.ks ? x * v.ks[k >> 1] : x;
+}
+
+// Exponent field of |x|, at least 1 (denormals share the exponent of the smallest normal numbers).
+__device__ __forceinline__ int exp_field(double x) {
+  return max(1, (int)((__double_as_longlong(x) >> 52) & 0x7ff));
+}
+
+// ---------------------------------------------------------------------------------------- packing
+constexpr int kPR = 32, kPK = 64, kPT = 256;  // rows and k of a packing CTA, its threads
+struct SgOperand {
+  SgView v;
+  int R, K, nq, tr;  // rows, contraction, chunks, rows of a tile (128 or 64)
+  int rfast;         // consecutive rows are closer in memory than consecutive k
+  unsigned char *dst;
+  int *e;            // exponent field of each row's largest magnitude
+};
+struct SgPack {
+  SgOperand op[4];
+  int first[5];  // first row block of each operand; first[n..4] = total
+};
+
+__device__ __forceinline__ void sg_load_tile(const SgOperand &o, int r0, int k0, double (*t)[kPK + 1]) {
+#pragma unroll
+  for (int q = 0; q < kPR * kPK / kPT; ++q) {
+    const int e = threadIdx.x + kPT * q;
+    const int r = o.rfast ? e % kPR : e / kPK, k = o.rfast ? e / kPR : e % kPK;
+    t[r][k] = (r0 + r < o.R && k0 + k < o.K) ? sg_at(o.v, r0 + r, k0 + k) : 0.0;
+  }
+}
+// The eight threads of a row: largest exponent field of its kPK elements (in all of them).
+__device__ __forceinline__ int sg_row_exp(const double (*t)[kPK + 1]) {
+  const int r = threadIdx.x >> 3, g = threadIdx.x & 7;
+  int m = 1;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) m = max(m, exp_field(t[r][g + 8 * j]));
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  return m;
+}
+__device__ __forceinline__ const SgOperand &sg_operand(const SgPack &P, int &rb) {
+  int i = 0;
+  while (i < 3 && (int)blockIdx.x >= P.first[i + 1]) ++i;
+  rb = (int)blockIdx.x - P.first[i];
+  return P.op[i];
+}
+
+// Row exponents of long contractions (e zeroed before): blockIdx.y = range of 64 k.
+__global__ void __launch_bounds__(kPT) k_sg_max(const __grid_constant__ SgPack P) {
+  __shared__ double t[kPR][kPK + 1];
+  int rb;
+  const SgOperand &o = sg_operand(P, rb);
+  const int r0 = rb * kPR;
+  sg_load_tile(o, r0, blockIdx.y * kPK, t);
+  __syncthreads();
+  const int m = sg_row_exp(t), r = r0 + (threadIdx.x >> 3);
+  if ((threadIdx.x & 7) == 0 && r < o.R) atomicMax(o.e + r, m);
+}
+
+// Digits: one thread per row and 8 k.  ONE: the whole contraction is one range (K <= 64), so the exponent
+// is found here; otherwise k_sg_max has left it in e.
+template <bool ONE>
+__global__ void __launch_bounds__(kPT) k_sg_pack(const __grid_constant__ SgPack P) {
+  __shared__ double t[kPR][kPK + 1];
+  int rb;
+  const SgOperand &o = sg_operand(P, rb);
+  const int r0 = rb * kPR, kb = ONE ? 0 : (int)blockIdx.y * kPK;
+  sg_load_tile(o, r0, kb, t);
+  __syncthreads();
+  const int rl = threadIdx.x >> 3, g = threadIdx.x & 7, r = r0 + rl;
+  const int em = ONE ? sg_row_exp(t) : (r < o.R ? o.e[r] : 1);
+  const int chunk = (kb >> 4) + (g >> 1);
+  if (r >= o.R || chunk >= o.nq) return;
+  if (ONE && g == 0) o.e[r] = em;
+  uint32_t lo[8], hi[8];  // the bytes of q + 0x80..80
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const long long b = __double_as_longlong(t[rl][8 * g + j]);
+    const int ex = (int)((b >> 52) & 0x7ff);
+    unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
+    if (ex) m |= 0x10000000000000ull;
+    const int s = max(ex, 1) - em + 9;  // q = m 2^s, rounded
+    unsigned long long q;
+    if (s >= 0)
+      q = m << s;
+    else
+      q = s < -54 ? 0ull : (m + (1ull << (-s - 1))) >> -s;
+    if (em == kNonFinite) q = 0ull;  // such rows are recomputed element by element
+    if (b < 0) q = 0ull - q;
+    q += 0x8080808080808080ull;
+    lo[j] = (uint32_t)q;
+    hi[j] = (uint32_t)(q >> 32);
+  }
+  const size_t blk = (size_t)kDig * o.tr * kCK * 2;
+  unsigned char *d = o.dst + ((size_t)(r / o.tr) * o.nq + chunk) * blk + (size_t)((r % o.tr) >> 3) * 256 + (g & 1) * 128 +
+                     (r & 7) * 16;
+  const __half2 off = __floats2half2_rn(1152.f, 1152.f);  // float16 bits 0x6400 | b are 1024 + b
+#pragma unroll
+  for (int s = 0; s < kDig; ++s) {  // digit s: byte 7 - s
+    uint32_t w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t a = s < 4 ? hi[2 * j] : lo[2 * j], c = s < 4 ? hi[2 * j + 1] : lo[2 * j + 1];
+      const uint32_t sel = 3 - (s & 3);
+      const uint32_t v = (__byte_perm(a, c, sel | ((sel + 4) << 8)) & 0x00ff00ffu) | 0x64006400u;
+      const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), off);
+      w[j] = *reinterpret_cast<const uint32_t *>(&h);
+    }
+    *reinterpret_cast<uint4 *>(d + (size_t)s * o.tr * kCK * 2) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// --------------------------------------------------------------------------------------- products
+struct SgProb {
+  const unsigned char *PA, *PB;
+  const int *eA, *eB;
+  int nq, ntn, ntiles;
+  SgProduct p;
+};
+struct SgArgs {
+  SgProb pr[2];
+  int tiles;  // of all products
+  unsigned *status;
+};
+// Tile u of a product: mode 0 row-major; otherwise the lower triangle, row tile tm having
+// mul (tm + 1) column tiles (mul = 1 for paired rows, 2 otherwise), cut off at the last one.
+__device__ __forceinline__ void sg_tile(const SgProb &P, int u, int &tm, int &tn) {
+  if (P.p.mode == 0) {
+    tm = u / P.ntn;
+    tn = u - tm * P.ntn;
+    return;
+  }
+  const int mul = P.p.cs ? 1 : 2;
+  tm = (int)((sqrtf(1.f + 8.f * (float)u / (float)mul) - 1.f) * 0.5f);
+  while (mul * (long long)tm * (tm + 1) / 2 > u) --tm;
+  while (mul * (long long)(tm + 1) * (tm + 2) / 2 <= u) ++tm;
+  tn = u - (int)(mul * (long long)tm * (tm + 1) / 2);
+}
+
+// A 96-bit two's complement integer, least significant word first.
+struct Fx {
+  uint32_t w0, w1, w2;
+};
+// x += v 2^32 and x += v
+__device__ __forceinline__ void fx_add_hi(Fx &x, long long v) {
+  asm("add.cc.u32 %0, %0, %2;\n addc.u32 %1, %1, %3;"
+      : "+r"(x.w1), "+r"(x.w2)
+      : "r"((uint32_t)v), "r"((uint32_t)((unsigned long long)v >> 32)));
+}
+__device__ __forceinline__ void fx_add_lo(Fx &x, long long v) {
+  const uint32_t h = (uint32_t)((unsigned long long)v >> 32);
+  asm("add.cc.u32 %0, %0, %3;\n addc.cc.u32 %1, %1, %4;\n addc.u32 %2, %2, %5;"
+      : "+r"(x.w0), "+r"(x.w1), "+r"(x.w2)
+      : "r"((uint32_t)v), "r"(h), "r"((uint32_t)((int)h >> 31)));
+}
+// Four adjacent levels of one element: v0 2^24 + v1 2^16 + v2 2^8 + v3.  SMALL: all below 2^22 in magnitude,
+// so that adding 1.5 2^23 leaves the integer in the low bits (the float-to-integer conversion runs on a pipe
+// a quarter as wide) and two levels still fit 32 bits.
+template <bool SMALL>
+__device__ __forceinline__ long long fx_levels(float v0, float v1, float v2, float v3) {
+  if (SMALL) {
+    constexpr uint32_t M = 0x4B400000u, B = M * 257u;
+    const uint32_t m0 = __float_as_uint(v0 + 12582912.f), m1 = __float_as_uint(v1 + 12582912.f);
+    const uint32_t m2 = __float_as_uint(v2 + 12582912.f), m3 = __float_as_uint(v3 + 12582912.f);
+    const int p = (int)((m0 << 8) + m1 - B), q = (int)((m2 << 8) + m3 - B);
+    return (long long)p * 65536 + q;
+  }
+  return (((long long)__float2int_rn(v0) * 256 + __float2int_rn(v1)) * 256 + __float2int_rn(v2)) * 256 + __float2int_rn(v3);
+}
+
+// x 2^E rounded to float64: the magnitude normalised by word moves and one funnel shift, some thirty 32-bit
+// instructions (converting 64-bit integers would take three float64 ones, 48 clocks of the SM's pipe per warp).
+__device__ __forceinline__ double fx_to_double(Fx x, int E) {
+  const uint32_t sg = (uint32_t)((int)x.w2 >> 31);
+  asm("add.cc.u32 %0, %0, %3;\n addc.cc.u32 %1, %1, %3;\n addc.u32 %2, %2, %3;"
+      : "+r"(x.w0), "+r"(x.w1), "+r"(x.w2)
+      : "r"(sg));  // -x = ~(x - 1)
+  uint32_t w0 = x.w0 ^ sg, w1 = x.w1 ^ sg, w2 = x.w2 ^ sg;
+  int k = E + 43;
+  if (w2 == 0u) {
+    w2 = w1;
+    w1 = w0;
+    w0 = 0u;
+    k -= 32;
+  }
+  if (w2 == 0u) {
+    if (w1 == 0u) return 0.0;
+    w2 = w1;
+    w1 = 0u;
+    k -= 32;
+  }
+  const int n = __clz(w2);
+  const uint32_t hi32 = __funnelshift_l(w1, w2, n), lo32 = __funnelshift_l(w0, w1, n);
+  k -= n;  // value = (hi32 : lo32) / 2^11 * 2^k, the leading bit set
+  const uint32_t f1 = hi32 >> 11, f0 = __funnelshift_r(lo32, hi32, 11), rnd = (lo32 >> 10) & 1u;
+  if ((unsigned)(k + 1073) < 2043u) {
+    const unsigned long long m = (((unsigned long long)(f1 + ((uint32_t)(k + 1074) << 20) + (sg & 0x80000000u)) << 32) | f0) + rnd;
+    return __longlong_as_double((long long)m);
+  }
+  // denormal, zero or overflow: scaled in two exact steps and one rounding
+  const int kc = min(max(k, -1140), 1030), ka = kc >> 1, kb = kc - ka;
+  const double v = (double)(long long)((((unsigned long long)f1 << 32) | f0) + rnd) * __hiloint2double((ka + 1023) << 20, 0) *
+                   __hiloint2double((kb + 1023) << 20, 0);
+  return sg ? -v : v;
+}
+
+// Element (i, j) of a row or column that holds an infinity or a NaN: the plain float64 sum.
+__device__ __noinline__ void sg_plain(const SgProduct &p, int i, int j) {
+  double a = 0.0;
+  for (int k = 0; k < p.K; ++k) a = fma(sg_at(p.A, i, k), sg_at(p.B, j, k), a);
+  if (p.neg) a = -a;
+  double *const c = p.C + (long long)(i >> 1) * p.crh + (long long)(i & 1) * p.crl + (long long)(j >> 1) * p.cch +
+                    (long long)(j & 1) * p.ccl;
+  if (p.beta) a += *c;
+  *c = a;
+  if (p.mode == 2 && i != j)
+    p.C[(long long)(j >> 1) * p.crh + (long long)(j & 1) * p.crl + (long long)(i >> 1) * p.cch + (long long)(i & 1) * p.ccl] = a;
+}
+
+// Four loads of 4 columns, `step` columns apart, under one wait.
+__device__ __forceinline__ void tmem_ld4x4(uint32_t taddr, uint32_t step, float (*v)[4]) {
+  uint32_t r[4][4];
+#pragma unroll
+  for (int l = 0; l < 4; ++l)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3])
+                 : "r"(taddr + l * step)
+                 : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int l = 0; l < 4; ++l)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[l][j] = __uint_as_float(r[l][j]);
+}
+
+// Range r of a tile is complete for levels 0-3 (accfull[0]) and 4-7 (accfull[1]); the drain warps give the
+// two halves back (accfree) as they finish with each, so that half of a drain overlaps the MMAs around it.
+struct SgShared {
+  uint64_t full[kStages], empty[kStages], accfull[2], accfree[2];
+  uint32_t tmem;
+};
+
+__global__ void __launch_bounds__(kSgThreads, 1) k_sg_mma(const __grid_constant__ SgArgs P) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ SgShared sh;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&sh.full[s], 1);
+      mbar_init(&sh.empty[s], 1);
+    }
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(&sh.accfull[h], 1);
+      mbar_init(&sh.accfree[h], kDrainWarps);
+    }
+    fence_mbar_init();
+  }
+  if (warp == kMmaWarp) {
+    tmem_alloc(&sh.tmem, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = sh.tmem;
+  unsigned *status = P.status;
+  const int n0 = P.pr[0].ntiles;
+
+  if (warp == kLoadWarp) {
+    // the copies run kStages chunks ahead of the MMAs, across tile boundaries
+    int gl = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < P.tiles && ok; t += gridDim.x) {
+      const SgProb &pr = P.pr[t < n0 ? 0 : 1];
+      int tm, tn;
+      sg_tile(pr, t < n0 ? t : t - n0, tm, tn);
+      const unsigned char *a = pr.PA + (size_t)tm * pr.nq * kABytes, *b = pr.PB + (size_t)tn * pr.nq * kBBytes;
+      const int nq = pr.nq;
+      for (int c = 0; c < nq && ok; ++c, ++gl, a += kABytes, b += kBBytes) {
+        const int s = gl % kStages;
+        if (gl >= kStages)
+          ok = __all_sync(0xffffffffu,
+                          mbar_wait(&sh.empty[s], (uint32_t)(gl / kStages - 1) & 1u, status, kErrTimeout, kWaitNs));
+        if (!ok) break;
+        if (lane == 0) {
+          mbar_arrive_tx(&sh.full[s], kStage);
+          bulk_g2s(smem + s * kStage, a, kABytes, &sh.full[s]);
+          bulk_g2s(smem + s * kStage + kABytes, b, kBBytes, &sh.full[s]);
+        }
+        __syncwarp();
+      }
+    }
+    // no copy may still be landing when the CTA exits
+    for (int c = max(0, gl - kStages); c < gl; ++c)
+      mbar_wait(&sh.full[c % kStages], (uint32_t)(c / kStages) & 1u, status, kErrTimeout, kWaitNs);
+  } else if (warp == kMmaWarp) {
+    // a tcgen05.mma blocks its issuer while the few places of the tensor pipe's queue are taken, so this
+    // warp does nothing else (with the copies issued from it too, a chunk took 2320 clocks instead of 1210)
+    const uint32_t sbase = smem_u32(smem);
+    int gc = 0, gb = 0;  // chunks issued, ranges begun
+    bool ok = true;
+    for (int t = blockIdx.x; t < P.tiles && ok; t += gridDim.x) {
+      const int nq = P.pr[t < n0 ? 0 : 1].nq;
+      for (int c = 0; c < nq; ++c, ++gc) {
+        const int s = gc % kStages, cr = c % kRangeChunks;
+        const bool first = cr == 0, last = cr == kRangeChunks - 1 || c == nq - 1;
+        if (first) ++gb;
+        const uint32_t fpar = (uint32_t)(gb - 2) & 1u;  // the range before this one has been drained
+        ok = mbar_wait(&sh.full[s], (uint32_t)(gc / kStages) & 1u, status, kErrTimeout, kWaitNs);
+        if (first && gb > 1) ok = ok && mbar_wait(&sh.accfree[0], fpar, status, kErrTimeout, kWaitNs);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t a0 = sdesc(sbase + s * kStage, 128, 256), b0 = sdesc(sbase + s * kStage + kABytes, 128, 256);
+        const uint32_t acc = first ? 0u : 1u;
+        constexpr uint64_t kAStep = kTM * kCK * 2 / 16, kBStep = kTN * kCK * 2 / 16;  // one digit's operand
+        if (elect_one()) {
+#pragma unroll
+          for (int d = 0; d < 4; ++d)  // levels d .. 3 (digits 0 .. 3 - d of the right operand)
+            mma_f16(tmem + kTN * d, a0 + d * kAStep, b0, idesc_f16(kTM, kTN * (4 - d)), d ? 1u : acc);
+          if (last) mma_commit(&sh.accfull[0]);
+        }
+        __syncwarp();
+        if (first && gb > 1) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&sh.accfree[1], fpar, status, kErrTimeout, kWaitNs));
+          if (!ok) break;
+          tc_fence_after();
+        }
+        if (elect_one()) {
+          // levels max(4, d) .. 7 (digits from max(4 - d, 0)); the short ones in the middle, so that the queue
+          // holds the longest MMAs while this warp turns to the next chunk
+          constexpr int order[kDig] = {0, 7, 6, 5, 4, 3, 2, 1};
+#pragma unroll
+          for (int q = 0; q < kDig; ++q) {
+            const int d = order[q], l0 = d < 4 ? 4 : d;
+            mma_f16(tmem + kTN * l0, a0 + d * kAStep, b0 + (l0 - d) * kBStep, idesc_f16(kTM, kTN * (8 - l0)), d ? 1u : acc);
+          }
+          mma_commit(&sh.empty[s]);
+          if (last) mma_commit(&sh.accfull[1]);
+        }
+        __syncwarp();
+      }
+    }
+    // the MMAs issued so far are complete before the tensor memory is given back
+    if (!ok && elect_one()) mma_commit(&sh.empty[gc % kStages]);
+    __syncwarp();
+    if (!ok || gc > 0) {
+      const int g = ok ? gc - 1 : gc;
+      if (!mbar_wait(&sh.empty[g % kStages], (uint32_t)(g / kStages) & 1u, status, kErrTimeout, kWaitNs) && lane == 0)
+        atomicOr(status, kErrInflight);
+    }
+  } else {
+    // warp w drains TMEM lanes 32 (w mod 4) .. + 31 (rows) and 16 columns from 16 (w / 4)
+    const int c0 = (warp >> 2) * 16;
+    const uint32_t lbase = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
+    int gb = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < P.tiles && ok; t += gridDim.x) {
+      const int pi = t < n0 ? 0 : 1;
+      const SgProb &pr = P.pr[pi];
+      const SgProduct &p = pr.p;
+      int tm, tn;
+      sg_tile(pr, pi ? t - n0 : t, tm, tn);
+      const int i = tm * kTM + (warp & 3) * 32 + lane, jb = tn * kTN + c0;
+      const bool rowok = i < p.M;
+      double *const Ci = p.C + (long long)(i >> 1) * p.crh + (long long)(i & 1) * p.crl + (long long)(jb >> 1) * p.cch;
+      if (p.beta && rowok && (lane & 15) == 0)  // the old values travel to L2 while the MMAs run
+        for (int j = 0; j < 16 && jb + j < p.N; ++j)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(Ci + (j >> 1) * p.cch + (j & 1) * p.ccl));
+      Fx x[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) x[j] = Fx{0u, 0u, 0u};
+      const int nr = (pr.nq + kRangeChunks - 1) / kRangeChunks;
+      for (int b = 0; b < nr && ok; ++b, ++gb) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(&sh.accfull[h], (uint32_t)gb & 1u, status, kErrTimeout, kWaitNs));
+          if (!ok) break;
+          tc_fence_after();
+#pragma unroll
+          for (int c4 = 0; c4 < 16; c4 += 4) {
+            float y[4][4];
+            tmem_ld4x4(lbase + kTN * 4 * h + c4, kTN, y);
+            float mx = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              mx = fmaxf(fmaxf(mx, fmaxf(fabsf(y[0][j]), fabsf(y[1][j]))), fmaxf(fabsf(y[2][j]), fabsf(y[3][j])));
+            if (__all_sync(0xffffffffu, mx < 4194304.f)) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const long long v = fx_levels<true>(y[0][j], y[1][j], y[2][j], y[3][j]);
+                if (h)
+                  fx_add_lo(x[c4 + j], v);
+                else
+                  fx_add_hi(x[c4 + j], v);
+              }
+            } else {  // digits that line up: sums up to 2^24
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const long long v = fx_levels<false>(y[0][j], y[1][j], y[2][j], y[3][j]);
+                if (h)
+                  fx_add_lo(x[c4 + j], v);
+                else
+                  fx_add_hi(x[c4 + j], v);
+              }
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.accfree[h]);
+        }
+      }
+      if (!ok) break;
+      const int ea = rowok ? __ldg(pr.eA + i) : 1;
+      const int4 *const eb4 = reinterpret_cast<const int4 *>(pr.eB + jb);
+      const uint32_t flip = p.neg ? 0x80000000u : 0u;
+      const int jend = p.mode == 0 ? p.N : min(p.N, (i >> p.cs) + 1);  // columns of this row that are wanted
+      const int jn = rowok ? jend - jb : 0;
+#pragma unroll
+      for (int j4 = 0; j4 < 16; j4 += 4) {
+        if (__all_sync(0xffffffffu, j4 >= jn)) break;
+        const int4 e4 = __ldg(eb4 + j4 / 4);
+        const int eb[4] = {e4.x, e4.y, e4.z, e4.w};
+        double *const Cj[2] = {Ci + (long long)(j4 >> 1) * p.cch, Ci + (long long)((j4 >> 1) + 1) * p.cch};
+        double old[4] = {0.0, 0.0, 0.0, 0.0};
+        if (p.beta) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (j4 + q < jn) old[q] = Cj[q >> 1][(q & 1) ? p.ccl : 0];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          double v = fx_to_double(x[j4 + q], ea + eb[q] - 2 * 1022 - 68);
+          v = __hiloint2double(__double2hiint(v) ^ flip, __double2loint(v));
+          if (p.beta) v += old[q];
+          if (j4 + q < jn && max(ea, eb[q]) != kNonFinite) {
+            Cj[q >> 1][(q & 1) ? p.ccl : 0] = v;
+            const int j = jb + j4 + q;
+            if (p.mode == 2 && i != j)
+              p.C[(long long)(j >> 1) * p.crh + (long long)(j & 1) * p.crl + (long long)(i >> 1) * p.cch +
+                  (long long)(i & 1) * p.ccl] = v;
+          }
+        }
+      }
+      // rows and columns with an infinity or a NaN
+      for (int j = jb; j < jb + 16; ++j)
+        if (j < jb + jn && max(ea, __ldg(pr.eB + j)) == kNonFinite) sg_plain(p, i, j);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) tmem_dealloc(tmem, 512);
+}
+
+constexpr size_t kAlign = 1024;
+size_t pad(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+}  // namespace
+
+size_t sg_bytes(long long rows, long long K) {
+  const size_t R = pad((size_t)rows, kTM) + 4 * kTM, k = pad((size_t)std::max<long long>(64, std::min<long long>(K, kSgK)), kCK);
+  return R * k * kDig * 2 + R * sizeof(int) + 16 * kAlign;
+}
+
+int sg_gemm(const SgProduct *pr, int np, const SgWork &ws, cudaStream_t st) {
+  if (np < 1 || np > 2) return GINT_EINVAL;
+  const int K = pr[0].K;
+  if (cudaFuncSetAttribute(k_sg_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSgSmem) != cudaSuccess)
+    return GINT_ECUDA;
+  for (int k0 = 0; k0 < std::max(K, 1); k0 += kSgK) {
+    const int kk = std::min(kSgK, K - k0), nq = std::max(1, (kk + kCK - 1) / kCK);
+    SgPack pk{};
+    SgArgs ar{};
+    ar.status = ws.status;
+    size_t off = 0;
+    unsigned char *base = ws.buf;
+    int nop = 0, blocks = 0, *e0 = nullptr;
+    long long erows = 0;
+    for (int q = 0; q < np; ++q) erows += pad(pr[q].M, kTM) + pad(pr[q].N, kTM);
+    if (pad((size_t)erows * sizeof(int), kAlign) > ws.bytes) return GINT_EINVAL;
+    e0 = reinterpret_cast<int *>(base);
+    off = pad((size_t)erows * sizeof(int), kAlign);
+    int *e = e0;
+    for (int q = 0; q < np; ++q) {
+      if (pr[q].K != K || pr[q].M < 0 || pr[q].N < 0) return GINT_EINVAL;
+      SgProb &pb = ar.pr[q];
+      pb.p = pr[q];
+      // the range [k0, k0 + kk) of the contraction (kSgK is even: part offsets stay aligned)
+      for (SgView *v : {&pb.p.A, &pb.p.B}) {
+        v->p += (long long)(k0 >> 1) * v->kh;
+        if (v->ks) v->ks += k0 >> 1;
+      }
+      pb.p.K = kk;
+      if (k0 > 0) pb.p.beta = 1;
+      pb.nq = nq;
+      pb.ntn = (pb.p.N + kTN - 1) / kTN;
+      const long long ntm = (pb.p.M + kTM - 1) / kTM;
+      long long tiles = 0;
+      if (pb.p.mode == 0) {
+        tiles = ntm * pb.ntn;
+      } else {
+        const int mul = pb.p.cs ? 1 : 2;
+        for (long long tm = 0; tm < ntm; ++tm) tiles += std::min<long long>(pb.ntn, mul * (tm + 1));
+      }
+      if (ar.tiles + tiles > 0x3fffffffLL) return GINT_EINVAL;
+      pb.ntiles = (int)tiles;
+      ar.tiles += (int)tiles;
+      for (int side = 0; side < 2; ++side) {
+        SgOperand &o = pk.op[nop];
+        o.v = side ? pb.p.B : pb.p.A;
+        o.R = side ? pb.p.N : pb.p.M;
+        o.K = kk;
+        o.nq = nq;
+        o.tr = side ? kTN : kTM;
+        const long long sr = o.v.rot ? o.v.rh / 2 : std::min(o.v.rl, o.v.rh), sk = o.v.rot ? o.v.kh / 2 : std::min(o.v.kl, o.v.kh);
+        o.rfast = sr <= sk;
+        o.dst = base + off;
+        o.e = e;
+        e += pad(o.R, kTM);
+        off += pad(o.R, o.tr) / o.tr * (size_t)nq * kDig * o.tr * kCK * 2;
+        (side ? pb.PB : pb.PA) = o.dst;
+        (side ? pb.eB : pb.eA) = o.e;
+        pk.first[nop++] = blocks;
+        blocks += (o.R + kPR - 1) / kPR;
+      }
+    }
+    if (off > ws.bytes) return GINT_EINVAL;
+    for (int q = nop; q < 5; ++q) pk.first[q] = blocks;
+    if (ar.tiles == 0) return GINT_OK;
+    if (kk <= kPK) {
+      k_sg_pack<true><<<blocks, kPT, 0, st>>>(pk);
+    } else {
+      if (cudaMemsetAsync(e0, 0, (size_t)erows * sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
+      const dim3 g((unsigned)blocks, (unsigned)((kk + kPK - 1) / kPK));
+      k_sg_max<<<g, kPT, 0, st>>>(pk);
+      k_sg_pack<false><<<g, kPT, 0, st>>>(pk);
+    }
+    k_sg_mma<<<std::min(ws.num_sms, ar.tiles), kSgThreads, kSgSmem, st>>>(ar);
+    if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA;
+  }
+  return GINT_OK;
+}
+
+}  // namespace gla
