@@ -122,6 +122,13 @@ struct gint_handle {
   int *pb_I = nullptr, *pb_J = nullptr, *pb_img_off = nullptr;
   long long *pb_off = nullptr;
   double *pb_img = nullptr;             // image positions of J per pair
+  GTabs pb_orb{};                       // orbital metadata with the offsets of pb_otab
+  double *pb_otab = nullptr;            // orbital tables of the overlap kernel
+  double2 *pb_phase = nullptr;          // weight x projector radial x phase at every quadrature point
+  double2 *pb_part = nullptr;           // [pb_groups][pb_nelems] partial sums
+  int *pb_order = nullptr;              // pairs by the shape of J; segments of equal shape start at pb_first
+  int pb_groups = 1;
+  std::vector<int> pb_shape, pb_first;
   double *red = nullptr;      // reduction partials
   double *scal = nullptr;     // device scalars
   unsigned *err_word = nullptr;

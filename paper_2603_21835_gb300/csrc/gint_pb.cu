@@ -8,9 +8,20 @@
 // available here, so a product rule of the same degree stands in: 9 Gauss-Legendre nodes in
 // cos(theta) times 18 equally spaced azimuths (162 points).
 //
-// GPU organisation (as the paper describes it): one CTA per (I, J) pair, one thread per angular
-// point, each thread accumulating its ray over all radial nodes; the sums over angular points are
-// warp-shuffle reductions followed by one shared-memory pass, no atomics.
+// GPU organisation.  Everything is float64, which this GPU runs at 2 multiply-adds per clock and SM: a
+// warp-wide float64 instruction occupies the SM's pipe for 16 clocks, and the kernel's time is the number of
+// those instructions.  So what does not depend on the pair is formed once per call (k_pb_phase: quadrature
+// weight times projector radial times the phase e^{-i A.x} of the point relative to tau_I; e^{-i A.tau_I}
+// multiplies the sums at the end), the orbital tables hold the knot differences, dr f' and the Y_lm
+// constants, and points outside an image's support cost the distance test only.  A warp takes 2 neighbouring rays
+// times 16 neighbouring radial nodes at a time, a compact patch that is mostly all inside or all outside
+// (32 rays of one radius, a band around the whole sphere, are rarely either), and 81 such ray pairs fill whole
+// warps where 162 rays leave the last of six with two.  k_psibeta: a CTA of 3 warps (four share an SM: one's
+// set-up and sums overlap the others' points; one CTA of 9 warps took 5.33 ms where this takes 4.77) works on a
+// pair and a group of its ray pairs; k_pb_sum adds the groups' sums in order (no atomics).
+// Per point and image inside the support 121 float64 instructions, outside a float32 test for the patch.
+// Bound: the float64 pipe (0.8 of its cycles active).  64-atom Si, 1,856 pairs x 22,680 points: 22.9 ms
+// (one CTA a pair and one thread a ray, every point evaluated in full) -> 4.77 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -22,12 +33,13 @@
 namespace {
 
 constexpr int kPbTheta = 9, kPbPhi = 18, kPbRays = kPbTheta * kPbPhi, kPbNr = 140;
-constexpr int kPbThreads = 192, kPbWarps = kPbThreads / 32;
+constexpr int kPbWarps = 3, kPbThreads = 32 * kPbWarps;
+constexpr int kPbRayPairs = kPbRays / 2, kPbSeg = 16;  // a warp's patch: 2 rays x 16 radial nodes
 constexpr int kPbMaxOrb = 16;  // orbitals of the neighbour atom (accumulators held in registers)
-constexpr int kPbGroup = 2;    // projector radials per pass over the ray
-constexpr int kPbRed = 2 * 5 * kPbMaxOrb;  // reduction slots of one projector radial (l <= 2)
+constexpr int kPbImages = 32;  // images of a pair staged in shared memory
+constexpr int kPbGroup = 2;    // projector radials per pass over the points
 constexpr double kPi = 3.14159265358979323846;
-static_assert(kPbRays <= kPbThreads, "one thread per angular point");
+static_assert(kPbRays % 2 == 0 && kPbRayPairs % 9 == 0, "ray pairs in ninths");
 
 __constant__ double c_ang[kPbRays][4];  // unit vector and weight (weights sum to 4 pi)
 __constant__ double c_rad[kPbNr][2];    // node in (0, 1) and weight of the rule on [0, 1]
@@ -41,6 +53,12 @@ struct GPb {
   const double *pos;
   const int *species;
   const double2 *tab, *ptab;  // orbital and projector tables, (f, f') per knot
+  const double *otab;         // orbital tables of this kernel: per knot and radial (f, df, dr f'_k, dr f'_k+1)
+  double2 *phase;             // [projector radial][ray][node]: weight x radial x e^{-i A.x}
+  const int *order;           // pairs of this launch
+  double *part;               // [group][complex element]
+  long long nelems;
+  int ngroups;                // CTAs per pair
 };
 
 // Gauss-Legendre nodes and weights on [-1, 1] (Newton iteration on P_n from the three-term
@@ -74,102 +92,235 @@ void gauss_legendre(int n, std::vector<double> &x, std::vector<double> &w) {
   }
 }
 
-// Sum over the CTA of v (threads beyond the rays hold 0): warp shuffles, then lane 0 of each warp
-// stores its warp's sum at red[warp][slot].
-__device__ __forceinline__ void warp_sum_to(double v, double (*red)[kPbRed], int slot) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][slot] = v;
+// One thread per (projector radial, ray, node).
+__global__ void __launch_bounds__(256) k_pb_phase(const __grid_constant__ GTabs prj, const __grid_constant__ GPb P) {
+  const int u = blockIdx.x * 256 + threadIdx.x, rad = blockIdx.y;
+  if (u >= kPbRays * kPbNr) return;
+  const int a = u / kPbNr, k = u - a * kPbNr;
+  double rcb = 0.0;
+  for (int s = 0; s < prj.nspecies; ++s)
+    if (rad >= prj.sp[s].rad0 && rad < prj.sp[s].rad0 + prj.sp[s].nrad) rcb = prj.sp[s].rcut;
+  const GRadial &R = prj.rad[rad];
+  const double r = rcb * c_rad[k][0], wk = rcb * c_rad[k][1] * r * r;
+  double f = 0.0, df;
+  if (r < R.rc) radial_eval<double>(P.ptab, R, r, f, df);
+  double s, c;
+  sincos(-r * (P.A[0] * c_ang[a][0] + P.A[1] * c_ang[a][1] + P.A[2] * c_ang[a][2]), &s, &c);
+  f *= wk;
+  P.phase[((long long)rad * kPbRays + a) * kPbNr + k] = make_double2(f * c, f * s);
 }
 
-__global__ void __launch_bounds__(kPbThreads) k_psibeta(const __grid_constant__ GTabs orb,
-                                                        const __grid_constant__ GTabs prj,
-                                                        const __grid_constant__ GPb P, double *__restrict__ out) {
-  __shared__ double red[kPbWarps][kPbRed];
-  const int p = blockIdx.x, I = P.pI[p], J = P.pJ[p];
-  const int spI = P.species[I], spJ = P.species[J];
-  const GSpecies &SJ = orb.sp[spJ];
-  const GSpecies &SB = prj.sp[spI];
-  const int noJ = SJ.norb;
-  const int a = threadIdx.x;
-  const bool ray = a < kPbRays;
-  const double ex = ray ? c_ang[a][0] : 0.0, ey = ray ? c_ang[a][1] : 0.0, ez = ray ? c_ang[a][2] : 0.0;
-  const double wa = ray ? c_ang[a][3] : 0.0;
-  const double tx = P.pos[3 * I], ty = P.pos[3 * I + 1], tz = P.pos[3 * I + 2];
-  const int i0 = P.img_off[p], i1 = P.img_off[p + 1];
-  const double rcb = SB.rcut;
-  double *o = out + 2 * P.poff[p];
-  int col = 0;  // first projector function of the group
-  for (int g0 = 0; g0 < SB.nrad; g0 += kPbGroup) {
-    const int ng = min(kPbGroup, SB.nrad - g0);
-    double acc[kPbGroup][kPbMaxOrb][2];
+// Orbitals of a shaped species (NS s, NP p, ND d radials on one knot grid) at displacement d with r2 = |d|^2
+// below the support: phi[m] += value.  Tables: the radial times the constant of Y_00, of Y_1m or of
+// Y_2,+-1 (the other d functions carry their ratio to it).
+template <int NS, int NP, int ND>
+__device__ __forceinline__ void pb_orbitals(const GTabs &g, const double *__restrict__ tab, const GSpecies &S, double dx,
+                                            double dy, double dz, double r2, double *phi) {
+  constexpr int NR = NS + NP + ND;
+  const GRadial &R0 = g.rad[S.rad0];
+  r2 = fmax(r2, 1e-300);  // on the atom: u = 0, so only the s functions remain
+  const double y = rsqrt(r2);
+  double r = r2 * y;
+  r = fma(fma(-r, r, r2), 0.5 * y, r);
+  // knot i = floor(r / dr), t in [0, 1] (a point on a knot may take either side)
+  const double x = r * R0.inv_dr, big = 6755399441055744.0;  // 1.5 2^52
+  const double xi = (x - 0.5) + big;  // its low bits: an integer within 1/2 of x - 1/2
+  const int i = min(max(__double2loint(xi), 0), R0.npts - 2);
+  const double t = x - (xi - big);
+  const double t2 = t * t, u = 1.0 - t, s = t2 * fma(-2.0, t, 3.0), c0 = t * u * u, c1 = -t2 * u;
+  const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)i * NR) * 2;
+  double f[NR];
 #pragma unroll
-    for (int g = 0; g < kPbGroup; ++g)
+  for (int k = 0; k < NR; ++k) {
+    const double2 a = __ldg(q + 2 * k), b = __ldg(q + 2 * k + 1);
+    f[k] = fma(b.y, c1, fma(b.x, c0, fma(a.y, s, a.x)));
+    if (S.kslot && !(r < g.rad[S.rad0 + k].rc)) f[k] = 0.0;  // kslot: the radials end at different radii
+  }
+  const double ux = dx * y, uy = dy * y, uz = dz * y;
 #pragma unroll
-      for (int m = 0; m < kPbMaxOrb; ++m) acc[g][m][0] = acc[g][m][1] = 0.0;
-    if (ray) {
-      for (int k = 0; k < kPbNr; ++k) {
-        const double r = rcb * c_rad[k][0], wk = rcb * c_rad[k][1] * r * r;
-        const double px = tx + r * ex, py = ty + r * ey, pz = tz + r * ez;
-        double fb[kPbGroup];
+  for (int k = 0; k < NS; ++k) phi[k] += f[k];
 #pragma unroll
-        for (int g = 0; g < kPbGroup; ++g) {
-          fb[g] = 0.0;
-          if (g < ng) {
-            const GRadial &R = prj.rad[SB.rad0 + g0 + g];
-            double df;
-            if (r < R.rc) radial_eval<double>(P.ptab, R, r, fb[g], df);
-          }
-        }
-        double phi[kPbMaxOrb];
+  for (int k = 0; k < NP; ++k) {
+    double *o = phi + NS + 3 * k;
+    o[0] = fma(f[NS + k], uz, o[0]);
+    o[1] = fma(f[NS + k], ux, o[1]);
+    o[2] = fma(f[NS + k], uy, o[2]);
+  }
+  if (ND > 0) {
+    const double xx = ux * ux, y0 = fma(2.0 * uz, uz, -fma(uy, uy, xx)), y3 = fma(-uy, uy, xx);
+    const double xz = ux * uz, yz = uy * uz, xy = ux * uy;
 #pragma unroll
-        for (int m = 0; m < kPbMaxOrb; ++m) phi[m] = 0.0;
-        for (int q = i0; q < i1; ++q) {
-          const double dx = px - P.img[3 * q], dy = py - P.img[3 * q + 1], dz = pz - P.img[3 * q + 2];
-          if (dx * dx + dy * dy + dz * dz < SJ.rcut2)
-            add_orbitals<double, true, false>(orb, P.tab, spJ, dx, dy, dz, phi, nullptr);
-        }
-        double s, c;
-        sincos(-(P.A[0] * px + P.A[1] * py + P.A[2] * pz), &s, &c);
-#pragma unroll
-        for (int g = 0; g < kPbGroup; ++g) {
-          const double wr = wk * fb[g], cr = wr * c, ci = wr * s;
-#pragma unroll
-          for (int m = 0; m < kPbMaxOrb; ++m) {
-            acc[g][m][0] += cr * phi[m];
-            acc[g][m][1] += ci * phi[m];
-          }
-        }
-      }
-    }
-    // angular factors w_a Y_lm(e_a) and the sums over the rays, one projector radial at a time
-    // (compile-time indices into the accumulators, which stay in registers)
-#pragma unroll
-    for (int g = 0; g < kPbGroup; ++g) {
-      if (g >= ng) break;
-      const int l = prj.rad[SB.rad0 + g0 + g].l, nm = 2 * l + 1;
-      double y[5], gy[5][3];
-      ylm_unit<double>(l, ex, ey, ez, y, gy);
-      for (int mm = 0; mm < nm; ++mm) {
-        const double f = ray ? wa * y[mm] : 0.0;
-#pragma unroll
-        for (int m = 0; m < kPbMaxOrb; ++m)
-          if (m < noJ) {
-            warp_sum_to(f * acc[g][m][0], red, 2 * (mm * noJ + m));
-            warp_sum_to(f * acc[g][m][1], red, 2 * (mm * noJ + m) + 1);
-          }
-      }
-      __syncthreads();
-      for (int u = threadIdx.x; u < 2 * nm * noJ; u += kPbThreads) {
-        double v = 0.0;
-        for (int w = 0; w < kPbWarps; ++w) v += red[w][u];
-        o[2 * col * noJ + u] = v;  // (projector col + u / (2 noJ), orbital (u / 2) mod noJ, re / im)
-      }
-      __syncthreads();
-      col += nm;
+    for (int k = 0; k < ND; ++k) {
+      double *o = phi + NS + 3 * NP + 5 * k;
+      const double fk = f[NS + NP + k];
+      o[0] = fma(fk * 0.28867513459481288225, y0, o[0]);  // sqrt(5/16) / sqrt(15/4)
+      o[1] = fma(fk, xz, o[1]);
+      o[2] = fma(fk, yz, o[2]);
+      o[3] = fma(fk * 0.5, y3, o[3]);
+      o[4] = fma(fk, xy, o[4]);
     }
   }
 }
+
+// v[0 .. 2 H) over the lanes that differ in bit `bit`: the lane whose bit is clear keeps the sums of the first
+// H, the other those of the second H.
+template <int H>
+__device__ __forceinline__ void halve(double *v, int bit) {
+  const bool up = threadIdx.x & bit;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const double keep = up ? v[i + H] : v[i], send = up ? v[i] : v[i + H];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+  }
+}
+
+// One pair (blockIdx.x) and group of ray pairs (blockIdx.y).  NO orbitals of J; NS = NP = ND = 0: the general
+// evaluator (any radial order and knot grids), NO = kPbMaxOrb.
+template <int NS, int NP, int ND, int NO>
+__global__ void __launch_bounds__(kPbThreads, 4) k_psibeta(const __grid_constant__ GTabs orb,
+                                                           const __grid_constant__ GTabs prj,
+                                                           const __grid_constant__ GPb P) {
+  constexpr int NV = 2 * kPbMaxOrb;  // (orbital, re / im) of one projector radial, padded
+  // after the reduction over a ray's 16 lanes a lane holds 2 of the 32 sums of each radial; here their sums over
+  // the warp's rays with the angular factors w_a Y_lm(e_a)
+  __shared__ double tot[kPbGroup][5][2][kPbThreads];
+  __shared__ double rk[kPbNr], sim[3 * kPbImages];  // radial nodes; tau_I - image of J
+  __shared__ float rkf[kPbNr], simf[3 * kPbImages];
+  const int p = P.order[blockIdx.x], I = P.pI[p], J = P.pJ[p];
+  const GSpecies &SJ = orb.sp[P.species[J]];
+  const GSpecies &SB = prj.sp[P.species[I]];
+  const int noJ = SJ.norb, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, kg = lane & (kPbSeg - 1);
+  for (int k = threadIdx.x; k < kPbNr; k += kPbThreads) {
+    rk[k] = SB.rcut * c_rad[k][0];
+    rkf[k] = (float)rk[k];
+  }
+  const double tx = P.pos[3 * I], ty = P.pos[3 * I + 1], tz = P.pos[3 * I + 2];
+  const int i0 = P.img_off[p], i1 = P.img_off[p + 1];
+  const bool staged = i1 - i0 <= kPbImages;
+  if (staged)
+    for (int u = threadIdx.x; u < 3 * (i1 - i0); u += kPbThreads) {
+      sim[u] = P.pos[3 * I + u % 3] - P.img[3 * i0 + u];
+      simf[u] = (float)sim[u];
+    }
+  // float32 coordinates of at most rc_phi + 2 rc_beta, a few roundings each: r^2 is off by less than 1e-6 of their
+  // square
+  const double ext = SJ.rcut + 2.0 * SB.rcut;
+  const float lim2 = (float)(SJ.rcut2 + 4e-6 * ext * ext);
+  __syncthreads();
+  const int np = kPbRayPairs / P.ngroups, rp0 = blockIdx.y * np;
+  double *o = P.part + 2 * (blockIdx.y * P.nelems + P.poff[p]);
+  int col = 0;  // first projector function of the pass
+  for (int g0 = 0; g0 < SB.nrad; g0 += kPbGroup) {
+    const int ng = min(kPbGroup, SB.nrad - g0);
+    for (int i = 0; i < kPbGroup * 10; ++i) (&tot[0][0][0][0])[i * kPbThreads + threadIdx.x] = 0.0;
+    for (int rp = rp0 + warp; rp < rp0 + np; rp += kPbWarps) {
+      const int a = 2 * rp + (lane >> 4);
+      const double ex = c_ang[a][0], ey = c_ang[a][1], ez = c_ang[a][2];
+      const float exf = (float)ex, eyf = (float)ey, ezf = (float)ez;
+      double acc[kPbGroup][NV];
+#pragma unroll
+      for (int g = 0; g < kPbGroup; ++g)
+#pragma unroll
+        for (int m = 0; m < NV; ++m) acc[g][m] = 0.0;
+      const double2 *ph = P.phase + ((long long)(SB.rad0 + g0) * kPbRays + a) * kPbNr;
+      for (int k = kg; k < (kPbNr + kPbSeg - 1) / kPbSeg * kPbSeg; k += kPbSeg) {
+        const bool pt = k < kPbNr;
+        const double r = pt ? rk[k] : 0.0;
+        const float rf = pt ? rkf[k] : 0.f;
+        double phi[NO];
+#pragma unroll
+        for (int m = 0; m < NO; ++m) phi[m] = 0.0;
+        bool any = false;
+        for (int q = i0; q < i1; ++q) {
+          // screened in float32 for the whole patch: a point beyond lim2 (four times the bound on the float32
+          // error of r^2 outside the support) is outside
+          double ox, oy, oz;  // tau_I - image
+          if (staged) {
+            const float fx = fmaf(rf, exf, simf[3 * (q - i0)]), fy = fmaf(rf, eyf, simf[3 * (q - i0) + 1]),
+                        fz = fmaf(rf, ezf, simf[3 * (q - i0) + 2]);
+            if (!__any_sync(0xffffffffu, pt && fx * fx + fy * fy + fz * fz < lim2)) continue;
+            ox = sim[3 * (q - i0)], oy = sim[3 * (q - i0) + 1], oz = sim[3 * (q - i0) + 2];
+          } else {
+            ox = tx - P.img[3 * q], oy = ty - P.img[3 * q + 1], oz = tz - P.img[3 * q + 2];
+          }
+          const double dx = fma(r, ex, ox), dy = fma(r, ey, oy), dz = fma(r, ez, oz);
+          const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+          if (pt && r2 < SJ.rcut2) {
+            any = true;
+            if constexpr (NS + NP + ND > 0)
+              pb_orbitals<NS, NP, ND>(orb, P.otab, SJ, dx, dy, dz, r2, phi);
+            else
+              add_orbitals<double, true, false>(orb, P.tab, P.species[J], dx, dy, dz, phi, nullptr);
+          }
+        }
+        if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+        for (int g = 0; g < kPbGroup; ++g) {
+          if (g >= ng) break;
+          const double2 w = pt ? __ldg(ph + (long long)g * kPbRays * kPbNr + k) : make_double2(0.0, 0.0);
+#pragma unroll
+          for (int m = 0; m < NO; ++m) {
+            acc[g][2 * m] = fma(w.x, phi[m], acc[g][2 * m]);
+            acc[g][2 * m + 1] = fma(w.y, phi[m], acc[g][2 * m + 1]);
+          }
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < kPbGroup; ++g) {
+        if (g >= ng) break;
+        halve<16>(acc[g], 8);
+        halve<8>(acc[g], 4);
+        halve<4>(acc[g], 2);
+        halve<2>(acc[g], 1);
+        double y[5], gy[5][3];
+        const int l = prj.rad[SB.rad0 + g0 + g].l;
+        ylm_unit<double>(l, ex, ey, ez, y, gy);
+#pragma unroll
+        for (int mm = 0; mm < 5; ++mm)
+          if (mm < 2 * l + 1) {
+            const double f = c_ang[a][3] * y[mm];
+            double *t = &tot[g][mm][0][threadIdx.x];
+            t[0] = fma(f, acc[g][0], t[0]);
+            t[kPbThreads] = fma(f, acc[g][1], t[kPbThreads]);
+          }
+      }
+    }
+    // the halvings left sums 2 kg, 2 kg + 1 (orbital, re / im) in the lanes kg of either half
+    __syncthreads();
+    for (int g = 0; g < ng; ++g) {
+      const int nm = 2 * prj.rad[SB.rad0 + g0 + g].l + 1;
+      for (int u = threadIdx.x; u < 2 * nm * noJ; u += kPbThreads) {
+        const int mm = u / (2 * noJ), e = u - mm * 2 * noJ;
+        const double *t = &tot[g][mm][e & 1][e >> 1];
+        double v = 0.0;
+        for (int w = 0; w < 2 * kPbWarps; ++w) v += t[w * kPbSeg];
+        o[2 * col * noJ + u] = v;  // (projector col + mm, orbital e / 2, re / im)
+      }
+      col += nm;
+    }
+    __syncthreads();
+  }
+}
+
+// out = e^{-i A.tau_I} times the sum of the groups' parts.
+__global__ void __launch_bounds__(128) k_pb_sum(const __grid_constant__ GPb P, double2 *__restrict__ out) {
+  const int p = blockIdx.x, I = P.pI[p];
+  const double2 *part = reinterpret_cast<const double2 *>(P.part);
+  double s, c;
+  sincos(-(P.A[0] * P.pos[3 * I] + P.A[1] * P.pos[3 * I + 1] + P.A[2] * P.pos[3 * I + 2]), &s, &c);
+  for (long long e = P.poff[p] + threadIdx.x; e < P.poff[p + 1]; e += blockDim.x) {
+    double re = 0.0, im = 0.0;
+    for (int g = 0; g < P.ngroups; ++g) {
+      const double2 v = part[g * P.nelems + e];
+      re += v.x;
+      im += v.y;
+    }
+    out[e] = make_double2(re * c - im * s, re * s + im * c);
+  }
+}
+
+// Orbital shapes (s, p, d radials) with a compiled evaluator, and their orbitals.
+#define GINT_PB_SHAPES(X) X(2, 2, 1, 13) X(2, 1, 0, 5) X(1, 1, 1, 9) X(1, 1, 0, 4) X(1, 0, 0, 1)
 
 template <typename T>
 void pfree(T *&p) {
@@ -197,6 +348,10 @@ void gint_pb_free(gint_handle *h) {
   pfree(h->pb_off);
   pfree(h->pb_img_off);
   pfree(h->pb_img);
+  pfree(h->pb_otab);
+  pfree(h->pb_order);
+  pfree(h->pb_phase);
+  pfree(h->pb_part);
   h->pb_ready = false;
   h->pb_npairs = 0;
   h->pb_nelems = 0;
@@ -299,15 +454,71 @@ int gint_pb_set(gint_handle *h, int nspecies, const gint_species *proj) {
     cudaGetLastError();
     return GINT_ECUDA;
   }
+  // orbital tables: per knot and radial (f, f_{k+1} - f_k, dr f'_k, dr f'_{k+1}), times the Y_lm constant;
+  // shapes without a compiled evaluator keep the general one
+  GTabs ot = g;
+  std::vector<double> otab;
+  std::vector<int> shape(g.nspecies, 0);
+  const double cl[3] = {0.28209479177387814347, 0.48860251190291992159, 1.09254843059207907054};
+  for (int s = 0; s < g.nspecies; ++s) {
+    GSpecies &S = ot.sp[s];
+    switch (S.shape) {
+#define CASE_PB(ns, np, nd, no) case GINT_SHAPE(ns, np, nd):
+      GINT_PB_SHAPES(CASE_PB)
+#undef CASE_PB
+      shape[s] = S.shape;
+      break;
+      default: continue;
+    }
+    S.ioff = (int)(otab.size() / 4);
+    S.kslot = 0;
+    for (int k = 0; k < S.nrad; ++k)
+      if (g.rad[S.rad0 + k].rc != S.rcut) S.kslot = 1;
+    for (int i = 0; i + 1 < g.rad[S.rad0].npts; ++i)
+      for (int k = 0; k < S.nrad; ++k) {
+        const GRadial &R = g.rad[S.rad0 + k];
+        const double c = cl[R.l];
+        const gint_radial &T = h->d_rad[S.rad0 + k];
+        otab.insert(otab.end(), {c * T.f[i], c * (T.f[i + 1] - T.f[i]), c * R.dr * T.df[i], c * R.dr * T.df[i + 1]});
+      }
+  }
+  // pairs in launch order: by the shape of J
+  std::vector<int> order(pI.size());
+  for (size_t q = 0; q < order.size(); ++q) order[q] = (int)q;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+    return shape[h->species_host[pJ[x]]] < shape[h->species_host[pJ[y]]];
+  });
   gint_pb_free(h);
   int rc;
+  const int npair = (int)pI.size();
+  // ray groups per pair (CTAs): enough CTAs for a few waves, no more (each group costs a reduction of its sums)
+  h->pb_groups = npair < 4 * h->num_sms ? 9 : npair < 64 * h->num_sms ? 3 : 1;
+  const size_t phase = (size_t)std::max(1, t.nrad) * kPbRays * kPbNr, part = (size_t)h->pb_groups * poff.back();
   if ((rc = upload(&h->pb_tab64, tab)) || (rc = upload(&h->pb_I, pI)) || (rc = upload(&h->pb_J, pJ)) ||
-      (rc = upload(&h->pb_off, poff)) || (rc = upload(&h->pb_img_off, img_off)) || (rc = upload(&h->pb_img, img))) {
+      (rc = upload(&h->pb_off, poff)) || (rc = upload(&h->pb_img_off, img_off)) || (rc = upload(&h->pb_img, img)) ||
+      (rc = upload(&h->pb_otab, otab)) || (rc = upload(&h->pb_order, order))) {
     gint_pb_free(h);
     return rc;
   }
+  if (cudaMalloc(&h->pb_phase, phase * sizeof(double2)) != cudaSuccess ||
+      cudaMalloc(&h->pb_part, std::max<size_t>(part, 1) * sizeof(double2)) != cudaSuccess) {
+    cudaGetLastError();
+    gint_pb_free(h);
+    return GINT_ENOMEM;
+  }
   h->pb_tabs = t;
-  h->pb_npairs = (int)pI.size();
+  h->pb_orb = ot;
+  h->pb_shape.clear();
+  h->pb_first.clear();
+  for (int q = 0; q < npair; ++q) {
+    const int sh = shape[h->species_host[pJ[order[q]]]];
+    if (q == 0 || sh != h->pb_shape.back()) {
+      h->pb_shape.push_back(sh);
+      h->pb_first.push_back(q);
+    }
+  }
+  h->pb_first.push_back(npair);
+  h->pb_npairs = npair;
   h->pb_nelems = poff.back();
   h->pb_pairs_host.resize(2 * pI.size());
   for (size_t q = 0; q < pI.size(); ++q) {
@@ -315,8 +526,9 @@ int gint_pb_set(gint_handle *h, int nspecies, const gint_species *proj) {
     h->pb_pairs_host[2 * q + 1] = pJ[q];
   }
   h->pb_off_host = poff;
-  h->pb_bytes = (long long)(tab.size() * sizeof(double2) + (2 * pI.size() + img_off.size()) * sizeof(int) +
-                            poff.size() * sizeof(long long) + img.size() * sizeof(double));
+  h->pb_bytes = (long long)(tab.size() * sizeof(double2) + (3 * pI.size() + img_off.size()) * sizeof(int) +
+                            poff.size() * sizeof(long long) + (img.size() + otab.size()) * sizeof(double) +
+                            (phase + part) * sizeof(double2));
   h->pb_ready = true;
   return GINT_OK;
 }
@@ -335,6 +547,24 @@ int gint_pb_run(gint_handle *h, const double A[3], double *out, cudaStream_t st)
   P.species = h->species_dev;
   P.tab = h->tab64;
   P.ptab = h->pb_tab64;
-  k_psibeta<<<(unsigned)h->pb_npairs, kPbThreads, 0, st>>>(h->geom, h->pb_tabs, P, out);
+  P.otab = h->pb_otab;
+  P.phase = h->pb_phase;
+  P.part = reinterpret_cast<double *>(h->pb_part);
+  P.nelems = h->pb_nelems;
+  P.ngroups = h->pb_groups;
+  if (h->pb_tabs.nrad == 0) return GINT_OK;
+  k_pb_phase<<<dim3((kPbRays * kPbNr + 255) / 256, (unsigned)h->pb_tabs.nrad), 256, 0, st>>>(h->pb_tabs, P);
+  for (size_t q = 0; q < h->pb_shape.size(); ++q) {
+    P.order = h->pb_order + h->pb_first[q];
+    const dim3 grid((unsigned)(h->pb_first[q + 1] - h->pb_first[q]), (unsigned)h->pb_groups);
+    switch (h->pb_shape[q]) {
+#define CASE_PB(ns, np, nd, no)                                                                        \
+  case GINT_SHAPE(ns, np, nd): k_psibeta<ns, np, nd, no><<<grid, kPbThreads, 0, st>>>(h->pb_orb, h->pb_tabs, P); break;
+      GINT_PB_SHAPES(CASE_PB)
+#undef CASE_PB
+      default: k_psibeta<0, 0, 0, kPbMaxOrb><<<grid, kPbThreads, 0, st>>>(h->pb_orb, h->pb_tabs, P);
+    }
+  }
+  k_pb_sum<<<(unsigned)h->pb_npairs, 128, 0, st>>>(P, reinterpret_cast<double2 *>(out));
   return cudaGetLastError() == cudaSuccess ? GINT_OK : GINT_ECUDA;
 }
