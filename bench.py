@@ -249,8 +249,8 @@ def run_reference(args):
 # ------------------------------------------------------------------------------ our arm
 # kernels of ours per step (density + local-H passes; memsets are not kernels):
 #   fp64: k_simt_rho, k_simt_vlocal;  fp32: k_to_f32, k_simt_rho, k_simt_vlocal;
-#   f16x3 / f16x1: k_prep, k_prep_scales, k_build_tiles, k_tc_fused (both passes), k_h_reduce
-KERNEL_LAUNCHES = {"fp64": 2, "fp32": 3, "f16x3": 5, "f16x1": 5}
+#   f16x3 / f16x1: k_prep, k_build_tiles, k_tc_fused (both passes), k_h_reduce
+KERNEL_LAUNCHES = {"fp64": 2, "fp32": 3, "f16x3": 4, "f16x1": 4}
 TENSOR_PRECISIONS = ("f16x3", "f16x1")
 
 

@@ -1558,10 +1558,18 @@ __device__ __forceinline__ void reduce_pair_t(const GTabs &g, const GRedSys &S, 
 #pragma unroll
         for (int q = 0; q < kRedE; ++q) add(q, v[jj][q]);
     }
-    for (; k < k1; ++k) {
-      const long long o = __ldg(src + k);
+    if (k < k1) {  // the last, partial batch: absent bricks re-read its first and add zero (exact)
 #pragma unroll
-      for (int q = 0; q < kRedE; ++q) add(q, __ldcg(hs + o + e[q]));
+      for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + (k + jj < k1 ? k + jj : k));
+      float v[kRedB][kRedE];
+#pragma unroll
+      for (int jj = 0; jj < kRedB; ++jj)
+#pragma unroll
+        for (int q = 0; q < kRedE; ++q) v[jj][q] = __ldcg(hs + o[jj] + e[q]);
+#pragma unroll
+      for (int jj = 0; jj < kRedB; ++jj)
+#pragma unroll
+        for (int q = 0; q < kRedE; ++q) add(q, k + jj < k1 ? v[jj][q] : 0.f);
     }
     if (grp > 0) {
 #pragma unroll
@@ -1605,8 +1613,17 @@ __device__ __forceinline__ void reduce_pair(const GTabs &g, const GRedSys &S, in
     reduce_pair_t<NG, false, PF>(g, S, u, tid, part_hi, part_lo, bar);
 }
 
-__global__ void __launch_bounds__(kRedThreads, 4) k_h_reduce(const __grid_constant__ GTabs g, const __grid_constant__ GRed R) {
-  __shared__ float part_hi[(kRedGroups - 1) * kRedE * kRedLanes], part_lo[(kRedGroups - 1) * kRedE * kRedLanes];
+// A system with at most kRedFewPairs upper pairs has them summed in kRedGroupsFew parts, others in kRedGroups: a
+// part's list is walked in batches of dependent loads, so in a launch of few pairs, which are those of small
+// cells and so have long lists, the length of a part sets the time (the 8-atom cell: 36 pairs of 864 bricks,
+// 42 us in 4 parts, 23.5 in 16).  Where the pairs fill the GPU the smaller CTAs are the faster (512-atom Si with its long
+// lists in 16 parts: 0.11 ms slower).  The rule looks at the system only, so its blocks do not depend on what
+// shares the launch.
+constexpr int kRedGroupsFew = 16, kRedFewPairs = 152;
+template <int NG>
+__global__ void __launch_bounds__(NG * kRedLanes, 1024 / (NG * kRedLanes))
+    k_h_reduce(const __grid_constant__ GTabs g, const __grid_constant__ GRed R) {
+  __shared__ float part_hi[(NG - 1) * kRedE * kRedLanes], part_lo[(NG - 1) * kRedE * kRedLanes];
   const long long gu = blockIdx.x;
   int lo = 0, hi = R.nsys - 1;
   while (lo < hi) {
@@ -1616,7 +1633,7 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_h_reduce(const __grid_consta
     else
       hi = mid - 1;
   }
-  reduce_pair<kRedGroups, true>(g, R.sys[lo], (int)(gu - R.start[lo]), threadIdx.x, part_hi, part_lo, 0);
+  reduce_pair<NG, true>(g, R.sys[lo], (int)(gu - R.start[lo]), threadIdx.x, part_hi, part_lo, 0);
 }
 
 // ------------------------------------------------------------------------------ batched preparation
@@ -1627,7 +1644,7 @@ struct GPrepSys {
   long long ngrid;
   double *F;        // zeroed here (the brick kernel accumulates into it)
   long long natoms;
-  unsigned *mx;     // [0] bits of max |D|, [1] bits of max |V| (atomicMax on non-negative floats)
+  unsigned *mx;     // [0] bits of max |D|, [1] bits of max |V| (atomicMax on non-negative floats), [2] blocks done
   float *scales;
   double phi_bound, w;
 };
@@ -1677,16 +1694,10 @@ __device__ __forceinline__ void prep_range(const GPrepSys &S, long long i0, long
   }
 }
 
-// blockIdx.y = system: prep_range over the whole arrays; also resets the work counter.
-__global__ void k_prep(const __grid_constant__ GPrep P) {
-  prep_range(P.sys[blockIdx.y], 0, 0x7fffffffffffffffLL, blockIdx.x * (long long)blockDim.x + threadIdx.x,
-             (long long)gridDim.x * blockDim.x);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *P.work = 0;
-}
-
-__device__ double pow2_scale(double lim, double m) {
-  if (!(m > 0)) return 1048576.0;
-  return exp2(floor(log2(lim / m)));
+// 2^floor(log2(lim / m)), the power of two read off the quotient's exponent (2^20 for m = 0).
+__device__ __forceinline__ float pow2_scale(double lim, double m) {
+  if (!(m > 0)) return 1048576.f;
+  return (float)__hiloint2double(__double2hiint(lim / m) & 0x7ff00000, 0);
 }
 
 // Power-of-two scales of a system ([0] orbitals, [1] D, [2] w V orbitals), with the largest scaled
@@ -1694,16 +1705,29 @@ __device__ double pow2_scale(double lim, double m) {
 // next call.  One thread.
 __device__ __forceinline__ void prep_scales(const GPrepSys &S) {
   const double pb = 4.0 * S.phi_bound;
-  S.scales[0] = (float)pow2_scale(30000.0, pb);
-  S.scales[1] = (float)pow2_scale(30000.0, (double)__uint_as_float(S.mx[0]));
-  S.scales[2] = (float)pow2_scale(30000.0, pb * S.w * (double)__uint_as_float(S.mx[1]));
+  S.scales[0] = pow2_scale(30000.0, pb);
+  S.scales[1] = pow2_scale(30000.0, (double)__uint_as_float(__ldcg(S.mx)));
+  S.scales[2] = pow2_scale(30000.0, pb * S.w * (double)__uint_as_float(__ldcg(S.mx + 1)));
   S.mx[0] = 0u;
   S.mx[1] = 0u;
 }
 
-// Thread s: the scales of system s.
-__global__ void k_prep_scales(const __grid_constant__ GPrep P) {
-  if (threadIdx.x < P.nsys) prep_scales(P.sys[threadIdx.x]);
+// blockIdx.y = system: prep_range over the whole arrays; the system's last block forms its scales (a launch of
+// its own, with float64 logarithms in one thread, took 8 us of every call); also resets the work counter.
+__global__ void __launch_bounds__(256) k_prep(const __grid_constant__ GPrep P) {
+  const GPrepSys &S = P.sys[blockIdx.y];
+  prep_range(S, 0, 0x7fffffffffffffffLL, blockIdx.x * (long long)blockDim.x + threadIdx.x,
+             (long long)gridDim.x * blockDim.x);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *P.work = 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();  // this block's maxima before its count
+    if (atomicAdd(S.mx + 2, 1u) == gridDim.x - 1) {
+      __threadfence();
+      prep_scales(S);
+      S.mx[2] = 0u;
+    }
+  }
 }
 
 struct GTileSys {
@@ -2149,8 +2173,7 @@ __global__ void __launch_bounds__(kT, 1)
         brick_body<FORCE>(g, S, b, do_rho, do_h, split3, dsmem, zero, tmem, sh, smem, cx);
         tc_fence_before();
       }
-    } else {  // H reduction: two upper pairs, one per 256 threads (named barriers 2, 3), split into parts
-      // exactly as k_h_reduce splits them, so the blocks equal those of the batched call bit for bit
+    } else {  // H reduction: two upper pairs, one per 256 threads (named barriers 2, 3), in four parts
       bool go = true;
       if (t == 0 && ld_acquire_s32(&JS.bricks) < J.nbricks) {
         flush();
@@ -2706,19 +2729,20 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
   GPrep P{};
   GTile TB{};
   GBatch B{};
-  GRed R{};
+  GRed R[2] = {};  // systems of few pairs, the others
   P.nsys = n;
   P.work = h0->work_ctr;
   bool force = false;
   int np = kRC;
-  long long items = 0, pairs = 0, uppers = 0;
-  int nt = 0, nr = 0;
+  long long items = 0, pairs = 0, uppers[2] = {0, 0}, span = 0;
+  int nt = 0;
   for (int i = 0; i < n; ++i) {
     const gint_task &T = tk[i];
     gint_handle *h = T.h;
     const bool dens = T.rho || T.F, loc = T.H_blocks != nullptr;
     force |= T.F != nullptr;
     fill_prep(P.sys[i], T);
+    span = std::max(span, std::max(h->nblock, h->geom.ngrid));
     if (dens && h->npairs > 0) {
       TB.start[nt] = pairs;
       fill_tile(TB.sys[nt++], T);
@@ -2729,12 +2753,12 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
     items += (dens || loc) ? h->geom.nbricks : 0;
     if (dens || loc) np = std::max(np, h->max_brick_porb);
     if (loc && (h->reduce_R ? h->r_nupper : h->nupper) > 0) {
-      R.start[nr] = uppers;
-      GRedSys &rs = R.sys[nr++];
+      GRedSys rs{};
       rs.hs = h->hs;
       rs.species = h->species_dev;
       rs.H = T.H_blocks;
       rs.fp64 = h->reduce_fp64 ? 1 : 0;
+      const int nu = h->reduce_R ? h->r_nupper : h->nupper, k = nu <= kRedFewPairs ? 0 : 1;
       if (h->reduce_R) {  // the same tiles keyed by (I, J, R): H(R) blocks
         rs.hu_pair = h->r_hu_key;
         rs.hu_off = h->r_hu_off;
@@ -2743,7 +2767,6 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
         rs.pair_J = h->r_kJ;
         rs.pair_T = h->r_kT;
         rs.pair_off = h->r_koff;
-        uppers += h->r_nupper;
       } else {
         rs.hu_pair = h->hu_pair;
         rs.hu_off = h->hu_off;
@@ -2752,8 +2775,10 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
         rs.pair_J = h->pair_col_dev;
         rs.pair_T = h->pair_T_dev;
         rs.pair_off = h->pair_off_dev;
-        uppers += h->nupper;
       }
+      R[k].start[R[k].nsys] = uppers[k];
+      R[k].sys[R[k].nsys++] = rs;
+      uppers[k] += nu;
     }
   }
   B.nsys = n;
@@ -2761,8 +2786,7 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
   TB.nsys = nt;
   TB.start[nt] = pairs;
   TB.fixed = (force && split3) ? 1 : 0;
-  R.nsys = nr;
-  R.start[nr] = uppers;
+  for (int k = 0; k < 2; ++k) R[k].start[R[k].nsys] = uppers[k];
   np = (np + 15) & ~15;
   // dynamic shared memory: P (hi, lo) | stage region (density chunk stages; afterwards the two W P
   // halves of the local-H pass) | tail pad read by the last 128-row A tile above NP
@@ -2773,9 +2797,11 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
   B.np_max = np;
   B.split3 = split3;
   B.dsmem = (int)smem;
-  const int bx = std::max(8, 2 * h0->num_sms / n);
+  // a few blocks of 256 threads per SM over all systems (8 loads of 8 bytes in flight per thread), no more than
+  // the largest array has work for
+  const long long bmax = std::max(1LL, (span + 2047) / 2048);
+  const int bx = (int)std::min<long long>(bmax, std::max(16, 8 * h0->num_sms / n));
   k_prep<<<dim3(bx, n), 256, 0, st>>>(P);
-  k_prep_scales<<<1, kMaxBatch, 0, st>>>(P);
   TC_CHECK(cudaGetLastError());
   if (pairs > 0) {
     k_build_tiles<<<(unsigned)((pairs + kTileWarps - 1) / kTileWarps), 32 * kTileWarps, 0, st>>>(tabs, TB);
@@ -2791,10 +2817,10 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
     TC_CHECK(cudaGetLastError());
     if (ev1) TC_CHECK(cudaEventRecord(ev1, st));
   }
-  if (uppers > 0) {
-    k_h_reduce<<<(unsigned)uppers, kRedThreads, 0, st>>>(tabs, R);
-    TC_CHECK(cudaGetLastError());
-  }
+  if (uppers[0] > 0)
+    k_h_reduce<kRedGroupsFew><<<(unsigned)uppers[0], kRedGroupsFew * kRedLanes, 0, st>>>(tabs, R[0]);
+  if (uppers[1] > 0) k_h_reduce<kRedGroups><<<(unsigned)uppers[1], kRedThreads, 0, st>>>(tabs, R[1]);
+  TC_CHECK(cudaGetLastError());
   return GINT_OK;
 }
 
