@@ -42,6 +42,8 @@ struct gint_handle {
   int *pair_I_dev = nullptr;  // row atom I of each pair
   // neighbour structure
   int *n_at = nullptr, *n_ent = nullptr, *n_orb = nullptr;
+  float *frac_dev = nullptr;  // fractional coordinates of the atoms (float32 screen of the neighbour kernels)
+  int4 *b_list = nullptr;     // first entries of each brick (counting pass -> filling pass)
   long long *b_at_off = nullptr, *b_ent_off = nullptr, *b_pair_off = nullptr;
   long long *scan_out = nullptr;
   int *s_atom = nullptr, *s_col = nullptr;
@@ -151,6 +153,7 @@ struct gint_handle {
 };
 
 // gint_nbr.cu
+constexpr long long kNbrListBytes = 64 * 16;  // of b_list per brick
 int gint_build_neighbours(gint_handle *h, cudaStream_t st);
 // gint_capi.cu
 int gint_reserve_nbr(gint_handle *h);
