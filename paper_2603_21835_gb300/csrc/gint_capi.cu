@@ -382,7 +382,7 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
   TRY(dalloc(&h->work_ctr, 4));
   TRYCU(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
   TRYCU(cudaMemset(h->err_word, 0, sizeof(unsigned)));
-  TRY(gint_tc_prepare(h));
+  TRY(gint_tc_prepare(h, st));
   TRYCU(cudaStreamSynchronize(st));
   *out = h;
   return GINT_OK;
@@ -522,7 +522,7 @@ int gint_set_positions(gint_handle *h, const double *pos_dev, void *stream) {
     return GINT_ECUDA;
   int rc = gint_build_neighbours(h, st);
   if (rc) return rc;
-  rc = gint_tc_refresh(h);
+  rc = gint_tc_prepare(h, st);
   if (rc) return rc;
   gint_hr_free(h);  // H(R) keys follow the new images (rebuilt on first use)
   if (cudaMemcpyAsync(h->pos_host.data(), h->pos_dev, 3 * sizeof(double) * h->geom.natoms, cudaMemcpyDeviceToHost,

@@ -94,10 +94,12 @@ struct gint_handle {
   uint4 *plan = nullptr;                  // per-brick plan records (brick metadata, prefetched by the kernel)
   long long *plan_off_dev = nullptr;      // [nbricks + 1] record offsets, 16-byte units
   long long tc_bytes = 0;                 // device bytes of the tensor-core workspace above
-  // the neighbour structure these layouts were built for (host copies: brick slot offsets, slot atoms,
-  // brick entry offsets); a rebuild for new positions that reproduces it refreshes the plan records only
-  std::vector<long long> tc_at_off, tc_ent_off;
-  std::vector<int> tc_satom;
+  // layout kernels: upper index of each pair (-1: lower), sizes per brick and list lengths, the ranges' counts per
+  // upper pair, totals; capacities of the buffers whose size follows the positions
+  int *pair_u = nullptr, *lay_cnt = nullptr;
+  long long *lay_sz = nullptr, *lay_tot = nullptr;
+  int lay_ranges = 0;
+  long long cap_hs = 0, cap_src = 0, cap_plan = 0;
   // local H per lattice vector (keys (I, J, R); built on first use by gint_hr_prepare)
   bool r_ready = false;
   int r_status = 0;           // GINT_OK, or why per-R output is unavailable for this geometry
@@ -171,8 +173,7 @@ int gint_tc_vlocal(gint_handle *h, int precision, const double *V, double *H, cu
 int gint_tc_batch(const gint_task *tasks, int n, int precision, cudaStream_t st, cudaEvent_t ev0,
                   cudaEvent_t ev1);
 int gint_tc_check_capacity(const gint_handle *h);
-int gint_tc_prepare(gint_handle *h);  // layouts and scratch of the tensor-core path (after neighbours)
-int gint_tc_refresh(gint_handle *h);  // after a neighbour rebuild: plan records only, or gint_tc_prepare
+int gint_tc_prepare(gint_handle *h, cudaStream_t st);  // layouts and scratch of the tensor-core path (after neighbours)
 void gint_tc_free(gint_handle *h);
 // gint_hr.cu
 int gint_hr_prepare(gint_handle *h);  // key tables of H(R) (GINT_EUNSUPPORTED if tiles mix R)

@@ -36,7 +36,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <thread>
 #include <vector>
 
 #include "gint_handle.cuh"
@@ -1871,6 +1870,232 @@ __global__ void __launch_bounds__(128) k_build_plans(const __grid_constant__ GTa
   }
 }
 
+// ------------------------------------------------------------------------------ layouts of a geometry
+// Scratch ranges, plan records and the per-pair contribution lists of the local-H reduction, built on the device
+// for every set of positions.  A pair's list holds the scratch offsets of its tiles in brick order (slot order
+// within a brick), so that the reduction's order is fixed: the bricks are cut into contiguous ranges, every
+// range's contributions are counted per pair, the counts scanned over the ranges, and each range then places
+// its own in order (one warp, the cursors of its pairs in shared memory where they fit).  On host threads this
+// took 1.5 of the 2.5 ms of new positions for the 64-atom cell, 9.7 of 13 ms for 512 atoms, with the lists
+// copied in and out.
+constexpr int kLayWarps = 4;
+constexpr int kLaySmem = 96 * 1024;  // cursors in shared memory up to this size
+
+// The warp's brick: norb of slot `lane` and `lane + 32`, the padded width and the sum of norb.
+__device__ __forceinline__ void lay_slots(const GTabs &g, const int *__restrict__ s_atom, const int *__restrict__ species,
+                                          long long s0, int na, int lane, int no[2], int &cur, int &cum) {
+  int po[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int a = lane + 32 * h;
+    const int sp = a < na ? species[s_atom[s0 + a]] : 0;
+    no[h] = a < na ? g.sp[sp].norb : 0;
+    po[h] = a < na ? g.sp[sp].porb : 0;
+  }
+  cur = cum = 0;
+  for (int a = 0; a < na; ++a) {
+    const int q = __shfl_sync(0xffffffffu, a < 32 ? po[0] : po[1], a & 31);
+    cur = place_slot(cur, q) + q;
+    cum += __shfl_sync(0xffffffffu, a < 32 ? no[0] : no[1], a & 31);
+  }
+}
+// Upper slot pair e (0 <= e < na (na + 1) / 2) in the order a ascending, then c from a.
+__device__ __forceinline__ void lay_pair(int e, int na, int &a, int &c) {
+  // row a starts at a na - a (a - 1) / 2
+  a = (int)(((float)(2 * na + 1) - sqrtf((float)((2 * na + 1) * (2 * na + 1) - 8 * e))) * 0.5f);
+  a = max(0, min(a, na - 1));
+  while (a > 0 && a * na - a * (a - 1) / 2 > e) --a;
+  while ((a + 1) * na - (a + 1) * a / 2 <= e) ++a;
+  c = a + e - (a * na - a * (a - 1) / 2);
+}
+
+// One warp per brick: scratch and plan sizes, the widest brick, and the range's contributions per upper pair.
+__global__ void __launch_bounds__(32 * kLayWarps)
+    k_lay_count(const __grid_constant__ GTabs g, GNbr nb, const long long *__restrict__ ent_off, long long nbricks,
+                const int *__restrict__ pair_u, int nu, long long per, int *tcnt, long long *hs_sz, long long *plan_sz,
+                int *npmax) {
+  const int lane = threadIdx.x & 31;
+  const long long b = (long long)blockIdx.x * kLayWarps + (threadIdx.x >> 5);
+  if (b >= nbricks) return;
+  const long long s0 = nb.b_at_off[b], p0 = nb.b_pair_off[b];
+  const int na = (int)(nb.b_at_off[b + 1] - s0);
+  int no[2], cur, cum;
+  lay_slots(g, nb.s_atom, nb.atom_species, s0, na, lane, no, cur, cum);
+  int sq = no[0] * no[0] + no[1] * no[1];
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if (lane == 0) {
+    const int np = (cur + 15) & ~15;
+    const long long tot = ((long long)cum * cum + sq) / 2;  // sum over upper slot pairs of norb norb
+    hs_sz[b] = (tot + 3) & ~3LL;                            // 16-byte aligned ranges (one bulk copy each)
+    plan_sz[b] = plan_words(na, (int)(ent_off[b + 1] - ent_off[b]), np) / 4;
+    atomicMax(npmax, np);
+  }
+  int *tc = tcnt + (b / per) * nu;
+  for (int e = lane; e < na * (na + 1) / 2; e += 32) {
+    int a, c;
+    lay_pair(e, na, a, c);
+    const int p = nb.b_pair[p0 + a * na + c];
+    if (p >= 0) atomicAdd(tc + pair_u[p], 1);
+  }
+}
+
+// Per upper pair: the ranges' counts become each range's first place in the pair's list; the total to cnt.
+__global__ void __launch_bounds__(128) k_lay_cols(int nu, int nranges, int *__restrict__ tcnt, long long *__restrict__ cnt) {
+  const int u = blockIdx.x * 128 + threadIdx.x;
+  if (u >= nu) return;
+  int run = 0;
+  for (int r0 = 0; r0 < nranges; r0 += 8) {
+    int v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = r0 + k < nranges ? tcnt[(long long)(r0 + k) * nu + u] : 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (r0 + k < nranges) {
+        tcnt[(long long)(r0 + k) * nu + u] = run;
+        run += v[k];
+      }
+  }
+  cnt[u] = run;
+}
+
+// Exclusive scans, one CTA per array: out[i] = sum of in[0 .. i), out[n] (and total) = the sum of all.
+struct LayScan {
+  const long long *in[3];
+  long long n[3];
+  long long *out[3];
+  long long *total;
+};
+__global__ void __launch_bounds__(1024) k_lay_scan(LayScan S) {
+  __shared__ long long ws[32];
+  const long long *in = S.in[blockIdx.x], n = S.n[blockIdx.x];
+  long long *out = S.out[blockIdx.x];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  long long carry = 0;
+  for (long long i0 = 0; i0 < n; i0 += 4096) {
+    const long long i = i0 + 4 * t;
+    long long v[4], s = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = i + k < n ? in[i + k] : 0;
+      s += v[k];
+    }
+    long long x = s;
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[w] = x;
+    __syncthreads();
+    if (w == 0) {
+      long long y = ws[lane];
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long z = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) y += z;
+      }
+      ws[lane] = y;
+    }
+    __syncthreads();
+    long long run = carry + (w > 0 ? ws[w - 1] : 0) + x - s;
+    carry += ws[31];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k < n) {
+        out[i + k] = run;
+        run += v[k];
+      }
+    __syncthreads();  // ws is rewritten in the next round
+  }
+  if (t == 0) {
+    out[n] = carry;
+    S.total[blockIdx.x] = carry;
+  }
+}
+
+// One warp per range of bricks: its contributions into the pairs' lists, in order.  SMEM: the range's cursors are
+// copied to shared memory first.
+template <bool SMEM>
+__global__ void __launch_bounds__(32) k_lay_fill(const __grid_constant__ GTabs g, GNbr nb, long long nbricks,
+                                                const int *__restrict__ pair_u, int nu, long long per, int *tcnt,
+                                                const long long *__restrict__ hs_off, const long long *__restrict__ uoff,
+                                                long long *__restrict__ src) {
+  extern __shared__ int cursors[];
+  __shared__ int s_no[64], s_cum[64];
+  __shared__ long long s_row[64];
+  const int lane = threadIdx.x;
+  int *cur = tcnt + (long long)blockIdx.x * nu;
+  if (SMEM) {
+    for (int u = lane; u < nu; u += 32) cursors[u] = cur[u];
+    cur = cursors;
+  }
+  __syncwarp();
+  for (long long b = blockIdx.x * per; b < min(nbricks, (blockIdx.x + 1) * per); ++b) {
+    const long long s0 = nb.b_at_off[b], p0 = nb.b_pair_off[b], h0 = hs_off[b];
+    const int na = (int)(nb.b_at_off[b + 1] - s0);
+    int no[2], width, cum;
+    lay_slots(g, nb.s_atom, nb.atom_species, s0, na, lane, no, width, cum);
+    // exclusive prefixes over the slots: norb, and rows of upper tiles norb (cum - cum_a)
+    int before = 0;
+    long long rows = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int x = no[h];
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      const int ca = before + x - no[h];
+      long long r = (long long)no[h] * (cum - ca), rs = r;
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, rs, o);
+        if (lane >= o) rs += y;
+      }
+      s_no[lane + 32 * h] = no[h];
+      s_cum[lane + 32 * h] = ca;
+      s_row[lane + 32 * h] = rows + rs - r;
+      before += __shfl_sync(0xffffffffu, x, 31);
+      rows += __shfl_sync(0xffffffffu, rs, 31);
+    }
+    __syncwarp();
+    const int ne = na * (na + 1) / 2;
+    for (int e0 = 0; e0 < ne; e0 += 128) {
+      // four rounds' table look-ups in flight together, then the rounds in order
+      int u[4];
+      long long at[4], to[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int e = e0 + 32 * r + lane;
+        int a = 0, c = 0;
+        if (e < ne) lay_pair(e, na, a, c);
+        u[r] = e < ne ? nb.b_pair[p0 + a * na + c] : -1;
+        to[r] = h0 + s_row[a] + (long long)s_no[a] * (s_cum[c] - s_cum[a]);
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) u[r] = u[r] >= 0 ? pair_u[u[r]] : -1;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) at[r] = u[r] >= 0 ? uoff[u[r]] : 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        // lanes of one pair (two images of one atom in an unfolded brick) take consecutive places
+        const unsigned same = __match_any_sync(0xffffffffu, u[r] >= 0 ? u[r] : -1 - lane);
+        const int rank = __popc(same & ((1u << lane) - 1u));
+        int base = 0;
+        if (u[r] >= 0) base = SMEM ? cur[u[r]] : __ldcg(cur + u[r]);
+        __syncwarp();
+        if (u[r] >= 0) {
+          src[at[r] + base + rank] = to[r];
+          if (rank == 0) {
+            if (SMEM)
+              cur[u[r]] = base + __popc(same);
+            else
+              __stcg(cur + u[r], base + __popc(same));
+          }
+        }
+        __syncwarp();
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------ resident serving kernel
 // Continuous batching: one resident launch drains a device work queue to which the host appends jobs
 // (one task: the density / force and local-H passes of one system) while it runs.  A job's items, in
@@ -2396,19 +2621,19 @@ void gint_tc_free(gint_handle *h) {
   dfree(h->hu_pair);
   dfree(h->hu_off);
   dfree(h->hu_src);
+  dfree(h->pair_u);
+  dfree(h->lay_sz);
+  dfree(h->lay_cnt);
+  dfree(h->lay_tot);
+  h->cap_hs = h->cap_src = h->cap_plan = 0;
 }
 
-// Layouts of the tensor-core path for the current neighbour lists: D tile offsets, the padded
-// brick width, the local-H scratch offsets and the per-pair contribution lists (host, fixed
-// brick order so that the float64 reduction order is deterministic).
-int gint_tc_prepare(gint_handle *h) {
-  gint_tc_free(h);
-  h->tc_at_off.clear();  // set again once every layout below is built
-  h->tc_ent_off.clear();
-  h->tc_satom.clear();
+// What depends on the pair set and the grid only: D tile offsets and buffers, the upper pairs, and the arrays of
+// the layout kernels.  Once per handle.
+static int tc_allocate(gint_handle *h) {
   const GGeom &g = h->geom;
   const int na_tot = g.natoms;
-  // D tiles: roundup(norb(I), 8) x porb(J) per pair
+  const long long nb = g.nbricks;
   // D tiles: porb(I) x porb(J) per pair, stored column-atom-major (for each J its row atoms I in
   // ascending order), so that a brick's consecutive row atoms of one chunk are one copy
   auto find_pair = [&](int I, int J) -> int {
@@ -2417,230 +2642,127 @@ int gint_tc_prepare(gint_handle *h) {
     return (it != e && *it == J) ? (int)(it - h->pair_col.begin()) : -1;
   };
   h->tile_off.assign(h->npairs + 1, 0);
-  {
-    long long off = 0;
-    for (int J = 0; J < na_tot; ++J)
-      for (int q = h->pair_row[J]; q < h->pair_row[J + 1]; ++q) {
-        const int I = h->pair_col[q];  // pair (J, I) exists, so (I, J) does too
-        const int p = find_pair(I, J);
-        if (p < 0) return GINT_EINVAL;
-        h->tile_off[p] = off;
-        off += (long long)g.sp[h->species_host[I]].porb * g.sp[h->species_host[J]].porb;
+  std::vector<int> upair, pair_u(std::max(h->npairs, 1), -1);
+  long long off = 0;
+  for (int J = 0; J < na_tot; ++J)
+    for (int q = h->pair_row[J]; q < h->pair_row[J + 1]; ++q) {
+      const int I = h->pair_col[q];  // pair (J, I) exists, so (I, J) does too
+      const int p = find_pair(I, J);
+      if (p < 0) return GINT_EINVAL;
+      h->tile_off[p] = off;
+      off += (long long)g.sp[h->species_host[I]].porb * g.sp[h->species_host[J]].porb;
+      if (I >= J) {  // q is the pair (J, I), an upper one
+        pair_u[q] = (int)upair.size();
+        upair.push_back(q);
       }
-    h->tile_off[h->npairs] = off;
-  }
-  h->ntile_elems = h->tile_off[h->npairs];
+    }
+  h->tile_off[h->npairs] = off;
+  h->ntile_elems = off;
+  h->nupper = (int)upair.size();
+  // ranges of bricks: enough warps for the GPU, at least 8 bricks each, the count table at most 64 MB
+  h->lay_ranges = (int)std::max<long long>(
+      1, std::min<long long>({2LL * h->num_sms, nb / 8, (16LL << 20) / std::max(1, h->nupper)}));
   const size_t tbytes = std::max<long long>(h->ntile_elems, 64) * sizeof(__half);
+  const size_t lay = (size_t)h->lay_ranges * std::max(h->nupper, 1) * sizeof(int);
   if (cudaMalloc(&h->Dt_hl, 2 * tbytes) != cudaSuccess || cudaMalloc(&h->Dt_hl2, 2 * tbytes) != cudaSuccess ||
       cudaMalloc(&h->zero_dev, 512) != cudaSuccess ||
       cudaMalloc(&h->tile_off_dev, (h->npairs + 1) * sizeof(long long)) != cudaSuccess ||
-      cudaMalloc(&h->scales, 8 * sizeof(float)) != cudaSuccess) {
+      cudaMalloc(&h->scales, 8 * sizeof(float)) != cudaSuccess ||
+      cudaMalloc(&h->hu_pair, std::max(h->nupper, 1) * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&h->pair_u, pair_u.size() * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&h->hu_off, (h->nupper + 1) * sizeof(long long)) != cudaSuccess ||
+      cudaMalloc(&h->hs_brick_off, (nb + 1) * sizeof(long long)) != cudaSuccess ||
+      cudaMalloc(&h->plan_off_dev, (nb + 1) * sizeof(long long)) != cudaSuccess ||
+      cudaMalloc(&h->lay_sz, (2 * nb + h->nupper + 1) * sizeof(long long)) != cudaSuccess ||
+      cudaMalloc(&h->lay_cnt, lay) != cudaSuccess || cudaMalloc(&h->lay_tot, 4 * sizeof(long long)) != cudaSuccess) {
     cudaGetLastError();
     return GINT_ENOMEM;
   }
+  h->tc_bytes = 4 * (long long)tbytes + 512 + 8 * sizeof(float) + (long long)lay + 4 * sizeof(long long) +
+                (h->npairs + 1 + 2 * h->nupper + 2 + 4 * nb + 2) * (long long)sizeof(long long) +
+                (h->nupper + h->npairs) * (long long)sizeof(int);
   TC_CHECK(cudaMemset(h->zero_dev, 0, 512));
   TC_CHECK(cudaMemset(h->scales, 0, 8 * sizeof(float)));
-  TC_CHECK(cudaMemcpy(h->tile_off_dev, h->tile_off.data(), (h->npairs + 1) * sizeof(long long),
-                      cudaMemcpyHostToDevice));
-  // brick slot lists on the host
-  const long long nb = g.nbricks;
-  std::vector<long long> at_off(nb + 1);
-  std::vector<int> satom(std::max<long long>(h->nslots, 1));
-  TC_CHECK(cudaMemcpy(at_off.data(), h->b_at_off, (nb + 1) * sizeof(long long), cudaMemcpyDeviceToHost));
-  if (h->nslots) TC_CHECK(cudaMemcpy(satom.data(), h->s_atom, h->nslots * sizeof(int), cudaMemcpyDeviceToHost));
-  std::vector<long long> hs_off(nb + 1, 0);
-  std::vector<long long> cnt(h->npairs + 1, 0);
-  int npmax = 0;
-  std::vector<long long> ent_off(nb + 1);
-  TC_CHECK(cudaMemcpy(ent_off.data(), h->b_ent_off, (nb + 1) * sizeof(long long), cudaMemcpyDeviceToHost));
-  std::vector<long long> plan_off(nb + 1, 0);  // plan records, 16-byte units
-  // the bricks' slot-pair tables (global pair index or -1, row slot major), from the neighbour build
-  std::vector<long long> bp_off(nb + 1);
-  std::vector<int> bpair(std::max<long long>(h->npairtab, 1));
-  TC_CHECK(cudaMemcpy(bp_off.data(), h->b_pair_off, (nb + 1) * sizeof(long long), cudaMemcpyDeviceToHost));
-  if (h->npairtab) TC_CHECK(cudaMemcpy(bpair.data(), h->b_pair, h->npairtab * sizeof(int), cudaMemcpyDeviceToHost));
-  // pass 1: sizes and counts, the bricks split into nthr contiguous ranges on host threads; each
-  // range counts its own contributions per pair (tcnt), so that pass 2 can place them in brick
-  // order without a shared cursor
-  const int nthr = (int)std::max<long long>(1, std::min<long long>({16, (long long)std::thread::hardware_concurrency(),
-                                                                      (nb + 1023) / 1024}));
-  std::vector<long long> bstart(nthr + 1);
-  for (int k = 0; k <= nthr; ++k) bstart[k] = nb * k / nthr;
-  std::vector<std::vector<long long>> tcnt(nthr, std::vector<long long>(h->npairs, 0));
-  std::vector<long long> hs_sz(nb), plan_sz(nb);
-  std::vector<int> np_thr(nthr, 0);
-  auto pass1 = [&](int k) {
-    std::vector<int> nol;
-    long long *tc = tcnt[k].data();
-    for (long long b = bstart[k]; b < bstart[k + 1]; ++b) {
-      const long long s0 = at_off[b], s1 = at_off[b + 1];
-      int cur = 0;
-      long long cum = 0;
-      nol.assign(s1 - s0, 0);
-      for (long long s = s0; s < s1; ++s) {
-        const GSpecies &S = g.sp[h->species_host[satom[s]]];
-        cur = place_slot(cur, S.porb) + S.porb;
-        nol[s - s0] = S.norb;
-        cum += S.norb;
-      }
-      np_thr[k] = std::max(np_thr[k], (cur + 15) & ~15);
-      plan_sz[b] = plan_words((int)(s1 - s0), (int)(ent_off[b + 1] - ent_off[b]), (cur + 15) & ~15) / 4;
-      long long tot = 0, rest = cum;
-      for (long long a = 0; a < s1 - s0; ++a) {
-        tot += (long long)nol[a] * rest;
-        rest -= nol[a];
-      }
-      hs_sz[b] = (tot + 3) & ~3LL;  // 16-byte aligned ranges (one bulk copy each)
-      const long long nab = s1 - s0;
-      const int *bpb = bpair.data() + bp_off[b];
-      for (long long a = 0; a < nab; ++a)
-        for (long long c = a; c < nab; ++c) {
-          const int p = bpb[a * nab + c];
-          if (p >= 0) tc[p]++;
-        }
-    }
-  };
-  auto run_threads = [&](auto &&fn) {  // ranges 1.. on new threads (serially if none can start), 0 here
-    std::vector<std::thread> th;
-    int k = 1;
-    try {
-      for (; k < nthr; ++k) th.emplace_back(fn, k);
-    } catch (...) {
-    }
-    for (int r = k; r < nthr; ++r) fn(r);
-    fn(0);
-    for (auto &t : th) t.join();
-  };
-  run_threads(pass1);
-  for (long long b = 0; b < nb; ++b) {
-    plan_off[b + 1] = plan_off[b] + plan_sz[b];
-    hs_off[b + 1] = hs_off[b] + hs_sz[b];
-  }
-  for (int k = 0; k < nthr; ++k) {
-    npmax = std::max(npmax, np_thr[k]);
-    for (long long p = 0; p < h->npairs; ++p) cnt[p + 1] += tcnt[k][p];
-  }
-  h->max_brick_porb = npmax;
-  h->hs_elems = hs_off[nb];
-  // upper pairs (I <= J) and their contribution lists (CSR, brick order)
-  std::vector<int> upair;
-  std::vector<long long> uoff(1, 0);
-  std::vector<long long> pstart(h->npairs, -1);
-  for (int I = 0; I < na_tot; ++I)
-    for (int p = h->pair_row[I]; p < h->pair_row[I + 1]; ++p)
-      if (h->pair_col[p] >= I) {
-        pstart[p] = uoff.back();
-        upair.push_back(p);
-        uoff.push_back(uoff.back() + cnt[p + 1]);
-      }
-  std::vector<long long> src(std::max<long long>(uoff.back(), 1));
-  // each range's first place in every pair's list: the pair's start plus the earlier ranges' counts
-  for (long long p = 0; p < h->npairs; ++p) {
-    long long at = pstart[p];
-    for (int k = 0; k < nthr; ++k) {
-      const long long n = tcnt[k][p];
-      tcnt[k][p] = at;
-      at += n;
-    }
-  }
-  auto pass2 = [&](int k) {
-    std::vector<int> nol;
-    long long *cur = tcnt[k].data();
-    for (long long b = bstart[k]; b < bstart[k + 1]; ++b) {
-      const long long s0 = at_off[b], s1 = at_off[b + 1];
-      nol.assign(s1 - s0, 0);
-      long long cum = 0;
-      for (long long s = s0; s < s1; ++s) {
-        nol[s - s0] = g.sp[h->species_host[satom[s]]].norb;
-        cum += nol[s - s0];
-      }
-      long long rowst = 0, cumno_a = 0;
-      const long long nab = s1 - s0;
-      const int *bpb = bpair.data() + bp_off[b];
-      for (long long a = 0; a < nab; ++a) {
-        long long cumno_c = cumno_a;
-        for (long long c = a; c < nab; ++c) {
-          const int p = bpb[a * nab + c];
-          if (p >= 0) src[cur[p]++] = hs_off[b] + rowst + (long long)nol[a] * (cumno_c - cumno_a);
-          cumno_c += nol[c];
-        }
-        rowst += (long long)nol[a] * (cum - cumno_a);
-        cumno_a += nol[a];
-      }
-    }
-  };
-  run_threads(pass2);
-  h->nupper = (int)upair.size();
-  if (cudaMalloc(&h->hs_brick_off, (nb + 1) * sizeof(long long)) != cudaSuccess ||
-      cudaMalloc(&h->hs, std::max<long long>(h->hs_elems, 1) * sizeof(float)) != cudaSuccess ||
-      cudaMalloc(&h->hu_pair, std::max<size_t>(upair.size(), 1) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&h->hu_off, uoff.size() * sizeof(long long)) != cudaSuccess ||
-      cudaMalloc(&h->hu_src, src.size() * sizeof(long long)) != cudaSuccess) {
-    cudaGetLastError();
-    return GINT_ENOMEM;
-  }
-  h->tc_bytes = 4 * (long long)tbytes + 512 + (h->npairs + 1) * (long long)sizeof(long long) + 8 * sizeof(float) +
-                (nb + 1) * (long long)sizeof(long long) + std::max<long long>(h->hs_elems, 1) * (long long)sizeof(float) +
-                (long long)std::max<size_t>(upair.size(), 1) * (long long)sizeof(int) +
-                (long long)(uoff.size() + src.size()) * (long long)sizeof(long long);
-  TC_CHECK(cudaMemcpy(h->hs_brick_off, hs_off.data(), (nb + 1) * sizeof(long long), cudaMemcpyHostToDevice));
-  if (!upair.empty())
-    TC_CHECK(cudaMemcpy(h->hu_pair, upair.data(), upair.size() * sizeof(int), cudaMemcpyHostToDevice));
-  TC_CHECK(cudaMemcpy(h->hu_off, uoff.data(), uoff.size() * sizeof(long long), cudaMemcpyHostToDevice));
-  TC_CHECK(cudaMemcpy(h->hu_src, src.data(), src.size() * sizeof(long long), cudaMemcpyHostToDevice));
-  // brick plan records, built on the device by the slow-path metadata code itself
-  if (cudaMalloc(&h->plan_off_dev, (nb + 1) * sizeof(long long)) != cudaSuccess ||
-      cudaMalloc(&h->plan, std::max<long long>(plan_off[nb], 1) * 16) != cudaSuccess) {
-    cudaGetLastError();
-    return GINT_ENOMEM;
-  }
-  h->tc_bytes += (nb + 1) * (long long)sizeof(long long) + std::max<long long>(plan_off[nb], 1) * 16;
-  TC_CHECK(cudaMemcpy(h->plan_off_dev, plan_off.data(), (nb + 1) * sizeof(long long), cudaMemcpyHostToDevice));
-  // (bricks beyond the kernels' capacity get no records: compute calls report GINT_ECAPACITY)
-  if (nb > 0 && h->max_brick_atoms <= kMAXA && h->max_brick_ent <= kMAXE && h->max_brick_porb <= kNPMAX) {
-    TC_CHECK(cudaMemset(h->err_word, 0, sizeof(unsigned)));
-    k_build_plans<<<(unsigned)nb, 128>>>(h->geom, static_cast<const GCell &>(h->geom), h->nbr(), h->tile_off_dev,
-                                         h->plan_off_dev, reinterpret_cast<uint32_t *>(h->plan), h->err_word);
-    TC_CHECK(cudaGetLastError());
-    TC_CHECK(cudaDeviceSynchronize());
-    unsigned err = 0;
-    TC_CHECK(cudaMemcpy(&err, h->err_word, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (err) return GINT_EDEVICE;
-  }
-  satom.resize(h->nslots);
-  h->tc_at_off.swap(at_off);
-  h->tc_ent_off.swap(ent_off);
-  h->tc_satom.swap(satom);
+  TC_CHECK(cudaMemcpy(h->tile_off_dev, h->tile_off.data(), (h->npairs + 1) * sizeof(long long), cudaMemcpyHostToDevice));
+  if (h->nupper) TC_CHECK(cudaMemcpy(h->hu_pair, upair.data(), upair.size() * sizeof(int), cudaMemcpyHostToDevice));
+  TC_CHECK(cudaMemcpy(h->pair_u, pair_u.data(), pair_u.size() * sizeof(int), cudaMemcpyHostToDevice));
   return GINT_OK;
 }
 
-// New positions, neighbour lists rebuilt: when every brick keeps its slots (the same atoms in the
-// same order) and its entry count, the D tile layout, the scratch ranges and the per-pair
-// contribution lists stay valid and only the plan records (entry positions relative to the brick)
-// change, so only k_build_plans runs again; otherwise the layouts are rebuilt (gint_tc_prepare).
-int gint_tc_refresh(gint_handle *h) {
-  const long long nb = h->geom.nbricks;
-  if (!h->Dt_hl || !h->plan || (long long)h->tc_at_off.size() != nb + 1 ||
-      (long long)h->tc_ent_off.size() != nb + 1 || (long long)h->tc_satom.size() != h->nslots)
-    return gint_tc_prepare(h);
-  std::vector<long long> at_off(nb + 1), ent_off(nb + 1);
-  std::vector<int> satom(std::max<long long>(h->nslots, 1));
-  TC_CHECK(cudaMemcpy(at_off.data(), h->b_at_off, (nb + 1) * sizeof(long long), cudaMemcpyDeviceToHost));
-  TC_CHECK(cudaMemcpy(ent_off.data(), h->b_ent_off, (nb + 1) * sizeof(long long), cudaMemcpyDeviceToHost));
-  if (h->nslots) TC_CHECK(cudaMemcpy(satom.data(), h->s_atom, h->nslots * sizeof(int), cudaMemcpyDeviceToHost));
-  satom.resize(h->nslots);
-  if (at_off != h->tc_at_off || ent_off != h->tc_ent_off || satom != h->tc_satom) return gint_tc_prepare(h);
-  if (nb > 0 && h->max_brick_atoms <= kMAXA && h->max_brick_ent <= kMAXE && h->max_brick_porb <= kNPMAX) {
-    TC_CHECK(cudaMemset(h->err_word, 0, sizeof(unsigned)));
-    k_build_plans<<<(unsigned)nb, 128>>>(h->geom, static_cast<const GCell &>(h->geom), h->nbr(), h->tile_off_dev,
-                                         h->plan_off_dev, reinterpret_cast<uint32_t *>(h->plan), h->err_word);
-    TC_CHECK(cudaGetLastError());
-    TC_CHECK(cudaDeviceSynchronize());
-    unsigned err = 0;
-    TC_CHECK(cudaMemcpy(&err, h->err_word, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (err) return GINT_EDEVICE;
+// A buffer of at least n elements of T: kept when it is large enough, otherwise replaced (exactly n the first
+// time, an eighth more after that, so that moving atoms do not reallocate at every step).
+template <typename T>
+static int tc_reserve(gint_handle *h, T *&p, long long &cap, long long n) {
+  n = std::max(n, 1LL);
+  if (p && n <= cap) return GINT_OK;
+  const long long want = p ? n + n / 8 : n;
+  dfree(p);
+  h->tc_bytes -= cap * (long long)sizeof(T);
+  cap = 0;
+  if (cudaMalloc(&p, want * sizeof(T)) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+    return GINT_ENOMEM;
   }
+  cap = want;
+  h->tc_bytes += cap * (long long)sizeof(T);
   return GINT_OK;
+}
+
+// Layouts of the tensor-core path for the current neighbour lists: scratch ranges, contribution lists and plan
+// records.  Synchronous on st.
+static int tc_layouts(gint_handle *h, cudaStream_t st) {
+  const GGeom &g = h->geom;
+  const long long nb = g.nbricks;
+  const int nu = h->nupper, nr = h->lay_ranges;
+  const long long per = (nb + nr - 1) / nr;
+  long long *hs_sz = h->lay_sz, *plan_sz = hs_sz + nb, *cnt = plan_sz + nb;
+  TC_CHECK(cudaMemsetAsync(h->lay_cnt, 0, (size_t)nr * std::max(nu, 1) * sizeof(int), st));
+  TC_CHECK(cudaMemsetAsync(h->lay_tot, 0, 4 * sizeof(long long), st));
+  const unsigned wg = (unsigned)((nb + kLayWarps - 1) / kLayWarps);
+  k_lay_count<<<wg, 32 * kLayWarps, 0, st>>>(g, h->nbr(), h->b_ent_off, nb, h->pair_u, nu, per, h->lay_cnt, hs_sz, plan_sz,
+                                            reinterpret_cast<int *>(h->lay_tot + 3));
+  k_lay_cols<<<(unsigned)((nu + 127) / 128), 128, 0, st>>>(nu, nr, h->lay_cnt, cnt);
+  const LayScan S{{hs_sz, plan_sz, cnt}, {nb, nb, nu}, {h->hs_brick_off, h->plan_off_dev, h->hu_off}, h->lay_tot};
+  k_lay_scan<<<3, 1024, 0, st>>>(S);
+  TC_CHECK(cudaGetLastError());
+  long long tot[4];
+  TC_CHECK(cudaMemcpyAsync(tot, h->lay_tot, sizeof(tot), cudaMemcpyDeviceToHost, st));
+  TC_CHECK(cudaStreamSynchronize(st));
+  h->hs_elems = tot[0];
+  h->max_brick_porb = (int)tot[3];
+  int rc;
+  if ((rc = tc_reserve(h, h->hs, h->cap_hs, tot[0])) || (rc = tc_reserve(h, h->plan, h->cap_plan, tot[1])) ||
+      (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2])))
+    return rc;
+  if ((size_t)nu * sizeof(int) <= kLaySmem) {
+    if ((rc = set_smem(k_lay_fill<true>, kLaySmem))) return rc;
+    k_lay_fill<true><<<(unsigned)nr, 32, nu * sizeof(int), st>>>(g, h->nbr(), nb, h->pair_u, nu, per, h->lay_cnt,
+                                                                h->hs_brick_off, h->hu_off, h->hu_src);
+  } else {
+    k_lay_fill<false><<<(unsigned)nr, 32, 0, st>>>(g, h->nbr(), nb, h->pair_u, nu, per, h->lay_cnt, h->hs_brick_off,
+                                                  h->hu_off, h->hu_src);
+  }
+  TC_CHECK(cudaGetLastError());
+  // brick plan records, built by the slow-path metadata code itself
+  // (bricks beyond the kernels' capacity get no records: compute calls report GINT_ECAPACITY)
+  unsigned err = 0;
+  if (nb > 0 && h->max_brick_atoms <= kMAXA && h->max_brick_ent <= kMAXE && h->max_brick_porb <= kNPMAX) {
+    TC_CHECK(cudaMemsetAsync(h->err_word, 0, sizeof(unsigned), st));
+    k_build_plans<<<(unsigned)nb, 128, 0, st>>>(h->geom, static_cast<const GCell &>(h->geom), h->nbr(), h->tile_off_dev,
+                                                h->plan_off_dev, reinterpret_cast<uint32_t *>(h->plan), h->err_word);
+    TC_CHECK(cudaGetLastError());
+    TC_CHECK(cudaMemcpyAsync(&err, h->err_word, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+  }
+  TC_CHECK(cudaStreamSynchronize(st));
+  return err ? GINT_EDEVICE : GINT_OK;
+}
+
+int gint_tc_prepare(gint_handle *h, cudaStream_t st) {
+  int rc = h->Dt_hl ? GINT_OK : tc_allocate(h);
+  if (!rc) rc = tc_layouts(h, st);
+  if (rc) gint_tc_free(h);  // compute calls report GINT_ECAPACITY
+  return rc;
 }
 
 int gint_tc_check_capacity(const gint_handle *h) {
