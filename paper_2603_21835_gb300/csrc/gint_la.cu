@@ -25,6 +25,18 @@
 namespace gla {
 namespace {
 
+// Programmatic dependent launch: the kernels below are launched while their predecessor runs; everything up to
+// here (arguments, index arithmetic) overlaps its tail, and this waits until its results are visible.  The
+// successor may be launched from here on.
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ double shfl(double x, int lane) { return __shfl_sync(0xffffffffu, x, lane); }
+__device__ __forceinline__ double2 shfl(double2 x, int lane) {
+  return make_double2(__shfl_sync(0xffffffffu, x.x, lane), __shfl_sync(0xffffffffu, x.y, lane));
+}
+
 // scalar arithmetic for T = double and T = double2 (complex, no conjugation anywhere)
 template <typename T>
 struct Ar;
@@ -33,7 +45,10 @@ struct Ar<double> {
   static __device__ __forceinline__ double zero() { return 0.0; }
   static __device__ __forceinline__ double fms(double a, double b, double c) { return ::fma(-a, b, c); }  // c - a b
   static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
-  static __device__ __forceinline__ double inv(double d) { return 1.0 / d; }
+  static __device__ __forceinline__ double scale(double a, double s) { return a * s; }
+  // reciprocal's denominator and numerator: 1 / d = num / den
+  static __device__ __forceinline__ double den(double d) { return d; }
+  static __device__ __forceinline__ double num(double) { return 1.0; }
   static __device__ __forceinline__ bool bad_pivot(double d, bool spd) { return spd ? !(d > 0.0) : !(d != 0.0 && isfinite(d)); }
 };
 template <>
@@ -42,14 +57,13 @@ struct Ar<double2> {
   static __device__ __forceinline__ double2 fms(double2 a, double2 b, double2 c) {
     return make_double2(::fma(a.y, b.y, ::fma(-a.x, b.x, c.x)), ::fma(-a.y, b.x, ::fma(-a.x, b.y, c.y)));
   }
+  static __device__ __forceinline__ double2 scale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
   static __device__ __forceinline__ double2 mul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
   }
   // 1 / d = conj(d) / |d|^2
-  static __device__ __forceinline__ double2 inv(double2 d) {
-    const double q = 1.0 / (d.x * d.x + d.y * d.y);
-    return make_double2(d.x * q, -d.y * q);
-  }
+  static __device__ __forceinline__ double den(double2 d) { return ::fma(d.y, d.y, d.x * d.x); }
+  static __device__ __forceinline__ double2 num(double2 d) { return make_double2(d.x, -d.y); }
   static __device__ __forceinline__ bool bad_pivot(double2 d, bool) {
     const double m = d.x * d.x + d.y * d.y;
     return !(m > 0.0 && isfinite(m));
@@ -59,66 +73,107 @@ struct Ar<double2> {
 // ------------------------------------------------------------------------ L D L^T, diagonal block
 constexpr int kDT = 256;
 
+// 1 / q to float64 rounding: the float32 reciprocal and one third-order Newton step, r (1 + e + e^2) with
+// e = 1 - q r below 2^-22: four dependent float64 instructions where the division is about ten.  Outside the
+// float32 range (and for zeros, infinities and NaNs) the division itself.
+__device__ __forceinline__ double recip(double q) {
+  const float f = (float)q;
+  if (!(fabsf(f) > 1e-30f && fabsf(f) < 1e30f)) return 1.0 / q;
+  const double r = (double)__frcp_rn(f), e = fma(-q, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // One CTA factors the nb x nb diagonal block, right-looking: at step j, l_kj = a_kj / d_j, then
-// a_ik -= a_ij l_kj for i >= k > j.  The elements stay in the registers of their threads (column-major
-// triangular order, so a thread's elements finish early); the column of the next step is published in
-// shared memory.  Warp 0 alone forms 1 / d_j and the scaled column: a float64 division is some forty
-// dependent instructions, and every further warp that repeats it takes the pipe from the others (the
-// former kernel, all eight warps dividing: 170 us for a complex block of 64; this one 22 us for one of 32).
+// a_ik -= a_ij l_kj for i >= k > j.  The float64 chain from one pivot to the next sets the time, so warp 0 does
+// nothing else: it holds column j + 1 (lane = row), applies step j to it, and forms its reciprocal and scaled
+// column while the other warps apply step j to the columns behind.  Their elements stay in registers, packed
+// from the triangle's last column backwards so that active ones fill whole warps; the column that warp 0 needs
+// next is published in shared memory.  One barrier a step.  (Complex, NB = 32: 34 us with two barriers and a
+// division in the chain, 30 us so; eight warps that all divided took 170 us for a block of 64.)
 template <typename T>
 __global__ void __launch_bounds__(kDT) k_ldl_diag(int nb, T *__restrict__ A, long long lda, int j0, int spd,
                                                   int *__restrict__ info, T *__restrict__ dinv) {
-  constexpr int NB = LdlBlock<T>::NB, NE = NB * (NB + 1) / 2, PER = (NE + kDT - 1) / kDT;
-  __shared__ T col[2][NB], lcol[NB];
+  constexpr int NB = LdlBlock<T>::NB, RL = NB / 32, NW = kDT - 32;
+  constexpr int NE = NB * (NB - 1) / 2, PER = (NE + NW - 1) / NW;  // elements of columns 1 .. NB - 1
+  __shared__ T pub[2][NB], cbuf[2][NB], lbuf[2][NB];
   const int tid = threadIdx.x;
-  T a[PER];
-  int ei[PER], ek[PER];
+  grid_wait();
+  if (tid < 32) {
+    const int lane = tid;
+    bool bad = false;
+    // column j of the factor: x (rows lane, lane + 32) final, published with l = x / d
+    auto finish = [&](int j, const T *x) {
+      T d = Ar<T>::zero();
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    int e = tid + kDT * q, k = 0;
-    ei[q] = ek[q] = -1;
-    a[q] = Ar<T>::zero();
-    if (e < NE) {
-      // column k starts at k NB - k (k - 1) / 2
-      k = (int)((2 * NB + 1 - sqrtf((float)((2 * NB + 1) * (2 * NB + 1) - 8 * e))) * 0.5f);
-      while (k > 0 && k * NB - k * (k - 1) / 2 > e) --k;
-      while ((k + 1) * NB - (k + 1) * k / 2 <= e) ++k;
-      const int i = k + (e - (k * NB - k * (k - 1) / 2));
-      if (i < nb && k < nb) {
-        ei[q] = i;
-        ek[q] = k;
-        a[q] = A[i + k * lda];
-        if (k == 0) col[0][i] = a[q];
+      for (int r = 0; r < RL; ++r) {
+        T v = shfl(x[r], j & 31);
+        if (r == (j >> 5)) d = v;
       }
-    }
-  }
-  bool bad = false;
-  for (int j = 0; j < nb; ++j) {
-    const T *c = col[j & 1];
-    __syncthreads();  // column j is published
-    if (tid < 32) {
-      const T d = c[j], di = Ar<T>::inv(d);
-      if (tid == 0) {
+      const double q = recip(Ar<T>::den(d));
+      const T nu = Ar<T>::num(d);
+#pragma unroll
+      for (int r = 0; r < RL; ++r) {
+        const int i = lane + 32 * r;
+        const T l = Ar<T>::scale(Ar<T>::mul(x[r], nu), q);
+        cbuf[j & 1][i] = x[r];
+        lbuf[j & 1][i] = l;
+        if (i > j && i < nb) A[i + j * lda] = l;
+      }
+      if (lane == 0) {
         if (!bad && Ar<T>::bad_pivot(d, spd)) {
           bad = true;
           atomicCAS(info, 0, j0 + j + 1);
         }
-        dinv[j] = di;
+        dinv[j] = Ar<T>::scale(nu, q);
         A[j + j * lda] = d;
       }
-      for (int k = j + 1 + tid; k < nb; k += 32) {
-        const T l = Ar<T>::mul(c[k], di);
-        lcol[k] = l;
-        A[k + j * lda] = l;
+    };
+    T x[RL];
+#pragma unroll
+    for (int r = 0; r < RL; ++r) x[r] = lane + 32 * r < nb ? A[lane + 32 * r] : Ar<T>::zero();
+    finish(0, x);
+    for (int j = 0; j + 1 < nb; ++j) {
+      __syncthreads();
+      const T lk = lbuf[j & 1][j + 1];
+#pragma unroll
+      for (int r = 0; r < RL; ++r) {
+        const int i = lane + 32 * r;
+        x[r] = i > j && i < nb ? Ar<T>::fms(cbuf[j & 1][i], lk, pub[(j + 1) & 1][i]) : Ar<T>::zero();
+      }
+      finish(j + 1, x);
+    }
+  } else {
+    T a[PER];
+    int ei[PER], ek[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      // position e from the end of the column-major triangle: column NB - 1 - c has c + 1 elements
+      const int e = tid - 32 + NW * q;
+      ei[q] = ek[q] = -1;
+      a[q] = Ar<T>::zero();
+      if (e < NE) {
+        int c = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+        while (c * (c + 1) / 2 > e) --c;
+        while ((c + 1) * (c + 2) / 2 <= e) ++c;
+        const int k = NB - 1 - c, i = k + (e - c * (c + 1) / 2);
+        if (i < nb) {
+          ei[q] = i;
+          ek[q] = k;
+          a[q] = A[i + k * lda];
+          if (k == 1) pub[1][i] = a[q];
+        }
       }
     }
-    __syncthreads();
+    for (int j = 0; j + 1 < nb; ++j) {
+      __syncthreads();
+      const T *c = cbuf[j & 1], *l = lbuf[j & 1];
 #pragma unroll
-    for (int q = 0; q < PER; ++q)
-      if (ek[q] > j) {
-        a[q] = Ar<T>::fms(c[ei[q]], lcol[ek[q]], a[q]);
-        if (ek[q] == j + 1) col[(j + 1) & 1][ei[q]] = a[q];
-      }
+      for (int q = 0; q < PER; ++q)
+        if (ek[q] >= j + 2) {
+          a[q] = Ar<T>::fms(c[ei[q]], l[ek[q]], a[q]);
+          if (ek[q] == j + 2) pub[(j + 2) & 1][ei[q]] = a[q];
+        }
+    }
   }
 }
 
@@ -145,6 +200,7 @@ __global__ void __launch_bounds__(NB * SV) k_trsv(int nb, const T *__restrict__ 
   T *Ls = reinterpret_cast<T *>(smem_raw);  // Ls[i + j NB] = L(i, j), or L(j, i) for TRANS
   T *xs = Ls + NB * NB;                     // [element][vector]
   const int tid = threadIdx.x, vl = tid % SV, i = tid / SV, v = blockIdx.x * SV + vl;
+  grid_wait();
   for (int e = tid; e < NB * NB; e += NB * SV) {
     const int r = e % NB, c = e / NB;
     if (r < nb && c < nb && (TRANS ? r < c : r > c)) Ls[e] = TRANS ? L[c + (long long)r * ldl] : L[r + (long long)c * ldl];
@@ -188,11 +244,6 @@ int set_smem(F *f, size_t bytes) {
              : GINT_ECUDA;
 }
 
-#define LA_CHECK()                                   \
-  do {                                               \
-    if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA; \
-  } while (0)
-
 // Operand views and C strides of real and complex column-major blocks.
 inline SgView left(const double *p, long long sr, long long sk) { return sg_real(p, sr, sk); }
 inline SgView left(const double2 *p, long long sr, long long sk) { return sg_cplx_left(p, sr, sk); }
@@ -226,10 +277,8 @@ int trsv(int nb, const T *L, long long ldl, int nv, Vecs<T> X, int nv2, Vecs<T> 
   constexpr int NB = LdlBlock<T>::NB;
   const size_t smem = (size_t)(NB * NB + NB * SV) * sizeof(T);
   if (set_smem(k_trsv<T, NB, SV, TRANS, PANEL>, smem) != GINT_OK) return GINT_ECUDA;
-  k_trsv<T, NB, SV, TRANS, PANEL><<<(unsigned)((nv + nv2 + SV - 1) / SV), NB * SV, smem, st>>>(nb, L, ldl, nv, X, nv2, X2,
-                                                                                               W, ldw, dinv);
-  LA_CHECK();
-  return GINT_OK;
+  return sg_launch(k_trsv<T, NB, SV, TRANS, PANEL>, dim3((unsigned)((nv + nv2 + SV - 1) / SV)), NB * SV, smem, st, nb, L, ldl,
+                   nv, X, nv2, X2, W, ldw, dinv);
 }
 
 }  // namespace
@@ -244,8 +293,7 @@ int ldl_factor_solve(int n, T *A, long long lda, int nrhs, T *B, long long ldb, 
   for (int j0 = 0; j0 < n; j0 += NB) {
     const int nb = std::min(NB, n - j0), m = n - j0 - nb;
     T *A11 = A + j0 + (long long)j0 * lda, *A21 = A11 + nb, *B1 = B + j0;
-    k_ldl_diag<T><<<1, kDT, 0, st>>>(nb, A11, lda, j0, spd ? 1 : 0, info, dinv + j0);
-    LA_CHECK();
+    if ((rc = sg_launch(k_ldl_diag<T>, dim3(1), kDT, 0, st, nb, A11, lda, j0, spd ? 1 : 0, info, dinv + j0))) return rc;
     // panel rows: W = A21 L11^-T, L21 = W D1^-1, and the same for the right-hand sides
     if (m + nrhs > 0 && (rc = trsv<T, 8, false, true>(nb, A11, lda, m, Vecs<T>{A21, 1, lda}, nrhs, Vecs<T>{B1, ldb, 1}, W,
                                                       ldw, dinv + j0, st)))

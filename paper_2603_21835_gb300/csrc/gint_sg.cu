@@ -55,6 +55,12 @@ constexpr unsigned kErrTimeout = 1u, kErrInflight = 2u;
 constexpr int kNonFinite = 2047;         // row exponent field of a row with an infinity or a NaN
 static_assert(kDig * kTN == 512, "the levels fill the tensor memory");
 
+// See sg_launch: wait for the predecessor's results, then let the successor be launched.
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ double sg_at(const SgView &v, int r, int k) {
   if (v.rot) {
     const double x = v.p[(long long)(r >> 1) * v.rh + (long long)(k >> 1) * v.kh + ((r ^ k) & 1)];
@@ -115,6 +121,7 @@ __global__ void __launch_bounds__(kPT) k_sg_max(const __grid_constant__ SgPack P
   int rb;
   const SgOperand &o = sg_operand(P, rb);
   const int r0 = rb * kPR;
+  grid_wait();
   sg_load_tile(o, r0, blockIdx.y * kPK, t);
   __syncthreads();
   const int m = sg_row_exp(t), r = r0 + (threadIdx.x >> 3);
@@ -129,6 +136,7 @@ __global__ void __launch_bounds__(kPT) k_sg_pack(const __grid_constant__ SgPack 
   int rb;
   const SgOperand &o = sg_operand(P, rb);
   const int r0 = rb * kPR, kb = ONE ? 0 : (int)blockIdx.y * kPK;
+  grid_wait();
   sg_load_tile(o, r0, kb, t);
   __syncthreads();
   const int rl = threadIdx.x >> 3, g = threadIdx.x & 7, r = r0 + rl;
@@ -329,6 +337,7 @@ __global__ void __launch_bounds__(kSgThreads, 1) k_sg_mma(const __grid_constant_
   const uint32_t tmem = sh.tmem;
   unsigned *status = P.status;
   const int n0 = P.pr[0].ntiles;
+  grid_wait();
 
   if (warp == kLoadWarp) {
     // the copies run kStages chunks ahead of the MMAs, across tile boundaries
@@ -480,23 +489,27 @@ __global__ void __launch_bounds__(kSgThreads, 1) k_sg_mma(const __grid_constant_
       const uint32_t flip = p.neg ? 0x80000000u : 0u;
       const int jend = p.mode == 0 ? p.N : min(p.N, (i >> p.cs) + 1);  // columns of this row that are wanted
       const int jn = rowok ? jend - jb : 0;
+      double old[2][4];  // the next four old values travel while the current four are converted
+      auto fetch = [&](int j4) {
+        double *const o = old[(j4 >> 2) & 1];
+        const double *const c = Ci + (long long)(j4 >> 1) * p.cch;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          o[q] = p.beta && j4 + q < jn ? c[(q >> 1) * p.cch + ((q & 1) ? p.ccl : 0)] : 0.0;
+      };
+      fetch(0);
 #pragma unroll
       for (int j4 = 0; j4 < 16; j4 += 4) {
         if (__all_sync(0xffffffffu, j4 >= jn)) break;
+        if (j4 < 12) fetch(j4 + 4);
         const int4 e4 = __ldg(eb4 + j4 / 4);
         const int eb[4] = {e4.x, e4.y, e4.z, e4.w};
         double *const Cj[2] = {Ci + (long long)(j4 >> 1) * p.cch, Ci + (long long)((j4 >> 1) + 1) * p.cch};
-        double old[4] = {0.0, 0.0, 0.0, 0.0};
-        if (p.beta) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (j4 + q < jn) old[q] = Cj[q >> 1][(q & 1) ? p.ccl : 0];
-        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           double v = fx_to_double(x[j4 + q], ea + eb[q] - 2 * 1022 - 68);
           v = __hiloint2double(__double2hiint(v) ^ flip, __double2loint(v));
-          if (p.beta) v += old[q];
+          if (p.beta) v += old[(j4 >> 2) & 1][q];
           if (j4 + q < jn && max(ea, eb[q]) != kNonFinite) {
             Cj[q >> 1][(q & 1) ? p.ccl : 0] = v;
             const int j = jb + j4 + q;
@@ -591,16 +604,17 @@ int sg_gemm(const SgProduct *pr, int np, const SgWork &ws, cudaStream_t st) {
     if (off > ws.bytes) return GINT_EINVAL;
     for (int q = nop; q < 5; ++q) pk.first[q] = blocks;
     if (ar.tiles == 0) return GINT_OK;
+    int rc;
     if (kk <= kPK) {
-      k_sg_pack<true><<<blocks, kPT, 0, st>>>(pk);
+      if ((rc = sg_launch(k_sg_pack<true>, dim3((unsigned)blocks), kPT, 0, st, pk))) return rc;
     } else {
       if (cudaMemsetAsync(e0, 0, (size_t)erows * sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
       const dim3 g((unsigned)blocks, (unsigned)((kk + kPK - 1) / kPK));
-      k_sg_max<<<g, kPT, 0, st>>>(pk);
-      k_sg_pack<false><<<g, kPT, 0, st>>>(pk);
+      k_sg_max<<<g, kPT, 0, st>>>(pk);  // after a copy engine's work: plain stream order
+      if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA;
+      if ((rc = sg_launch(k_sg_pack<false>, g, kPT, 0, st, pk))) return rc;
     }
-    k_sg_mma<<<std::min(ws.num_sms, ar.tiles), kSgThreads, kSgSmem, st>>>(ar);
-    if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA;
+    if ((rc = sg_launch(k_sg_mma, dim3((unsigned)std::min(ws.num_sms, ar.tiles)), kSgThreads, kSgSmem, st, ar))) return rc;
   }
   return GINT_OK;
 }

@@ -5,7 +5,28 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
+#include <utility>
+
+#include "gint.h"
+
 namespace gla {
+
+// Launch in stream order with programmatic serialization: the kernel may begin while its predecessor on the
+// stream is still running and must execute griddepcontrol.wait before it touches what that one wrote.
+template <typename... P, typename... Q>
+int sg_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Q &&...args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kern, static_cast<P>(std::forward<Q>(args))...) == cudaSuccess ? GINT_OK : GINT_ECUDA;
+}
 
 // Real operand view of a product: element (r, k), r the output row (or column) index and k the
 // contraction index, is
