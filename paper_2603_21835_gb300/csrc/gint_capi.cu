@@ -47,10 +47,11 @@ void dfree(T *&p) {
 }
 
 void free_all(gint_handle *h) {
-  dfree(h->tab64); dfree(h->tab32); dfree(h->tab32i); dfree(h->dtab32); dfree(h->dtab32i);
+  dfree(h->tab64); dfree(h->otab64); dfree(h->tab32); dfree(h->tab32i); dfree(h->dtab32); dfree(h->dtab32i);
   dfree(h->pos_dev); dfree(h->species_dev);
   dfree(h->pair_row_dev); dfree(h->pair_col_dev); dfree(h->pair_off_dev); dfree(h->pair_T_dev); dfree(h->pair_I_dev);
   dfree(h->n_at); dfree(h->n_ent); dfree(h->n_orb); dfree(h->frac_dev); dfree(h->b_list);
+  dfree(h->fx_eD); dfree(h->atom_off_dev);
   dfree(h->b_at_off); dfree(h->b_ent_off); dfree(h->b_pair_off); dfree(h->scan_out);
   dfree(h->s_atom); dfree(h->s_col); dfree(h->s_ent); dfree(h->e_shift); dfree(h->b_pair);
   dfree(h->D32); dfree(h->work_ctr); dfree(h->red); dfree(h->scal); dfree(h->err_word);
@@ -313,6 +314,37 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
   TRY(dalloc(&h->dtab32i, d32i.size()));
   TRYCU(cudaMemcpy(h->dtab32, d32.data(), d32.size() * sizeof(float), cudaMemcpyHostToDevice));
   TRYCU(cudaMemcpy(h->dtab32i, d32i.data(), d32i.size() * sizeof(float), cudaMemcpyHostToDevice));
+  // tables of the float64 evaluators: per knot and radial (f, f_{k+1} - f_k, dr f'_k, dr f'_{k+1}), times the Y_lm
+  // constant of the shell
+  {
+    h->tabs64 = g;
+    std::vector<double> o;
+    const double cl[3] = {0.28209479177387814347, 0.48860251190291992159, 1.09254843059207907054};
+    for (int s = 0; s < d->nspecies; ++s) {
+      GSpecies &S = h->tabs64.sp[s];
+      S.ioff = (int)(o.size() / 4);
+      S.kslot = 0;
+      switch (S.shape) {
+#define CASE_O64(ns, np, nd, no) case GINT_SHAPE(ns, np, nd):
+        GINT_O64_SHAPES(CASE_O64)
+#undef CASE_O64
+        break;
+        default: S.shape = 0; continue;
+      }
+      for (int k = 0; k < S.nrad; ++k)
+        if (g.rad[S.rad0 + k].rc != S.rcut) S.kslot = 1;
+      for (int i = 0; i + 1 < g.rad[S.rad0].npts; ++i)
+        for (int k = 0; k < S.nrad; ++k) {
+          const GRadial &R = g.rad[S.rad0 + k];
+          const double2 *T = t64.data() + R.off + i;
+          const double c = cl[R.l];
+          for (double x : {T[0].x, T[1].x - T[0].x, R.dr * T[0].y, R.dr * T[1].y}) o.push_back(c * x);
+        }
+    }
+    h->notab64 = (long long)o.size();
+    TRY(dalloc(&h->otab64, o.size()));
+    if (!o.empty()) TRYCU(cudaMemcpy(h->otab64, o.data(), o.size() * sizeof(double), cudaMemcpyHostToDevice));
+  }
   // atoms
   h->pos_host.assign(d->pos, d->pos + 3 * (size_t)d->natoms);
   h->species_host.assign(d->species, d->species + d->natoms);
@@ -324,6 +356,9 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
     h->atom_off[a + 1] = h->atom_off[a] + h->atom_norb[a];
   }
   h->norb = h->atom_off[d->natoms];
+  TRY(dalloc(&h->atom_off_dev, (size_t)d->natoms + 1));
+  TRY(dalloc(&h->fx_eD, (size_t)h->norb));
+  TRYCU(cudaMemcpy(h->atom_off_dev, h->atom_off.data(), (d->natoms + 1) * sizeof(int), cudaMemcpyHostToDevice));
   TRY(dalloc(&h->pos_dev, 3 * (size_t)d->natoms));
   TRY(dalloc(&h->species_dev, (size_t)d->natoms));
   TRYCU(cudaMemcpy(h->pos_dev, h->pos_host.data(), h->pos_host.size() * sizeof(double), cudaMemcpyHostToDevice));
@@ -500,8 +535,9 @@ int gint_brick_lists(const gint_handle *h, long long *nslots, long long *nentrie
 int gint_memory(const gint_handle *h, long long *device_bytes) {
   if (!h || !device_bytes) return GINT_EINVAL;
   const long long nb = h->geom.nbricks, na = h->geom.natoms, np = h->npairs, L = sizeof(long long);
-  long long b = h->nknots * (long long)(sizeof(double2) + sizeof(float2) + sizeof(float)) + h->nknots_i * 12;  // tables
-  b += na * (3 * (long long)sizeof(double) + 4);                                            // atoms
+  long long b = h->nknots * (long long)(sizeof(double2) + sizeof(float2) + sizeof(float)) + h->nknots_i * 12 +
+                h->notab64 * (long long)sizeof(double);  // tables
+  b += na * (3 * (long long)sizeof(double) + 4) + (na + 1 + h->norb) * 4;                    // atoms
   b += (na + 1) * 4 + np * 4 + (np + 1) * L + 2 * np * 4;                                  // pair set
   b += nb * (3 * 4 + kNbrListBytes) + (nb + 1) * 3 * L + 8 * L + na * 3 * 4;                // brick counts and lists
   b += h->cap_slots * 8 + (h->cap_slots + 1) * L + h->cap_ent * 3 * (long long)sizeof(double) +
@@ -539,13 +575,25 @@ static int check_precision(int precision) {
              : GINT_EINVAL;
 }
 
+// Float64 passes: the digit products on the tensor cores where the handle has scratch for them, else (and in
+// float32) the CUDA-core kernels.
+static int cuda_rho(gint_handle *h, bool fp64, const double *D, double *rho, const double *V, double *F, cudaStream_t st) {
+  if (fp64 && h->fx_batch > 0) return gint_fx_rho(h, D, rho, V, F, st);
+  return gint_simt_rho(h, fp64, D, rho, V, F, st);
+}
+static int cuda_vlocal(gint_handle *h, bool fp64, const double *V, double *H, cudaStream_t st) {
+  // (bricks of more than 453 orbitals are refused on either path: GINT_ECAPACITY)
+  if (fp64 && h->fx_batch > 0 && h->max_brick_orb <= 453) return gint_fx_vlocal(h, V, H, st);
+  return gint_simt_vlocal(h, fp64, V, H, st);
+}
+
 int gint_rho(gint_handle *h, int precision, const double *D_blocks, double *rho, void *stream) {
   if (!h || !D_blocks || !rho) return GINT_EINVAL;
   if (check_precision(precision)) return GINT_EINVAL;
   DeviceGuard guard(h->device);
   cudaStream_t st = (cudaStream_t)stream;
   if (precision == GINT_FP64 || precision == GINT_FP32)
-    return gint_simt_rho(h, precision == GINT_FP64, D_blocks, rho, nullptr, nullptr, st);
+    return cuda_rho(h, precision == GINT_FP64, D_blocks, rho, nullptr, nullptr, st);
   return gint_tc_rho(h, precision, D_blocks, rho, nullptr, nullptr, st);
 }
 
@@ -556,7 +604,7 @@ int gint_vlocal(gint_handle *h, int precision, const double *V, double *H_blocks
   cudaStream_t st = (cudaStream_t)stream;
   if (precision == GINT_FP64 || precision == GINT_FP32) {
     if (cudaMemsetAsync(H_blocks, 0, sizeof(double) * (size_t)h->nblock, st) != cudaSuccess) return GINT_ECUDA;
-    return gint_simt_vlocal(h, precision == GINT_FP64, V, H_blocks, st);
+    return cuda_vlocal(h, precision == GINT_FP64, V, H_blocks, st);
   }
   return gint_tc_vlocal(h, precision, V, H_blocks, st);  // every block element is written
 }
@@ -634,7 +682,7 @@ int gint_force(gint_handle *h, int precision, const double *D_blocks, const doub
   cudaStream_t st = (cudaStream_t)stream;
   if (precision == GINT_FP64 || precision == GINT_FP32) {
     if (cudaMemsetAsync(F, 0, sizeof(double) * 3 * (size_t)h->geom.natoms, st) != cudaSuccess) return GINT_ECUDA;
-    return gint_simt_rho(h, precision == GINT_FP64, D_blocks, rho, V, F, st);
+    return cuda_rho(h, precision == GINT_FP64, D_blocks, rho, V, F, st);
   }
   return gint_tc_rho(h, precision, D_blocks, rho, V, F, st);  // F is zeroed by the preparation kernel
 }
@@ -669,14 +717,14 @@ int gint_run_batch_timed(const gint_task *tasks, int ntasks, int precision, void
     int rc = GINT_OK;
     if (T.F) {
       if (cudaMemsetAsync(T.F, 0, sizeof(double) * 3 * (size_t)h->geom.natoms, st) != cudaSuccess) return GINT_ECUDA;
-      rc = gint_simt_rho(h, fp64, T.D_blocks, T.rho, T.V, T.F, st);
+      rc = cuda_rho(h, fp64, T.D_blocks, T.rho, T.V, T.F, st);
     } else if (T.rho) {
-      rc = gint_simt_rho(h, fp64, T.D_blocks, T.rho, nullptr, nullptr, st);
+      rc = cuda_rho(h, fp64, T.D_blocks, T.rho, nullptr, nullptr, st);
     }
     if (rc) return rc;
     if (T.H_blocks) {
       if (cudaMemsetAsync(T.H_blocks, 0, sizeof(double) * (size_t)h->nblock, st) != cudaSuccess) return GINT_ECUDA;
-      rc = gint_simt_vlocal(h, fp64, T.V, T.H_blocks, st);
+      rc = cuda_vlocal(h, fp64, T.V, T.H_blocks, st);
       if (rc) return rc;
     }
   }

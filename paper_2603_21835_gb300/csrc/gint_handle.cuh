@@ -14,6 +14,9 @@ struct gint_handle {
   GGeom geom{};
   // radial tables, (f, f') per knot
   double2 *tab64 = nullptr;
+  double *otab64 = nullptr;  // tables of the float64 evaluators of shaped species, and the species metadata with
+  GTabs tabs64{};            // their offsets (shape 0: no compiled evaluator)
+  long long notab64 = 0;
   float2 *tab32 = nullptr;
   float2 *tab32i = nullptr;  // interleaved per-species copy of tab32 ([knot][radial]) for shaped species
   // float32 knot differences f_{k+1} - f_k formed in float64 (parallel to tab32 / tab32i): the
@@ -100,6 +103,9 @@ struct gint_handle {
   long long *lay_sz = nullptr, *lay_tot = nullptr;
   int lay_ranges = 0;
   long long cap_hs = 0, cap_src = 0, cap_plan = 0;
+  // float64 passes on digit products (gint_fx.cu): scratch in hs, for fx_batch bricks at a time (0: not available)
+  int fx_batch = 0;
+  int *fx_eD = nullptr, *atom_off_dev = nullptr;  // exponents of D's rows; first orbital of each atom
   // local H per lattice vector (keys (I, J, R); built on first use by gint_hr_prepare)
   bool r_ready = false;
   int r_status = 0;           // GINT_OK, or why per-R output is unavailable for this geometry
@@ -126,8 +132,6 @@ struct gint_handle {
   int *pb_I = nullptr, *pb_J = nullptr, *pb_img_off = nullptr;
   long long *pb_off = nullptr;
   double *pb_img = nullptr;             // image positions of J per pair
-  GTabs pb_orb{};                       // orbital metadata with the offsets of pb_otab
-  double *pb_otab = nullptr;            // orbital tables of the overlap kernel
   double2 *pb_phase = nullptr;          // weight x projector radial x phase at every quadrature point
   double2 *pb_part = nullptr;           // [pb_groups][pb_nelems] partial sums
   int *pb_order = nullptr;              // pairs by the shape of J; segments of equal shape start at pb_first
@@ -166,6 +170,10 @@ int gint_simt_vlocal(gint_handle *h, bool fp64, const double *V, double *H, cuda
 int gint_convert_D32(gint_handle *h, const double *D, cudaStream_t st);
 int gint_reduce_dot(gint_handle *h, const double *a, const double *b, long long n, double scale, double *out,
                     cudaStream_t st);
+// gint_fx.cu
+long long gint_fx_bytes(const gint_handle *h, int bricks);  // scratch for that many bricks at a time (0: not supported)
+int gint_fx_rho(gint_handle *h, const double *D, double *rho, const double *V, double *F, cudaStream_t st);
+int gint_fx_vlocal(gint_handle *h, const double *V, double *H, cudaStream_t st);
 // gint_tc.cu
 int gint_tc_rho(gint_handle *h, int precision, const double *D, double *rho, const double *V, double *F,
                 cudaStream_t st);

@@ -223,6 +223,146 @@ __device__ __forceinline__ void add_orbitals(const GTabs &g, const typename Tab2
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// Float64 evaluators of l-sorted species on one knot grid (NS s, NP p, ND d radials), for the kernels whose time is
+// the number of float64 instructions (a warp-wide one occupies the SM's pipe for 16 clocks).  Tables (otab64 of the
+// handle): per knot and radial (f, f_{k+1} - f_k, dr f'_k, dr f'_{k+1}), times the constant of Y_00, of Y_1m or of
+// Y_2,+-1 (the other d functions carry their ratio to it); GSpecies::ioff: first table entry, kslot: the radials end
+// at different radii.
+#define GINT_O64_SHAPES(X) X(2, 2, 1, 13) X(2, 1, 0, 5) X(1, 1, 1, 9) X(1, 1, 0, 4) X(1, 0, 0, 1) X(3, 3, 2, 22)
+
+// 1 / r, r and the knot position of a point with r2 = |d|^2 (below 1e-36 it counts as 1e-36).
+struct Knot64 {
+  double y, r, t;
+  int i;
+};
+__device__ __forceinline__ Knot64 knot64(const GRadial &R0, double r2) {
+  Knot64 K;
+  if (r2 < 1e-36) {  // on the atom: f / r keeps its limit, u = d / r vanishes
+    K.y = 1e18;
+    K.r = 1e-18;
+  } else {
+    // one third-order step from the float32 reciprocal root (relative error below 2^-22): y (1 + e / 2 + 3 e^2 / 8)
+    // with e = 1 - r2 y^2; r by a Newton step with an exact residual, almost correctly rounded.  Against rsqrt() the
+    // evaluation kernels lost a fifth of their time (float64 instructions at 16 cycles each).
+    const double y = (double)rsqrtf((float)r2), e = fma(-(r2 * y), y, 1.0);
+    K.y = fma(y, e * fma(e, 0.375, 0.5), y);
+    K.r = r2 * K.y;
+    K.r = fma(fma(-K.r, K.r, r2), 0.5 * K.y, K.r);
+  }
+  // knot i = floor(r / dr), t in [0, 1] (a point on a knot may take either side)
+  const double x = K.r * R0.inv_dr, big = 6755399441055744.0;  // 1.5 2^52
+  const double xi = (x - 0.5) + big;  // its low bits: an integer within 1/2 of x - 1/2
+  K.i = min(max(__double2loint(xi), 0), R0.npts - 2);
+  K.t = x - (xi - big);
+  return K;
+}
+
+// phi[m] += the orbitals at displacement (dx, dy, dz), r2 below the support.
+template <int NS, int NP, int ND>
+__device__ __forceinline__ void orbitals64(const GTabs &g, const double *__restrict__ tab, const GSpecies &S, double dx,
+                                           double dy, double dz, double r2, double *phi) {
+  constexpr int NR = NS + NP + ND;
+  const Knot64 K = knot64(g.rad[S.rad0], r2);
+  const double t = K.t, t2 = t * t, u = 1.0 - t, s = t2 * fma(-2.0, t, 3.0), c0 = t * u * u, c1 = -t2 * u;
+  const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)K.i * NR) * 2;
+  double f[NR];
+#pragma unroll
+  for (int k = 0; k < NR; ++k) {
+    const double2 a = __ldg(q + 2 * k), b = __ldg(q + 2 * k + 1);
+    f[k] = fma(b.y, c1, fma(b.x, c0, fma(a.y, s, a.x)));
+    if (S.kslot && !(K.r < g.rad[S.rad0 + k].rc)) f[k] = 0.0;
+  }
+  const double ux = dx * K.y, uy = dy * K.y, uz = dz * K.y;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) phi[k] += f[k];
+#pragma unroll
+  for (int k = 0; k < NP; ++k) {
+    double *o = phi + NS + 3 * k;
+    o[0] = fma(f[NS + k], uz, o[0]);
+    o[1] = fma(f[NS + k], ux, o[1]);
+    o[2] = fma(f[NS + k], uy, o[2]);
+  }
+  if (ND > 0) {
+    const double xx = ux * ux, y0 = fma(2.0 * uz, uz, -fma(uy, uy, xx)), y3 = fma(-uy, uy, xx);
+    const double xz = ux * uz, yz = uy * uz, xy = ux * uy;
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+      double *o = phi + NS + 3 * NP + 5 * k;
+      const double fk = f[NS + NP + k];
+      o[0] = fma(fk * 0.28867513459481288225, y0, o[0]);  // sqrt(5/16) / sqrt(15/4)
+      o[1] = fma(fk, xz, o[1]);
+      o[2] = fma(fk, yz, o[2]);
+      o[3] = fma(fk * 0.5, y3, o[3]);
+      o[4] = fma(fk, xy, o[4]);
+    }
+  }
+}
+
+// rho += sum_m c_m phi_m and (gx, gy, gz) += sum_m c_m grad phi_m at the displacement, shell by shell:
+// phi = R Y(u), grad phi = u (R' - l R / r) Y + (R / r) grad Y with Y the homogeneous polynomial, so a radial needs
+// Y and grad Y contracted with its coefficients only.
+template <int NS, int NP, int ND>
+__device__ __forceinline__ void contract64(const GTabs &g, const double *__restrict__ tab, const GSpecies &S, double dx,
+                                           double dy, double dz, double r2, const double *c, double &rho, double &gx,
+                                           double &gy, double &gz) {
+  constexpr int NR = NS + NP + ND;
+  const GRadial &R0 = g.rad[S.rad0];
+  const bool at0 = r2 < 1e-24;
+  const Knot64 K = knot64(R0, r2);
+  const double t = K.t, t2 = t * t, u = 1.0 - t, s = t2 * fma(-2.0, t, 3.0), c0 = t * u * u, c1 = -t2 * u;
+  const double ds = 6.0 * t * u, d0 = u * fma(-3.0, t, 1.0), d1 = t * fma(3.0, t, -2.0), idr = R0.inv_dr;
+  const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)K.i * NR) * 2;
+  const double ux = at0 ? 0.0 : dx * K.y, uy = at0 ? 0.0 : dy * K.y, uz = at0 ? 0.0 : dz * K.y;
+  double rad = 0.0;  // coefficient of u
+  auto radial = [&](int k, double &R, double &dR) {
+    const double2 a = __ldg(q + 2 * k), b = __ldg(q + 2 * k + 1);
+    R = fma(b.y, c1, fma(b.x, c0, fma(a.y, s, a.x)));
+    dR = fma(b.y, d1, fma(b.x, d0, a.y * ds)) * idr;
+    if (S.kslot && !(K.r < g.rad[S.rad0 + k].rc)) R = dR = 0.0;
+  };
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    double R, dR;
+    radial(k, R, dR);
+    rho = fma(c[k], R, rho);
+    rad = fma(c[k], dR, rad);
+  }
+#pragma unroll
+  for (int k = 0; k < NP; ++k) {
+    const double *o = c + NS + 3 * k;  // z, x, y
+    double R, dR;
+    radial(NS + k, R, dR);
+    const double Rr = at0 ? dR : R * K.y, y = fma(o[0], uz, fma(o[1], ux, o[2] * uy));
+    rho = fma(at0 ? 0.0 : R, y, rho);
+    rad = fma(dR - Rr, y, rad);
+    gx = fma(Rr, o[1], gx);
+    gy = fma(Rr, o[2], gy);
+    gz = fma(Rr, o[0], gz);
+  }
+  if (ND > 0) {
+    const double xx = ux * ux, y0 = fma(2.0 * uz, uz, -fma(uy, uy, xx)), y3 = fma(-uy, uy, xx);
+    const double xz = ux * uz, yz = uy * uz, xy = ux * uy;
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+      const double *o = c + NS + 3 * NP + 5 * k;
+      double R, dR;
+      radial(NS + NP + k, R, dR);
+      const double a0 = o[0] * 0.28867513459481288225, a3 = o[3] * 0.5;
+      const double y = fma(a0, y0, fma(o[1], xz, fma(o[2], yz, fma(a3, y3, o[4] * xy))));
+      const double Rr = at0 ? 0.0 : R * K.y;
+      rho = fma(at0 ? 0.0 : R, y, rho);
+      rad = fma(fma(-2.0, Rr, dR), y, rad);
+      gx = fma(Rr, fma(2.0 * (a3 - a0), ux, fma(o[1], uz, o[4] * uy)), gx);
+      gy = fma(Rr, fma(-2.0 * (a3 + a0), uy, fma(o[2], uz, o[4] * ux)), gy);
+      gz = fma(Rr, fma(4.0 * a0, uz, fma(o[1], ux, o[2] * uy)), gz);
+    }
+  }
+  gx = fma(rad, ux, gx);
+  gy = fma(rad, uy, gy);
+  gz = fma(rad, uz, gz);
+}
+
 // Device error word bits.
 #define GINT_ERRBIT_CAPACITY 1u
 #define GINT_ERRBIT_SKIN 2u

@@ -53,7 +53,7 @@ struct GPb {
   const double *pos;
   const int *species;
   const double2 *tab, *ptab;  // orbital and projector tables, (f, f') per knot
-  const double *otab;         // orbital tables of this kernel: per knot and radial (f, df, dr f'_k, dr f'_k+1)
+  const double *otab;         // orbital tables of orbitals64
   double2 *phase;             // [projector radial][ray][node]: weight x radial x e^{-i A.x}
   const int *order;           // pairs of this launch
   double *part;               // [group][complex element]
@@ -108,58 +108,6 @@ __global__ void __launch_bounds__(256) k_pb_phase(const __grid_constant__ GTabs 
   sincos(-r * (P.A[0] * c_ang[a][0] + P.A[1] * c_ang[a][1] + P.A[2] * c_ang[a][2]), &s, &c);
   f *= wk;
   P.phase[((long long)rad * kPbRays + a) * kPbNr + k] = make_double2(f * c, f * s);
-}
-
-// Orbitals of a shaped species (NS s, NP p, ND d radials on one knot grid) at displacement d with r2 = |d|^2
-// below the support: phi[m] += value.  Tables: the radial times the constant of Y_00, of Y_1m or of
-// Y_2,+-1 (the other d functions carry their ratio to it).
-template <int NS, int NP, int ND>
-__device__ __forceinline__ void pb_orbitals(const GTabs &g, const double *__restrict__ tab, const GSpecies &S, double dx,
-                                            double dy, double dz, double r2, double *phi) {
-  constexpr int NR = NS + NP + ND;
-  const GRadial &R0 = g.rad[S.rad0];
-  r2 = fmax(r2, 1e-300);  // on the atom: u = 0, so only the s functions remain
-  const double y = rsqrt(r2);
-  double r = r2 * y;
-  r = fma(fma(-r, r, r2), 0.5 * y, r);
-  // knot i = floor(r / dr), t in [0, 1] (a point on a knot may take either side)
-  const double x = r * R0.inv_dr, big = 6755399441055744.0;  // 1.5 2^52
-  const double xi = (x - 0.5) + big;  // its low bits: an integer within 1/2 of x - 1/2
-  const int i = min(max(__double2loint(xi), 0), R0.npts - 2);
-  const double t = x - (xi - big);
-  const double t2 = t * t, u = 1.0 - t, s = t2 * fma(-2.0, t, 3.0), c0 = t * u * u, c1 = -t2 * u;
-  const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)i * NR) * 2;
-  double f[NR];
-#pragma unroll
-  for (int k = 0; k < NR; ++k) {
-    const double2 a = __ldg(q + 2 * k), b = __ldg(q + 2 * k + 1);
-    f[k] = fma(b.y, c1, fma(b.x, c0, fma(a.y, s, a.x)));
-    if (S.kslot && !(r < g.rad[S.rad0 + k].rc)) f[k] = 0.0;  // kslot: the radials end at different radii
-  }
-  const double ux = dx * y, uy = dy * y, uz = dz * y;
-#pragma unroll
-  for (int k = 0; k < NS; ++k) phi[k] += f[k];
-#pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    double *o = phi + NS + 3 * k;
-    o[0] = fma(f[NS + k], uz, o[0]);
-    o[1] = fma(f[NS + k], ux, o[1]);
-    o[2] = fma(f[NS + k], uy, o[2]);
-  }
-  if (ND > 0) {
-    const double xx = ux * ux, y0 = fma(2.0 * uz, uz, -fma(uy, uy, xx)), y3 = fma(-uy, uy, xx);
-    const double xz = ux * uz, yz = uy * uz, xy = ux * uy;
-#pragma unroll
-    for (int k = 0; k < ND; ++k) {
-      double *o = phi + NS + 3 * NP + 5 * k;
-      const double fk = f[NS + NP + k];
-      o[0] = fma(fk * 0.28867513459481288225, y0, o[0]);  // sqrt(5/16) / sqrt(15/4)
-      o[1] = fma(fk, xz, o[1]);
-      o[2] = fma(fk, yz, o[2]);
-      o[3] = fma(fk * 0.5, y3, o[3]);
-      o[4] = fma(fk, xy, o[4]);
-    }
-  }
 }
 
 // v[0 .. 2 H) over the lanes that differ in bit `bit`: the lane whose bit is clear keeps the sums of the first
@@ -248,7 +196,7 @@ __global__ void __launch_bounds__(kPbThreads, 4) k_psibeta(const __grid_constant
           if (pt && r2 < SJ.rcut2) {
             any = true;
             if constexpr (NS + NP + ND > 0)
-              pb_orbitals<NS, NP, ND>(orb, P.otab, SJ, dx, dy, dz, r2, phi);
+              orbitals64<NS, NP, ND>(orb, P.otab, SJ, dx, dy, dz, r2, phi);
             else
               add_orbitals<double, true, false>(orb, P.tab, P.species[J], dx, dy, dz, phi, nullptr);
           }
@@ -348,7 +296,6 @@ void gint_pb_free(gint_handle *h) {
   pfree(h->pb_off);
   pfree(h->pb_img_off);
   pfree(h->pb_img);
-  pfree(h->pb_otab);
   pfree(h->pb_order);
   pfree(h->pb_phase);
   pfree(h->pb_part);
@@ -454,34 +401,16 @@ int gint_pb_set(gint_handle *h, int nspecies, const gint_species *proj) {
     cudaGetLastError();
     return GINT_ECUDA;
   }
-  // orbital tables: per knot and radial (f, f_{k+1} - f_k, dr f'_k, dr f'_{k+1}), times the Y_lm constant;
-  // shapes without a compiled evaluator keep the general one
-  GTabs ot = g;
-  std::vector<double> otab;
+  // shapes without a compiled kernel take the general one
   std::vector<int> shape(g.nspecies, 0);
-  const double cl[3] = {0.28209479177387814347, 0.48860251190291992159, 1.09254843059207907054};
-  for (int s = 0; s < g.nspecies; ++s) {
-    GSpecies &S = ot.sp[s];
-    switch (S.shape) {
+  for (int s = 0; s < g.nspecies; ++s) switch (h->tabs64.sp[s].shape) {
 #define CASE_PB(ns, np, nd, no) case GINT_SHAPE(ns, np, nd):
       GINT_PB_SHAPES(CASE_PB)
 #undef CASE_PB
-      shape[s] = S.shape;
+      shape[s] = h->tabs64.sp[s].shape;
       break;
-      default: continue;
+      default: break;
     }
-    S.ioff = (int)(otab.size() / 4);
-    S.kslot = 0;
-    for (int k = 0; k < S.nrad; ++k)
-      if (g.rad[S.rad0 + k].rc != S.rcut) S.kslot = 1;
-    for (int i = 0; i + 1 < g.rad[S.rad0].npts; ++i)
-      for (int k = 0; k < S.nrad; ++k) {
-        const GRadial &R = g.rad[S.rad0 + k];
-        const double c = cl[R.l];
-        const gint_radial &T = h->d_rad[S.rad0 + k];
-        otab.insert(otab.end(), {c * T.f[i], c * (T.f[i + 1] - T.f[i]), c * R.dr * T.df[i], c * R.dr * T.df[i + 1]});
-      }
-  }
   // pairs in launch order: by the shape of J
   std::vector<int> order(pI.size());
   for (size_t q = 0; q < order.size(); ++q) order[q] = (int)q;
@@ -496,7 +425,7 @@ int gint_pb_set(gint_handle *h, int nspecies, const gint_species *proj) {
   const size_t phase = (size_t)std::max(1, t.nrad) * kPbRays * kPbNr, part = (size_t)h->pb_groups * poff.back();
   if ((rc = upload(&h->pb_tab64, tab)) || (rc = upload(&h->pb_I, pI)) || (rc = upload(&h->pb_J, pJ)) ||
       (rc = upload(&h->pb_off, poff)) || (rc = upload(&h->pb_img_off, img_off)) || (rc = upload(&h->pb_img, img)) ||
-      (rc = upload(&h->pb_otab, otab)) || (rc = upload(&h->pb_order, order))) {
+      (rc = upload(&h->pb_order, order))) {
     gint_pb_free(h);
     return rc;
   }
@@ -507,7 +436,6 @@ int gint_pb_set(gint_handle *h, int nspecies, const gint_species *proj) {
     return GINT_ENOMEM;
   }
   h->pb_tabs = t;
-  h->pb_orb = ot;
   h->pb_shape.clear();
   h->pb_first.clear();
   for (int q = 0; q < npair; ++q) {
@@ -527,7 +455,7 @@ int gint_pb_set(gint_handle *h, int nspecies, const gint_species *proj) {
   }
   h->pb_off_host = poff;
   h->pb_bytes = (long long)(tab.size() * sizeof(double2) + (3 * pI.size() + img_off.size()) * sizeof(int) +
-                            poff.size() * sizeof(long long) + (img.size() + otab.size()) * sizeof(double) +
+                            poff.size() * sizeof(long long) + img.size() * sizeof(double) +
                             (phase + part) * sizeof(double2));
   h->pb_ready = true;
   return GINT_OK;
@@ -547,7 +475,7 @@ int gint_pb_run(gint_handle *h, const double A[3], double *out, cudaStream_t st)
   P.species = h->species_dev;
   P.tab = h->tab64;
   P.ptab = h->pb_tab64;
-  P.otab = h->pb_otab;
+  P.otab = h->otab64;
   P.phase = h->pb_phase;
   P.part = reinterpret_cast<double *>(h->pb_part);
   P.nelems = h->pb_nelems;
@@ -559,10 +487,10 @@ int gint_pb_run(gint_handle *h, const double A[3], double *out, cudaStream_t st)
     const dim3 grid((unsigned)(h->pb_first[q + 1] - h->pb_first[q]), (unsigned)h->pb_groups);
     switch (h->pb_shape[q]) {
 #define CASE_PB(ns, np, nd, no)                                                                        \
-  case GINT_SHAPE(ns, np, nd): k_psibeta<ns, np, nd, no><<<grid, kPbThreads, 0, st>>>(h->pb_orb, h->pb_tabs, P); break;
+  case GINT_SHAPE(ns, np, nd): k_psibeta<ns, np, nd, no><<<grid, kPbThreads, 0, st>>>(h->tabs64, h->pb_tabs, P); break;
       GINT_PB_SHAPES(CASE_PB)
 #undef CASE_PB
-      default: k_psibeta<0, 0, 0, kPbMaxOrb><<<grid, kPbThreads, 0, st>>>(h->pb_orb, h->pb_tabs, P);
+      default: k_psibeta<0, 0, 0, kPbMaxOrb><<<grid, kPbThreads, 0, st>>>(h->tabs64, h->pb_tabs, P);
     }
   }
   k_pb_sum<<<(unsigned)h->pb_npairs, 128, 0, st>>>(P, reinterpret_cast<double2 *>(out));

@@ -2732,6 +2732,14 @@ static int tc_layouts(gint_handle *h, cudaStream_t st) {
   h->hs_elems = tot[0];
   h->max_brick_porb = (int)tot[3];
   int rc;
+  // the scratch tiles' buffer also serves the float64 passes: enlarged (small systems) to hold a brick per SM for
+  // them if memory allows
+  h->fx_batch = 0;
+  if (gint_fx_bytes(h, 1) > 0) {
+    const int want = (int)std::min<long long>(h->num_sms, nb);
+    const long long fx = (gint_fx_bytes(h, want) + 3) / 4;
+    if (tc_reserve(h, h->hs, h->cap_hs, std::max(tot[0], fx)) == GINT_OK) h->fx_batch = want;
+  }
   if ((rc = tc_reserve(h, h->hs, h->cap_hs, tot[0])) || (rc = tc_reserve(h, h->plan, h->cap_plan, tot[1])) ||
       (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2])))
     return rc;

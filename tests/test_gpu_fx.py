@@ -1,0 +1,94 @@
+"""Float64 density, force and local-H passes on exact digit products, over the forms their kernels tell apart:
+orbital counts of a brick that are no multiple of the 16-, 64- and 128-column tiles, atoms across a tile edge,
+every compiled orbital shape and the general evaluator, radials that end early, atoms on grid points, ragged and
+one-brick grids, empty bricks, bricks of more than 512 columns (the CUDA-core kernels), infinities and NaNs.
+Tolerances of the float64 path: 1e-12 of the largest element for rho and H, 1e-11 for F, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle.oracle import Oracle
+from paper_2603_21835_gb300 import inputs
+from tests.test_gpu_psibeta_shapes import ORB, _shorter, _sp
+
+pytestmark = pytest.mark.gpu
+
+
+def _system(names, nat, box, grid, on_grid=False):
+    rng = np.random.default_rng(nat)
+    sp = []
+    for n in names:
+        s = _sp(n, ORB[n.split()[0]])
+        sp.append(_shorter(s, 1, 3.3337) if n.endswith("short") else s)
+    cell = np.diag([box, box * 1.1, box * 0.95])
+    frac = rng.random((nat, 3))
+    if on_grid:
+        frac = np.floor(frac * grid) / grid
+    return inputs.System(cell=cell, pos=frac @ cell, species=(np.arange(nat) % len(names)).astype(np.int32), sp=sp, grid=grid)
+
+
+@pytest.mark.parametrize("names,nat,box,grid,on_grid", [
+    (("100",), 1, 11.0, (4, 4, 8), False), (("110",), 3, 15.0, (11, 9, 13), False), (("221", "110"), 9, 12.0, (8, 8, 8), False),
+    (("221", "100"), 17, 12.0, (8, 5, 16), False), (("111", "210"), 6, 10.0, (12, 8, 8), True), (("unsorted",), 5, 13.0, (8, 8, 8), True),
+    (("dd", "grids"), 7, 10.0, (8, 8, 8), False), (("221 short", "111 short"), 6, 9.0, (8, 8, 9), False),
+    (("221",), 2, 40.0, (20, 20, 24), False), (("221",), 34, 10.0, (4, 8, 8), False), (("221",), 44, 10.0, (4, 8, 8), False)])
+def test_passes_match_the_oracle(names, nat, box, grid, on_grid):
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    s = _system(names, nat, box, grid, on_grid)
+    rng = np.random.default_rng(nat + 1)
+    o = Oracle(s)
+    C = rng.normal(size=(o.norb, 5)) / 4
+    D = C @ C.T
+    V = rng.normal(size=int(np.prod(grid)))
+    rho_o, H_o, F_o = o.rho(D).reshape(-1), o.vlocal(V), o.force(D, V)
+    g = G.Gint(s)
+    Db, Vd = torch.from_numpy(g.dense_to_blocks(D)).cuda(), torch.from_numpy(V).cuda()
+    for _ in range(2):  # again: the scratch holds the last call's
+        rho = g.rho(Db, G.FP64).cpu().numpy().reshape(-1)
+        if nat < 44:
+            H = g.blocks_to_dense(g.vlocal(Vd, G.FP64).cpu().numpy())
+        else:  # more than 453 orbitals in a brick: refused in float64
+            with pytest.raises(G.GintError):
+                g.vlocal(Vd, G.FP64)
+            H = H_o
+        F = g.force(Db, Vd, G.FP64)
+        F = (F[0] if isinstance(F, tuple) else F).cpu().numpy()
+        g.sync()
+        assert np.abs(rho - rho_o).max() <= 1e-12 * np.abs(rho_o).max()
+        assert np.abs(H - H_o).max() <= 1e-12 * np.abs(H_o).max()
+        assert np.abs(F - F_o).max() <= 1e-11 * np.abs(F_o).max()
+    g.close()
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_non_finite_inputs_reach_the_same_results(bad):
+    """One bad point of V, or one bad element of D: the same elements are non-finite as on the CUDA cores (FP32), the
+    rest equals the clean run's."""
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    s = _system(("221", "110"), 6, 16.0, (16, 12, 16))
+    rng = np.random.default_rng(3)
+    g = G.Gint(s)
+    C = rng.normal(size=(g.norb, 5)) / 4
+    D = torch.from_numpy(g.dense_to_blocks(C @ C.T)).cuda()
+    V = torch.from_numpy(rng.normal(size=g.ngrid)).cuda()
+    H0, rho0 = g.vlocal(V, G.FP64).clone(), g.rho(D, G.FP64).clone()
+    Vb = V.clone()
+    Vb[g.ngrid // 2 + 37] = bad
+    Hb, Hs = g.vlocal(Vb, G.FP64).clone(), g.vlocal(Vb, G.FP32).clone()
+    ok = torch.isfinite(Hb)
+    assert torch.equal(ok, torch.isfinite(Hs)) and not ok.all() and ok.any()
+    assert float((Hb - H0)[ok].abs().max()) <= 1e-12 * float(H0.abs().max())
+    M = C @ C.T
+    M[3, 20] = M[20, 3] = bad
+    Db = torch.from_numpy(g.dense_to_blocks(M)).cuda()
+    rb, rs = g.rho(Db, G.FP64).clone().reshape(-1), g.rho(Db, G.FP32).clone().reshape(-1)
+    ok = torch.isfinite(rb)
+    assert torch.equal(ok, torch.isfinite(rs)) and not ok.all() and ok.any()
+    assert float((rb - rho0.reshape(-1))[ok].abs().max()) <= 1e-12 * float(rho0.abs().max())
+    g.sync()
+    g.close()
