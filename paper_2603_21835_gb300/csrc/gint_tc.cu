@@ -347,7 +347,6 @@ struct BrickSh {
   float e_hi[kMAXE][3], e_lo[kMAXE][3];  // entry positions relative to the brick origin
   float pt_hi[128][3], pt_lo[128][3];    // grid point positions relative to the brick origin
   unsigned char col2slot[kNPMAX];
-  double fpart[kMAXA][3];
   union alignas(8) {
     float rpart[4][128];  // density / force epilogues, fixed-point rows: per-slice partials of a point
     // local-H epilogue (after those): per 8-column group h of the padded columns, (dense index of
@@ -356,6 +355,7 @@ struct BrickSh {
   };
   union {
     float rpartl[4][128];  // density epilogue: compensation terms of the groups' partial sums
+    float fpart[4][3 * kMAXA];  // force epilogue: per quarter of the points, 2 w V sum(Y grad phi) of each slot
     double vd[128];        // V at the brick's points, copied asynchronously (formed into wv after the
                            // orbitals, before the density epilogue uses rpartl)
   };
@@ -411,7 +411,6 @@ __device__ void load_brick(const GCell &g, const GTabs &tb, const GNbr &nb, cons
     sh.s_no[a] = tb.sp[sp].norb;
     sh.s_po[a] = tb.sp[sp].porb;
     sh.s_e0[a] = (int)(nb.s_ent[s0 + a] - e_begin);
-    sh.fpart[a][0] = sh.fpart[a][1] = sh.fpart[a][2] = 0.0;
   }
   for (int k = t; k < kNPMAX; k += blockDim.x) sh.col2slot[k] = kNoSlot;
   __syncthreads();
@@ -479,7 +478,6 @@ __device__ void unpack_plan(BrickSh &sh, bool wait_store = false) {
     sh.s_e0[a] = (int)q[5];
     sh.s_cumno[a] = (int)q[6];
     sh.s_rowst[a] = (int)q[7];
-    sh.fpart[a][0] = sh.fpart[a][1] = sh.fpart[a][2] = 0.0;
   }
   if (t == 0) {
     sh.na = na;
@@ -557,6 +555,10 @@ __device__ __forceinline__ void slot_values(const GTabs &g, const float2 *__rest
 }
 
 // Species shapes with a static fast path; others use the generic evaluator (NS=NPR=ND=0).
+// DZP: the kernels' instances for launches whose species are all double-zeta with one polarisation shell
+// (2s 2p 1d, 2s 1p).  The other shapes' code in the same kernel costs registers in every path (force instance:
+// 1.9 KB of spills a thread with all six, 0.1 KB with these two).
+__host__ __device__ constexpr bool is_dzp(int shape) { return shape == GINT_SHAPE(2, 2, 1) || shape == GINT_SHAPE(2, 1, 0); }
 #define GINT_FOR_SHAPES(X) X(2, 2, 1) X(2, 1, 0) X(1, 1, 1) X(1, 1, 0) X(1, 0, 0) X(3, 3, 2)
 
 // --- per-atom jobs ---
@@ -596,19 +598,170 @@ __device__ __forceinline__ void job_P(const GTabs &g, const float2 *__restrict__
   store_P<PO>(v, sh.s_pcol[a], p, Sphi, Ph, Pl, sboP);
 }
 
-// Force epilogue: y[PO] (true Y values of slot a's columns) -> rho part and force components.
+// One image's rho and force contributions of slot a at a point, the terms and their order those of add_image_fast with
+// the sums over orbitals behind it (job_F), without the 4 PO accumulators: the table entries of all radials are loaded
+// together (they come from L2 as often as not, the first-level cache is what shared memory leaves of it).  The fused
+// multiply-adds are written out: the roundings are those of the summed form, term by term.
+template <int NS, int NPR, int ND>
+__device__ __forceinline__ void single_F(const GTabs &g, const float2 *__restrict__ tabi,
+                                         const float *__restrict__ dtabi, const GSpecies &S, const float dh[3],
+                                         const float dl[3], bool in, const float *y, float &rp, float &fx, float &fy,
+                                         float &fz) {
+  constexpr int NR = NS + NPR + ND, KS = (NR + 1) & ~1, NO = NS + 3 * NPR + 5 * ND;
+  float r = 0.f, rl, ir = 0.f, t = 0.f;
+  bool at0 = false;
+  int i = 0;
+  if (in) {
+    dist_df(dh, dl, r, rl, ir, at0);
+    in = knot_df(g.rad[S.rad0], r, rl, i, t);
+  }
+  if (!in) {  // beyond the support: 0 times y (a non-finite y reaches the sums)
+    float z = 0.f;
+#pragma unroll
+    for (int k = 0; k < NO; ++k) z = fmaf(0.f, y[k], z);
+    rp += z;
+    fx += z;
+    fy += z;
+    fz += z;
+    return;
+  }
+  const float2 *q2 = tabi + S.ioff + (long long)i * KS;
+  const float4 *q = reinterpret_cast<const float4 *>(q2);
+  const float2 *qd = reinterpret_cast<const float2 *>(dtabi + S.ioff + (long long)i * KS);
+  float2 ka[KS], kb[KS];
+  float kd[KS];
+#pragma unroll
+  for (int h = 0; h < KS / 2; ++h) {
+    const float4 x = __ldg(q + h), z = __ldg(q + KS / 2 + h);
+    const float2 d = __ldg(qd + h);
+    ka[2 * h] = make_float2(x.x, x.y);
+    ka[2 * h + 1] = make_float2(x.z, x.w);
+    kb[2 * h] = make_float2(z.x, z.y);
+    kb[2 * h + 1] = make_float2(z.z, z.w);
+    kd[2 * h] = d.x;
+    kd[2 * h + 1] = d.y;
+  }
+  const Basis B = hermite_basis(t);
+  const float drf = g.rad[S.rad0].dr_f, idr = g.rad[S.rad0].idr_hi;
+  auto radial_k = [&](int k, float &f, float &df) {
+    const float2 a = ka[k], b = kb[k];
+    const float dlt = kd[k];
+    f = a.x + dlt * B.s + drf * (a.y * B.c0 + b.y * B.c1);
+    df = fmaf(dlt, B.ds, drf * fmaf(a.y, B.d0, b.y * B.d1)) * idr;
+    if (!(r < g.rad[S.rad0 + k].rc_f)) f = df = 0.f;
+  };
+  const float ux = dh[0] * ir, uy = dh[1] * ir, uz = dh[2] * ir;
+  const float Y0 = 0.28209479177387814347f;
+  float y1[3], gy1[3][3], y2[5], gy2[5][3];
+  if (NPR > 0) ylm_unit<float>(1, ux, uy, uz, y1, gy1);
+  if (ND > 0) ylm_unit<float>(2, ux, uy, uz, y2, gy2);
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    float f, df;
+    radial_k(k, f, df);
+    const float v = f * Y0, a = at0 ? 0.f : df * Y0;
+    rp += v * y[k];
+    fx = fmaf(a * ux, y[k], fx);
+    fy = fmaf(a * uy, y[k], fy);
+    fz = fmaf(a * uz, y[k], fz);
+  }
+#pragma unroll
+  for (int k = 0; k < NPR; ++k) {
+    const int col = NS + 3 * k;
+    float f, df;
+    radial_k(NS + k, f, df);
+    if (at0) {
+      const float c = 0.48860251190291992159f * df;
+      fz += c * y[col];
+      fx += c * y[col + 1];
+      fy += c * y[col + 2];
+      continue;
+    }
+    const float fr = f * ir;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const float v = f * y1[m], a = fmaf(df, y1[m], -(fr * y1[m]));
+      rp += v * y[col + m];
+      fx = fmaf(fmaf(a, ux, fr * gy1[m][0]), y[col + m], fx);
+      fy = fmaf(fmaf(a, uy, fr * gy1[m][1]), y[col + m], fy);
+      fz = fmaf(fmaf(a, uz, fr * gy1[m][2]), y[col + m], fz);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < ND; ++k) {
+    const int col = NS + 3 * NPR + 5 * k;
+    float f, df;
+    radial_k(NS + NPR + k, f, df);
+    if (at0) f = df = 0.f;
+    const float fr = f * ir;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+      const float v = f * y2[m], a = fmaf(df, y2[m], -(2.f * fr * y2[m]));
+      rp += v * y[col + m];
+      const float tx = m == 0 || m == 4 ? fmaf(fr, gy2[m][0], a * ux) : fmaf(a, ux, fr * gy2[m][0]);
+      fx = fmaf(tx, y[col + m], fx);
+      fy = fmaf(fmaf(a, uy, fr * gy2[m][1]), y[col + m], fy);
+      fz = fmaf(fmaf(a, uz, fr * gy2[m][2]), y[col + m], fz);
+    }
+  }
+}
+
+// N Y columns of a point (float32, times inv) from tensor memory.
+template <int N>
+__device__ __forceinline__ void load_Y(uint32_t ty, uint32_t tcorr, float inv, float *y) {
+  static_assert(N == 8 || N == 16, "");  // (an 8-column atom may end the accumulator: no load reaches past it)
+  float yc[N];
+  if (N == 16) {
+    if (tcorr)
+      tmem_ld16x2(ty, ty + tcorr, y, yc);
+    else
+      tmem_ld16(ty, y);
+  } else {
+    tmem_ld8(ty, y);
+    if (tcorr) tmem_ld8(ty + tcorr, yc);
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if (tcorr) y[i] += yc[i];
+    y[i] *= inv;
+  }
+}
+
+// Force epilogue of slot a: rho part and force components of a point.  Y is loaded where it is used: before the
+// orbitals of an only image, behind the sums over several (their accumulators leave it no registers).  The epilogue is
+// bound by instruction issue and by the table loads' latency; it took 33 of an item's 62 thousand cycles (64-atom Si)
+// with Y in local memory, 4 PO accumulators and one radial's loads at a time: 1496 us of forces -> 1041 us.
 template <int NS, int NPR, int ND, int PO>
 __device__ __forceinline__ void job_F(const GTabs &g, const float2 *__restrict__ tab, const float *__restrict__ dtab,
-                                      const BrickSh &sh, int a, int p, bool valid, const float *y, float &rp, float &fx,
-                                      float &fy, float &fz) {
+                                      const BrickSh &sh, int a, int p, bool valid, uint32_t ty, uint32_t tcorr, float inv,
+                                      float &rp, float &fx, float &fy, float &fz) {
+  if (sh.s_e0[a + 1] - sh.s_e0[a] == 1) {
+    float y[PO];
+#pragma unroll
+    for (int h = 0; h + 16 <= PO; h += 16) load_Y<16>(ty + h, tcorr, inv, y + h);
+    if (PO & 8) load_Y<8>(ty + (PO & ~15), tcorr, inv, y + (PO & ~15));
+    const GSpecies &S = g.sp[sh.s_sp[a]];
+    float dh[3], dl[3];
+    rel_disp_df(sh, point_df(sh, p), sh.s_e0[a], dh, dl);
+    const bool in = valid && dh[0] * dh[0] + dh[1] * dh[1] + dh[2] * dh[2] < S.rcut2f;
+    single_F<NS, NPR, ND>(g, tab, dtab, S, dh, dl, in, y, rp, fx, fy, fz);
+    __syncwarp();
+    return;
+  }
   float v[PO], gv[3 * PO];
   slot_values<NS, NPR, ND, true>(g, tab, dtab, sh, a, point_df(sh, p), valid, v, gv);
+  __syncwarp();
 #pragma unroll
-  for (int i = 0; i < PO; ++i) {
-    rp += v[i] * y[i];
-    fx += gv[3 * i] * y[i];
-    fy += gv[3 * i + 1] * y[i];
-    fz += gv[3 * i + 2] * y[i];
+  for (int h = 0; h < PO; h += 8) {
+    float y[8];
+    load_Y<8>(ty + h, tcorr, inv, y);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      rp += v[h + i] * y[i];
+      fx += gv[3 * (h + i)] * y[i];
+      fy += gv[3 * (h + i) + 1] * y[i];
+      fz += gv[3 * (h + i) + 2] * y[i];
+    }
   }
 }
 
@@ -640,9 +793,11 @@ __device__ __noinline__ void job_P_generic(const GTabs &g, const float2 *__restr
 }
 __device__ __noinline__ void job_F_generic(const GTabs &g, const float2 *__restrict__ tab,
                                            const float *__restrict__ dtab, const BrickSh &sh, int a, int p, bool valid,
-                                           const float *y, float &rp, float &fx, float &fy, float &fz) {
-  float v[GINT_MAX_ORB_ATOM], gv[3 * GINT_MAX_ORB_ATOM];
+                                           uint32_t ty, uint32_t tcorr, float inv, float &rp, float &fx, float &fy,
+                                           float &fz) {
+  float y[GINT_MAX_ORB_ATOM], v[GINT_MAX_ORB_ATOM], gv[3 * GINT_MAX_ORB_ATOM];
   const int no = sh.s_no[a];
+  for (int h = 0; h < sh.s_po[a]; h += 8) load_Y<8>(ty + h, tcorr, inv, y + h);
   for (int i = 0; i < no; ++i) v[i] = gv[3 * i] = gv[3 * i + 1] = gv[3 * i + 2] = 0.f;
   if (valid) {
     const GSpecies &S = g.sp[sh.s_sp[a]];
@@ -736,7 +891,7 @@ struct ItemCtx {
   bool vpend;     // V of the brick's points is wanted in sh.vd: orbital slice 3 (the last four warps)
                   // copies one value per thread asynchronously during the orbital phase
 };
-template <bool FORCE>
+template <bool FORCE, bool DZP>
 __device__ __forceinline__ void brick_body(const GTabs &g, const GSys &S, long long b, bool do_rho, bool do_h,
                                            int split3, int dsmem, const __half *__restrict__ zero, uint32_t tmem,
                                            BrickSh &sh, unsigned char *smem, ItemCtx &cx) {
@@ -880,6 +1035,7 @@ __device__ __forceinline__ void brick_body(const GTabs &g, const GSys &S, long l
         switch (shp) {
 #define CASE_P(ns, np_, nd)                                                                                      \
 case GINT_SHAPE(ns, np_, nd):                                                                                \
+  if constexpr (DZP && !is_dzp(GINT_SHAPE(ns, np_, nd))) {} else                                                  \
   if (pair)                                                                                                  \
     job_P2<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, sh, a, a1, P, p, valid, Sphi, Ph, Pl, sboP); \
   else                                                                                                       \
@@ -888,18 +1044,19 @@ case GINT_SHAPE(ns, np_, nd):                                                   
           GINT_FOR_SHAPES(CASE_P)
 #undef CASE_P
           default:
-            job_P_generic(g, tab, sh, a, p, valid, Sphi, Ph, Pl, sboP);
+            if constexpr (!DZP) job_P_generic(g, tab, sh, a, p, valid, Sphi, Ph, Pl, sboP);
         }
         if (a1 < na && !(pair && shp != 0)) {
           switch (g.sp[sh.s_sp[a1]].shape) {
 #define CASE_P1(ns, np_, nd)                                                                                      \
 case GINT_SHAPE(ns, np_, nd):                                                                                 \
+  if constexpr (!DZP || is_dzp(GINT_SHAPE(ns, np_, nd)))                                                      \
   job_P<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, sh, a1, P, p, valid, Sphi, Ph, Pl, sboP);    \
   break;
             GINT_FOR_SHAPES(CASE_P1)
 #undef CASE_P1
             default:
-              job_P_generic(g, tab, sh, a1, p, valid, Sphi, Ph, Pl, sboP);
+              if constexpr (!DZP) job_P_generic(g, tab, sh, a1, p, valid, Sphi, Ph, Pl, sboP);
           }
         }
       }
@@ -1092,39 +1249,18 @@ case GINT_SHAPE(ns, np_, nd):                                                   
       const float wv = (valid && S.V) ? sh.wv[p] : 0.f;
       float rp = 0.f;
       for (int a = q; a < na; a += 4) {
-        const int pc = sh.s_pcol[a], po = sh.s_po[a];
-        // the atom's own columns only (an 8-column atom may end the accumulator: a 16-column
-        // load there would reach past the tensor-memory allocation)
-        float y[GINT_MAX_ORB_ATOM], yc[16];
-        for (int h = 0; h < po; h += 16) {
-          if (po - h >= 16) {
-            if (split3 && corr_base) {
-              tmem_ld16x2(tmem + lane_base + pc + h, tmem + lane_base + corr_base + pc + h, y + h, yc);
-#pragma unroll
-              for (int i = 0; i < 16; ++i) y[h + i] += yc[i];
-            } else {
-              tmem_ld16(tmem + lane_base + pc + h, y + h);
-            }
-          } else {
-            tmem_ld8(tmem + lane_base + pc + h, y + h);
-            if (split3 && corr_base) {
-              tmem_ld8(tmem + lane_base + corr_base + pc + h, yc);
-#pragma unroll
-              for (int i = 0; i < 8; ++i) y[h + i] += yc[i];
-            }
-          }
-        }
-        for (int i = 0; i < po; ++i) y[i] *= inv;
+        const uint32_t ty = tmem + lane_base + (uint32_t)sh.s_pcol[a], tcorr = split3 ? corr_base : 0u;
         float fx = 0.f, fy = 0.f, fz = 0.f;
         switch (g.sp[sh.s_sp[a]].shape) {
 #define CASE_F(ns, np_, nd)                                                                          \
 case GINT_SHAPE(ns, np_, nd):                                                                    \
-  job_F<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, S.dtabi, sh, a, p, valid, y, rp, fx, fy, fz); \
+  if constexpr (!DZP || is_dzp(GINT_SHAPE(ns, np_, nd)))                                         \
+  job_F<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, S.dtabi, sh, a, p, valid, ty, tcorr, inv, rp, fx, fy, fz); \
   break;
           GINT_FOR_SHAPES(CASE_F)
 #undef CASE_F
           default:
-            job_F_generic(g, tab, S.dtab, sh, a, p, valid, y, rp, fx, fy, fz);
+            if constexpr (!DZP) job_F_generic(g, tab, S.dtab, sh, a, p, valid, ty, tcorr, inv, rp, fx, fy, fz);
         }
         fx *= 2.f * wv;
         fy *= 2.f * wv;
@@ -1135,9 +1271,10 @@ case GINT_SHAPE(ns, np_, nd):                                                   
           fz += __shfl_xor_sync(0xffffffffu, fz, o);
         }
         if (lane == 0) {
-          atomicAdd(&sh.fpart[a][0], (double)fx);
-          atomicAdd(&sh.fpart[a][1], (double)fy);
-          atomicAdd(&sh.fpart[a][2], (double)fz);
+          float *const fp = &sh.fpart[warp & 3][3 * a];
+          fp[0] = fx;
+          fp[1] = fy;
+          fp[2] = fz;
         }
       }
       sh.rpart[q][p] = rp;
@@ -1146,11 +1283,10 @@ case GINT_SHAPE(ns, np_, nd):                                                   
         S.rho[gidx] =
             (double)sh.rpart[0][p] + (double)sh.rpart[1][p] + (double)sh.rpart[2][p] + (double)sh.rpart[3][p];
       if (S.F)
-        for (int a = t; a < na; a += kT) {
-          const int I = sh.s_atom[a];
-          atomicAdd(S.F + 3 * I + 0, sh.fpart[a][0]);
-          atomicAdd(S.F + 3 * I + 1, sh.fpart[a][1]);
-          atomicAdd(S.F + 3 * I + 2, sh.fpart[a][2]);
+        for (int u = t; u < 3 * na; u += kT) {
+          const int a = u / 3;
+          atomicAdd(S.F + 3 * sh.s_atom[a] + (u - 3 * a), (((double)sh.fpart[0][u] + (double)sh.fpart[1][u]) +
+                                                           (double)sh.fpart[2][u]) + (double)sh.fpart[3][u]);
         }
     }
     }  // do_rho
@@ -1346,7 +1482,7 @@ case GINT_SHAPE(ns, np_, nd):                                                   
   }
 }
 
-template <bool FORCE>
+template <bool FORCE, bool DZP>
 __global__ void __launch_bounds__(kT, 1)
     k_tc_fused(const __grid_constant__ GTabs g, const __grid_constant__ GBatch B, const __half *__restrict__ zero,
                int *work) {
@@ -1445,7 +1581,7 @@ __global__ void __launch_bounds__(kT, 1)
     }
     if (t == kNextT) next_item(nclaim);  // every thread has read sh.item and sh.plan_pref
     ItemCtx cx{fpar, dpar, GH, ok, vpend};
-    brick_body<FORCE>(g, S, b, do_rho, do_h, split3, B.dsmem, zero, tmem, sh, smem, cx);
+    brick_body<FORCE, DZP>(g, S, b, do_rho, do_h, split3, B.dsmem, zero, tmem, sh, smem, cx);
     fpar = cx.fpar;
     dpar = cx.dpar;
     GH = cx.GH;
@@ -2395,7 +2531,7 @@ __global__ void __launch_bounds__(kT, 1)
           }
         }
         if (t < 128) sh.wv[t] = wvv;  // read by brick_body after its barriers
-        brick_body<FORCE>(g, S, b, do_rho, do_h, split3, dsmem, zero, tmem, sh, smem, cx);
+        brick_body<FORCE, false>(g, S, b, do_rho, do_h, split3, dsmem, zero, tmem, sh, smem, cx);
         tc_fence_before();
       }
     } else {  // H reduction: two upper pairs, one per 256 threads (named barriers 2, 3), in four parts
@@ -2922,7 +3058,8 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
   // halves of the local-H pass) | tail pad read by the last 128-row A tile above NP
   // all the shared memory a CTA may have: items lay out P and as many stages as fit for their own
   // width (at least two stages at the widest brick of the launch)
-  static const uint32_t smem = std::min(dyn_smem_limit(k_tc_fused<false>), dyn_smem_limit(k_tc_fused<true>));
+  static const uint32_t smem = std::min(std::min(dyn_smem_limit(k_tc_fused<false, false>), dyn_smem_limit(k_tc_fused<true, false>)),
+                                        std::min(dyn_smem_limit(k_tc_fused<false, true>), dyn_smem_limit(k_tc_fused<true, true>)));
   if (rho_smem_bytes(np, 2) + kHTail > smem) return GINT_ECAPACITY;
   B.np_max = np;
   B.split3 = split3;
@@ -2939,7 +3076,10 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
   }
   if (items > 0) {
     const unsigned grid = (unsigned)std::min<long long>(h0->num_sms, items);
-    auto kern = force ? k_tc_fused<true> : k_tc_fused<false>;
+    bool dzp = true;
+    for (int s = 0; s < tabs.nspecies; ++s) dzp = dzp && is_dzp(tabs.sp[s].shape);
+    auto kern = force ? (dzp ? k_tc_fused<true, true> : k_tc_fused<true, false>)
+                      : (dzp ? k_tc_fused<false, true> : k_tc_fused<false, false>);
     int rc = set_smem(kern, smem);
     if (rc) return rc;
     if (ev0) TC_CHECK(cudaEventRecord(ev0, st));
