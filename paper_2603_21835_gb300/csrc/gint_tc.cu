@@ -562,40 +562,56 @@ __host__ __device__ constexpr bool is_dzp(int shape) { return shape == GINT_SHAP
 #define GINT_FOR_SHAPES(X) X(2, 2, 1) X(2, 1, 0) X(1, 1, 1) X(1, 1, 0) X(1, 0, 0) X(3, 3, 2)
 
 // --- per-atom jobs ---
-// Density phase A: scaled orbitals of slot a at point p -> P row p, columns [pcol, pcol + PO).
-template <int PO>
-__device__ __forceinline__ void store_P(const float *v, int pc, int p, float Sphi, unsigned char *Ph,
-                                        unsigned char *Pl, uint32_t sboP) {
+// Scaled orbitals of 8 columns at a point -> P row p, split; fixp (force launches with the three-term split): the
+// values the split stands for as float32 in the same 32 bytes, for the fixed-point split once the row's scale is known,
+// and their largest |value| in m (the rows' maxima and the second split took two passes over the split values before:
+// 64-atom forces 1041 -> 1016 us).
+template <bool FORCE>
+__device__ __forceinline__ void store_P8(const float *v, uint32_t off, float Sphi, unsigned char *Ph, unsigned char *Pl,
+                                         bool fixp, float &m) {
+  uint32_t wh[4], wl[4];
 #pragma unroll
-  for (int k = 0; k < PO; k += 8) {
-    uint32_t wh[4], wl[4];
+  for (int e = 0; e < 4; ++e) split_h2(v[2 * e] * Sphi, v[2 * e + 1] * Sphi, wh[e], wl[e]);
+  if (FORCE && fixp) {
+    uint32_t x[8];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      split_h2(v[k + 2 * e] * Sphi, v[k + 2 * e + 1] * Sphi, wh[e], wl[e]);
+      const float2 hf = __half22float2(*reinterpret_cast<const __half2 *>(&wh[e]));
+      const float2 lf = __half22float2(*reinterpret_cast<const __half2 *>(&wl[e]));
+      const float a = hf.x + lf.x, b = hf.y + lf.y;
+      m = fmaxf(m, fmaxf(fabsf(a), fabsf(b)));
+      x[2 * e] = __float_as_uint(a);
+      x[2 * e + 1] = __float_as_uint(b);
     }
-    const uint32_t off = (p >> 3) * sboP + ((pc + k) >> 3) * 128 + (p & 7) * 16;
-    *reinterpret_cast<uint4 *>(Ph + off) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
-    *reinterpret_cast<uint4 *>(Pl + off) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+    *reinterpret_cast<uint4 *>(Ph + off) = make_uint4(x[0], x[1], x[2], x[3]);
+    *reinterpret_cast<uint4 *>(Pl + off) = make_uint4(x[4], x[5], x[6], x[7]);
+    return;
   }
+  *reinterpret_cast<uint4 *>(Ph + off) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
+  *reinterpret_cast<uint4 *>(Pl + off) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
 }
-// Two atoms of the same shape at once (two independent evaluation chains per thread).
-template <int NS, int NPR, int ND, int PO>
-__device__ __forceinline__ void job_P2(const GTabs &g, const float2 *__restrict__ tab, const BrickSh &sh, int a0,
-                                       int a1, const PointDF &P, int p, bool valid, float Sphi, unsigned char *Ph,
-                                       unsigned char *Pl, uint32_t sboP) {
-  float v0[PO], v1[PO];
-  slot_values<NS, NPR, ND, false>(g, tab, nullptr, sh, a0, P, valid, v0, nullptr);
-  slot_values<NS, NPR, ND, false>(g, tab, nullptr, sh, a1, P, valid, v1, nullptr);
-  store_P<PO>(v0, sh.s_pcol[a0], p, Sphi, Ph, Pl, sboP);
-  store_P<PO>(v1, sh.s_pcol[a1], p, Sphi, Ph, Pl, sboP);
+template <int PO, bool FORCE>
+__device__ __forceinline__ void store_P(const float *v, int pc, int p, float Sphi, unsigned char *Ph,
+                                        unsigned char *Pl, uint32_t sboP, bool fixp, float &m) {
+#pragma unroll
+  for (int k = 0; k < PO; k += 8)
+    store_P8<FORCE>(v + k, (p >> 3) * sboP + ((pc + k) >> 3) * 128 + (p & 7) * 16, Sphi, Ph, Pl, fixp, m);
 }
-template <int NS, int NPR, int ND, int PO>
-__device__ __forceinline__ void job_P(const GTabs &g, const float2 *__restrict__ tab, const BrickSh &sh, int a,
+// Scaled orbitals of slot a0 (and of slot a1 of the same shape, if a1 >= 0) at point p -> P row p.
+template <int NS, int NPR, int ND, int PO, bool FORCE>
+__device__ __forceinline__ void job_P(const GTabs &g, const float2 *__restrict__ tab, const BrickSh &sh, int a0, int a1,
                                       const PointDF &P, int p, bool valid, float Sphi, unsigned char *Ph,
-                                      unsigned char *Pl, uint32_t sboP) {
+                                      unsigned char *Pl, uint32_t sboP, bool fixp, float &m) {
   float v[PO];
-  slot_values<NS, NPR, ND, false>(g, tab, nullptr, sh, a, P, valid, v, nullptr);
-  store_P<PO>(v, sh.s_pcol[a], p, Sphi, Ph, Pl, sboP);
+  slot_values<NS, NPR, ND, false>(g, tab, nullptr, sh, a0, P, valid, v, nullptr);
+  if (a1 >= 0) {
+    float v1[PO];
+    slot_values<NS, NPR, ND, false>(g, tab, nullptr, sh, a1, P, valid, v1, nullptr);
+    store_P<PO, FORCE>(v, sh.s_pcol[a0], p, Sphi, Ph, Pl, sboP, fixp, m);
+    store_P<PO, FORCE>(v1, sh.s_pcol[a1], p, Sphi, Ph, Pl, sboP, fixp, m);
+  } else {
+    store_P<PO, FORCE>(v, sh.s_pcol[a0], p, Sphi, Ph, Pl, sboP, fixp, m);
+  }
 }
 
 // One image's rho and force contributions of slot a at a point, the terms and their order those of add_image_fast with
@@ -768,7 +784,7 @@ __device__ __forceinline__ void job_F(const GTabs &g, const float2 *__restrict__
 // Generic-shape jobs (any species up to GINT_MAX_ORB_ATOM orbitals).
 __device__ __noinline__ void job_P_generic(const GTabs &g, const float2 *__restrict__ tab, const BrickSh &sh, int a,
                                            int p, bool valid, float Sphi, unsigned char *Ph,
-                                           unsigned char *Pl, uint32_t sboP) {
+                                           unsigned char *Pl, uint32_t sboP, bool fixp, float &m) {
   float v[GINT_MAX_ORB_ATOM];
   const int po = sh.s_po[a], pc = sh.s_pcol[a];
   for (int i = 0; i < po; ++i) v[i] = 0.f;
@@ -781,15 +797,8 @@ __device__ __noinline__ void job_P_generic(const GTabs &g, const float2 *__restr
         add_image_generic<false>(g, tab, nullptr, S, dh, dl, v, nullptr);
     }
   }
-  for (int k = 0; k < po; k += 8) {
-    uint32_t wh[4], wl[4];
-    for (int e = 0; e < 4; ++e) {
-      split_h2(v[k + 2 * e] * Sphi, v[k + 2 * e + 1] * Sphi, wh[e], wl[e]);
-    }
-    const uint32_t off = (p >> 3) * sboP + ((pc + k) >> 3) * 128 + (p & 7) * 16;
-    *reinterpret_cast<uint4 *>(Ph + off) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
-    *reinterpret_cast<uint4 *>(Pl + off) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-  }
+  for (int k = 0; k < po; k += 8)
+    store_P8<true>(v + k, (p >> 3) * sboP + ((pc + k) >> 3) * 128 + (p & 7) * 16, Sphi, Ph, Pl, fixp, m);
 }
 __device__ __noinline__ void job_F_generic(const GTabs &g, const float2 *__restrict__ tab,
                                            const float *__restrict__ dtab, const BrickSh &sh, int a, int p, bool valid,
@@ -1010,6 +1019,7 @@ __device__ __forceinline__ void brick_body(const GTabs &g, const GSys &S, long l
       const int li = prefetch_index(warp);
       if (li >= 0 && li < nch && li < nst) issue_copies(S, li, li, NP, na);
     }
+    float pmax = 0.f;  // fixp: the largest |value| of this thread's slots at its point
     // ---- phase A: scaled orbitals of all atoms at every point -> P (hi, lo), zero padding
     for (int a = q; a < na; a += 4) {
       const int gap0 = gap_begin(sh, a), pc = sh.s_pcol[a];
@@ -1029,55 +1039,30 @@ __device__ __forceinline__ void brick_body(const GTabs &g, const GSys &S, long l
       const float2 *tab = S.tab, *tabi = S.tabi;
       const PointDF P = point_df(sh, p);
       for (int a = q; a < na; a += 8) {
-        const int a1 = a + 4;
         const int shp = g.sp[sh.s_sp[a]].shape;
-        const bool pair = a1 < na && g.sp[sh.s_sp[a1]].shape == shp;
-        switch (shp) {
-#define CASE_P(ns, np_, nd)                                                                                      \
-case GINT_SHAPE(ns, np_, nd):                                                                                \
-  if constexpr (DZP && !is_dzp(GINT_SHAPE(ns, np_, nd))) {} else                                                  \
-  if (pair)                                                                                                  \
-    job_P2<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, sh, a, a1, P, p, valid, Sphi, Ph, Pl, sboP); \
-  else                                                                                                       \
-    job_P<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, sh, a, P, p, valid, Sphi, Ph, Pl, sboP);    \
+        int a1 = a + 4 < na && shp != 0 && g.sp[sh.s_sp[a + 4]].shape == shp ? a + 4 : -1, a0 = a;
+        for (;;) {  // a pair of one shape, or one after the other
+          switch (g.sp[sh.s_sp[a0]].shape) {
+#define CASE_P(ns, np_, nd)                                                                                            \
+case GINT_SHAPE(ns, np_, nd):                                                                                          \
+  if constexpr (!DZP || is_dzp(GINT_SHAPE(ns, np_, nd)))                                                               \
+  job_P<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8, FORCE>(g, tabi, sh, a0, a1, P, p, valid, Sphi, Ph, Pl, sboP, \
+                                                                 fixp, pmax);                                          \
   break;
-          GINT_FOR_SHAPES(CASE_P)
+            GINT_FOR_SHAPES(CASE_P)
 #undef CASE_P
-          default:
-            if constexpr (!DZP) job_P_generic(g, tab, sh, a, p, valid, Sphi, Ph, Pl, sboP);
-        }
-        if (a1 < na && !(pair && shp != 0)) {
-          switch (g.sp[sh.s_sp[a1]].shape) {
-#define CASE_P1(ns, np_, nd)                                                                                      \
-case GINT_SHAPE(ns, np_, nd):                                                                                 \
-  if constexpr (!DZP || is_dzp(GINT_SHAPE(ns, np_, nd)))                                                      \
-  job_P<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, sh, a1, P, p, valid, Sphi, Ph, Pl, sboP);    \
-  break;
-            GINT_FOR_SHAPES(CASE_P1)
-#undef CASE_P1
             default:
-              if constexpr (!DZP) job_P_generic(g, tab, sh, a1, p, valid, Sphi, Ph, Pl, sboP);
+              if constexpr (!DZP) job_P_generic(g, tab, sh, a0, p, valid, Sphi, Ph, Pl, sboP, fixp, pmax);
           }
+          if (a1 >= 0 || a0 != a || a + 4 >= na) break;
+          a0 = a + 4;
         }
       }
     }
     if (fixp) {
       // ---- fixed-point rows: s_p from the row's largest |value| (the four slices' maxima), then
-      // every element x = (hi + lo) s_p re-split as hi = rint(x), lo = x - hi (float16)
-      float m = 0.f;
-      for (int a = q; a < na; a += 4)
-        for (int k = sh.s_pcol[a]; k < sh.s_pcol[a] + sh.s_po[a]; k += 8) {
-          const uint32_t off = (p >> 3) * sboP + (k >> 3) * 128 + (p & 7) * 16;
-          const uint4 wh = *reinterpret_cast<const uint4 *>(Ph + off), wl = *reinterpret_cast<const uint4 *>(Pl + off);
-          const uint32_t hw[4] = {wh.x, wh.y, wh.z, wh.w}, lw[4] = {wl.x, wl.y, wl.z, wl.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 hf = __half22float2(*reinterpret_cast<const __half2 *>(&hw[e]));
-            const float2 lf = __half22float2(*reinterpret_cast<const __half2 *>(&lw[e]));
-            m = fmaxf(m, fmaxf(fabsf(hf.x + lf.x), fabsf(hf.y + lf.y)));
-          }
-        }
-      sh.rpart[q][p] = m;
+      // every element x s_p split as hi = rint(x s_p), lo = x s_p - hi (float16)
+      sh.rpart[q][p] = pmax;
       __syncthreads();
       const float rm = fmaxf(fmaxf(sh.rpart[0][p], sh.rpart[1][p]), fmaxf(sh.rpart[2][p], sh.rpart[3][p]));
       int ex = 0;
@@ -1087,15 +1072,12 @@ case GINT_SHAPE(ns, np_, nd):                                                   
       for (int a = q; a < na; a += 4)
         for (int k = sh.s_pcol[a]; k < sh.s_pcol[a] + sh.s_po[a]; k += 8) {
           const uint32_t off = (p >> 3) * sboP + (k >> 3) * 128 + (p & 7) * 16;
-          const uint4 wh = *reinterpret_cast<const uint4 *>(Ph + off), wl = *reinterpret_cast<const uint4 *>(Pl + off);
-          const uint32_t hw[4] = {wh.x, wh.y, wh.z, wh.w}, lw[4] = {wl.x, wl.y, wl.z, wl.w};
+          const float4 x = *reinterpret_cast<const float4 *>(Ph + off), y = *reinterpret_cast<const float4 *>(Pl + off);
           uint32_t oh[4], ol[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 hf = __half22float2(*reinterpret_cast<const __half2 *>(&hw[e]));
-            const float2 lf = __half22float2(*reinterpret_cast<const __half2 *>(&lw[e]));
-            split_fx2((hf.x + lf.x) * sp, (hf.y + lf.y) * sp, oh[e], ol[e]);
-          }
+          split_fx2(x.x * sp, x.y * sp, oh[0], ol[0]);
+          split_fx2(x.z * sp, x.w * sp, oh[1], ol[1]);
+          split_fx2(y.x * sp, y.y * sp, oh[2], ol[2]);
+          split_fx2(y.z * sp, y.w * sp, oh[3], ol[3]);
           *reinterpret_cast<uint4 *>(Ph + off) = make_uint4(oh[0], oh[1], oh[2], oh[3]);
           *reinterpret_cast<uint4 *>(Pl + off) = make_uint4(ol[0], ol[1], ol[2], ol[3]);
         }
