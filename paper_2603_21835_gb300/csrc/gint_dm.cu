@@ -15,11 +15,14 @@
 // k_dm_pack: operands -> hi/lo core-matrix blocks: block (row tile t, chunk q) is 32 KB,
 //   [hi 16 KB | lo 16 KB], each 128 rows x 64 k float16, core matrix (row group g, k group h) at
 //   byte (g * 8 + h) * 128 (K-major, no swizzle: LBO 128, SBO 1024).  Rows >= n, k >= 2 nocc: 0.
-// k_dm_mma: one CTA of 16 warps per tile pair I <= J of D (128 x 128).  Lane 0 of warp 0 streams
-//   the A (tile I) and B (tile J) blocks of each chunk by two bulk copies into a 3-stage ring and
-//   issues 12 MMAs per chunk (4 K steps x 3 products); all 16 warps drain the hi hi accumulators
-//   (row = TMEM lane, 32 columns a warp) and write D[i, j] and D[j, i] from one value, so D is
-//   symmetric bit for bit.  (Sixteen warps keep the register cap at 128 for the Kahan sums.)
+// k_dm_mma: one CTA of 18 warps per tile pair I <= J of D (128 x 128).  A load warp streams the A (tile I) and B
+//   (tile J) blocks of each chunk by two bulk copies into a 3-stage ring, an MMA warp issues 12 MMAs per chunk (4 K
+//   steps x 3 products), and 16 warps drain the hi hi accumulators (row = TMEM lane, 32 columns a warp) and write
+//   D[i, j] and D[j, i] from one value, so D is symmetric bit for bit.  (A tcgen05.mma holds its issuer up while the
+//   queue is full: loads and drains by the same warp waited behind it.)
+//   6656 orbitals, 1024 states: 755 us with warp 0 loading, issuing and draining, 650 us with warps of their own, 446 us
+//   with panels of tiles, whole-line stores and two float64 instructions a result instead of six (a warp's takes 16
+//   clocks of the SM; a quarter of the time is left there, a quarter in the tensor pipe, the drains issue for half).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -43,9 +46,12 @@ constexpr uint32_t kHalfBytes = kTile * kKC * 2;  // one float16 part of a block
 constexpr uint32_t kBlockBytes = 2 * kHalfBytes;  // hi then lo
 constexpr uint32_t kStageBytes = 2 * kBlockBytes;  // A block then B block
 constexpr uint32_t kSmemBytes = kStages * kStageBytes;
+constexpr int kLdD = kTile + 1;  // doubles a row of the D tile takes in shared memory
+static_assert(kTile * kLdD * 8 <= kSmemBytes, "D tile over the stages");
 constexpr int kDrainWarps = 16;                   // four per TMEM lane quarter, 32 columns each
 constexpr int kDrainCols = kTile / (kDrainWarps / 4);
-constexpr int kDmThreads = 32 * kDrainWarps;
+constexpr int kMmaWarp = kDrainWarps, kLoadWarp = kDrainWarps + 1;
+constexpr int kDmThreads = 32 * (kDrainWarps + 2);
 static_assert(kCrossCol + 128 <= kTmemCols, "tensor memory columns");
 constexpr long long kWaitNs = 2000000000LL;  // bounded waits: 2 s
 constexpr unsigned kErrTimeout = 1u;
@@ -107,6 +113,22 @@ __device__ __forceinline__ void split_f16(float x, __half &hi, __half &lo) {
   lo = __float2half_rn(x - __half2float(hi));
 }
 
+__device__ __noinline__ float scaled_f32_slow(double x, int e) { return (float)(x * ldexp(1.0, e)); }
+// (k_dm_pack was bound by float64 instructions, 6 a state and thread: 114 us -> 40 us for 109 MB in and 109 MB out.)
+// (float)(x 2^e) rounded to nearest even, in integer arithmetic while the result is a normal float32 (a float64
+// multiplication and a conversion take the SM's float64 pipe 32 clocks a warp).
+__device__ __forceinline__ float scaled_f32(double x, int e) {
+  e = max(e, -3000);  // (a scale of 0: infinite maximum)
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int te = (int)((hi >> 20) & 0x7ffu) - 1023 + 127 + e;
+  if (te > 0 && te < 254 && (hi & 0x7ff00000u)) {
+    const uint32_t m = ((uint32_t)te << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29), rem = lo & 0x1fffffffu;
+    return __uint_as_float(((hi & 0x80000000u) | m) + (rem + (m & 1u) > 0x10000000u ? 1u : 0u));
+  }
+  if ((hi << 1 | lo) == 0u) return __uint_as_float(hi);
+  return scaled_f32_slow(x, e);
+}
+
 // Block (x, y): rows i = 128 x + t of the operands, groups of 8 k (4 states) kg = y, y + gridDim.y,
 // ...; each thread reads psi[s][i] (coalesced over i) and writes one 16-byte core-matrix row of hi
 // and of lo, for A and for B.  B = 2^sigmaB psi is scaled in float64 (exact) and rounded to float32
@@ -116,9 +138,12 @@ __global__ void __launch_bounds__(kTile) k_dm_pack(int n, int nocc, int nq, cons
                                                    const double *__restrict__ f, const unsigned long long *__restrict__ m,
                                                    unsigned char *__restrict__ PA, unsigned char *__restrict__ PB) {
   const int sa = dm_sigma(m[0]), sb = dm_sigma(m[1]);
-  const double scb = ldexp(1.0, sb), rab = ldexp(1.0, sa - sb);
+  __shared__ float s_f[4];
   const int t = blockIdx.x, r = threadIdx.x, i = t * kTile + r;
   for (int kg = blockIdx.y; kg < nq * (kKC / 8); kg += gridDim.y) {
+    __syncthreads();
+    if (r < 4) s_f[r] = kg * 4 + r < nocc ? scaled_f32(f[kg * 4 + r], sa - sb) : 0.f;
+    __syncthreads();
     __align__(16) __half ah[8], al[8], bh[8], bl[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -126,9 +151,9 @@ __global__ void __launch_bounds__(kTile) k_dm_pack(int n, int nocc, int nq, cons
       float bx = 0.f, by = 0.f, fa = 0.f;
       if (i < n && s < nocc) {
         const double2 p = psi[(long long)s * n + i];
-        bx = (float)(p.x * scb);
-        by = (float)(p.y * scb);
-        fa = (float)(f[s] * rab);
+        bx = scaled_f32(p.x, sb);
+        by = scaled_f32(p.y, sb);
+        fa = s_f[j];
       }
       split_f16(bx * fa, ah[2 * j], al[2 * j]);
       split_f16(by * fa, ah[2 * j + 1], al[2 * j + 1]);
@@ -157,6 +182,46 @@ struct DmShared {
   uint32_t tmem;
 };
 
+__device__ __noinline__ double times_pow2_slow(double x, int e) { return x * ldexp(1.0, e); }
+// p = J (J + 1) / 2 + I, 0 <= I <= J.
+__device__ __forceinline__ void tri_index(long long p, int &I, int &J) {
+  J = (int)((sqrt(8.0 * (double)p + 1.0) - 1.0) * 0.5);
+  while ((long long)J * (J + 1) / 2 > p) --J;
+  while ((long long)(J + 1) * (J + 2) / 2 <= p) ++J;
+  I = (int)(p - (long long)J * (J + 1) / 2);
+}
+// Tile pair p -> (I, J), I <= J < T, by panels of kPanel columns J, rows I first: the CTAs that run at one time read
+// about kPanel row tiles of A and kPanel of B (a chunk of theirs is 1.5 MB in L2, 24 tiles of K = 2048 24 MB), not
+// all of A for one column of B.
+constexpr int kPanel = 12;
+__device__ __forceinline__ void dm_tile(long long p, int T, int &I, int &J) {
+  int x, y;
+  tri_index(p, x, y);
+  const int J0 = y / kPanel * kPanel, w = min(kPanel, T - J0);
+  const long long q = p - (long long)J0 * (J0 + 1) / 2;
+  if (q < (long long)J0 * w) {
+    I = (int)(q / w);
+    J = J0 + (int)(q - (long long)I * w);
+  } else {
+    tri_index(q - (long long)J0 * w, x, y);
+    I = J0 + x;
+    J = J0 + y;
+  }
+}
+// (double)x for a normal x or zero (smaller values count as zero) in integer arithmetic: a conversion takes the SM's
+// float64 pipe 16 clocks a warp.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), m = b & 0x7fffffu, e = (b >> 23) & 0xffu;
+  return e ? __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | (m >> 3)), (int)(m << 29)) : 0.0;
+}
+// x 2^e for a result in the normal range, else by multiplication.
+__device__ __forceinline__ double times_pow2(double x, int e) {
+  const int hi = __double2hiint(x), t = ((hi >> 20) & 0x7ff) + e;
+  if ((hi & 0x7ff00000) && (unsigned)(t - 1) < 2045u && (hi & 0x7ff00000) != 0x7ff00000)
+    return __hiloint2double(hi + (e << 20), __double2loint(x));
+  return times_pow2_slow(x, e);
+}
+
 // Copies of chunk c (A tile I, B tile J) into its stage.
 __device__ __forceinline__ void dm_load(DmShared &sh, unsigned char *smem, const unsigned char *PA,
                                         const unsigned char *PB, int I, int J, int nq, int c) {
@@ -176,11 +241,11 @@ __device__ __forceinline__ bool dm_drain(DmShared &sh, uint32_t lane_base, int c
   if (!ok) return false;
   tc_fence_after();
 #pragma unroll
-  for (int g = 0; g < kDrainCols / 16; ++g) {
-    float y[16];
-    tmem_ld16(lane_base + (uint32_t)a * 128u + (uint32_t)g * 16u, y);
+  for (int g = 0; g < kDrainCols / 8; ++g) {  // (by 8 columns: 18 warps leave a thread 96 registers, 64 of them sums)
+    float y[8];
+    tmem_ld8(lane_base + (uint32_t)a * 128u + (uint32_t)g * 8u, y);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) kahan_add(sum[g * 16 + j], cmp[g * 16 + j], y[j]);
+    for (int j = 0; j < 8; ++j) kahan_add(sum[g * 8 + j], cmp[g * 8 + j], y[j]);
   }
   tc_fence_before();
   __syncwarp();
@@ -194,12 +259,8 @@ __global__ void __launch_bounds__(kDmThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ DmShared sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // tile pair p -> (I, J), I <= J, p = J (J + 1) / 2 + I
-  const long long p = blockIdx.x;
-  int J = (int)((sqrt(8.0 * (double)p + 1.0) - 1.0) * 0.5);
-  while ((long long)J * (J + 1) / 2 > p) --J;
-  while ((long long)(J + 1) * (J + 2) / 2 <= p) ++J;
-  const int I = (int)(p - (long long)J * (J + 1) / 2);
+  int I, J;
+  dm_tile(blockIdx.x, (n + kTile - 1) / kTile, I, J);
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -213,7 +274,7 @@ __global__ void __launch_bounds__(kDmThreads, 1)
     mbar_init(&sh.done, 1);
     fence_mbar_init();
   }
-  if (warp == 0) {
+  if (warp == kMmaWarp) {
     tmem_alloc(&sh.tmem, kTmemCols);
     tmem_relinquish();
   }
@@ -230,96 +291,97 @@ __global__ void __launch_bounds__(kDmThreads, 1)
   for (int j = 0; j < kDrainCols; ++j) sum[j] = cmp[j] = 0.f;
   bool ok = true;
 
-  if (warp == 0) {
-    // the warp runs the issue loop together (warp-uniform descriptor arithmetic; one elected lane
-    // issues, which keeps the tensor pipe fed better than a loop confined to one lane): chunk c's
-    // MMAs (hi hi into ring slot c mod kHH, hi lo + lo hi into the cross slot), then the refill of
-    // chunk c - 1's stage once its MMAs are done (lane 0 issues the copies); the warp drains chunk
-    // c - 2 (the slot the MMAs of chunk c + 1 will take).  Wait results are lane 0's, broadcast.
+  if (warp == kLoadWarp) {
+    int c = 0;
+    for (; c < nq; ++c) {
+      if (c >= kStages)
+        ok = __all_sync(0xffffffffu, mbar_wait(&sh.empty[c % kStages], (uint32_t)(c / kStages - 1) & 1u, status, kErrTimeout,
+                                               kWaitNs));
+      if (!ok) break;
+      if (lane == 0) dm_load(sh, smem, PA, PB, I, J, nq, c);
+      __syncwarp();
+    }
+    // no copy may still be landing in shared memory when the CTA exits
+    for (int k = max(0, c - kStages); k < c; ++k)
+      mbar_wait(&sh.full[k % kStages], (uint32_t)(k / kStages) & 1u, status, kErrTimeout, kWaitNs);
+  } else if (warp == kMmaWarp) {
+    // the warp runs the issue loop together (warp-uniform descriptor arithmetic; one elected lane issues): chunk c's
+    // MMAs, hi hi into ring slot c mod kHH, hi lo + lo hi into the cross slot
     const uint32_t idesc = idesc_f16(kTile, kTile), sbase = smem_u32(smem), dx = tmem + kCrossCol;
-    int issued = 0, consumed = 0;
-    for (; issued < min(kStages, nq); ++issued)
-      if (lane == 0) dm_load(sh, smem, PA, PB, I, J, nq, issued);
-    for (int c = 0; c < nq && ok; ++c) {
+    for (int c = 0; c < nq; ++c) {
       const int s = c % kStages, a = c % kHH;
-      bool lok = mbar_wait(&sh.full[s], (uint32_t)(c / kStages) & 1u, status, kErrTimeout, kWaitNs);
-      lok = __shfl_sync(0xffffffffu, lok, 0);
-      if (lok) consumed = c + 1;
-      if (lok && c >= kHH)
-        lok = __shfl_sync(0xffffffffu,
-                          mbar_wait(&sh.hfree[a], (uint32_t)((c / kHH) - 1) & 1u, status, kErrTimeout, kWaitNs), 0);
-      if (lok) {
-        tc_fence_after();
-        const uint32_t sa = sbase + s * kStageBytes, sb = sa + kBlockBytes;
-        const uint32_t dh = tmem + (uint32_t)a * 128u;
-        if (elect_one()) {
+      ok = mbar_wait(&sh.full[s], (uint32_t)(c / kStages) & 1u, status, kErrTimeout, kWaitNs);
+      if (c >= kHH) ok = ok && mbar_wait(&sh.hfree[a], (uint32_t)((c / kHH) - 1) & 1u, status, kErrTimeout, kWaitNs);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t sa = sbase + s * kStageBytes, dh = tmem + (uint32_t)a * 128u;
+      const uint64_t ah0 = sdesc(sa, 128, 1024), al0 = sdesc(sa + kHalfBytes, 128, 1024);
+      const uint64_t bh0 = sdesc(sa + kBlockBytes, 128, 1024), bl0 = sdesc(sa + kBlockBytes + kHalfBytes, 128, 1024);
+      if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < kKC / 16; ++ks) {
-            const uint32_t o = ks * 256;  // two core matrices along K per step
-            const uint64_t ah = sdesc(sa + o, 128, 1024), al = sdesc(sa + kHalfBytes + o, 128, 1024);
-            const uint64_t bh = sdesc(sb + o, 128, 1024), bl = sdesc(sb + kHalfBytes + o, 128, 1024);
-            mma_f16(dh, ah, bh, idesc, ks > 0 ? 1u : 0u);
-            mma_f16(dx, ah, bl, idesc, (c > 0 || ks > 0) ? 1u : 0u);
-            mma_f16(dx, al, bh, idesc, 1u);
-          }
-          mma_commit(&sh.empty[s]);
-          mma_commit(&sh.hfull[a]);
+        for (int ks = 0; ks < kKC / 16; ++ks) {
+          const uint64_t o = (uint64_t)(ks * (256 >> 4));  // two core matrices along K per step
+          mma_f16(dh, ah0 + o, bh0 + o, idesc, ks > 0 ? 1u : 0u);
+          mma_f16(dx, ah0 + o, bl0 + o, idesc, (c > 0 || ks > 0) ? 1u : 0u);
+          mma_f16(dx, al0 + o, bh0 + o, idesc, 1u);
         }
-        __syncwarp();
-        if (c >= 1 && issued < nq) {
-          lok = __shfl_sync(0xffffffffu,
-                            mbar_wait(&sh.empty[(c - 1) % kStages], (uint32_t)((c - 1) / kStages) & 1u, status,
-                                      kErrTimeout, kWaitNs),
-                            0);
-          if (lok) {
-            if (lane == 0) dm_load(sh, smem, PA, PB, I, J, nq, issued);
-            ++issued;
-          }
-        }
+        mma_commit(&sh.empty[s]);
+        mma_commit(&sh.hfull[a]);
       }
-      ok = lok;
-      if (ok && c >= 2) ok = dm_drain(sh, lane_base, c - 2, sum, cmp, status);
+      __syncwarp();
     }
     if (elect_one()) mma_commit(&sh.done);  // the lane that issued the MMAs
     __syncwarp();
-    if (lane == 0) {
-      // no copy may still be landing in shared memory when the CTA exits
-      for (int c = consumed; c < issued; ++c)
-        mbar_wait(&sh.full[c % kStages], (uint32_t)(c / kStages) & 1u, status, kErrTimeout, kWaitNs);
-    }
-    for (int c = max(0, nq - 2); c < nq && ok; ++c) ok = dm_drain(sh, lane_base, c, sum, cmp, status);
   } else {
     for (int c = 0; c < nq && ok; ++c) ok = dm_drain(sh, lane_base, c, sum, cmp, status);
   }
 
-  ok = __all_sync(0xffffffffu, ok && mbar_wait(&sh.done, 0u, status, kErrTimeout, kWaitNs));
+  ok = ok && mbar_wait(&sh.done, 0u, status, kErrTimeout, kWaitNs);
+  ok = __syncthreads_and(ok);  // (one answer for the CTA: the epilogue has a barrier)
   tc_fence_after();
-  if (ok) {
-    const double scale = ldexp(1.0, -(dm_sigma(m[0]) + dm_sigma(m[1])));
+  if (ok && warp < kDrainWarps) {
+    // D[j, i] leaves from the registers (lanes along i), D[i, j] through shared memory (the stages are free), rows of
+    // kLdD doubles: both in whole cache lines
+    const int es = -(dm_sigma(m[0]) + dm_sigma(m[1]));
     const long long i = (long long)I * kTile + r;
+    double *const T = reinterpret_cast<double *>(smem);
 #pragma unroll
-    for (int g = 0; g < kDrainCols / 16; ++g) {
-      float x[16];
-      tmem_ld16(lane_base + kCrossCol + (uint32_t)g * 16u, x);
+    for (int g = 0; g < kDrainCols / 8; ++g) {
+      float x[8];
+      tmem_ld8(lane_base + kCrossCol + (uint32_t)g * 8u, x);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const long long jj = (long long)J * kTile + c0 + g * 16 + j;
-        if (i < n && jj < n && (I != J || jj >= i)) {
-          const double v = (((double)sum[g * 16 + j] - (double)cmp[g * 16 + j]) + (double)x[j]) * scale;
-          D[i * n + jj] = v;
-          D[jj * n + i] = v;
+      for (int j = 0; j < 8; ++j) {
+        const float a = sum[g * 8 + j], b = cmp[g * 8 + j];
+        double v;
+        if (fabsf(a) < INFINITY && fabsf(b) < INFINITY && fabsf(x[j]) < INFINITY)
+          v = times_pow2((widen(a) - widen(b)) + widen(x[j]), es);
+        else
+          v = (((double)a - (double)b) + (double)x[j]) * ldexp(1.0, es);
+        const int c = c0 + g * 8 + j;
+        const long long jj = (long long)J * kTile + c;
+        if (I != J || c >= r) {
+          T[r * kLdD + c] = v;
+          if (I == J) T[c * kLdD + r] = v;
+          if (I != J && i < n && jj < n) D[jj * n + i] = v;
         }
       }
     }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kDrainWarps) : "memory");
+    for (int u = warp; u < kTile * (kTile / 32); u += kDrainWarps) {
+      const int rr = u / (kTile / 32), c = (u % (kTile / 32)) * 32 + lane;
+      const long long ii = (long long)I * kTile + rr, jj = (long long)J * kTile + c;
+      if (ii < n && jj < n) D[ii * n + jj] = T[rr * kLdD + c];
+    }
   }
-  if (!ok && warp == 0 && lane == 0) {
+  if (!ok && warp == kMmaWarp && lane == 0) {
     // before the tensor memory is released: once more (bounded) for the MMAs issued so far, which
     // complete by themselves; if they still have not, say so
     if (!mbar_wait(&sh.done, 0u, status, kErrTimeout, 4 * kWaitNs)) atomicOr(status, kErrInflight);
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+  if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
 }
 
 }  // namespace
