@@ -250,7 +250,7 @@ def run_reference(args):
 # kernels of ours per step (density + local-H passes; memsets are not kernels):
 #   fp64: k_simt_rho, k_simt_vlocal;  fp32: k_to_f32, k_simt_rho, k_simt_vlocal;
 #   f16x3 / f16x1: k_prep, k_build_tiles, k_tc_fused (both passes), k_h_reduce
-KERNEL_LAUNCHES = {"fp64": 2, "fp32": 3, "f16x3": 4, "f16x1": 4}
+KERNEL_LAUNCHES = {"fp64": None, "fp32": 3, "f16x3": 4, "f16x1": 4}
 TENSOR_PRECISIONS = ("f16x3", "f16x1")
 
 
@@ -477,14 +477,17 @@ def run_cn(n, nocc, steps, stream):
     # (n^3 / 3), solves with n right-hand sides (2 n^3)
     fl_step = 12.0 * n * n * nocc + 4.0 / 3.0 * n ** 3
     fl_d, fl_e = 2.0 * n * n * nocc, (4.0 + 1.0 / 3.0) * n ** 3
+    peaks, peak_kind = load_peaks()
+    peak = peaks["bf16_tflops"] / 36
     step_tf, dm_tf, edm_tf = (fl / (ms * 1e-3) / 1e12 for fl, ms in ((fl_step, ms_s), (fl_d, ms_d), (fl_e, ms_e)))
     return {"n": n, "nocc": nocc, "ms_step": ms_s, "step_tflops": step_tf,
             "ms_density_matrix": ms_d, "dm_tflops": dm_tf,
             "ms_energy_density_matrix": ms_e, "edm_tflops": edm_tf,
-            "fp64": {"kernels": "k_gemm, k_ldl_diag, k_trsv (hand-written float64 on the CUDA cores)",
-                     "bound": "fp64", "peak_tflops": FP64_NOMINAL_TFLOPS, "peak_source": "nominal (none measured)",
-                     "step_frac": step_tf / FP64_NOMINAL_TFLOPS, "dm_frac": dm_tf / FP64_NOMINAL_TFLOPS,
-                     "edm_frac": edm_tf / FP64_NOMINAL_TFLOPS},
+            # float64 products as 36 exact float16 digit products (k_sg_*): their ceiling is the tensor rate over 36;
+            # diagonal blocks and substitutions run on the CUDA cores (1.25 TFLOP/s nominal)
+            "fp64": {"kernels": "k_sg_pack, k_sg_mma (exact digit products), k_ldl_diag, k_trsv",
+                     "bound": "tensor", "peak_tflops": peak, "peak_source": f"{peak_kind} bf16 burst / 36 digit products",
+                     "step_frac": step_tf / peak, "dm_frac": dm_tf / peak, "edm_frac": edm_tf / peak},
             "ms_density_matrix_f16x3": ms_t, "dm_f16x3_tflops_real_part": 4.0 * n * n * nocc / (ms_t * 1e-3) / 1e12,
             "dm_f16x3_tensor_tflops": tc_flops / (ms_t * 1e-3) / 1e12,
             "solver_info": info, "precision": "c128 / f64; f16x3 tensor-core D build"}
@@ -663,15 +666,17 @@ def main():
     else:
         mr = statistics.mean(a.elapsed_time(b) for a, b in evr)
         mh = statistics.mean(a.elapsed_time(b) for a, b in evh)
-        dom, tdom = ("k_simt_rho", mr) if mr >= mh else ("k_simt_vlocal", mh)
+        k64 = args.precision == "fp64"  # orbital evaluation and digit products per batch of bricks
+        dom, tdom = (("k_fx_eval + k_fx_mma (density)" if k64 else "k_simt_rho", mr) if mr >= mh else
+                     ("k_fx_eval + k_fx_mma (local H)" if k64 else "k_simt_vlocal", mh))
         flops = 2.0 * W  # one pass per launch, 2 flops per ordered orbital pair per grid point
     if tensor:
         peak = peaks.get("bf16_tflops")
         bound, punit = "tensor", "TFLOP/s"
         pdesc = f"f16 dense = {peak_kind} bf16 burst (nominal f16 and bf16 dense rates are equal)"
     elif args.precision == "fp64":
-        peak = FP64_NOMINAL_TFLOPS
-        bound, punit, pdesc = "alu", "TFLOP/s", "fp64 nominal 1.25 TFLOP/s (GB300)"
+        peak = peaks.get("bf16_tflops") / 36
+        bound, punit, pdesc = "tensor", "TFLOP/s", f"{peak_kind} bf16 burst / 36 float16 digit products"
     else:
         mhz = clocks.get("sm_mhz") or 2070.0
         peak = FP32_SIMT_TFLOPS_PER_GHZ * mhz / 1e3
@@ -736,6 +741,10 @@ def main():
         cn = run_cn(g.norb, 128 if g.norb < 2048 else 1024, 3 if g.norb < 2048 else 2, stream)
 
     launches = KERNEL_LAUNCHES.get(args.precision)
+    if args.precision == "fp64":  # digits of D, two kernels a batch of bricks and pass (one brick per SM), the mirror
+        n1, n2, n3 = w.system.grid
+        bricks = -(-n1 // 4) * -(-n2 // 4) * -(-n3 // 8)
+        launches = 3 + 4 * -(-bricks // torch.cuda.get_device_properties(dev).multi_processor_count)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": max(3, args.warmup), "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",

@@ -21,17 +21,11 @@
 
 #include "gint.h"
 #include "gint_la.cuh"
+#include "gint_sgpack.cuh"
 
 namespace gla {
 namespace {
 
-// Programmatic dependent launch: the kernels below are launched while their predecessor runs; everything up to
-// here (arguments, index arithmetic) overlaps its tail, and this waits until its results are visible.  The
-// successor may be launched from here on.
-__device__ __forceinline__ void grid_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
 __device__ __forceinline__ double shfl(double x, int lane) { return __shfl_sync(0xffffffffu, x, lane); }
 __device__ __forceinline__ double2 shfl(double2 x, int lane) {
   return make_double2(__shfl_sync(0xffffffffu, x.x, lane), __shfl_sync(0xffffffffu, x.y, lane));
@@ -177,6 +171,85 @@ __global__ void __launch_bounds__(kDT) k_ldl_diag(int nb, T *__restrict__ A, lon
   }
 }
 
+// ------------------------------------------------- digits of the next product's operands (gint_sgpack.cuh)
+// A launch of its own for them took 9 us a panel, as long as the solve before it: the solve's CTAs cut the vectors they
+// have just formed, and in the backward substitution, where the left operand is part of the factor and waits for
+// nothing, further CTAs of the same launch cut that one.
+__device__ __forceinline__ void pack_left(const SgOperand &o, int rb, double (*t)[kPK + 1]) {
+  const int tid = threadIdx.x, r0 = rb * kPR;
+  grid_wait();  // (the digits' place was read by the product before)
+  if (tid < kPT) sg_load_tile(o, tid, r0, 0, t);
+  __syncthreads();
+  const int r = r0 + (tid >> 3);
+  if (tid >= kPT) return;
+  const int em = sg_row_exp(t, tid);
+  if (r >= o.R) return;
+  if ((tid & 7) == 0) o.e[r] = em;
+  sg_store_group(o, r, tid & 7, em, [&](int j) { return t[tid >> 3][8 * (tid & 7) + j]; });
+}
+__device__ __forceinline__ void put(double *t, int i, double x) { t[i] = x; }
+__device__ __forceinline__ void put(double *t, int i, double2 x) {
+  t[2 * i] = x.x;
+  t[2 * i + 1] = x.y;
+}
+// Vectors v0 .. v0 + SV - 1 of a solve, element i of vector vl: x (before the division by D) and y.
+//   PANEL: vectors v < nv are rows v of the left operand W and of the right operand L of product 0 and of the left
+//   operand L of product 1; the others rows of the right operand W of product 1.  Otherwise all are rows of the right
+//   operand of product 0.  (Rows of a complex left operand come in pairs, see SgView.)
+template <typename T, int SV, bool PANEL>
+__device__ __forceinline__ void pack_vectors(const SgPack &pk, int npk, int v0, int nv, int nv2, int i, int vl, T x, T y,
+                                             double (*t)[kPK + 1]) {
+  constexpr bool C = sizeof(T) == 16;
+  static_assert(SV == 8, "");
+  __shared__ int s_e[2 * SV];
+  const int tid = threadIdx.x;
+  put(t[vl], i, x);
+  put(t[SV + vl], i, y);
+  __syncthreads();
+  if (tid < 2 * SV * 16) {
+    int m = 1;
+#pragma unroll
+    for (int q = 0; q < kPK / 16; ++q) m = max(m, exp_field(t[tid >> 4][(tid & 15) + 16 * q]));
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((tid & 15) == 0) s_e[tid >> 4] = m;
+  }
+  __syncthreads();
+  for (int u = tid; u < 5 * SV * 8; u += blockDim.x) {
+    const int slot = u / (SV * 8), l = (u >> 3) & (SV - 1), g = u & 7, v = v0 + l;
+    if (v >= nv + nv2) continue;
+    int op = -1, r = v, part = -1, src = l;  // operand, its row, row of a complex pair, row of t
+    if (PANEL && v >= nv) {
+      if (slot == 2) op = 3;
+      r = v - nv;
+    } else if (slot == 2) {
+      op = 1;
+      if (PANEL) src = SV + l;
+    } else if (PANEL && (C || !(slot & 1 || slot == 4))) {
+      op = slot < 2 ? 0 : 2;
+      part = C ? (slot < 2 ? slot : slot - 3) : -1;
+      r = C ? 2 * v + part : v;
+      if (slot >= 2) src = SV + l;
+    }
+    if (!C && slot == 3 && PANEL && v < nv) {
+      op = 2;
+      r = v;
+      src = SV + l;
+    }
+    if (op < 0 || op >= npk) continue;
+    const SgOperand &o = pk.op[op];
+    const double *row = t[src];
+    const int em = s_e[src];
+    if (g == 0) o.e[r] = em;
+    sg_store_group(o, r, g, em, [&](int j) {
+      const int k = 8 * g + j;
+      if (part < 0) return row[k];
+      const double z = row[(k & ~1) | ((k ^ part) & 1)];
+      return part == 0 && (k & 1) ? -z : z;
+    });
+  }
+}
+
 // ------------------------------------------------------------- unit-triangular multi-vector solves
 // Vectors v < nv, element i < nb at X[v vs + i es]; the nb x nb block L (element (i, j) at
 // L[i + j ldl]) in shared memory:
@@ -195,8 +268,13 @@ struct Vecs {
 template <typename T, int NB, int SV, bool TRANS, bool PANEL>
 __global__ void __launch_bounds__(NB * SV) k_trsv(int nb, const T *__restrict__ L, long long ldl, int nv, Vecs<T> X,
                                                   int nv2, Vecs<T> X2, T *__restrict__ W, long long ldw,
-                                                  const T *__restrict__ dinv) {
+                                                  const T *__restrict__ dinv, const __grid_constant__ SgPack pk, int npk,
+                                                  int nsolve) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if ((int)blockIdx.x >= nsolve) {
+    pack_left(pk.op[0], (int)blockIdx.x - nsolve, reinterpret_cast<double(*)[kPK + 1]>(smem_raw));
+    return;
+  }
   T *Ls = reinterpret_cast<T *>(smem_raw);  // Ls[i + j NB] = L(i, j), or L(j, i) for TRANS
   T *xs = Ls + NB * NB;                     // [element][vector]
   const int tid = threadIdx.x, vl = tid % SV, i = tid / SV, v = blockIdx.x * SV + vl;
@@ -228,12 +306,18 @@ __global__ void __launch_bounds__(NB * SV) k_trsv(int nb, const T *__restrict__ 
       }
     }
   }
-  if (!act) return;
-  if (PANEL) {
-    W[v + (long long)i * ldw] = xi;
-    *x = Ar<T>::mul(xi, dinv[i]);
-  } else {
-    *x = xi;
+  T yi = xi;
+  if (act) {
+    if (PANEL) {
+      W[v + (long long)i * ldw] = xi;
+      yi = Ar<T>::mul(xi, dinv[i]);
+    }
+    *x = yi;
+  }
+  if (npk > 0) {
+    __syncthreads();  // L and the vectors in shared memory have been read
+    pack_vectors<T, SV, PANEL>(pk, npk, blockIdx.x * SV, nv, nv2, i, vl, xi, yi,
+                               reinterpret_cast<double(*)[kPK + 1]>(smem_raw));
   }
 }
 
@@ -273,12 +357,13 @@ SgProduct update(int mode, int M, int N, int K, SgView A, SgView B, T *C, long l
 
 template <typename T, int SV, bool TRANS, bool PANEL>
 int trsv(int nb, const T *L, long long ldl, int nv, Vecs<T> X, int nv2, Vecs<T> X2, T *W, long long ldw, const T *dinv,
-         cudaStream_t st) {
+         const SgPack &pk, int npk, cudaStream_t st) {
   constexpr int NB = LdlBlock<T>::NB;
   const size_t smem = (size_t)(NB * NB + NB * SV) * sizeof(T);
   if (set_smem(k_trsv<T, NB, SV, TRANS, PANEL>, smem) != GINT_OK) return GINT_ECUDA;
-  return sg_launch(k_trsv<T, NB, SV, TRANS, PANEL>, dim3((unsigned)((nv + nv2 + SV - 1) / SV)), NB * SV, smem, st, nb, L, ldl,
-                   nv, X, nv2, X2, W, ldw, dinv);
+  const int nsolve = (nv + nv2 + SV - 1) / SV, nleft = !PANEL && npk > 0 ? pk.first[1] : 0;
+  return sg_launch(k_trsv<T, NB, SV, TRANS, PANEL>, dim3((unsigned)(nsolve + nleft)), NB * SV, smem, st, nb, L, ldl, nv, X, nv2,
+                   X2, W, ldw, dinv, pk, npk, nsolve);
 }
 
 }  // namespace
@@ -294,27 +379,33 @@ int ldl_factor_solve(int n, T *A, long long lda, int nrhs, T *B, long long ldb, 
     const int nb = std::min(NB, n - j0), m = n - j0 - nb;
     T *A11 = A + j0 + (long long)j0 * lda, *A21 = A11 + nb, *B1 = B + j0;
     if ((rc = sg_launch(k_ldl_diag<T>, dim3(1), kDT, 0, st, nb, A11, lda, j0, spd ? 1 : 0, info, dinv + j0))) return rc;
-    // panel rows: W = A21 L11^-T, L21 = W D1^-1, and the same for the right-hand sides
-    if (m + nrhs > 0 && (rc = trsv<T, 8, false, true>(nb, A11, lda, m, Vecs<T>{A21, 1, lda}, nrhs, Vecs<T>{B1, ldb, 1}, W,
-                                                      ldw, dinv + j0, st)))
-      return rc;
-    if (m == 0) continue;
     // A22 -= W21 L21^T (lower triangle), B2 -= L21 W_B^T
     const SgProduct pr[2] = {
         update<T>(1, m, m, nb, left(W, 1, ldw), right(A21, 1, lda), A21 + (long long)nb * lda, lda),
         update<T>(0, m, nrhs, nb, left(A21, 1, lda), right(W + m, 1, ldw), B1 + nb, ldb)};
-    if ((rc = sg_gemm(pr, nrhs > 0 ? 2 : 1, ws, st))) return rc;
+    const int np = nrhs > 0 ? 2 : 1;
+    SgPack pk{};
+    if (m > 0 && (rc = sg_operands(pr, np, ws, &pk))) return rc;
+    // panel rows: W = A21 L11^-T, L21 = W D1^-1, and the same for the right-hand sides
+    if (m + nrhs > 0 && (rc = trsv<T, 8, false, true>(nb, A11, lda, m, Vecs<T>{A21, 1, lda}, nrhs, Vecs<T>{B1, ldb, 1}, W,
+                                                      ldw, dinv + j0, pk, m > 0 ? 2 * np : 0, st)))
+      return rc;
+    if (m == 0) continue;
+    if ((rc = sg_gemm(pr, np, ws, st, true))) return rc;
   }
   // L^T X = Y, last block first, then the rows above
   for (int k0 = ((n - 1) / NB) * NB; k0 >= 0 && nrhs > 0; k0 -= NB) {
     const int nb = std::min(NB, n - k0);
     const T *Lkk = A + k0 + (long long)k0 * lda;
-    if ((rc = trsv<T, 8, true, false>(nb, Lkk, lda, nrhs, Vecs<T>{B + k0, ldb, 1}, 0, Vecs<T>{}, nullptr, 0, nullptr, st)))
-      return rc;
-    if (k0 == 0) continue;
     // rows i < k0: B_i -= sum_k L[k0 + k, i] X[k0 + k]
     const SgProduct pr = update<T>(0, k0, nrhs, nb, left(A + k0, lda, 1), right(B + k0, ldb, 1), B, ldb);
-    if ((rc = sg_gemm(&pr, 1, ws, st))) return rc;
+    SgPack pk{};
+    if (k0 > 0 && (rc = sg_operands(&pr, 1, ws, &pk))) return rc;
+    if ((rc = trsv<T, 8, true, false>(nb, Lkk, lda, nrhs, Vecs<T>{B + k0, ldb, 1}, 0, Vecs<T>{}, nullptr, 0, nullptr, pk,
+                                      k0 > 0 ? 2 : 0, st)))
+      return rc;
+    if (k0 == 0) continue;
+    if ((rc = sg_gemm(&pr, 1, ws, st, true))) return rc;
   }
   return GINT_OK;
 }

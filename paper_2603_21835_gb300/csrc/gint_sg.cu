@@ -35,7 +35,7 @@
 #include "gint.h"
 #include "gint_ptx.cuh"
 #include "gint_sg.cuh"
-#include "gint_sgdev.cuh"
+#include "gint_sgpack.cuh"
 
 namespace gla {
 namespace {
@@ -48,48 +48,7 @@ constexpr int kDrainWarps = 16, kMmaWarp = 16, kLoadWarp = 17, kSgThreads = 32 *
 constexpr long long kWaitNs = 2000000000LL;  // bounded waits: 2 s
 constexpr unsigned kErrTimeout = 1u, kErrInflight = 2u;
 
-__device__ __forceinline__ double sg_at(const SgView &v, int r, int k) {
-  if (v.rot) {
-    const double x = v.p[(long long)(r >> 1) * v.rh + (long long)(k >> 1) * v.kh + ((r ^ k) & 1)];
-    return (!(r & 1) && (k & 1)) ? -x : x;
-  }
-  const double x = v.p[(long long)(r >> 1) * v.rh + (long long)(r & 1) * v.rl + (long long)(k >> 1) * v.kh +
-                       (long long)(k & 1) * v.kl];
-  return v.ks ? x * v.ks[k >> 1] : x;
-}
-
 // ---------------------------------------------------------------------------------------- packing
-constexpr int kPR = 32, kPK = 64, kPT = 256;  // rows and k of a packing CTA, its threads
-struct SgOperand {
-  SgView v;
-  int R, K, nq, tr;  // rows, contraction, chunks, rows of a tile (128 or 64)
-  int rfast;         // consecutive rows are closer in memory than consecutive k
-  unsigned char *dst;
-  int *e;            // exponent field of each row's largest magnitude
-};
-struct SgPack {
-  SgOperand op[4];
-  int first[5];  // first row block of each operand; first[n..4] = total
-};
-
-__device__ __forceinline__ void sg_load_tile(const SgOperand &o, int r0, int k0, double (*t)[kPK + 1]) {
-#pragma unroll
-  for (int q = 0; q < kPR * kPK / kPT; ++q) {
-    const int e = threadIdx.x + kPT * q;
-    const int r = o.rfast ? e % kPR : e / kPK, k = o.rfast ? e / kPR : e % kPK;
-    t[r][k] = (r0 + r < o.R && k0 + k < o.K) ? sg_at(o.v, r0 + r, k0 + k) : 0.0;
-  }
-}
-// The eight threads of a row: largest exponent field of its kPK elements (in all of them).
-__device__ __forceinline__ int sg_row_exp(const double (*t)[kPK + 1]) {
-  const int r = threadIdx.x >> 3, g = threadIdx.x & 7;
-  int m = 1;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) m = max(m, exp_field(t[r][g + 8 * j]));
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  return m;
-}
 __device__ __forceinline__ const SgOperand &sg_operand(const SgPack &P, int &rb) {
   int i = 0;
   while (i < 3 && (int)blockIdx.x >= P.first[i + 1]) ++i;
@@ -104,9 +63,9 @@ __global__ void __launch_bounds__(kPT) k_sg_max(const __grid_constant__ SgPack P
   const SgOperand &o = sg_operand(P, rb);
   const int r0 = rb * kPR;
   grid_wait();
-  sg_load_tile(o, r0, blockIdx.y * kPK, t);
+  sg_load_tile(o, threadIdx.x, r0, blockIdx.y * kPK, t);
   __syncthreads();
-  const int m = sg_row_exp(t), r = r0 + (threadIdx.x >> 3);
+  const int m = sg_row_exp(t, threadIdx.x), r = r0 + (threadIdx.x >> 3);
   if ((threadIdx.x & 7) == 0 && r < o.R) atomicMax(o.e + r, m);
 }
 
@@ -119,17 +78,13 @@ __global__ void __launch_bounds__(kPT) k_sg_pack(const __grid_constant__ SgPack 
   const SgOperand &o = sg_operand(P, rb);
   const int r0 = rb * kPR, kb = ONE ? 0 : (int)blockIdx.y * kPK;
   grid_wait();
-  sg_load_tile(o, r0, kb, t);
+  sg_load_tile(o, threadIdx.x, r0, kb, t);
   __syncthreads();
-  const int rl = threadIdx.x >> 3, g = threadIdx.x & 7, r = r0 + rl;
-  const int em = ONE ? sg_row_exp(t) : (r < o.R ? o.e[r] : 1);
-  const int chunk = (kb >> 4) + (g >> 1);
-  if (r >= o.R || chunk >= o.nq) return;
-  if (ONE && g == 0) o.e[r] = em;
-  const size_t blk = (size_t)kDig * o.tr * kCK * 2;
-  unsigned char *d = o.dst + ((size_t)(r / o.tr) * o.nq + chunk) * blk + (size_t)((r % o.tr) >> 3) * 256 + (g & 1) * 128 +
-                     (r & 7) * 16;
-  store_digits([&](int j) { return t[rl][8 * g + j]; }, em, d, (size_t)o.tr * kCK * 2);
+  const int rl = threadIdx.x >> 3, r = r0 + rl;
+  const int em = ONE ? sg_row_exp(t, threadIdx.x) : (r < o.R ? o.e[r] : 1);
+  if (r >= o.R) return;
+  if (ONE && (threadIdx.x & 7) == 0) o.e[r] = em;
+  sg_store_group(o, r, kb / 8 + (threadIdx.x & 7), em, [&](int j) { return t[rl][8 * (threadIdx.x & 7) + j]; });
 }
 
 // --------------------------------------------------------------------------------------- products
@@ -369,77 +324,94 @@ size_t sg_bytes(long long rows, long long K) {
   return R * k * kDig * 2 + R * sizeof(int) + 16 * kAlign;
 }
 
-int sg_gemm(const SgProduct *pr, int np, const SgWork &ws, cudaStream_t st) {
-  if (np < 1 || np > 2) return GINT_EINVAL;
+// Layout and arguments of the launch for the contraction range [k0, k0 + kk).
+static int sg_plan(const SgProduct *pr, int np, const SgWork &ws, int k0, int kk, SgPack &pk, SgArgs &ar, int **pe0, long long &erows) {
+  const int K = pr[0].K, nq = std::max(1, (kk + kCK - 1) / kCK);
+  ar.status = ws.status;
+  size_t off = 0;
+  unsigned char *base = ws.buf;
+  int nop = 0, blocks = 0;
+  for (int q = 0; q < np; ++q) erows += pad(pr[q].M, kTM) + pad(pr[q].N, kTM);
+  if (pad((size_t)erows * sizeof(int), kAlign) > ws.bytes) return GINT_EINVAL;
+  int *const e0 = *pe0 = reinterpret_cast<int *>(base);
+  off = pad((size_t)erows * sizeof(int), kAlign);
+  int *e = e0;
+  for (int q = 0; q < np; ++q) {
+    if (pr[q].K != K || pr[q].M < 0 || pr[q].N < 0) return GINT_EINVAL;
+    SgProb &pb = ar.pr[q];
+    pb.p = pr[q];
+    // the range [k0, k0 + kk) of the contraction (kSgK is even: part offsets stay aligned)
+    for (SgView *v : {&pb.p.A, &pb.p.B}) {
+      v->p += (long long)(k0 >> 1) * v->kh;
+      if (v->ks) v->ks += k0 >> 1;
+    }
+    pb.p.K = kk;
+    if (k0 > 0) pb.p.beta = 1;
+    pb.nq = nq;
+    pb.ntn = (pb.p.N + kTN - 1) / kTN;
+    const long long ntm = (pb.p.M + kTM - 1) / kTM;
+    long long tiles = 0;
+    if (pb.p.mode == 0) {
+      tiles = ntm * pb.ntn;
+    } else {
+      const int mul = pb.p.cs ? 1 : 2;
+      for (long long tm = 0; tm < ntm; ++tm) tiles += std::min<long long>(pb.ntn, mul * (tm + 1));
+    }
+    if (ar.tiles + tiles > 0x3fffffffLL) return GINT_EINVAL;
+    pb.ntiles = (int)tiles;
+    ar.tiles += (int)tiles;
+    for (int side = 0; side < 2; ++side) {
+      SgOperand &o = pk.op[nop];
+      o.v = side ? pb.p.B : pb.p.A;
+      o.R = side ? pb.p.N : pb.p.M;
+      o.K = kk;
+      o.nq = nq;
+      o.tr = side ? kTN : kTM;
+      const long long sr = o.v.rot ? o.v.rh / 2 : std::min(o.v.rl, o.v.rh), sk = o.v.rot ? o.v.kh / 2 : std::min(o.v.kl, o.v.kh);
+      o.rfast = sr <= sk;
+      o.dst = base + off;
+      o.e = e;
+      e += pad(o.R, kTM);
+      off += pad(o.R, o.tr) / o.tr * (size_t)nq * kDig * o.tr * kCK * 2;
+      (side ? pb.PB : pb.PA) = o.dst;
+      (side ? pb.eB : pb.eA) = o.e;
+      pk.first[nop++] = blocks;
+      blocks += (o.R + kPR - 1) / kPR;
+    }
+  }
+  if (off > ws.bytes) return GINT_EINVAL;
+  for (int q = nop; q < 5; ++q) pk.first[q] = blocks;
+  return GINT_OK;
+}
+
+int sg_operands(const SgProduct *pr, int np, const SgWork &ws, SgPack *pk) {
+  if (np < 1 || np > 2 || pr[0].K > kPK) return GINT_EINVAL;
+  SgArgs ar{};
+  int *e0;
+  long long erows = 0;
+  return sg_plan(pr, np, ws, 0, pr[0].K, *pk, ar, &e0, erows);
+}
+
+int sg_gemm(const SgProduct *pr, int np, const SgWork &ws, cudaStream_t st, bool packed) {
+  if (np < 1 || np > 2 || (packed && pr[0].K > kPK)) return GINT_EINVAL;
   const int K = pr[0].K;
   if (cudaFuncSetAttribute(k_sg_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSgSmem) != cudaSuccess)
     return GINT_ECUDA;
   for (int k0 = 0; k0 < std::max(K, 1); k0 += kSgK) {
-    const int kk = std::min(kSgK, K - k0), nq = std::max(1, (kk + kCK - 1) / kCK);
+    const int kk = std::min(kSgK, K - k0);
     SgPack pk{};
     SgArgs ar{};
-    ar.status = ws.status;
-    size_t off = 0;
-    unsigned char *base = ws.buf;
-    int nop = 0, blocks = 0, *e0 = nullptr;
+    int *e0 = nullptr;
     long long erows = 0;
-    for (int q = 0; q < np; ++q) erows += pad(pr[q].M, kTM) + pad(pr[q].N, kTM);
-    if (pad((size_t)erows * sizeof(int), kAlign) > ws.bytes) return GINT_EINVAL;
-    e0 = reinterpret_cast<int *>(base);
-    off = pad((size_t)erows * sizeof(int), kAlign);
-    int *e = e0;
-    for (int q = 0; q < np; ++q) {
-      if (pr[q].K != K || pr[q].M < 0 || pr[q].N < 0) return GINT_EINVAL;
-      SgProb &pb = ar.pr[q];
-      pb.p = pr[q];
-      // the range [k0, k0 + kk) of the contraction (kSgK is even: part offsets stay aligned)
-      for (SgView *v : {&pb.p.A, &pb.p.B}) {
-        v->p += (long long)(k0 >> 1) * v->kh;
-        if (v->ks) v->ks += k0 >> 1;
-      }
-      pb.p.K = kk;
-      if (k0 > 0) pb.p.beta = 1;
-      pb.nq = nq;
-      pb.ntn = (pb.p.N + kTN - 1) / kTN;
-      const long long ntm = (pb.p.M + kTM - 1) / kTM;
-      long long tiles = 0;
-      if (pb.p.mode == 0) {
-        tiles = ntm * pb.ntn;
-      } else {
-        const int mul = pb.p.cs ? 1 : 2;
-        for (long long tm = 0; tm < ntm; ++tm) tiles += std::min<long long>(pb.ntn, mul * (tm + 1));
-      }
-      if (ar.tiles + tiles > 0x3fffffffLL) return GINT_EINVAL;
-      pb.ntiles = (int)tiles;
-      ar.tiles += (int)tiles;
-      for (int side = 0; side < 2; ++side) {
-        SgOperand &o = pk.op[nop];
-        o.v = side ? pb.p.B : pb.p.A;
-        o.R = side ? pb.p.N : pb.p.M;
-        o.K = kk;
-        o.nq = nq;
-        o.tr = side ? kTN : kTM;
-        const long long sr = o.v.rot ? o.v.rh / 2 : std::min(o.v.rl, o.v.rh), sk = o.v.rot ? o.v.kh / 2 : std::min(o.v.kl, o.v.kh);
-        o.rfast = sr <= sk;
-        o.dst = base + off;
-        o.e = e;
-        e += pad(o.R, kTM);
-        off += pad(o.R, o.tr) / o.tr * (size_t)nq * kDig * o.tr * kCK * 2;
-        (side ? pb.PB : pb.PA) = o.dst;
-        (side ? pb.eB : pb.eA) = o.e;
-        pk.first[nop++] = blocks;
-        blocks += (o.R + kPR - 1) / kPR;
-      }
-    }
-    if (off > ws.bytes) return GINT_EINVAL;
-    for (int q = nop; q < 5; ++q) pk.first[q] = blocks;
+    int rc = sg_plan(pr, np, ws, k0, kk, pk, ar, &e0, erows);
+    if (rc) return rc;
     if (ar.tiles == 0) return GINT_OK;
-    int rc;
-    if (kk <= kPK) {
-      if ((rc = sg_launch(k_sg_pack<true>, dim3((unsigned)blocks), kPT, 0, st, pk))) return rc;
+    if (packed) {  // K <= 64: one range
+    } else if (kk <= kPK) {
+      if ((rc = sg_launch(k_sg_pack<true>, dim3((unsigned)pk.first[4]), kPT, 0, st, pk))) return rc;
     } else {
       if (cudaMemsetAsync(e0, 0, (size_t)erows * sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
-      const dim3 g((unsigned)blocks, (unsigned)((kk + kPK - 1) / kPK));
+      const dim3 g((unsigned)pk.first[4], (unsigned)((kk + kPK - 1) / kPK));
       k_sg_max<<<g, kPT, 0, st>>>(pk);  // after a copy engine's work: plain stream order
       if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA;
       if ((rc = sg_launch(k_sg_pack<false>, g, kPT, 0, st, pk))) return rc;

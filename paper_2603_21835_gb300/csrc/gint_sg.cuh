@@ -74,7 +74,23 @@ struct SgWork {
 // 128) and contraction at most K (longer contractions are cut into ranges of kSgK).
 size_t sg_bytes(long long rows, long long K);
 
+// Where a launch's operand digits go: left and right operand of each product in turn.
+struct SgOperand {
+  SgView v;
+  int R, K, nq, tr;    // rows, contraction, chunks of 16 k, rows of a tile (128 left, 64 right)
+  int rfast;           // consecutive rows are closer in memory than consecutive k
+  unsigned char *dst;  // digit blocks, see gint_sg.cu
+  int *e;              // exponent field of each row's largest magnitude
+};
+constexpr int kPackRows = 32;  // rows of a packing block
+struct SgPack {
+  SgOperand op[4];
+  int first[5];  // first row block of each operand; first[n..4] = total
+};
+
 // np (1 or 2) products of the same K in one launch (K <= 64: packed in one pass), asynchronous on st.
-int sg_gemm(const SgProduct *pr, int np, const SgWork &ws, cudaStream_t st);
+// packed (K <= 64): the operands' digits and exponents are already where sg_operands says.
+int sg_gemm(const SgProduct *pr, int np, const SgWork &ws, cudaStream_t st, bool packed = false);
+int sg_operands(const SgProduct *pr, int np, const SgWork &ws, SgPack *pk);
 
 }  // namespace gla
