@@ -633,7 +633,7 @@ def main():
     ms_per_step = max_over_ranks(sum(t_steps), world, dev) / args.steps
     value = world * 2.0 * W / (ms_per_step * 1e-3) / 1e9
 
-    # the float64 GPU path on the same workload and inputs (CUDA cores; the comparator of the
+    # the float64 GPU path on the same workload and inputs (the comparator of the
     # mixed-precision path), timed the same way: density + local-H passes, L2 flushed
     fp64_gpu = None
     if args.precision != "fp64" and args.fp64_steps > 0:
@@ -653,7 +653,7 @@ def main():
         ms64 = max_over_ranks(statistics.mean(t64), world, dev)
         v64 = world * 2.0 * W / (ms64 * 1e-3) / 1e9
         fp64_gpu = {"value": v64, "unit": UNIT, "ms_per_step": ms64, "steps": args.fp64_steps,
-                    "kernels": "k_simt_rho, k_simt_vlocal (float64 CUDA cores)",
+                    "kernels": "k_fx_eval, k_fx_mma (float64 orbitals, exact digit products)",
                     "mixed_over_fp64": value / v64}
 
     # roofline of the dominant kernel (per-launch mean over the timed region, CUDA events on its stream)

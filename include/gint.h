@@ -60,7 +60,7 @@ extern "C" {
  * GINT_F16X3 forces (gint_force, and force tasks of gint_run_batch) split orbitals and D in fixed point
  * instead: hi = the nearest integer at a common scale (so the tensor core's float32 accumulation of
  * hi * hi is exact), lo = the float16 remainder, and four products hi*hi + hi*lo + lo*hi + lo*lo. */
-#define GINT_FP64 0  /* float64 everywhere (CUDA cores) */
+#define GINT_FP64 0  /* float64 everywhere */
 #define GINT_FP32 1  /* float32 orbitals and CUDA-core contractions */
 #define GINT_F16X3 2 /* float32 orbitals; tensor-core contractions on operands split into two float16
                         parts (hi + lo, 22 significant bits, power-of-two scaled), products
@@ -230,8 +230,8 @@ int gint_psibeta(gint_handle *h, const double *A, double *out, void *stream);
 
 /* Dense steps of real-time propagation around the grid passes (paper Sec. 2): the density matrix
  * from coefficients and occupations, and one Crank-Nicolson step of the coefficients, in float64 on
- * the library's own kernels (a tiled GEMM, a blocked L D L^T factorisation without pivoting and its
- * triangular solves).  A context holds all
+ * the library's own kernels (products as exact digit products on the tensor cores, a blocked L D L^T
+ * factorisation without pivoting and its triangular solves).  A context holds all
  * buffers for an n x n problem with nocc states (allocated by gint_cn_create on the current device),
  * so the compute calls allocate nothing.  Matrices are float64 n x n, symmetric (any order); psi is
  * complex float64 n x nocc column-major (state j is psi[j n .. j n + n)), re / im interleaved; all

@@ -2,8 +2,8 @@
 //
 // Set-up mirrors the paper's GintInfo (Sec. 3.3.1, Fig. 2): geometry, the fine grid and its
 // coarse blocks ("bricks"), the brick -> atom neighbour relation (built on the device), and
-// the atom-pair block layout of the matrices.  Compute calls dispatch to the SIMT (FP64,
-// FP32) or tensor-core (F16x3, F16x1) kernels.
+// the atom-pair block layout of the matrices.  Compute calls dispatch to the float64 digit-product
+// (FP64), SIMT (FP32, FP64 of very wide bricks) or tensor-core (F16x3, F16x1) kernels.
 #include <cuda_runtime.h>
 
 #include <algorithm>
