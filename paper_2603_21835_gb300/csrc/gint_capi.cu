@@ -314,8 +314,8 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
   TRY(dalloc(&h->dtab32i, d32i.size()));
   TRYCU(cudaMemcpy(h->dtab32, d32.data(), d32.size() * sizeof(float), cudaMemcpyHostToDevice));
   TRYCU(cudaMemcpy(h->dtab32i, d32i.data(), d32i.size() * sizeof(float), cudaMemcpyHostToDevice));
-  // tables of the float64 evaluators: per knot and radial (f, f_{k+1} - f_k, dr f'_k, dr f'_{k+1}), times the Y_lm
-  // constant of the shell
+  // tables of the float64 evaluators: per knot and radial the cubic Hermite interpolant's coefficients in t, times
+  // the Y_lm constant of the shell
   {
     h->tabs64 = g;
     std::vector<double> o;
@@ -338,7 +338,8 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
           const GRadial &R = g.rad[S.rad0 + k];
           const double2 *T = t64.data() + R.off + i;
           const double c = cl[R.l];
-          for (double x : {T[0].x, T[1].x - T[0].x, R.dr * T[0].y, R.dr * T[1].y}) o.push_back(c * x);
+          const double df = T[1].x - T[0].x, m0 = R.dr * T[0].y, m1 = R.dr * T[1].y;
+          for (double x : {T[0].x, m0, 3.0 * df - (2.0 * m0 + m1), (m0 + m1) - 2.0 * df}) o.push_back(c * x);
         }
     }
     h->notab64 = (long long)o.size();

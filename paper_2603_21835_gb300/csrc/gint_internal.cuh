@@ -226,9 +226,10 @@ __device__ __forceinline__ void add_orbitals(const GTabs &g, const typename Tab2
 // ------------------------------------------------------------------------------------------
 // Float64 evaluators of l-sorted species on one knot grid (NS s, NP p, ND d radials), for the kernels whose time is
 // the number of float64 instructions (a warp-wide one occupies the SM's pipe for 16 clocks).  Tables (otab64 of the
-// handle): per knot and radial (f, f_{k+1} - f_k, dr f'_k, dr f'_{k+1}), times the constant of Y_00, of Y_1m or of
+// handle): per knot and radial the interpolant a + t (b + t (c + t d)), times the constant of Y_00, of Y_1m or of
 // Y_2,+-1 (the other d functions carry their ratio to it); GSpecies::ioff: first table entry, kslot: the radials end
-// at different radii.
+// at different radii.  (Three instructions a radial, two more with its derivative, and no basis: with knot values and
+// slopes the basis functions of t took 7 and 13 more an image.)
 #define GINT_O64_SHAPES(X) X(2, 2, 1, 13) X(2, 1, 0, 5) X(1, 1, 1, 9) X(1, 1, 0, 4) X(1, 0, 0, 1) X(3, 3, 2, 22)
 
 // 1 / r, r and the knot position of a point with r2 = |d|^2 (below 1e-36 it counts as 1e-36).
@@ -264,13 +265,13 @@ __device__ __forceinline__ void orbitals64(const GTabs &g, const double *__restr
                                            double dy, double dz, double r2, double *phi) {
   constexpr int NR = NS + NP + ND;
   const Knot64 K = knot64(g.rad[S.rad0], r2);
-  const double t = K.t, t2 = t * t, u = 1.0 - t, s = t2 * fma(-2.0, t, 3.0), c0 = t * u * u, c1 = -t2 * u;
+  const double t = K.t;
   const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)K.i * NR) * 2;
   double f[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) {
     const double2 a = __ldg(q + 2 * k), b = __ldg(q + 2 * k + 1);
-    f[k] = fma(b.y, c1, fma(b.x, c0, fma(a.y, s, a.x)));
+    f[k] = fma(fma(fma(b.y, t, b.x), t, a.y), t, a.x);
     if (S.kslot && !(K.r < g.rad[S.rad0 + k].rc)) f[k] = 0.0;
   }
   const double ux = dx * K.y, uy = dy * K.y, uz = dz * K.y;
@@ -310,15 +311,15 @@ __device__ __forceinline__ void contract64(const GTabs &g, const double *__restr
   const GRadial &R0 = g.rad[S.rad0];
   const bool at0 = r2 < 1e-24;
   const Knot64 K = knot64(R0, r2);
-  const double t = K.t, t2 = t * t, u = 1.0 - t, s = t2 * fma(-2.0, t, 3.0), c0 = t * u * u, c1 = -t2 * u;
-  const double ds = 6.0 * t * u, d0 = u * fma(-3.0, t, 1.0), d1 = t * fma(3.0, t, -2.0), idr = R0.inv_dr;
+  const double t = K.t, idr = R0.inv_dr;
   const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)K.i * NR) * 2;
   const double ux = at0 ? 0.0 : dx * K.y, uy = at0 ? 0.0 : dy * K.y, uz = at0 ? 0.0 : dz * K.y;
   double rad = 0.0;  // coefficient of u
   auto radial = [&](int k, double &R, double &dR) {
     const double2 a = __ldg(q + 2 * k), b = __ldg(q + 2 * k + 1);
-    R = fma(b.y, c1, fma(b.x, c0, fma(a.y, s, a.x)));
-    dR = fma(b.y, d1, fma(b.x, d0, a.y * ds)) * idr;
+    const double h = fma(b.y, t, b.x), g1 = fma(h, t, a.y);
+    R = fma(g1, t, a.x);
+    dR = fma(fma(b.y, t, h), t, g1) * idr;
     if (S.kslot && !(K.r < g.rad[S.rad0 + k].rc)) R = dR = 0.0;
   };
 #pragma unroll
