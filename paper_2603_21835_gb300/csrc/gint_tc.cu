@@ -2851,12 +2851,16 @@ static int tc_layouts(gint_handle *h, cudaStream_t st) {
   h->max_brick_porb = (int)tot[3];
   int rc;
   // the scratch tiles' buffer also serves the float64 passes: enlarged (small systems) to hold a brick per SM for
-  // them if memory allows
+  // them, to no more than twice the tiles and 96 MB (a server keeps many small handles), if memory allows.  A batch
+  // of fewer than 64 bricks would leave the chip to launch tails; the CUDA-core kernels are then as fast.
   h->fx_batch = 0;
-  if (gint_fx_bytes(h, 1) > 0) {
-    const int want = (int)std::min<long long>(h->num_sms, nb);
-    const long long fx = (gint_fx_bytes(h, want) + 3) / 4;
-    if (tc_reserve(h, h->hs, h->cap_hs, std::max(tot[0], fx)) == GINT_OK) h->fx_batch = want;
+  const long long fx0 = gint_fx_bytes(h, 0), fx1 = gint_fx_bytes(h, 1) - fx0;
+  if (fx1 > 0) {
+    const long long room = (2 * tot[0] * 4 + (96LL << 20) - fx0) / fx1;
+    const int want = (int)std::min<long long>({(long long)h->num_sms, nb, std::max(room, 0LL)});
+    if (want >= std::min<long long>(nb, 64) && want > 0 &&
+        tc_reserve(h, h->hs, h->cap_hs, std::max(tot[0], (gint_fx_bytes(h, want) + 3) / 4)) == GINT_OK)
+      h->fx_batch = want;
   }
   if ((rc = tc_reserve(h, h->hs, h->cap_hs, tot[0])) || (rc = tc_reserve(h, h->plan, h->cap_plan, tot[1])) ||
       (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2])))
