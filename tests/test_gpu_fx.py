@@ -92,3 +92,53 @@ def test_non_finite_inputs_reach_the_same_results(bad):
     assert float((rb - rho0.reshape(-1))[ok].abs().max()) <= 1e-12 * float(rho0.abs().max())
     g.sync()
     g.close()
+
+
+def test_captured_passes_replay():
+    """The float64 passes and the dense steps around them in one CUDA graph, replayed on new inputs: the direct calls'
+    results (force and H sums in another order of atomics: 1e-13)."""
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    s = _system(("221", "110"), 6, 12.0, (16, 12, 16))
+    rng = np.random.default_rng(5)
+    g = G.Gint(s)
+    n = g.norb
+    C = rng.normal(size=(n, 5)) / 4
+    D0, V0 = torch.from_numpy(g.dense_to_blocks(C @ C.T)).cuda(), torch.from_numpy(rng.normal(size=g.ngrid)).cuda()
+    cn = G.CrankNicolson(n, 5)
+    S = torch.eye(n, dtype=torch.float64, device="cuda")
+    A = torch.from_numpy(rng.normal(size=(n, n))).cuda()
+    A = 0.5 * (A + A.T)
+    psi0 = torch.from_numpy(np.ascontiguousarray((rng.normal(size=(n, 5)) + 1j * rng.normal(size=(n, 5))).T)).cuda()
+    f = torch.ones(5, dtype=torch.float64, device="cuda")
+    D, V, psi = D0.clone(), V0.clone(), psi0.clone()
+    out = [torch.empty(g.grid, dtype=torch.float64, device="cuda"), torch.empty_like(D), torch.empty((6, 3), dtype=torch.float64, device="cuda"),
+           torch.empty_like(psi), torch.empty((n, n), dtype=torch.float64, device="cuda")]
+
+    def calls():
+        g.rho(D, G.FP64, out=out[0])
+        g.vlocal(V, G.FP64, out=out[1])
+        g.force(D, V, G.FP64, out=out[2])
+        cn.step(S, A, 0.05, psi, out=out[3])
+        cn.density_matrix(out[3], f, out=out[4])
+
+    calls()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls()
+    for scale in (1.0, -0.5):
+        D.copy_(scale * D0)
+        V.copy_(scale * V0)
+        psi.copy_(scale * psi0)
+        graph.replay()
+        torch.cuda.synchronize()
+        got = [x.clone() for x in out]
+        calls()
+        torch.cuda.synchronize()
+        for a, b in zip(got, out):
+            assert float((a - b).abs().max()) <= 1e-13 * float(b.abs().max())
+    cn.close()
+    g.close()
