@@ -747,11 +747,13 @@ __device__ __forceinline__ void load_Y(uint32_t ty, uint32_t tcorr, float inv, f
 // orbitals of an only image, behind the sums over several (their accumulators leave it no registers).  The epilogue is
 // bound by instruction issue and by the table loads' latency; it took 33 of an item's 62 thousand cycles (64-atom Si)
 // with Y in local memory, 4 PO accumulators and one radial's loads at a time: 1496 us of forces -> 1041 us.
-template <int NS, int NPR, int ND, int PO>
+// ONE: the way of an only image is compiled (the instances of all shapes go without it: six of them spill 2 KB a
+// thread and a served job took 10 % longer, 1s 1p 1d forces 1.31 ms -> 1.11 ms this way).
+template <int NS, int NPR, int ND, int PO, bool ONE>
 __device__ __forceinline__ void job_F(const GTabs &g, const float2 *__restrict__ tab, const float *__restrict__ dtab,
                                       const BrickSh &sh, int a, int p, bool valid, uint32_t ty, uint32_t tcorr, float inv,
                                       float &rp, float &fx, float &fy, float &fz) {
-  if (sh.s_e0[a + 1] - sh.s_e0[a] == 1) {
+  if (ONE && sh.s_e0[a + 1] - sh.s_e0[a] == 1) {
     float y[PO];
 #pragma unroll
     for (int h = 0; h + 16 <= PO; h += 16) load_Y<16>(ty + h, tcorr, inv, y + h);
@@ -1237,7 +1239,7 @@ case GINT_SHAPE(ns, np_, nd):                                                   
 #define CASE_F(ns, np_, nd)                                                                          \
 case GINT_SHAPE(ns, np_, nd):                                                                    \
   if constexpr (!DZP || is_dzp(GINT_SHAPE(ns, np_, nd)))                                         \
-  job_F<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8>(g, tabi, S.dtabi, sh, a, p, valid, ty, tcorr, inv, rp, fx, fy, fz); \
+  job_F<ns, np_, nd, (ns + 3 * np_ + 5 * nd + 7) / 8 * 8, DZP>(g, tabi, S.dtabi, sh, a, p, valid, ty, tcorr, inv, rp, fx, fy, fz); \
   break;
           GINT_FOR_SHAPES(CASE_F)
 #undef CASE_F
@@ -2284,7 +2286,7 @@ __device__ __forceinline__ bool wait_count(const int *cnt, long long target, uns
   return true;
 }
 
-template <bool FORCE>
+template <bool FORCE, bool DZP>
 __global__ void __launch_bounds__(kT, 1)
     k_serve(const __grid_constant__ GTabs g, GServeCtl *ctl, const GJob *__restrict__ jobs, GJobState *st,
             const long long *__restrict__ job_end, volatile unsigned long long *done, const __half *__restrict__ zero,
@@ -2513,7 +2515,7 @@ __global__ void __launch_bounds__(kT, 1)
           }
         }
         if (t < 128) sh.wv[t] = wvv;  // read by brick_body after its barriers
-        brick_body<FORCE, false>(g, S, b, do_rho, do_h, split3, dsmem, zero, tmem, sh, smem, cx);
+        brick_body<FORCE, DZP>(g, S, b, do_rho, do_h, split3, dsmem, zero, tmem, sh, smem, cx);
         tc_fence_before();
       }
     } else {  // H reduction: two upper pairs, one per 256 threads (named barriers 2, 3), in four parts
@@ -2975,6 +2977,13 @@ static void fill_red_gamma(GRedSys &rs, const gint_task &T) {
   rs.fp64 = h->reduce_fp64 ? 1 : 0;
 }
 
+// Every species has one of the shapes of the kernels' DZP instances.
+static bool all_dzp(const GTabs &tabs) {
+  bool dzp = true;
+  for (int s = 0; s < tabs.nspecies; ++s) dzp = dzp && is_dzp(tabs.sp[s].shape);
+  return dzp;
+}
+
 static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1) {
   gint_handle *h0 = tk[0].h;
   const GTabs &tabs = h0->geom;
@@ -3062,8 +3071,7 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
   }
   if (items > 0) {
     const unsigned grid = (unsigned)std::min<long long>(h0->num_sms, items);
-    bool dzp = true;
-    for (int s = 0; s < tabs.nspecies; ++s) dzp = dzp && is_dzp(tabs.sp[s].shape);
+    const bool dzp = all_dzp(tabs);
     auto kern = force ? (dzp ? k_tc_fused<true, true> : k_tc_fused<true, false>)
                       : (dzp ? k_tc_fused<false, true> : k_tc_fused<false, false>);
     int rc = set_smem(kern, smem);
@@ -3177,7 +3185,7 @@ static int server_launch(gint_server *v) {
   if (cudaMemcpyAsync(&v->ctl->first_seq, v->stage_misc, sizeof(unsigned long long), cudaMemcpyHostToDevice,
                       v->kstream) != cudaSuccess)
     return GINT_ECUDA;
-  auto kern = v->forces ? k_serve<true> : k_serve<false>;
+  auto kern = v->forces ? (all_dzp(v->tabs) ? k_serve<true, true> : k_serve<true, false>) : k_serve<false, false>;
   kern<<<v->num_sms, kT, v->dsmem, v->kstream>>>(v->tabs, v->ctl, v->jobs, v->st, v->job_end, v->done_d, v->zero,
                                                   v->split3, v->dsmem, v->idle_ns);
   if (cudaGetLastError() != cudaSuccess || cudaEventRecord(v->kdone, v->kstream) != cudaSuccess) return GINT_ECUDA;
@@ -3200,7 +3208,7 @@ extern "C" int gint_server_create(int precision, int forces, double idle_s, gint
     server_free(v);
     return GINT_ECUDA;
   }
-  v->dsmem = (int)std::min(dyn_smem_limit(k_serve<false>), dyn_smem_limit(k_serve<true>));
+  v->dsmem = (int)std::min(dyn_smem_limit(k_serve<false, false>), std::min(dyn_smem_limit(k_serve<true, false>), dyn_smem_limit(k_serve<true, true>)));
   bool okm = cudaMalloc(&v->ctl, sizeof(GServeCtl)) == cudaSuccess &&
              cudaMalloc(&v->jobs, kServeRing * sizeof(GJob)) == cudaSuccess &&
              cudaMalloc(&v->st, kServeRing * sizeof(GJobState)) == cudaSuccess &&
@@ -3225,7 +3233,8 @@ extern "C" int gint_server_create(int precision, int forces, double idle_s, gint
       cudaStreamCreateWithFlags(&v->cstream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&v->kdone, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&v->ev_in, cudaEventDisableTiming) != cudaSuccess ||
-      set_smem(k_serve<true>, (uint32_t)v->dsmem) != GINT_OK || set_smem(k_serve<false>, (uint32_t)v->dsmem) != GINT_OK) {
+      set_smem(k_serve<true, false>, (uint32_t)v->dsmem) != GINT_OK || set_smem(k_serve<true, true>, (uint32_t)v->dsmem) != GINT_OK ||
+      set_smem(k_serve<false, false>, (uint32_t)v->dsmem) != GINT_OK) {
     cudaGetLastError();
     server_free(v);
     return GINT_ECUDA;
