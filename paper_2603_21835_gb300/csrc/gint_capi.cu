@@ -462,10 +462,12 @@ int make_twin(gint_handle *h) {
 // brick of h sees two images of one atom (its tiles mix several R), h's unfolded twin.
 int hr_handle(gint_handle *h, gint_handle **t) {
   *t = h;
+  if (h->geom_status) return h->geom_status;
   if (h->folded && !h->unfold) {
     const int rc = make_twin(h);
     if (rc) return rc;
     *t = h->twin;
+    if (h->twin->geom_status) return h->twin->geom_status;
   }
   return gint_hr_prepare(*t);
 }
@@ -520,6 +522,7 @@ int gint_stats(const gint_handle *h, double *W, double *W_exec, long long *nbric
 int gint_brick_lists(const gint_handle *h, long long *nslots, long long *nentries, long long *b_off, int *slot_atom,
                      long long *slot_ent, double *ent_pos) {
   if (!h) return GINT_EINVAL;
+  if (h->geom_status) return h->geom_status;
   long long ns = h->nslots, ne = 0;
   if (cudaMemcpy(&ne, h->s_ent + ns, sizeof(long long), cudaMemcpyDeviceToHost) != cudaSuccess) return GINT_ECUDA;
   if (nslots) *nslots = ns;
@@ -550,10 +553,7 @@ int gint_memory(const gint_handle *h, long long *device_bytes) {
   return GINT_OK;
 }
 
-int gint_set_positions(gint_handle *h, const double *pos_dev, void *stream) {
-  if (!h || !pos_dev) return GINT_EINVAL;
-  DeviceGuard guard(h->device);
-  cudaStream_t st = (cudaStream_t)stream;
+static int rebuild_geometry(gint_handle *h, const double *pos_dev, cudaStream_t st) {
   if (cudaMemcpyAsync(h->pos_dev, pos_dev, 3 * sizeof(double) * h->geom.natoms, cudaMemcpyDeviceToDevice, st) !=
       cudaSuccess)
     return GINT_ECUDA;
@@ -566,7 +566,15 @@ int gint_set_positions(gint_handle *h, const double *pos_dev, void *stream) {
                       st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return GINT_ECUDA;
-  if (h->twin) return gint_set_positions(h->twin, pos_dev, stream);
+  return GINT_OK;
+}
+
+int gint_set_positions(gint_handle *h, const double *pos_dev, void *stream) {
+  if (!h || !pos_dev) return GINT_EINVAL;
+  DeviceGuard guard(h->device);
+  h->geom_status = rebuild_geometry(h, pos_dev, (cudaStream_t)stream);
+  if (h->geom_status) return h->geom_status;
+  if (h->twin) return gint_set_positions(h->twin, pos_dev, stream);  // (its status holds back the per-R calls only)
   return GINT_OK;
 }
 
@@ -591,6 +599,7 @@ static int cuda_vlocal(gint_handle *h, bool fp64, const double *V, double *H, cu
 int gint_rho(gint_handle *h, int precision, const double *D_blocks, double *rho, void *stream) {
   if (!h || !D_blocks || !rho) return GINT_EINVAL;
   if (check_precision(precision)) return GINT_EINVAL;
+  if (h->geom_status) return h->geom_status;
   DeviceGuard guard(h->device);
   cudaStream_t st = (cudaStream_t)stream;
   if (precision == GINT_FP64 || precision == GINT_FP32)
@@ -601,6 +610,7 @@ int gint_rho(gint_handle *h, int precision, const double *D_blocks, double *rho,
 int gint_vlocal(gint_handle *h, int precision, const double *V, double *H_blocks, void *stream) {
   if (!h || !V || !H_blocks) return GINT_EINVAL;
   if (check_precision(precision)) return GINT_EINVAL;
+  if (h->geom_status) return h->geom_status;
   DeviceGuard guard(h->device);
   cudaStream_t st = (cudaStream_t)stream;
   if (precision == GINT_FP64 || precision == GINT_FP32) {
@@ -655,6 +665,7 @@ int gint_bloch(gint_handle *h, const double *H_R, int nk, const double *kfrac, d
 
 int gint_set_projectors(gint_handle *h, int nspecies, const gint_species *proj) {
   if (!h) return GINT_EINVAL;
+  if (h->geom_status) return h->geom_status;
   DeviceGuard guard(h->device);
   return gint_pb_set(h, nspecies, proj);
 }
@@ -671,6 +682,7 @@ int gint_psibeta_layout(const gint_handle *h, int *npairs, long long *nelems, co
 
 int gint_psibeta(gint_handle *h, const double *A, double *out, void *stream) {
   if (!h || !A || !out) return GINT_EINVAL;
+  if (h->geom_status) return h->geom_status;
   DeviceGuard guard(h->device);
   return gint_pb_run(h, A, out, (cudaStream_t)stream);
 }
@@ -679,6 +691,7 @@ int gint_force(gint_handle *h, int precision, const double *D_blocks, const doub
                void *stream) {
   if (!h || !D_blocks || !V || !F) return GINT_EINVAL;
   if (check_precision(precision)) return GINT_EINVAL;
+  if (h->geom_status) return h->geom_status;
   DeviceGuard guard(h->device);
   cudaStream_t st = (cudaStream_t)stream;
   if (precision == GINT_FP64 || precision == GINT_FP32) {
@@ -702,6 +715,8 @@ int gint_run_batch_timed(const gint_task *tasks, int ntasks, int precision, void
     if ((T.rho || T.F) && !T.D_blocks) return GINT_EINVAL;
     if ((T.H_blocks || T.F) && !T.V) return GINT_EINVAL;
   }
+  for (int i = 0; i < ntasks; ++i)
+    if (tasks[i].h->geom_status) return tasks[i].h->geom_status;
   if (ntasks == 0) return GINT_OK;
   DeviceGuard guard(tasks[0].h->device);
   cudaStream_t st = (cudaStream_t)stream;

@@ -7,6 +7,7 @@
 
 #include <vector>
 
+#include "gint.h"
 #include "gint_internal.cuh"
 
 struct gint_handle {
@@ -43,6 +44,9 @@ struct gint_handle {
   long long *pair_off_dev = nullptr;
   int *pair_T_dev = nullptr;  // index of the transposed pair (J, I)
   int *pair_I_dev = nullptr;  // row atom I of each pair
+  // GINT_OK, or why the last gint_set_positions failed: lists, layouts and scratch sizes may then be of different
+  // positions (or absent), so every call that reads them returns this code
+  int geom_status = GINT_OK;
   // neighbour structure
   int *n_at = nullptr, *n_ent = nullptr, *n_orb = nullptr;
   float *frac_dev = nullptr;  // fractional coordinates of the atoms (float32 screen of the neighbour kernels)

@@ -3250,6 +3250,7 @@ extern "C" int gint_server_submit(gint_server *v, const gint_task *T, void *stre
   if ((!dens && !loc) || (dens && !T->D_blocks) || ((loc || T->F) && !T->V)) return GINT_EINVAL;
   if (T->F && !v->forces) return GINT_EINVAL;
   if (h->device != v->device) return GINT_EINVAL;
+  if (h->geom_status) return h->geom_status;
   int rc = gint_tc_check_capacity(h);
   if (rc) return rc;
   if (loc && h->max_brick_porb > kNPMAXH) return GINT_ECAPACITY;
@@ -3358,6 +3359,7 @@ extern "C" int gint_orbitals(gint_handle *h, int precision, long long npts, cons
                              double *grad) {
   if (!h || npts < 0 || (npts > 0 && (!pts || !phi))) return GINT_EINVAL;
   if (precision != GINT_FP64 && precision != GINT_F16X3) return GINT_EUNSUPPORTED;
+  if (h->geom_status) return h->geom_status;
   if (h->max_species_norb > GINT_MAX_ORB_ATOM) return GINT_ECAPACITY;
   if (npts == 0) return GINT_OK;
   const int norb = h->norb, na = h->geom.natoms;

@@ -329,6 +329,7 @@ class Gint:
         self.weight = float(_lib.gint_weight(h))
         self._pos_host = pos.copy()
         self._pos_dev = None
+        self._pos_valid = True  # the handle is at _pos_dev (or, while that is None, at its creation's positions)
 
     # -- bookkeeping
     def stats(self) -> dict:
@@ -507,16 +508,17 @@ class Gint:
     def set_positions(self, pos: torch.Tensor, stream=None):
         """New positions (device float64 [natoms, 3]); neighbour lists are rebuilt on the device."""
         pos = pos.detach().contiguous()
-        _check(_lib.gint_set_positions(self._h, _dptr(pos, numel=3 * self.natoms), _stream(stream)),
-               "gint_set_positions")
-        self._pos_dev = pos.clone()
+        ptr = _dptr(pos, numel=3 * self.natoms)
+        self._pos_valid = False  # refused positions leave the handle at none
         self.__dict__.pop("nblock_R", None)  # H(R) keys follow the new images
+        _check(_lib.gint_set_positions(self._h, ptr, _stream(stream)), "gint_set_positions")
+        self._pos_dev, self._pos_valid = pos.clone(), True
 
     def ensure_positions(self, pos: torch.Tensor, stream=None):
         """Rebuilds the neighbour lists only if pos differs from the current geometry."""
         if self._pos_dev is None:
             self._pos_dev = torch.from_numpy(self._pos_host).to(pos.device)
-        if not torch.equal(self._pos_dev, pos.detach()):
+        if not self._pos_valid or not torch.equal(self._pos_dev, pos.detach()):
             self.set_positions(pos, stream)
 
     # -- layout helpers (host, numpy): dense <-> atom-pair blocks

@@ -1,0 +1,94 @@
+"""A set_positions that fails leaves the handle at no positions: calls that read the geometry return its error, launch
+nothing, and work again once a set_positions succeeds."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2603_21835_gb300 import inputs
+
+from . import fake_cudart
+
+ESKIN, EDEVICE = -7, -5
+
+
+def _calls(G, g, dev="cpu"):
+    D, V = torch.zeros(g.nblock, dtype=torch.float64, device=dev), torch.zeros(g.ngrid, dtype=torch.float64, device=dev)
+    out = lambda n: torch.zeros(n, dtype=torch.float64, device=dev)
+    calls = {}
+    for p in (G.FP64, G.FP32, G.F16X3):
+        calls[f"rho{p}"] = lambda p=p: g.rho(D, p, out=out(g.ngrid))
+        calls[f"vlocal{p}"] = lambda p=p: g.vlocal(V, p, out=out(g.nblock))
+        calls[f"force{p}"] = lambda p=p: g.force(D, V, p, out=out(3 * g.natoms))
+        calls[f"run{p}"] = lambda p=p: g.run(D, V, p, rho=out(g.ngrid), H=out(g.nblock))
+    calls["layout_R"] = g.layout_R
+    calls["orbitals"] = lambda: g.orbitals(np.zeros((1, 3)))
+    calls["brick_lists"] = g.brick_lists
+    calls["set_projectors"] = lambda: g.set_projectors([inputs.si_species()])
+    return calls
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return fake_cudart.load(tmp_path_factory.mktemp("fake"))
+
+
+@pytest.mark.parametrize("cause, code", [("fake_refuse", ESKIN), ("fake_plan_error", EDEVICE)])
+def test_no_launch_after_a_refused_geometry(fake, cause, code):
+    G, lib = fake
+    lib.fake_refuse(0)
+    lib.fake_plan_error(0)
+    w = inputs.si_workload((1, 1, 1), (16, 16, 16), seed=0)
+    g = G.Gint(w.system)
+    pos = torch.from_numpy(w.system.pos.copy())
+    lib.fake_clear()
+    g.rho(torch.zeros(g.nblock, dtype=torch.float64), G.FP64, out=torch.zeros(g.ngrid, dtype=torch.float64))
+    assert b"k_fx_eval" in lib.fake_log()  # (so the refusals below are not for want of scratch)
+    getattr(lib, cause)(1)
+    with pytest.raises(G.GintError) as e:
+        g.set_positions(pos + 1.0)
+    assert e.value.code == code
+    for name, call in _calls(G, g).items():
+        lib.fake_clear()
+        with pytest.raises(G.GintError) as e:
+            call()
+        assert e.value.code == code and lib.fake_log() == b"", name
+    # going back to the old positions is a rebuild, not the skip of unchanged ones
+    getattr(lib, cause)(0)
+    lib.fake_clear()
+    g.ensure_positions(pos)
+    assert b"k_brick_count" in lib.fake_log()
+    lib.fake_clear()
+    g.rho(torch.zeros(g.nblock, dtype=torch.float64), G.FP64, out=torch.zeros(g.ngrid, dtype=torch.float64))
+    assert b"k_fx_eval" in lib.fake_log()
+    g.close()
+
+
+@pytest.mark.gpu
+def test_refused_and_recovered_on_the_gpu():
+    from paper_2603_21835_gb300 import gint as G
+
+    w = inputs.si_workload((1, 1, 1), (24, 24, 24), seed=0)
+    # a cell with vacuum, so that some pairs have no block
+    cell = 3.0 * np.asarray(w.system.cell)
+    s = inputs.System(cell=cell, pos=w.system.pos[:2], species=w.system.species[:2], sp=w.system.sp, grid=(24, 24, 24))
+    far = s.pos.copy()
+    far[1] = far[0] + cell.sum(0) / 2
+    s = inputs.System(cell=cell, pos=far, species=s.species, sp=s.sp, grid=s.grid)
+    g = G.Gint(s)
+    D = torch.randn(g.nblock, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    V = torch.randn(g.ngrid, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    Db = torch.from_numpy(g.dense_to_blocks((lambda M: M + M.T)(g.blocks_to_dense(D.cpu().numpy())))).cuda()
+    before = g.rho(Db, G.FP64).clone()
+    near = far.copy()
+    near[1] = near[0] + 2.0
+    with pytest.raises(G.GintError) as e:
+        g.set_positions(torch.from_numpy(near).cuda())
+    assert e.value.code == ESKIN
+    for name, call in _calls(G, g, "cuda").items():
+        with pytest.raises(G.GintError) as e:
+            call()
+        assert e.value.code == ESKIN, name
+    g.ensure_positions(torch.from_numpy(far).cuda())
+    assert torch.equal(g.rho(Db, G.FP64), before)
+    g.vlocal(V, G.F16X3)
+    g.sync()
