@@ -2729,6 +2729,7 @@ void dfree(T *&p) {
 
 void gint_tc_free(gint_handle *h) {
   h->tc_bytes = 0;
+  h->fx_batch = 0;  // (its scratch is hs)
   dfree(h->plan);
   dfree(h->plan_off_dev);
   dfree(h->Dt_hl);
@@ -2810,19 +2811,20 @@ static int tc_allocate(gint_handle *h) {
 }
 
 // A buffer of at least n elements of T: kept when it is large enough, otherwise replaced (exactly n the first
-// time, an eighth more after that, so that moving atoms do not reallocate at every step).
+// time, an eighth more after that if memory allows, so that moving atoms do not reallocate at every step).
 template <typename T>
 static int tc_reserve(gint_handle *h, T *&p, long long &cap, long long n) {
   n = std::max(n, 1LL);
   if (p && n <= cap) return GINT_OK;
-  const long long want = p ? n + n / 8 : n;
+  long long want = p ? n + n / 8 : n;
   dfree(p);
   h->tc_bytes -= cap * (long long)sizeof(T);
   cap = 0;
-  if (cudaMalloc(&p, want * sizeof(T)) != cudaSuccess) {
+  while (cudaMalloc(&p, want * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
     p = nullptr;
-    return GINT_ENOMEM;
+    if (want == n) return GINT_ENOMEM;
+    want = n;
   }
   cap = want;
   h->tc_bytes += cap * (long long)sizeof(T);
@@ -2852,10 +2854,12 @@ static int tc_layouts(gint_handle *h, cudaStream_t st) {
   h->hs_elems = tot[0];
   h->max_brick_porb = (int)tot[3];
   int rc;
+  h->fx_batch = 0;
+  if ((rc = tc_reserve(h, h->plan, h->cap_plan, tot[1])) || (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2]))) return rc;
   // the scratch tiles' buffer also serves the float64 passes: enlarged (small systems) to hold a brick per SM for
   // them, to no more than twice the tiles and 96 MB (a server keeps many small handles), if memory allows.  A batch
-  // of fewer than 64 bricks would leave the chip to launch tails; the CUDA-core kernels are then as fast.
-  h->fx_batch = 0;
+  // of fewer than 64 bricks would leave the chip to launch tails; the CUDA-core kernels are then as fast.  (After the
+  // buffers that every pass needs, so that it never takes their memory.)
   const long long fx0 = gint_fx_bytes(h, 0), fx1 = gint_fx_bytes(h, 1) - fx0;
   if (fx1 > 0) {
     const long long room = (2 * tot[0] * 4 + (96LL << 20) - fx0) / fx1;
@@ -2864,9 +2868,7 @@ static int tc_layouts(gint_handle *h, cudaStream_t st) {
         tc_reserve(h, h->hs, h->cap_hs, std::max(tot[0], (gint_fx_bytes(h, want) + 3) / 4)) == GINT_OK)
       h->fx_batch = want;
   }
-  if ((rc = tc_reserve(h, h->hs, h->cap_hs, tot[0])) || (rc = tc_reserve(h, h->plan, h->cap_plan, tot[1])) ||
-      (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2])))
-    return rc;
+  if ((rc = tc_reserve(h, h->hs, h->cap_hs, tot[0]))) return rc;
   if ((size_t)nu * sizeof(int) <= kLaySmem) {
     if ((rc = set_smem(k_lay_fill<true>, kLaySmem))) return rc;
     k_lay_fill<true><<<(unsigned)nr, 32, nu * sizeof(int), st>>>(g, h->nbr(), nb, h->pair_u, nu, per, h->lay_cnt,

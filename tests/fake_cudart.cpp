@@ -18,7 +18,8 @@ std::map<const void *, std::string> &names() {
 std::string g_log;
 size_t g_live = 0, g_limit = ~(size_t)0;
 std::map<void *, size_t> g_blocks;
-int g_refuse = 0, g_err_plans = 0, g_porb = 16;
+int g_refuse = 0, g_err_plans = 0;
+long long g_tot[4] = {1000, 100, 50, 16};
 struct Cfg {
   dim3 g, b;
   size_t s;
@@ -43,7 +44,7 @@ void launched(const void *f, void **args) {
       long long *total;
     };
     long long *t = ((S *)args[0])->total;
-    t[0] = 1000, t[1] = 100, t[2] = 50, t[3] = g_porb;  // (t[3]: k_lay_count's widest brick)
+    memcpy(t, g_tot, sizeof(g_tot));  // (t[3]: k_lay_count's widest brick)
   } else if (is("k_build_plans") && g_err_plans) {
     **(unsigned **)args[6] |= 4u;
   }
@@ -58,7 +59,7 @@ void fake_refuse(int on) { g_refuse = on; }       // the next geometries overlap
 void fake_plan_error(int on) { g_err_plans = on; }
 void fake_limit(size_t bytes) { g_limit = bytes; }  // device memory
 size_t fake_live() { return g_live; }
-void fake_width(int porb) { g_porb = porb; }
+void fake_list_entries(long long n) { g_tot[2] = n; }
 
 // what nvcc's host code calls
 void **__cudaRegisterFatBinary(void *) {

@@ -63,6 +63,57 @@ def test_no_launch_after_a_refused_geometry(fake, cause, code):
     g.close()
 
 
+def _rho64(G, lib, g):
+    lib.fake_clear()
+    g.rho(torch.zeros(g.nblock, dtype=torch.float64), G.FP64, out=torch.zeros(g.ngrid, dtype=torch.float64))
+    return lib.fake_log()
+
+
+def test_scratch_of_the_float64_passes_takes_no_memory_that_others_need(fake):
+    """A handle whose buffers fit without the float64 scratch is created without it, and its float64 passes run on the
+    CUDA-core kernels; one that loses its buffers in a failed set_positions launches nothing."""
+    G, lib = fake
+    lib.fake_refuse(0)
+    lib.fake_plan_error(0)
+    unlimited = 2 ** 63
+    w = inputs.si_workload((1, 1, 1), (16, 16, 16), seed=0)
+    pos = torch.from_numpy(w.system.pos.copy())
+    before = lib.fake_live()
+    g = G.Gint(w.system)
+    full = lib.fake_live() - before
+    assert b"k_fx_eval" in _rho64(G, lib, g)
+    g.close()
+    assert lib.fake_live() == before
+    try:
+        lib.fake_limit(before + full - 1)
+        g = G.Gint(w.system)
+        small = lib.fake_live() - before
+        log = _rho64(G, lib, g)
+        assert small < full and b"k_fx" not in log and b"k_simt_rho" in log
+        # a list that grows to exactly what is left
+        n = 4000
+        lib.fake_list_entries(n)
+        lib.fake_limit(before + small + 8 * (n - 50))
+        g.set_positions(pos)
+        assert b"k_simt_rho" in _rho64(G, lib, g)
+        # ... and beyond it
+        lib.fake_list_entries(2 * n)
+        with pytest.raises(G.GintError) as e:
+            g.set_positions(pos)
+        assert e.value.code == -2
+        with pytest.raises(G.GintError):
+            _rho64(G, lib, g)
+        assert lib.fake_log() == b""
+        lib.fake_limit(unlimited)
+        g.set_positions(pos)
+        assert b"k_fx_eval" in _rho64(G, lib, g)
+        g.close()
+    finally:
+        lib.fake_limit(unlimited)
+        lib.fake_list_entries(50)
+    assert lib.fake_live() == before
+
+
 @pytest.mark.gpu
 def test_refused_and_recovered_on_the_gpu():
     from paper_2603_21835_gb300 import gint as G
