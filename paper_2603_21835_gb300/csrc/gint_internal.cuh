@@ -232,10 +232,12 @@ __device__ __forceinline__ void add_orbitals(const GTabs &g, const typename Tab2
 // slopes the basis functions of t took 7 and 13 more an image.)
 #define GINT_O64_SHAPES(X) X(2, 2, 1, 13) X(2, 1, 0, 5) X(1, 1, 1, 9) X(1, 1, 0, 4) X(1, 0, 0, 1) X(3, 3, 2, 22)
 
-// 1 / r, r and the knot position of a point with r2 = |d|^2 (below 1e-36 it counts as 1e-36).
+// 1 / r, r and the knot position of a point with r2 = |d|^2 (below 1e-36 it counts as 1e-36).  end: at or beyond the
+// last knot, where the radials are 0 (r2 may lie below the squared support radius and r round up to the radius).
 struct Knot64 {
   double y, r, t;
   int i;
+  bool end;
 };
 __device__ __forceinline__ Knot64 knot64(const GRadial &R0, double r2) {
   Knot64 K;
@@ -254,8 +256,10 @@ __device__ __forceinline__ Knot64 knot64(const GRadial &R0, double r2) {
   // knot i = floor(r / dr), t in [0, 1] (a point on a knot may take either side)
   const double x = K.r * R0.inv_dr, big = 6755399441055744.0;  // 1.5 2^52
   const double xi = (x - 0.5) + big;  // its low bits: an integer within 1/2 of x - 1/2
-  K.i = min(max(__double2loint(xi), 0), R0.npts - 2);
+  K.i = __double2loint(xi);
   K.t = x - (xi - big);
+  K.end = false;
+  if (K.i >= R0.npts - 2) K.end = K.i > R0.npts - 2 || K.t >= 1.0;
   return K;
 }
 
@@ -265,6 +269,7 @@ __device__ __forceinline__ void orbitals64(const GTabs &g, const double *__restr
                                            double dy, double dz, double r2, double *phi) {
   constexpr int NR = NS + NP + ND;
   const Knot64 K = knot64(g.rad[S.rad0], r2);
+  if (K.end) return;
   const double t = K.t;
   const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)K.i * NR) * 2;
   double f[NR];
@@ -311,6 +316,7 @@ __device__ __forceinline__ void contract64(const GTabs &g, const double *__restr
   const GRadial &R0 = g.rad[S.rad0];
   const bool at0 = r2 < 1e-24;
   const Knot64 K = knot64(R0, r2);
+  if (K.end) return;
   const double t = K.t, idr = R0.inv_dr;
   const double2 *q = reinterpret_cast<const double2 *>(tab) + ((long long)S.ioff + (long long)K.i * NR) * 2;
   const double ux = at0 ? 0.0 : dx * K.y, uy = at0 ? 0.0 : dy * K.y, uz = at0 ? 0.0 : dz * K.y;

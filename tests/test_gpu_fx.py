@@ -142,3 +142,38 @@ def test_captured_passes_replay():
             assert float((a - b).abs().max()) <= 1e-13 * float(b.abs().max())
     cn.close()
     g.close()
+
+
+@pytest.mark.parametrize("rc,dr", [(5.0, 0.01), (5.0, 0.2), (10.0, 0.01), (10.0, 10.0 / 1023), (5.0, 5.0)])
+def test_no_support_where_r_rounds_up_to_the_radius(rc, dr):
+    """A grid point with r2 one ulp below rc^2, so that r rounds to rc, the last knot: outside, as for the oracle and
+    the CUDA-core evaluator, whatever the parity of the knot count and the values at the table's end."""
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    sp = _sp("a", [(0, 0.3, rc)], dr)
+    sp.radials[0].f[:] = 1.0
+    sp.radials[0].df[:] = 0.0
+    a, b = 3.0 * rc / 5.0, np.nextafter(4.0 * rc / 5.0, 0.0)
+    r2 = b * b + a * a  # (the kernels' order: fma(dy, dy, dx dx), the product of b exact enough to agree)
+    assert r2 == np.nextafter(rc * rc, 0.0) and np.sqrt(r2) == rc
+    s = inputs.System(cell=np.diag([4.0 * rc] * 3), pos=np.array([[a, b, 0.0]]), species=np.zeros(1, np.int32), sp=[sp],
+                      grid=(8, 8, 8))
+    o = Oracle(s)
+    D = np.array([[3.0]])
+    V = np.ones(512)
+    ref = o.rho(D).reshape(-1)
+    assert ref[0] == 0.0 and ref.max() > 0.2
+    g = G.Gint(s)
+    Db, Vd = torch.from_numpy(g.dense_to_blocks(D)).cuda(), torch.from_numpy(V).cuda()
+    rho = g.rho(Db, G.FP64).cpu().numpy().reshape(-1)
+    rho_f = torch.empty(512, dtype=torch.float64, device="cuda")
+    F = g.force(Db, Vd, G.FP64, rho_out=rho_f).cpu().numpy()
+    H = g.vlocal(Vd, G.FP64).cpu().numpy()
+    g.sync()
+    assert rho[0] == 0.0 and rho_f[0].item() == 0.0
+    assert np.abs(rho - ref).max() <= 1e-12 * ref.max() and np.abs(rho_f.cpu().numpy() - ref).max() <= 1e-12 * ref.max()
+    assert np.abs(H - o.vlocal(V).reshape(-1)).max() <= 1e-12 * np.abs(o.vlocal(V)).max()
+    assert np.abs(F - o.force(D, V)).max() <= 1e-11
+    g.close()
