@@ -259,7 +259,12 @@ __device__ __forceinline__ Knot64 knot64(const GRadial &R0, double r2) {
   K.i = __double2loint(xi);
   K.t = x - (xi - big);
   K.end = false;
-  if (K.i >= R0.npts - 2) K.end = K.i > R0.npts - 2 || K.t >= 1.0;
+  if (K.i >= R0.npts - 2) {  // (x rounded: above, the multiplication may be fused into x - 0.5 and t)
+    const double xr = __dmul_rn(K.r, R0.inv_dr);
+    K.i = R0.npts - 2;
+    K.t = xr - (double)K.i;
+    K.end = K.t >= 1.0;
+  }
   return K;
 }
 
