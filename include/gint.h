@@ -136,7 +136,7 @@ int gint_brick_lists(const gint_handle *h, long long *nslots, long long *nentrie
 
 /* Diagnostic: the periodised orbitals Phi_mu (Eqs. 1-2 at k = 0, all lattice images within the support)
  * and their gradients at arbitrary points, evaluated by the brick kernels' own evaluators:
- * GINT_FP64 (the float64 CUDA-core evaluator) or GINT_F16X3 (the tensor-core path's float32 evaluator:
+ * GINT_FP64 (the evaluators of the float64 passes) or GINT_F16X3 (the tensor-core path's float32 evaluator:
  * double-float distance and knot parameter, float32 Hermite interpolation with derivative differences
  * formed in float64, float32 Y_lm).  pts [npts][3] (host, Cartesian Bohr); phi [npts][norb] and grad
  * [npts][norb][3] (host outputs, grad may be NULL).  Synchronous; allocates temporary device memory.

@@ -2565,9 +2565,22 @@ __global__ void __launch_bounds__(kT, 1)
 // ------------------------------------------------------------------------------ orbital diagnostic
 // One thread per (point, atom): the periodised orbitals of the atom and their gradients at an
 // arbitrary point, summed over the lattice images whose support covers it, by the brick kernels'
-// own evaluators: float64 (the CUDA-core path's add_orbitals) or float32 (the tensor-core path's
-// double-float distance, knot and Hermite evaluation, difference tables for the derivatives).
-__global__ void k_orbitals(const __grid_constant__ GGeom g, const double2 *__restrict__ tab64,
+// own evaluators: float64 (orbitals64, and contract64 with one coefficient at a time for the gradients; add_orbitals
+// for species without a compiled shape) or float32 (the tensor-core path's double-float distance, knot and Hermite
+// evaluation, difference tables for the derivatives).
+template <int NS, int NP, int ND, int NO>
+__device__ __forceinline__ void orbitals_point64(const GTabs &t, const double *__restrict__ otab, const GSpecies &S,
+                                                 const double dd[3], double r2, double *v, double (*gv)[3]) {
+  orbitals64<NS, NP, ND>(t, otab, S, dd[0], dd[1], dd[2], r2, v);
+  for (int m = 0; m < NO; ++m) {
+    double c[NO], rho = 0.0;
+#pragma unroll
+    for (int i = 0; i < NO; ++i) c[i] = i == m ? 1.0 : 0.0;
+    contract64<NS, NP, ND>(t, otab, S, dd[0], dd[1], dd[2], r2, c, rho, gv[m][0], gv[m][1], gv[m][2]);
+  }
+}
+__global__ void k_orbitals(const __grid_constant__ GGeom g, const __grid_constant__ GTabs t64,
+                           const double *__restrict__ otab64, const double2 *__restrict__ tab64,
                            const float2 *__restrict__ tab, const float2 *__restrict__ tabi,
                            const float *__restrict__ dtab, const float *__restrict__ dtabi, const double *__restrict__ pos,
                            const int *__restrict__ species, const int *__restrict__ aoff, long long npts, int norb,
@@ -2597,9 +2610,17 @@ __global__ void k_orbitals(const __grid_constant__ GGeom g, const double2 *__res
       for (int n2 = lo[2]; n2 <= hi[2]; ++n2) {
         double dd[3];
         for (int d = 0; d < 3; ++d) dd[d] = d0[d] - (n0 * g.cell[d] + n1 * g.cell[3 + d] + n2 * g.cell[6 + d]);
-        if (dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2] >= S.rcut2) continue;
+        const double r2 = fma(dd[2], dd[2], fma(dd[1], dd[1], dd[0] * dd[0]));
+        if (r2 >= S.rcut2) continue;
         if (fp64) {
-          add_orbitals<double, true, true>(g, tab64, sp, dd[0], dd[1], dd[2], v64, gv64);
+          switch (t64.sp[sp].shape) {
+#define CASE_O64(ns, np_, nd, no_) \
+  case GINT_SHAPE(ns, np_, nd): orbitals_point64<ns, np_, nd, no_>(t64, otab64, t64.sp[sp], dd, r2, v64, gv64); break;
+            GINT_O64_SHAPES(CASE_O64)
+#undef CASE_O64
+            default:
+              add_orbitals<double, true, true>(g, tab64, sp, dd[0], dd[1], dd[2], v64, gv64);
+          }
         } else {
           float dh[3], dl[3];
           for (int d = 0; d < 3; ++d) split2(dd[d], dh[d], dl[d]);
@@ -3380,7 +3401,7 @@ extern "C" int gint_orbitals(gint_handle *h, int precision, long long npts, cons
     rc = GINT_ECUDA;
   if (!rc) {
     const long long nt = npts * na;
-    k_orbitals<<<(unsigned)((nt + 127) / 128), 128>>>(h->geom, h->tab64, h->tab32, h->tab32i, h->dtab32, h->dtab32i,
+    k_orbitals<<<(unsigned)((nt + 127) / 128), 128>>>(h->geom, h->tabs64, h->otab64, h->tab64, h->tab32, h->tab32i, h->dtab32, h->dtab32i,
                                                       h->pos_dev, h->species_dev, daoff, npts, norb, dp,
                                                       precision == GINT_FP64 ? 1 : 0, dphi, dgrad);
     if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) rc = GINT_ECUDA;

@@ -131,3 +131,25 @@ def test_orbital_evaluators_match_oracle_at_edge_radii(prec, tol, gtol):
     assert np.all(np.abs(ref_phi[0, off[0]:off[1]][l_of > 0]) == 0.0)
     assert np.abs(own[l_of > 0]).max() <= tol * np.abs(ref_phi).max()
     g.close()
+
+
+def test_float64_orbitals_are_those_of_the_float64_passes():
+    """gint_orbitals evaluates as the passes do: with one s orbital and D = 1 the digits hold the orbital itself, so the
+    density is the square of the orbital bit for bit."""
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    L, grid = 13.0, (12, 8, 16)
+    sp = inputs.Species(name="s", radials=[inputs.make_radial(0, 0.3, 6.0, 0.01)])
+    s = inputs.System(cell=np.diag([L] * 3), pos=np.array([[6.3, 6.7, 6.55]]), species=np.zeros(1, np.int32), sp=[sp],
+                      grid=grid)
+    g = G.Gint(s)
+    x = [np.arange(n) / n * L for n in grid]
+    pts = np.stack(np.meshgrid(*x, indexing="ij"), -1).reshape(-1, 3)
+    phi, _ = g.orbitals(pts, G.FP64)
+    rho = g.rho(torch.ones(1, dtype=torch.float64, device="cuda"), G.FP64).cpu().numpy().reshape(-1)
+    g.sync()
+    one = np.linalg.norm(pts - s.pos[0], axis=1) < 6.4  # (of the other points some see an image, formed in another order)
+    assert one.sum() > 500 and np.array_equal(rho[one], phi[one, 0] ** 2)
+    g.close()
