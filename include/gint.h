@@ -247,6 +247,13 @@ int gint_psibeta(gint_handle *h, const double *A, double *out, void *stream);
  * definite Hermitian part S) is factored as L D L^T without pivoting.
  * gint_dm_build: D = Re(psi diag(f) psi^dagger), f [nocc] (device) occupations; D is symmetric bit
  * for bit.
+ * Accuracy of the float64 products: an operand is held to 2^-62 of its row's largest element, so that an
+ * element's error is below 2^-58 per term of the product of the two rows' maxima, plus one rounding.
+ * In norms that is no worse than a float64 chain; elements far below both maxima (a density-matrix
+ * element of two functions that overlap in their tails only) keep fewer significant bits than a chain
+ * would leave them.  gint_cn_step and gint_edm work in the basis scaled by powers of two to norms next to
+ * 1 and balance the factor's pivots: results do not depend on such a scaling, and the solve is as
+ * backward stable as plain float64 elimination.
  * gint_dm_build_f16x3: the same D on the tensor cores: D = A B^T with A_ik = f_s psi_is, B_ik = psi_is
  * (k = 2 s + real / imaginary part), each operand scaled by a power of two and split into float16
  * hi + lo, three float16 products per term (lo lo dropped).  The hi hi products of each chunk of 64 k

@@ -20,31 +20,62 @@
 
 namespace {
 
-// A = S + i dt/2 H (S, H real symmetric: row- and column-major alike)
-__global__ void k_cn_mat(long long nn, const double *__restrict__ S, const double *__restrict__ H, double half_dt,
-                         double2 *__restrict__ A) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nn; e += (long long)gridDim.x * blockDim.x)
-    A[e] = make_double2(S[e], half_dt * H[e]);
+// The steps work in the basis t_i phi_i, t_i the power of two that brings the norm sqrt(S_ii) next to 1 (between
+// 2^-1/2 and 2^1/2).  Digit products scale an operand by its rows' largest elements, so a contraction over basis
+// functions of very different norms would lose the bits of the small ones, which float64's own exponents keep; scaled
+// by powers of two, nothing is rounded, and the results do not depend on such a scaling of the basis at all.  Normalised
+// functions have t = 1.
+__device__ __forceinline__ int eq_exp(double s) {  // t = 2^-eq_exp
+  const int e = (__double2hiint(s) >> 20) & 0x7ff;
+  return e == 0 || e == 0x7ff ? 0 : (e - 1023 + 1) >> 1;
 }
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// X <- 2 X - psi
-__global__ void k_cn_finish(long long m, const double2 *__restrict__ psi, double2 *__restrict__ X) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < m; e += (long long)gridDim.x * blockDim.x) {
+// F = t S t, or (H not null) the complex t (S + i dt/2 H) t (S, H real symmetric: row- and column-major alike);
+// eq[0 .. n) = t, eq[n .. 2 n) = 1 / t
+template <typename T>
+__global__ void __launch_bounds__(256) k_cn_mat(int n, const double *__restrict__ S, const double *__restrict__ H,
+                                                double half_dt, T *__restrict__ F, double *__restrict__ eq) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  const int p = eq_exp(S[i + (long long)i * n]);
+  const double ti = pow2(-p);
+  if (blockIdx.y == 0) {
+    eq[i] = ti;
+    eq[n + i] = pow2(p);
+  }
+  for (int j = blockIdx.y; j < n; j += gridDim.y) {
+    const double tj = pow2(-eq_exp(S[j + (long long)j * n]));
+    const long long e = i + (long long)j * n;
+    if constexpr (sizeof(T) == 16)
+      F[e] = make_double2(S[e] * ti * tj, half_dt * H[e] * ti * tj);
+    else
+      F[e] = S[e] * ti * tj;
+  }
+}
+dim3 mat_grid(int n) { return dim3((unsigned)((n + 255) / 256), (unsigned)std::min(n, 16384)); }
+
+// X <- 2 t X - psi (rows of n)
+__global__ void k_cn_finish(int n, int k, const double2 *__restrict__ psi, double2 *__restrict__ X,
+                            const double *__restrict__ t) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  const double s = 2.0 * t[i];
+  for (int c = blockIdx.y; c < k; c += gridDim.y) {
+    const long long e = i + (long long)c * n;
     const double2 x = X[e], p = psi[e];
-    X[e] = make_double2(2.0 * x.x - p.x, 2.0 * x.y - p.y);
+    X[e] = make_double2(s * x.x - p.x, s * x.y - p.y);
   }
 }
 
-// E = (X + X^T) / 2 (n x n)
-__global__ void k_sym_half(int n, const double *__restrict__ X, double *__restrict__ E) {
-  const long long nn = (long long)n * n;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nn; e += (long long)gridDim.x * blockDim.x) {
-    const long long i = e / n, j = e - i * n;
-    E[e] = 0.5 * (X[e] + X[j * n + i]);
-  }
+// E = (t X + (t X)^T) / 2 (n x n; X column-major)
+__global__ void k_sym_half(int n, const double *__restrict__ X, const double *__restrict__ t, double *__restrict__ E) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  const double ti = t[i];
+  for (int j = blockIdx.y; j < n; j += gridDim.y)
+    E[i + (long long)j * n] = 0.5 * (ti * X[i + (long long)j * n] + t[j] * X[j + (long long)i * n]);
 }
-
-unsigned blocks_for(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 4096); }
 
 }  // namespace
 
@@ -53,6 +84,7 @@ struct gint_cn {
   double2 *A = nullptr;        // n x n: the factor (complex), or two real n x n matrices (gint_edm)
   double2 *work = nullptr;     // the factorisation's panel workspace (gla::ldl_work)
   gla::SgWork sg{};            // scratch of the float64 products
+  double *eq = nullptr;        // 2 n: the basis scaling of the call (k_cn_mat)
   int *info = nullptr;
   void *dmw = nullptr;         // tensor-core density-matrix build: packed operands and scales
   unsigned *status = nullptr;  // its device error word
@@ -66,6 +98,7 @@ int gint_cn_destroy(gint_cn *c) {
   cudaFree(c->A);
   cudaFree(c->work);
   cudaFree(c->sg.buf);
+  cudaFree(c->eq);
   cudaFree(c->info);
   cudaFree(c->dmw);
   cudaFree(c->status);
@@ -88,7 +121,7 @@ int gint_cn_create(int n, int nocc, gint_cn **out) {
                           gla::sg_bytes(gla::ldl_rows<double2>(n, nocc), 64), gla::sg_bytes(gla::ldl_rows<double>(n, n), 64)});
   if (cudaDeviceGetAttribute(&c->sg.num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
       cudaMalloc(&c->A, nn * sizeof(double2)) != cudaSuccess || cudaMalloc(&c->work, work) != cudaSuccess ||
-      cudaMalloc(&c->sg.buf, c->sg.bytes) != cudaSuccess ||
+      cudaMalloc(&c->sg.buf, c->sg.bytes) != cudaSuccess || cudaMalloc(&c->eq, 2 * (size_t)n * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&c->info, sizeof(int)) != cudaSuccess || cudaMalloc(&c->dmw, gint_dm_tc_bytes(n, nocc)) != cudaSuccess ||
       cudaMalloc(&c->status, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(c->info, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->status, 0, sizeof(unsigned)) != cudaSuccess) {
@@ -109,14 +142,16 @@ int gint_cn_step(gint_cn *c, const double *S, const double *H, double dt, const 
   const long long nn = (long long)n * n;
   double2 *X = reinterpret_cast<double2 *>(psi_out);
   if (cudaMemsetAsync(c->info, 0, sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
-  k_cn_mat<<<blocks_for(nn), 256, 0, st>>>(nn, S, H, 0.5 * dt, c->A);
+  k_cn_mat<double2><<<mat_grid(n), 256, 0, st>>>(n, S, H, 0.5 * dt, c->A, c->eq);
   if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA;
-  // X = S psi as one real product: column 2 c + part of the interleaved complex arrays
+  // X = (t S t) (psi / t) as one real product: column 2 c + part of the interleaved complex arrays
   gla::SgProduct p{};
   p.M = p.K = n;
   p.N = 2 * k;
   p.A = gla::sg_real(S, 1, n);
   p.B = gla::SgView{psi, 2LL * n, 1, 4, 2, 0, nullptr};
+  p.A.rs = p.A.ks = c->eq;
+  p.B.ks = c->eq + n;
   p.C = psi_out;
   p.crh = 4;
   p.crl = 2;
@@ -125,7 +160,8 @@ int gint_cn_step(gint_cn *c, const double *S, const double *H, double dt, const 
   int rc = gla::sg_gemm(&p, 1, c->sg, st);
   if (rc) return rc;
   if ((rc = gla::ldl_factor_solve<double2>(n, c->A, n, k, X, n, c->work, c->info, false, c->sg, st))) return rc;
-  k_cn_finish<<<blocks_for((long long)n * k), 256, 0, st>>>((long long)n * k, reinterpret_cast<const double2 *>(psi), X);
+  k_cn_finish<<<dim3((unsigned)((n + 255) / 256), (unsigned)std::min(k, 16384)), 256, 0, st>>>(
+      n, k, reinterpret_cast<const double2 *>(psi), X, c->eq);
   return cudaGetLastError() == cudaSuccess ? GINT_OK : GINT_ECUDA;
 }
 
@@ -138,7 +174,7 @@ int gint_dm_build(gint_cn *c, const double *psi, const double *f, double *D, voi
   p.M = p.N = n;
   p.K = 2 * c->nocc;
   p.mode = 2;
-  p.A = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f};
+  p.A = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 1};
   p.B = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, nullptr};
   p.C = D;
   p.crh = 2;
@@ -159,14 +195,16 @@ int gint_edm(gint_cn *c, const double *S, const double *H, const double *D, doub
   const int n = c->n;
   // the complex n x n buffer holds two real n x n matrices: F (the factor of S) and X
   double *F = reinterpret_cast<double *>(c->A), *X = F + (size_t)n * n;
-  if (cudaMemsetAsync(c->info, 0, sizeof(int), st) != cudaSuccess ||
-      cudaMemcpyAsync(F, S, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return GINT_ECUDA;
-  // X = H D, then X <- S^{-1} X (S = L D L^T), E = (X + X^T) / 2
+  if (cudaMemsetAsync(c->info, 0, sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
+  k_cn_mat<double><<<mat_grid(n), 256, 0, st>>>(n, S, nullptr, 0.0, F, c->eq);
+  if (cudaGetLastError() != cudaSuccess) return GINT_ECUDA;
+  // X = (t H t) (D / t), then X <- (t S t)^{-1} X (t S t = L D L^T), E = (t X + (t X)^T) / 2
   gla::SgProduct p{};
   p.M = p.N = p.K = n;
   p.A = gla::sg_real(H, 1, n);
   p.B = gla::sg_real(D, n, 1);
+  p.A.rs = p.A.ks = c->eq;
+  p.B.ks = c->eq + n;
   p.C = X;
   p.crh = 2;
   p.crl = 1;
@@ -176,7 +214,7 @@ int gint_edm(gint_cn *c, const double *S, const double *H, const double *D, doub
   if (rc) return rc;
   if ((rc = gla::ldl_factor_solve<double>(n, F, n, n, X, n, reinterpret_cast<double *>(c->work), c->info, true, c->sg, st)))
     return rc;
-  k_sym_half<<<blocks_for((long long)n * n), 256, 0, st>>>(n, X, E);
+  k_sym_half<<<mat_grid(n), 256, 0, st>>>(n, X, c->eq, E);
   return cudaGetLastError() == cudaSuccess ? GINT_OK : GINT_ECUDA;
 }
 

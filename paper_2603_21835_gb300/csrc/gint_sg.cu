@@ -11,6 +11,10 @@
 //   less 128), exact in float16;
 //   sum_k x_ik y_jk = 2^(..) sum_{l = s + t} 256^(14 - l) sum_k d_s d_t, levels l = 0..7 kept (the
 //   dropped ones are below 2^-60 of the largest products: float64 rounding of one product is 2^-53).
+//   An element's error is below 2^-58 per term of the product of its two rows' largest magnitudes, and one float64
+//   rounding: in norms that is better than a float64 chain, but terms far below the maxima of both rows lose bits that
+//   a chain keeps.  Callers balance a contraction index whose magnitudes run against each other in the two operands
+//   (basis functions of unequal norms, pivots) with powers of two.
 //
 // The MMAs of level l add at most 8 x 128 products of magnitude 2^14 per accumulator in a range of 128 k:
 // at most 2^24, so every float32 partial sum is an exact integer whatever the tensor core's rounding.
@@ -343,7 +347,7 @@ static int sg_plan(const SgProduct *pr, int np, const SgWork &ws, int k0, int kk
     // the range [k0, k0 + kk) of the contraction (kSgK is even: part offsets stay aligned)
     for (SgView *v : {&pb.p.A, &pb.p.B}) {
       v->p += (long long)(k0 >> 1) * v->kh;
-      if (v->ks) v->ks += k0 >> 1;
+      if (v->ks) v->ks += k0 >> v->ksh;
     }
     pb.p.K = kk;
     if (k0 > 0) pb.p.beta = 1;

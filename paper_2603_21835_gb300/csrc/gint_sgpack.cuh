@@ -12,9 +12,11 @@ __device__ __forceinline__ double sg_at(const SgView &v, int r, int k) {
     const double x = v.p[(long long)(r >> 1) * v.rh + (long long)(k >> 1) * v.kh + ((r ^ k) & 1)];
     return (!(r & 1) && (k & 1)) ? -x : x;
   }
-  const double x = v.p[(long long)(r >> 1) * v.rh + (long long)(r & 1) * v.rl + (long long)(k >> 1) * v.kh +
-                       (long long)(k & 1) * v.kl];
-  return v.ks ? x * v.ks[k >> 1] : x;
+  double x = v.p[(long long)(r >> 1) * v.rh + (long long)(r & 1) * v.rl + (long long)(k >> 1) * v.kh +
+                 (long long)(k & 1) * v.kl];
+  if (v.ks) x *= v.ks[k >> v.ksh];
+  if (v.rs) x *= v.rs[r];
+  return x;
 }
 
 constexpr int kPR = kPackRows, kPK = 64, kPT = 256;  // rows and k of a packing block, its threads
