@@ -249,6 +249,7 @@ int gint_psibeta(gint_handle *h, const double *A, double *out, void *stream);
  * for bit.
  * Accuracy of the float64 products: an operand is held to 2^-62 of its row's largest element, so that an
  * element's error is below 2^-58 per term of the product of the two rows' maxima, plus one rounding.
+ * (gint_dm_build: of f^(1/2) psi, so below (2 nocc) 2^-57 (D_ii D_jj)^(1/2) for occupations >= 0.)
  * In norms that is no worse than a float64 chain; elements far below both maxima (a density-matrix
  * element of two functions that overlap in their tails only) keep fewer significant bits than a chain
  * would leave them.  gint_cn_step and gint_edm work in the basis scaled by powers of two to norms next to

@@ -168,14 +168,16 @@ int gint_cn_step(gint_cn *c, const double *S, const double *H, double dt, const 
 int gint_dm_build(gint_cn *c, const double *psi, const double *f, double *D, void *stream) {
   if (!c || !psi || !f || !D) return GINT_EINVAL;
   const int n = c->n;
-  // D = A B^T over k = 2 s + (real, imaginary part): A_ik = f_s psi_is, B_ik = psi_is (real views);
+  // D = A B^T over k = 2 s + (real, imaginary part): A_ik = f_s psi_is, B_ik = psi_is (real views), with the power of
+  // two next to |f_s|^(1/2) moved from A to B: the row maxima that the digits are relative to are then at most
+  // about D_ii^(1/2), so a function that lives in states of small occupation keeps its bits;
   // the lower triangle is computed and mirrored, so D is symmetric bit for bit
   gla::SgProduct p{};
   p.M = p.N = n;
   p.K = 2 * c->nocc;
   p.mode = 2;
-  p.A = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 1};
-  p.B = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, nullptr};
+  p.A = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 1, nullptr, 1};
+  p.B = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 1, nullptr, 2};
   p.C = D;
   p.crh = 2;
   p.crl = 1;

@@ -70,3 +70,29 @@ def test_small_pivots_leave_the_solve_backward_stable(small, cols):
     Sl, Hl = S.astype(np.longdouble), H.astype(np.longdouble)
     R = Sl @ X + 0.5j * dt * (Hl @ X) - Sl @ psi.astype(np.clongdouble)
     assert np.abs(R).max() <= n * 2.0**-53 * np.abs(X).max()
+
+
+def test_density_matrix_of_functions_in_states_of_small_occupation():
+    """Half of the functions have all their weight in states of occupation 1e-12: the error is relative to
+    (D_ii D_jj)^(1/2), the operands' digits being those of f^(1/2) psi."""
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    n, nocc = 70, 40
+    rng = np.random.default_rng(3)
+    psi = rng.normal(size=(n, nocc)) + 1j * rng.normal(size=(n, nocc))
+    f = np.where(np.arange(nocc) < 10, 1.3, 1.7e-12)
+    psi[: n // 2, :10] *= 1e-7
+    cn = G.CrankNicolson(n, nocc)
+    D = cn.density_matrix(torch.from_numpy(np.ascontiguousarray(psi.T)).cuda(), torch.from_numpy(f).cuda()).cpu().numpy()
+    assert cn.info() == 0
+    cn.close()
+    a = np.stack([psi.real, psi.imag], -1).reshape(n, 2 * nocc).astype(np.longdouble)
+    fa = a * np.repeat(f, 2)
+    ref = fa @ a.T
+    d = np.sqrt(np.diag(ref))
+    # the factor f psi and the sum are rounded once each
+    bound = 2.0**-53 * (np.abs(fa) @ np.abs(a.T) + np.abs(ref)) + 2 * nocc * 2.0**-57 * np.outer(d, d)
+    assert (np.abs(D - ref) <= bound).all()
+    assert np.array_equal(D, D.T)
