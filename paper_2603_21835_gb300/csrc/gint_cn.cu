@@ -17,6 +17,7 @@
 #include "gint.h"
 #include "gint_dm.cuh"
 #include "gint_la.cuh"
+#include "gint_sgpack.cuh"
 
 namespace {
 
@@ -29,38 +30,37 @@ __device__ __forceinline__ int eq_exp(double s) {  // t = 2^-eq_exp
   const int e = (__double2hiint(s) >> 20) & 0x7ff;
   return e == 0 || e == 0x7ff ? 0 : (e - 1023 + 1) >> 1;
 }
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
 // F = t S t, or (H not null) the complex t (S + i dt/2 H) t (S, H real symmetric: row- and column-major alike);
-// eq[0 .. n) = t, eq[n .. 2 n) = 1 / t
+// eq[0 .. n) = log2 t, eq[n .. 2 n) = -log2 t
 template <typename T>
 __global__ void __launch_bounds__(256) k_cn_mat(int n, const double *__restrict__ S, const double *__restrict__ H,
-                                                double half_dt, T *__restrict__ F, double *__restrict__ eq) {
+                                                double half_dt, T *__restrict__ F, int *__restrict__ eq) {
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= n) return;
   const int p = eq_exp(S[i + (long long)i * n]);
-  const double ti = pow2(-p);
   if (blockIdx.y == 0) {
-    eq[i] = ti;
-    eq[n + i] = pow2(p);
+    eq[i] = -p;
+    eq[n + i] = p;
   }
   for (int j = blockIdx.y; j < n; j += gridDim.y) {
-    const double tj = pow2(-eq_exp(S[j + (long long)j * n]));
     const long long e = i + (long long)j * n;
+    const double s = S[e];
+    const int q = -p - eq_exp(S[j + (long long)j * n]);
     if constexpr (sizeof(T) == 16)
-      F[e] = make_double2(S[e] * ti * tj, half_dt * H[e] * ti * tj);
+      F[e] = make_double2(gla::times_pow2(s, q), gla::times_pow2(half_dt * H[e], q));
     else
-      F[e] = S[e] * ti * tj;
+      F[e] = gla::times_pow2(s, q);
   }
 }
 dim3 mat_grid(int n) { return dim3((unsigned)((n + 255) / 256), (unsigned)std::min(n, 16384)); }
 
 // X <- 2 t X - psi (rows of n)
 __global__ void k_cn_finish(int n, int k, const double2 *__restrict__ psi, double2 *__restrict__ X,
-                            const double *__restrict__ t) {
+                            const int *__restrict__ lt) {
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= n) return;
-  const double s = 2.0 * t[i];
+  const double s = __hiloint2double((1023 + 1 + lt[i]) << 20, 0);
   for (int c = blockIdx.y; c < k; c += gridDim.y) {
     const long long e = i + (long long)c * n;
     const double2 x = X[e], p = psi[e];
@@ -69,12 +69,12 @@ __global__ void k_cn_finish(int n, int k, const double2 *__restrict__ psi, doubl
 }
 
 // E = (t X + (t X)^T) / 2 (n x n; X column-major)
-__global__ void k_sym_half(int n, const double *__restrict__ X, const double *__restrict__ t, double *__restrict__ E) {
+__global__ void k_sym_half(int n, const double *__restrict__ X, const int *__restrict__ lt, double *__restrict__ E) {
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= n) return;
-  const double ti = t[i];
+  const int li = lt[i];
   for (int j = blockIdx.y; j < n; j += gridDim.y)
-    E[i + (long long)j * n] = 0.5 * (ti * X[i + (long long)j * n] + t[j] * X[j + (long long)i * n]);
+    E[i + (long long)j * n] = 0.5 * (gla::times_pow2(X[i + (long long)j * n], li) + gla::times_pow2(X[j + (long long)i * n], lt[j]));
 }
 
 }  // namespace
@@ -84,7 +84,7 @@ struct gint_cn {
   double2 *A = nullptr;        // n x n: the factor (complex), or two real n x n matrices (gint_edm)
   double2 *work = nullptr;     // the factorisation's panel workspace (gla::ldl_work)
   gla::SgWork sg{};            // scratch of the float64 products
-  double *eq = nullptr;        // 2 n: the basis scaling of the call (k_cn_mat)
+  int *eq = nullptr;           // 2 n: the basis scaling of the call (k_cn_mat)
   int *info = nullptr;
   void *dmw = nullptr;         // tensor-core density-matrix build: packed operands and scales
   unsigned *status = nullptr;  // its device error word
@@ -121,7 +121,7 @@ int gint_cn_create(int n, int nocc, gint_cn **out) {
                           gla::sg_bytes(gla::ldl_rows<double2>(n, nocc), 64), gla::sg_bytes(gla::ldl_rows<double>(n, n), 64)});
   if (cudaDeviceGetAttribute(&c->sg.num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
       cudaMalloc(&c->A, nn * sizeof(double2)) != cudaSuccess || cudaMalloc(&c->work, work) != cudaSuccess ||
-      cudaMalloc(&c->sg.buf, c->sg.bytes) != cudaSuccess || cudaMalloc(&c->eq, 2 * (size_t)n * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&c->sg.buf, c->sg.bytes) != cudaSuccess || cudaMalloc(&c->eq, 2 * (size_t)n * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&c->info, sizeof(int)) != cudaSuccess || cudaMalloc(&c->dmw, gint_dm_tc_bytes(n, nocc)) != cudaSuccess ||
       cudaMalloc(&c->status, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(c->info, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->status, 0, sizeof(unsigned)) != cudaSuccess) {
@@ -150,8 +150,8 @@ int gint_cn_step(gint_cn *c, const double *S, const double *H, double dt, const 
   p.N = 2 * k;
   p.A = gla::sg_real(S, 1, n);
   p.B = gla::SgView{psi, 2LL * n, 1, 4, 2, 0, nullptr};
-  p.A.rs = p.A.ks = c->eq;
-  p.B.ks = c->eq + n;
+  p.A.rp = p.A.kp = c->eq;
+  p.B.kp = c->eq + n;
   p.C = psi_out;
   p.crh = 4;
   p.crl = 2;
@@ -176,8 +176,8 @@ int gint_dm_build(gint_cn *c, const double *psi, const double *f, double *D, voi
   p.M = p.N = n;
   p.K = 2 * c->nocc;
   p.mode = 2;
-  p.A = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 1, nullptr, 1};
-  p.B = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 1, nullptr, 2};
+  p.A = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 1};
+  p.B = gla::SgView{psi, 4, 2, 2LL * n, 1, 0, f, 2};
   p.C = D;
   p.crh = 2;
   p.crl = 1;
@@ -205,8 +205,8 @@ int gint_edm(gint_cn *c, const double *S, const double *H, const double *D, doub
   p.M = p.N = p.K = n;
   p.A = gla::sg_real(H, 1, n);
   p.B = gla::sg_real(D, n, 1);
-  p.A.rs = p.A.ks = c->eq;
-  p.B.ks = c->eq + n;
+  p.A.rp = p.A.kp = c->eq;
+  p.B.kp = c->eq + n;
   p.C = X;
   p.crh = 2;
   p.crl = 1;

@@ -40,6 +40,7 @@ struct Ar<double> {
   static __device__ __forceinline__ double fms(double a, double b, double c) { return ::fma(-a, b, c); }  // c - a b
   static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
   static __device__ __forceinline__ double scale(double a, double s) { return a * s; }
+  static __device__ __forceinline__ double pow2(double a, int e) { return times_pow2(a, e); }
   // reciprocal's denominator and numerator: 1 / d = num / den
   static __device__ __forceinline__ double den(double d) { return d; }
   static __device__ __forceinline__ double num(double) { return 1.0; }
@@ -52,6 +53,7 @@ struct Ar<double2> {
     return make_double2(::fma(a.y, b.y, ::fma(-a.x, b.x, c.x)), ::fma(-a.y, b.x, ::fma(-a.x, b.y, c.y)));
   }
   static __device__ __forceinline__ double2 scale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
+  static __device__ __forceinline__ double2 pow2(double2 a, int e) { return make_double2(times_pow2(a.x, e), times_pow2(a.y, e)); }
   static __device__ __forceinline__ double2 mul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
   }
@@ -300,6 +302,7 @@ __global__ void __launch_bounds__(NB * SV) k_trsv(int nb, const T *__restrict__ 
   T *x = nullptr;
   if (act) x = v < nv ? X.X + v * X.vs + i * X.es : X2.X + (v - nv) * X2.vs + i * X2.es;
   T xi = act ? *x : Ar<T>::zero();
+  const T di = PANEL && act ? dinv[i] : Ar<T>::zero();
   if (i == (TRANS ? nb - 1 : 0)) xs[tid] = xi;
   // step j reads element j (final and published after step j - 1) and changes later elements only
   if (!TRANS) {
@@ -319,11 +322,10 @@ __global__ void __launch_bounds__(NB * SV) k_trsv(int nb, const T *__restrict__ 
       }
     }
   }
-  T yi = xi, di = Ar<T>::zero();
+  T yi = xi;
   if (act) {
     if (PANEL) {
       W[v + (long long)i * ldw] = xi;
-      di = dinv[i];
       yi = Ar<T>::mul(xi, di);
     }
     *x = yi;
@@ -331,8 +333,8 @@ __global__ void __launch_bounds__(NB * SV) k_trsv(int nb, const T *__restrict__ 
   if (npk > 0) {
     if (PANEL) {
       const int b = pivot_balance(di);
-      xi = Ar<T>::scale(xi, __hiloint2double((1023 + b) << 20, 0));
-      yi = Ar<T>::scale(yi, __hiloint2double((1023 - b) << 20, 0));
+      xi = Ar<T>::pow2(xi, b);
+      yi = Ar<T>::pow2(yi, -b);
     }
     __syncthreads();  // L and the vectors in shared memory have been read
     pack_vectors<T, SV, PANEL>(pk, npk, blockIdx.x * SV, nv, nv2, i, vl, xi, yi,

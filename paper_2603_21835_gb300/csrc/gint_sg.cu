@@ -347,7 +347,8 @@ static int sg_plan(const SgProduct *pr, int np, const SgWork &ws, int k0, int kk
     // the range [k0, k0 + kk) of the contraction (kSgK is even: part offsets stay aligned)
     for (SgView *v : {&pb.p.A, &pb.p.B}) {
       v->p += (long long)(k0 >> 1) * v->kh;
-      if (v->ks) v->ks += k0 >> v->ksh;
+      if (v->ks) v->ks += k0 >> 1;
+      if (v->kp) v->kp += k0;
     }
     pb.p.K = kk;
     if (k0 > 0) pb.p.beta = 1;

@@ -30,9 +30,9 @@ int sg_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cuda
 
 // Real operand view of a product: element (r, k), r the output row (or column) index and k the
 // contraction index, is
-//   p[(r >> 1) rh + (r & 1) rl + (k >> 1) kh + (k & 1) kl], times ks[k >> ksh] when ks is not null and times rs[r]
-//   when rs is not null; half: ks in two factors, ks 2^-h (1) for the left operand and 2^h (2) for the right one, 2^h
-//   next to |ks|^(1/2),
+//   p[(r >> 1) rh + (r & 1) rl + (k >> 1) kh + (k & 1) kl], times ks[k >> 1] when ks is not null; half: ks in
+//   two factors, ks 2^-h (1) for the left operand and 2^h (2) for the right one, 2^h next to |ks|^(1/2); and times
+//   2^(kp[k] + rp[r]) when kp is not null (rp null: 0),
 // or, for `rot` (the left operand of a complex product seen as a real one: output rows 2 i = real and
 // 2 i + 1 = imaginary part, contraction 2 k = real and 2 k + 1 = imaginary part of the right operand),
 //   +- p[(r >> 1) rh + (k >> 1) kh + ((r ^ k) & 1)], minus when r is even and k odd.
@@ -41,9 +41,8 @@ struct SgView {
   long long rh, rl, kh, kl;
   int rot;
   const double *ks;
-  int ksh;
-  const double *rs;
   int half;
+  const int *kp, *rp;
 };
 inline SgView sg_real(const double *p, long long sr, long long sk) {
   return SgView{p, 2 * sr, sr, 2 * sk, sk, 0, nullptr};

@@ -30,6 +30,18 @@ __device__ __forceinline__ int exp_field(double x) {
   return max(1, (int)((__double_as_longlong(x) >> 52) & 0x7ff));
 }
 
+static __device__ __noinline__ double times_pow2_slow(double x, int e) {
+  const int a = e >> 1, b = e - a;  // (|e| <= 2044)
+  return x * __hiloint2double((1023 + a) << 20, 0) * __hiloint2double((1023 + b) << 20, 0);
+}
+// x 2^e: on the integer pipe while x and the result are normal (a float64 multiplication takes the SM's pipe 16 clocks
+// a warp), |e| <= 2044.
+__device__ __forceinline__ double times_pow2(double x, int e) {
+  const int hi = __double2hiint(x), t = (hi >> 20) & 0x7ff;
+  if (e == 0 || ((hi & 0x7fffffff) | __double2loint(x)) == 0) return x;
+  if (t != 0 && t != 0x7ff && (unsigned)(t + e - 1) < 2046u) return __hiloint2double(hi + (e << 20), __double2loint(x));
+  return times_pow2_slow(x, e);
+}
 // Digits of the eight values x(0 .. 7) of one row, whose largest magnitude has exponent field em: q = x 2^(62 - e)
 // rounded to an integer, its balanced base-256 digits as float16, digit s as 16 bytes at d + s step.  em ==
 // kNonFinite: zeros (such rows are summed without digits).

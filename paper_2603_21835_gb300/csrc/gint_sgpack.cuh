@@ -15,14 +15,14 @@ __device__ __forceinline__ double sg_at(const SgView &v, int r, int k) {
   double x = v.p[(long long)(r >> 1) * v.rh + (long long)(r & 1) * v.rl + (long long)(k >> 1) * v.kh +
                  (long long)(k & 1) * v.kl];
   if (v.ks) {
-    double s = v.ks[k >> v.ksh];
+    double s = v.ks[k >> 1];
     if (v.half) {
       const int e = (__double2hiint(s) >> 20) & 0x7ff, h = e == 0 || e == 0x7ff ? 0 : (e - 1023) >> 1;
       s = v.half == 1 ? s * __hiloint2double((1023 - h) << 20, 0) : __hiloint2double((1023 + h) << 20, 0);
     }
     x *= s;
   }
-  if (v.rs) x *= v.rs[r];
+  if (v.kp) x = times_pow2(x, v.kp[k] + (v.rp ? v.rp[r] : 0));
   return x;
 }
 
