@@ -47,7 +47,7 @@ void dfree(T *&p) {
 }
 
 void free_all(gint_handle *h) {
-  dfree(h->tab64); dfree(h->otab64); dfree(h->tab32); dfree(h->tab32i); dfree(h->dtab32); dfree(h->dtab32i);
+  dfree(h->tab64); dfree(h->otab64); dfree(h->otab64q); dfree(h->tab32); dfree(h->tab32i); dfree(h->dtab32); dfree(h->dtab32i);
   dfree(h->pos_dev); dfree(h->species_dev);
   dfree(h->pair_row_dev); dfree(h->pair_col_dev); dfree(h->pair_off_dev); dfree(h->pair_T_dev); dfree(h->pair_I_dev);
   dfree(h->n_at); dfree(h->n_ent); dfree(h->n_orb); dfree(h->frac_dev); dfree(h->b_list);
@@ -318,7 +318,7 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
   // the Y_lm constant of the shell
   {
     h->tabs64 = g;
-    std::vector<double> o;
+    std::vector<double> o, oq;
     const double cl[3] = {0.28209479177387814347, 0.48860251190291992159, 1.09254843059207907054};
     for (int s = 0; s < d->nspecies; ++s) {
       GSpecies &S = h->tabs64.sp[s];
@@ -331,6 +331,14 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
         break;
         default: S.shape = 0; continue;
       }
+      int q[16];
+      for (int k = 0, i = 0; k < S.nrad; ++k) {
+        const GRadial &R = g.rad[S.rad0 + k];
+        double m = 0.0;
+        for (int t = 0; t < R.npts; ++t) m = std::max(m, std::fabs(t64[R.off + t].x));
+        q[k] = m > 0.0 && std::isfinite(m) ? std::min(std::max(std::ilogb(m), -60), 60) : 0;
+        for (int e = 0; e < 2 * R.l + 1; ++e) h->fx_q[s][i++] = (signed char)q[k];
+      }
       for (int k = 0; k < S.nrad; ++k)
         if (g.rad[S.rad0 + k].rc != S.rcut) S.kslot = 1;
       for (int i = 0; i + 1 < g.rad[S.rad0].npts; ++i)
@@ -339,12 +347,19 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
           const double2 *T = t64.data() + R.off + i;
           const double c = cl[R.l];
           const double df = T[1].x - T[0].x, m0 = R.dr * T[0].y, m1 = R.dr * T[1].y;
-          for (double x : {T[0].x, m0, 3.0 * df - (2.0 * m0 + m1), (m0 + m1) - 2.0 * df}) o.push_back(c * x);
+          for (double x : {T[0].x, m0, 3.0 * df - (2.0 * m0 + m1), (m0 + m1) - 2.0 * df}) {
+            o.push_back(c * x);
+            oq.push_back(std::ldexp(c * x, -q[k]));
+          }
         }
     }
     h->notab64 = (long long)o.size();
     TRY(dalloc(&h->otab64, o.size()));
-    if (!o.empty()) TRYCU(cudaMemcpy(h->otab64, o.data(), o.size() * sizeof(double), cudaMemcpyHostToDevice));
+    TRY(dalloc(&h->otab64q, o.size()));
+    if (!o.empty()) {
+      TRYCU(cudaMemcpy(h->otab64, o.data(), o.size() * sizeof(double), cudaMemcpyHostToDevice));
+      TRYCU(cudaMemcpy(h->otab64q, oq.data(), o.size() * sizeof(double), cudaMemcpyHostToDevice));
+    }
   }
   // atoms
   h->pos_host.assign(d->pos, d->pos + 3 * (size_t)d->natoms);
@@ -358,7 +373,7 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
   }
   h->norb = h->atom_off[d->natoms];
   TRY(dalloc(&h->atom_off_dev, (size_t)d->natoms + 1));
-  TRY(dalloc(&h->fx_eD, (size_t)h->norb));
+  TRY(dalloc(&h->fx_eD, 2 * (size_t)h->norb));
   TRYCU(cudaMemcpy(h->atom_off_dev, h->atom_off.data(), (d->natoms + 1) * sizeof(int), cudaMemcpyHostToDevice));
   TRY(dalloc(&h->pos_dev, 3 * (size_t)d->natoms));
   TRY(dalloc(&h->species_dev, (size_t)d->natoms));
@@ -540,8 +555,8 @@ int gint_memory(const gint_handle *h, long long *device_bytes) {
   if (!h || !device_bytes) return GINT_EINVAL;
   const long long nb = h->geom.nbricks, na = h->geom.natoms, np = h->npairs, L = sizeof(long long);
   long long b = h->nknots * (long long)(sizeof(double2) + sizeof(float2) + sizeof(float)) + h->nknots_i * 12 +
-                h->notab64 * (long long)sizeof(double);  // tables
-  b += na * (3 * (long long)sizeof(double) + 4) + (na + 1 + h->norb) * 4;                    // atoms
+                2 * h->notab64 * (long long)sizeof(double);  // tables
+  b += na * (3 * (long long)sizeof(double) + 4) + (na + 1 + 2 * h->norb) * 4;                // atoms
   b += (na + 1) * 4 + np * 4 + (np + 1) * L + 2 * np * 4;                                  // pair set
   b += nb * (3 * 4 + kNbrListBytes) + (nb + 1) * 3 * L + 8 * L + na * 3 * 4;                // brick counts and lists
   b += h->cap_slots * 8 + (h->cap_slots + 1) * L + h->cap_ent * 3 * (long long)sizeof(double) +

@@ -9,7 +9,8 @@
 // 36 us, k_fx_grad 76 us.  Errors against extended precision on that system (Frobenius norm, mean of five geometries),
 // CUDA cores -> here: rho 6.9e-16 -> 6.1e-16, H 1.7e-15 -> 9.1e-16, F 2.0e-15 -> 1.9e-15.
 //
-//   k_fx_dmax, k_fx_ddigits   D rows' exponents and digits, per pair in 8 x 8 core matrices
+//   k_fx_dmax, k_fx_ddigits   D rows' exponents and digits, per pair in 8 x 8 core matrices (a row on one scale in
+//               all its pairs: a brick without the pair that sets it may have far less of it, see kMaxGap)
 //   k_fx_eval   one CTA per brick: orbitals (float64) and their digits into scratch
 //     density: rows = points (scale: the point's largest orbital), contraction = orbitals
 //     local H: rows = orbitals (scale: the orbital's largest value in the brick, with and without w V),
@@ -26,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "gint_handle.cuh"
 #include "gint_ptx.cuh"
@@ -65,20 +67,36 @@ __host__ __device__ inline FxLayout fx_layout(int np) {
 
 enum { kRho = 0, kY = 1, kH = 2 };
 
+// An orbital's digits are relative to the largest at the point, D's to its row's largest: orbitals of very different
+// size (unnormalised bases) would run against each other in the two operands of Y = D P.  Density and forces therefore
+// work with P 2^-q (tables that carry the factor) and D 2^q under the contraction index, 2^q the power of two next to
+// the orbital's largest radial value: nothing is rounded, and results do not depend on such a scaling of the basis.
+struct FxScale {
+  signed char q[GINT_MAX_SPECIES][GINT_MAX_ORB_ATOM];  // 0: species without a compiled shape
+};
+// Columns whose row of D reaches more than 2^kMaxGap beyond what the brick has of it are summed in float64 (digits
+// keep 2^-58 of the row's maximum per term, a float64 chain 2^-53 of its own terms).
+constexpr int kMaxGap = 4;
+constexpr int kLookGap = 1 << 16;                                    // in the second half of eD
+constexpr int kPlain = 1 << 20, kPlainInf = kPlain, kPlainGap = kPlain + 1;  // in FxShared::eB
+
 struct FxArgs {
   GCell c;
   GNbr nb;
-  const double *otab;        // tables of orbitals64
+  const double *otab, *otabq;  // tables of orbitals64, and times 2^-q
   const double2 *tab;        // radial tables (general evaluator)
   const double *D, *V;
   double *rho, *F, *H;
   const unsigned char *Dd;   // D digits
-  const int *eD, *atom_off;  // exponents of D's rows by orbital; first orbital of each atom
+  const int *eD, *atom_off;  // exponents of D's rows by orbital, then those with kLookGap; first orbital of each atom
+  int norb;
   const long long *tile_off;
   unsigned char *scr;
   FxLayout L;
   unsigned *err;
   long long b0;              // first brick of the launch
+  FxScale q;
+  bool upper;                // the density alone reads the pairs I <= J
 };
 
 // ------------------------------------------------------------------------------------------- D digits
@@ -89,7 +107,8 @@ struct FxD {
   const int *atom_off;
   int *eD;
   unsigned char *Dd;
-  int npairs;
+  int npairs, norb;
+  FxScale q;
   bool upper;  // the density alone reads the pairs I <= J (the others are their transposes), as every precision does
 };
 // Element (i, j) of pair p at D[ri i + rj j].
@@ -107,8 +126,10 @@ __global__ void __launch_bounds__(256) k_fx_dmax(const __grid_constant__ GTabs g
   if (i >= nI) return;
   int ri, rj, m = 1;
   const double *D = d_block(P, p, nI, nJ, ri, rj);
-  for (int j = 0; j < nJ; ++j) m = max(m, exp_field(D[i * ri + j * rj]));
+  const signed char *q = P.q.q[P.species[J]];
+  for (int j = 0; j < nJ; ++j) m = max(m, exp_field(times_pow2(D[i * ri + j * rj], q[j])));
   atomicMax(P.eD + P.atom_off[I] + i, m);
+  if (I == J) P.eD[P.norb + P.atom_off[I] + i] = m;
 }
 // One warp per pair, units of (row, 8 columns); core matrix (row group, column group): 1 KB, digit s at 128 s.
 __global__ void __launch_bounds__(256) k_fx_ddigits(const __grid_constant__ GTabs g, FxD P) {
@@ -117,14 +138,19 @@ __global__ void __launch_bounds__(256) k_fx_ddigits(const __grid_constant__ GTab
   const int I = P.pair_I[p], J = P.pair_J[p];
   const GSpecies &SI = g.sp[P.species[I]], &SJ = g.sp[P.species[J]];
   const int nI = SI.norb, nJ = SJ.norb, gJ = SJ.porb >> 3;
+  const signed char *q = P.q.q[P.species[J]];
   int ri, rj;
   const double *D = d_block(P, p, nI, nJ, ri, rj);
   unsigned char *dst = P.Dd + P.tile_off[p] * 16;
+  if (I == J && lane < nI) {  // (rows whose maximum lies far above the own block's: k_fx_mma looks at the brick's part)
+    const int o = P.atom_off[I] + lane, e = P.eD[o];
+    P.eD[P.norb + o] = e < kNonFinite && e - P.eD[P.norb + o] > kMaxGap ? e | kLookGap : e;
+  }
   for (int u = lane; u < SI.porb * gJ; u += 32) {
     const int i = u / gJ, kg = u - i * gJ;
     const int em = i < nI ? P.eD[P.atom_off[I] + i] : 1;
-    store_digits([&](int j) { return i < nI && 8 * kg + j < nJ ? D[i * ri + (8 * kg + j) * rj] : 0.0; }, em,
-                 dst + (size_t)((i >> 3) * gJ + kg) * 1024 + (i & 7) * 16, 128);
+    store_digits([&](int j) { return i < nI && 8 * kg + j < nJ ? times_pow2(D[i * ri + (8 * kg + j) * rj], q[8 * kg + j]) : 0.0; },
+                 em, dst + (size_t)((i >> 3) * gJ + kg) * 1024 + (i & 7) * 16, 128);
   }
 }
 
@@ -192,7 +218,7 @@ __device__ __forceinline__ void fx_position(const FxArgs &P, const double *fr, i
 // ----------------------------------------------------------------------------------------- evaluation
 // Orbitals of slot a at the thread's point into column-major P64 (rows 0 .. porb, padding zero); returns the
 // largest exponent field.
-template <int NS, int NP, int ND, int NO>
+template <int NS, int NP, int ND, int NO, bool RHO>
 __device__ __forceinline__ int eval_slot(const GTabs &g, const FxArgs &P, const Slots &S, int a, const double r[3], bool valid,
                                          double *out) {
   const GSpecies &G = g.sp[S.sp[a]];
@@ -205,7 +231,7 @@ __device__ __forceinline__ int eval_slot(const GTabs &g, const FxArgs &P, const 
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
       if (r2 < G.rcut2) {
         if constexpr (NS + NP + ND > 0)
-          orbitals64<NS, NP, ND>(g, P.otab, G, dx, dy, dz, r2, v);
+          orbitals64<NS, NP, ND>(g, RHO ? P.otabq : P.otab, G, dx, dy, dz, r2, v);
         else
           add_orbitals<double, true, false>(g, P.tab, S.sp[a], dx, dy, dz, v, nullptr);
       }
@@ -250,10 +276,10 @@ __global__ void __launch_bounds__(kEvalT) k_fx_eval(const __grid_constant__ GTab
     double *out = P64 + (long long)S.col[a] * 128 + p;
     switch (g.sp[S.sp[a]].shape) {
 #define CASE_E(ns, np_, nd, no) \
-  case GINT_SHAPE(ns, np_, nd): em = max(em, eval_slot<ns, np_, nd, no>(g, P, S, a, r, valid, out)); break;
+  case GINT_SHAPE(ns, np_, nd): em = max(em, eval_slot<ns, np_, nd, no, RHO>(g, P, S, a, r, valid, out)); break;
       GINT_O64_SHAPES(CASE_E)
 #undef CASE_E
-      default: em = max(em, eval_slot<0, 0, 0, GINT_MAX_ORB_ATOM>(g, P, S, a, r, valid, out));
+      default: em = max(em, eval_slot<0, 0, 0, GINT_MAX_ORB_ATOM, RHO>(g, P, S, a, r, valid, out));
     }
   }
   const int n16 = (np + 15) & ~15;
@@ -316,6 +342,26 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool in) 
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
 
+// Element (i, j) of slots (a, c)' block at D[ri i + rj j]; null: no pair.
+__device__ __forceinline__ const double *slot_block(const GTabs &g, const FxArgs &P, const Slots &S, long long b, int a, int c,
+                                                    int &ri, int &rj) {
+  const bool t = P.upper && S.atom[a] > S.atom[c];
+  const int pr = P.nb.b_pair[P.nb.b_pair_off[b] + (t ? c * S.na + a : a * S.na + c)];
+  ri = t ? 1 : g.sp[S.sp[c]].norb;
+  rj = t ? g.sp[S.sp[a]].norb : 1;
+  return pr < 0 ? nullptr : P.D + P.nb.pair_off[pr];
+}
+// Largest exponent of D 2^q in the brick's part of row i of slot a's atom.
+__device__ __noinline__ int fx_brick_row(const GTabs &g, const FxArgs &P, const Slots &S, long long b, int a, int i) {
+  int m = 1;
+  for (int c = 0; c < S.na; ++c) {
+    int ri, rj;
+    const double *D = slot_block(g, P, S, b, a, c, ri, rj);
+    if (!D) continue;
+    for (int j = 0; j < g.sp[S.sp[c]].norb; ++j) m = max(m, exp_field(times_pow2(D[i * ri + j * rj], P.q.q[S.sp[c]][j])));
+  }
+  return m;
+}
 // Sums without digits, where a row holds an infinity or a NaN: over the atoms that reach one of the point's 32
 // (the CUDA-core path's slabs, whose rule decides which results a non-finite input reaches).
 __device__ __forceinline__ bool fx_reaches(const GTabs &g, const Slots &S, const double *P64, int a, int slab) {
@@ -328,12 +374,15 @@ __device__ __forceinline__ bool fx_reaches(const GTabs &g, const Slots &S, const
 __device__ __noinline__ double fx_plain_y(const GTabs &g, const FxArgs &P, const FxShared &sh, long long b, const double *P64,
                                           int n, int p) {
   const int na = sh.S.na, c = sh.grp_slot[n >> 3], i = sh.col_orb[n];
+  const bool finite = sh.eB[n] == kPlainGap;  // (an atom that does not reach adds zeros)
   double y = 0.0;
-  if (!fx_reaches(g, sh.S, P64, c, p >> 5)) return y;
+  if (!finite && !fx_reaches(g, sh.S, P64, c, p >> 5)) return y;
   for (int a = 0; a < na; ++a) {
-    const int pr = P.nb.b_pair[P.nb.b_pair_off[b] + c * na + a], no = g.sp[sh.S.sp[a]].norb;
-    if (pr < 0 || !fx_reaches(g, sh.S, P64, a, p >> 5)) continue;
-    for (int j = 0; j < no; ++j) y = fma(P.D[P.nb.pair_off[pr] + (long long)i * no + j], P64[(sh.S.col[a] + j) * 128 + p], y);
+    int ri, rj;
+    const double *D = slot_block(g, P, sh.S, b, c, a, ri, rj);
+    if (!D || (!finite && !fx_reaches(g, sh.S, P64, a, p >> 5))) continue;
+    for (int j = 0; j < g.sp[sh.S.sp[a]].norb; ++j)
+      y = fma(D[i * ri + j * rj], times_pow2(P64[(sh.S.col[a] + j) * 128 + p], P.q.q[sh.S.sp[a]][j]), y);
   }
   return y;
 }
@@ -383,7 +432,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_fx_mma(const __grid_constant_
     for (int k = 0; k < 8; ++k) {
       const int i = 8 * G + k - sh.S.col[a];
       sh.col_orb[8 * G + k] = (short)(i < no ? i : -1);
-      if (MODE != kH) sh.eB[8 * G + k] = i < no ? P.eD[P.atom_off[sh.S.atom[a]] + i] : 1;
     }
   }
   const int ng8 = np / 8;
@@ -401,6 +449,16 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_fx_mma(const __grid_constant_
   __syncthreads();
   tc_fence_after();
   if (MODE != kH) {
+    // the row's exponent (density: that of Y 2^q, to meet P 2^-q), or why the column is summed in float64: an infinity or
+    // a NaN, or the brick's part of the row too far below its maximum (looked at only where the own atom's block, which
+    // every brick of the atom has, is)
+    for (int c = tid; c < np; c += kFxThreads) {
+      const int a = sh.grp_slot[c >> 3], i = sh.col_orb[c];
+      int e = i < 0 ? 1 : P.eD[P.norb + P.atom_off[sh.S.atom[a]] + i];
+      const bool gap = e >= kLookGap && e - kLookGap - fx_brick_row(g, P, sh.S, b, a, i) > kMaxGap;
+      e &= kLookGap - 1;
+      sh.eB[c] = gap ? kPlainGap : e == kNonFinite ? kPlainInf : MODE == kRho && i >= 0 ? e + P.q.q[sh.S.sp[a]][i] : e;
+    }
     for (int e = tid; e < ng8 * ng8; e += kFxThreads) {
       const int n = e / ng8, k = e - n * ng8, sn = sh.grp_slot[n], sk = sh.grp_slot[k];
       const int p = P.nb.b_pair[P.nb.b_pair_off[b] + sn * na + sk];
@@ -587,18 +645,18 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_fx_mma(const __grid_constant_
             const double v = fx_to_double(x[j8 + j], ea + eb - 2 * 1022 - 68);
             if (MODE == kY)
               Y[col * 128 + row] = v;
-            else if (eb != kNonFinite)
+            else if (eb < kPlain)
               racc = fma(pv[j], v, racc);
-            if (eb == kNonFinite) plain |= 1u << j;
+            if (eb >= kPlain) plain |= 1u << j;
           }
-          while (plain) {  // rows of D with an infinity or a NaN
+          while (plain) {
             const int col = jb + j8 + __ffs(plain) - 1;
             plain &= plain - 1;
             const double v = fx_plain_y(g, P, sh, b, P64, col, row);
             if (MODE == kY)
               Y[col * 128 + row] = v;
             else
-              racc = fma(P64[col * 128 + row], v, racc);
+              racc = fma(times_pow2(P64[col * 128 + row], P.q.q[sh.S.sp[sh.grp_slot[col >> 3]]][sh.col_orb[col]]), v, racc);
           }
         }
       }
@@ -707,12 +765,16 @@ int fx_args(gint_handle *h, FxArgs &P) {
   P.c = static_cast<const GCell &>(h->geom);
   P.nb = h->nbr();
   P.otab = h->otab64;
+  P.otabq = h->otab64q;
   P.tab = h->tab64;
   P.tile_off = h->tile_off_dev;
   unsigned char *s = reinterpret_cast<unsigned char *>(h->hs);
   P.Dd = s;
   P.scr = s + fx_dbytes(h);
   P.eD = h->fx_eD;
+  P.norb = h->norb;
+  static_assert(sizeof(P.q.q) == sizeof(h->fx_q), "");
+  memcpy(P.q.q, h->fx_q, sizeof(P.q.q));
   P.atom_off = h->atom_off_dev;
   P.L = fx_layout(h->max_brick_porb);
   P.err = h->err_word;
@@ -742,9 +804,10 @@ int gint_fx_rho(gint_handle *h, const double *D, double *rho, const double *V, d
   P.V = V;
   P.rho = rho;
   P.F = F;
+  P.upper = F == nullptr;
   FxD Q{D, h->pair_I_dev, h->pair_col_dev, h->pair_T_dev, h->species_dev, h->pair_off_dev, h->tile_off_dev, h->atom_off_dev,
-        h->fx_eD, const_cast<unsigned char *>(P.Dd), h->npairs, F == nullptr};
-  if (cudaMemsetAsync(h->fx_eD, 0, h->norb * sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
+        h->fx_eD, const_cast<unsigned char *>(P.Dd), h->npairs, h->norb, P.q, F == nullptr};
+  if (cudaMemsetAsync(h->fx_eD, 0, 2 * (size_t)h->norb * sizeof(int), st) != cudaSuccess) return GINT_ECUDA;
   const unsigned pg = (unsigned)((h->npairs + 7) / 8);
   k_fx_dmax<<<pg, 256, 0, st>>>(h->tabs64, Q);
   k_fx_ddigits<<<pg, 256, 0, st>>>(h->tabs64, Q);

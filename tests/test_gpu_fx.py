@@ -177,3 +177,69 @@ def test_no_support_where_r_rounds_up_to_the_radius(rc, dr):
     assert np.abs(H - o.vlocal(V).reshape(-1)).max() <= 1e-12 * np.abs(o.vlocal(V)).max()
     assert np.abs(F - o.force(D, V)).max() <= 1e-11
     g.close()
+
+
+def test_density_does_not_depend_on_the_scale_of_the_radials():
+    """Radials times powers of two, D divided by them: the same density bit for bit, alone and in the force pass."""
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    power = [-20, 13, 5, -30, -9]
+    names, nat, box, grid = ("221",), 9, 12.0, (8, 8, 16)
+    s = _system(names, nat, box, grid)
+    t = _system(names, nat, box, grid)
+    for r, a in zip(t.sp[0].radials, power):
+        r.f *= 2.0**a
+        r.df *= 2.0**a
+    c = np.tile(2.0 ** np.repeat(power, [2 * r.l + 1 for r in s.sp[0].radials]), nat)
+    rng = np.random.default_rng(4)
+    C = rng.normal(size=(len(c), 5)) / 4
+    D, V = C @ C.T, rng.normal(size=int(np.prod(grid)))
+    out = []
+    for sys_, D_ in ((s, D), (t, D / c[:, None] / c)):
+        g = G.Gint(sys_)
+        Db, Vd = torch.from_numpy(g.dense_to_blocks(D_)).cuda(), torch.from_numpy(V).cuda()
+        rho_f = torch.empty(V.size, dtype=torch.float64, device="cuda")
+        g.force(Db, Vd, G.FP64, rho_out=rho_f)
+        out.append((g.rho(Db, G.FP64).cpu().numpy().reshape(-1), rho_f.cpu().numpy()))
+        g.sync()
+        g.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+def test_a_large_block_elsewhere_costs_a_brick_no_bits():
+    """Atoms 0 and 1 share a block of D 2^40 above the rest: in bricks (4 x 4 x 8 points) that atom 1 does not reach, the
+    density and the forces' density are those of a float64 chain, although the rows of atom 0 hold that block too."""
+    import torch
+
+    from paper_2603_21835_gb300 import gint as G
+
+    L, grid = 30.0, (16, 16, 16)
+    sp = [_sp("a", ORB["221"])]
+    s = inputs.System(cell=np.diag([L] * 3), pos=np.array([[10.1, 15.2, 14.9], [18.3, 15.1, 15.2], [11.9, 13.0, 15.0]]),
+                      species=np.zeros(3, np.int32), sp=sp, grid=grid)
+    o = Oracle(s)
+    rng = np.random.default_rng(8)
+    D = rng.normal(size=(o.norb, o.norb))
+    D = D + D.T
+    D[:13, 13:26] *= 2.0**40
+    D[13:26, :13] *= 2.0**40
+    x = [np.arange(n) / n * L for n in grid]
+    pts = np.stack(np.meshgrid(*x, indexing="ij"), -1).reshape(-1, 3)
+    near = (np.linalg.norm(pts - s.pos[1], axis=1) < 6.0).reshape(4, 4, 4, 4, 2, 8)
+    far = np.broadcast_to(~near.any(axis=(1, 3, 5), keepdims=True), near.shape).reshape(-1)
+    ref = o.rho(D).reshape(-1)
+    g = G.Gint(s)
+    Db, Vd = torch.from_numpy(g.dense_to_blocks(D)).cuda(), torch.ones(ref.size, dtype=torch.float64, device="cuda")
+    rho_f = torch.empty_like(Vd)
+    F = g.force(Db, Vd, G.FP64, rho_out=rho_f).cpu().numpy()
+    rho = g.rho(Db, G.FP64).cpu().numpy().reshape(-1)
+    g.sync()
+    # the tolerance of the float64 path on either set of points
+    for got in (rho, rho_f.cpu().numpy()):
+        assert np.abs(got - ref)[far].max() <= 1e-12 * np.abs(ref[far]).max()
+        assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
+    Fo = o.force(D, np.ones(ref.size))
+    assert np.abs(F - Fo).max() <= 1e-11 * np.abs(Fo).max()
+    g.close()
