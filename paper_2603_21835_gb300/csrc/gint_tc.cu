@@ -1609,11 +1609,12 @@ constexpr int kRedLanes = 64, kRedGroups = 4, kRedThreads = kRedLanes * kRedGrou
 __device__ __forceinline__ void bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-// Upper pair u of system S by NG groups of kRedLanes threads (tid in [0, NG kRedLanes)); part_hi and
-// part_lo hold (NG - 1) kRedE kRedLanes floats each; the groups synchronise on barrier `bar`.
+// Upper pair u of system S in NP parts by NG groups of kRedLanes threads (tid in [0, NG kRedLanes)), NP / NG parts each;
+// part_hi and part_lo hold (NP - 1) kRedE kRedLanes floats each; the groups synchronise on barrier `bar`.  The result
+// depends on NP, not on NG.
 // F64: every tile value converted and added in float64 (a part's float64 sum travels between the
 // groups as the two 32-bit halves of its bits in part_lo / part_hi), the same parts and order.
-template <int NG, bool F64, bool PF>
+template <int NP, int NG, bool F64, bool PF>
 __device__ __forceinline__ void reduce_pair_t(const GTabs &g, const GRedSys &S, int u, int tid, float *part_hi,
                                               float *part_lo, int bar) {
   const int p = S.hu_pair[u];
@@ -1621,8 +1622,7 @@ __device__ __forceinline__ void reduce_pair_t(const GTabs &g, const GRedSys &S, 
   const int nI = g.sp[S.species[I]].norb, nJ = g.sp[S.species[J]].norb;
   const int ln = tid % kRedLanes, grp = tid / kRedLanes;
   const long long kk0 = S.hu_off[u], kk1 = S.hu_off[u + 1];
-  const long long per = (kk1 - kk0 + NG - 1) / NG;
-  const long long k0 = min(kk1, kk0 + grp * per), k1 = min(kk1, k0 + per);
+  const long long per = (kk1 - kk0 + NP - 1) / NP;
   const float *__restrict__ hs = S.hs;
   const long long *__restrict__ src = S.hu_src;
   const int ne = nI * nJ;
@@ -1636,70 +1636,77 @@ __device__ __forceinline__ void reduce_pair_t(const GTabs &g, const GRedSys &S, 
       e[q] = base + q * kRedLanes + ln;
       act[q] = e[q] < ne;
       if (!act[q]) e[q] = 0;  // a valid address; its loads are discarded
-      ah[q] = al[q] = 0.f;
-      ad[q] = 0.0;
     }
-    auto add = [&](int q, float x) {
-      if (F64) {
-        ad[q] += (double)x;
-      } else {
-        float sum, err;
-        two_sum(ah[q], x, sum, err);
-        ah[q] = sum;
-        al[q] += err;
-      }
-    };
-    long long k = k0;
-    // PF: the next batch's tile offsets are loaded while the current batch's values are summed, so
-    // the offset and value loads of a batch are not two round trips in a row (the standalone
-    // reduction; the resident kernel keeps the lighter loop, its registers being spoken for)
-    long long o[kRedB];
-    if (PF && k + kRedB <= k1) {
+#pragma unroll 1
+    for (int part = (grp + 1) * (NP / NG) - 1; part >= grp * (NP / NG); --part) {  // (part 0 last: it stays in registers)
+      const long long k0 = min(kk1, kk0 + part * per), k1 = min(kk1, k0 + per);
 #pragma unroll
-      for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + k + jj);
-    }
-    for (; k + kRedB <= k1; k += kRedB) {
-      if (!PF) {
+      for (int q = 0; q < kRedE; ++q) {
+        ah[q] = al[q] = 0.f;
+        ad[q] = 0.0;
+      }
+      auto add = [&](int q, float x) {
+        if (F64) {
+          ad[q] += (double)x;
+        } else {
+          float sum, err;
+          two_sum(ah[q], x, sum, err);
+          ah[q] = sum;
+          al[q] += err;
+        }
+      };
+      long long k = k0;
+      // PF: the next batch's tile offsets are loaded while the current batch's values are summed, so
+      // the offset and value loads of a batch are not two round trips in a row (the standalone
+      // reduction; the resident kernel keeps the lighter loop, its registers being spoken for)
+      long long o[kRedB];
+      if (PF && k + kRedB <= k1) {
 #pragma unroll
         for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + k + jj);
       }
-      float v[kRedB][kRedE];
+      for (; k + kRedB <= k1; k += kRedB) {
+        if (!PF) {
 #pragma unroll
-      for (int jj = 0; jj < kRedB; ++jj)
+          for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + k + jj);
+        }
+        float v[kRedB][kRedE];
 #pragma unroll
-        for (int q = 0; q < kRedE; ++q) v[jj][q] = __ldcg(hs + o[jj] + e[q]);  // written by this or another launch
-      if (PF && k + 2 * kRedB <= k1) {
+        for (int jj = 0; jj < kRedB; ++jj)
 #pragma unroll
-        for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + k + kRedB + jj);
+          for (int q = 0; q < kRedE; ++q) v[jj][q] = __ldcg(hs + o[jj] + e[q]);  // written by this or another launch
+        if (PF && k + 2 * kRedB <= k1) {
+#pragma unroll
+          for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + k + kRedB + jj);
+        }
+#pragma unroll
+        for (int jj = 0; jj < kRedB; ++jj)
+#pragma unroll
+          for (int q = 0; q < kRedE; ++q) add(q, v[jj][q]);
       }
+      if (k < k1) {  // the last, partial batch: absent bricks re-read its first and add zero (exact)
 #pragma unroll
-      for (int jj = 0; jj < kRedB; ++jj)
+        for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + (k + jj < k1 ? k + jj : k));
+        float v[kRedB][kRedE];
 #pragma unroll
-        for (int q = 0; q < kRedE; ++q) add(q, v[jj][q]);
-    }
-    if (k < k1) {  // the last, partial batch: absent bricks re-read its first and add zero (exact)
+        for (int jj = 0; jj < kRedB; ++jj)
 #pragma unroll
-      for (int jj = 0; jj < kRedB; ++jj) o[jj] = __ldg(src + (k + jj < k1 ? k + jj : k));
-      float v[kRedB][kRedE];
+          for (int q = 0; q < kRedE; ++q) v[jj][q] = __ldcg(hs + o[jj] + e[q]);
 #pragma unroll
-      for (int jj = 0; jj < kRedB; ++jj)
+        for (int jj = 0; jj < kRedB; ++jj)
 #pragma unroll
-        for (int q = 0; q < kRedE; ++q) v[jj][q] = __ldcg(hs + o[jj] + e[q]);
+          for (int q = 0; q < kRedE; ++q) add(q, k + jj < k1 ? v[jj][q] : 0.f);
+      }
+      if (part > 0) {
 #pragma unroll
-      for (int jj = 0; jj < kRedB; ++jj)
-#pragma unroll
-        for (int q = 0; q < kRedE; ++q) add(q, k + jj < k1 ? v[jj][q] : 0.f);
-    }
-    if (grp > 0) {
-#pragma unroll
-      for (int q = 0; q < kRedE; ++q) {
-        const int w = ((grp - 1) * kRedE + q) * kRedLanes + ln;
-        if (F64) {
-          part_hi[w] = __int_as_float(__double2hiint(ad[q]));
-          part_lo[w] = __int_as_float(__double2loint(ad[q]));
-        } else {
-          part_hi[w] = ah[q];
-          part_lo[w] = al[q];
+        for (int q = 0; q < kRedE; ++q) {
+          const int w = ((part - 1) * kRedE + q) * kRedLanes + ln;
+          if (F64) {
+            part_hi[w] = __int_as_float(__double2hiint(ad[q]));
+            part_lo[w] = __int_as_float(__double2loint(ad[q]));
+          } else {
+            part_hi[w] = ah[q];
+            part_lo[w] = al[q];
+          }
         }
       }
     }
@@ -1709,7 +1716,7 @@ __device__ __forceinline__ void reduce_pair_t(const GTabs &g, const GRedSys &S, 
       for (int q = 0; q < kRedE; ++q) {
         if (!act[q]) continue;
         double acc = F64 ? ad[q] : (double)ah[q] + (double)al[q];
-        for (int g2 = 0; g2 < NG - 1; ++g2) {
+        for (int g2 = 0; g2 < NP - 1; ++g2) {
           const int w = (g2 * kRedE + q) * kRedLanes + ln;
           acc += F64 ? __hiloint2double(__float_as_int(part_hi[w]), __float_as_int(part_lo[w]))
                      : (double)part_hi[w] + (double)part_lo[w];
@@ -1723,22 +1730,22 @@ __device__ __forceinline__ void reduce_pair_t(const GTabs &g, const GRedSys &S, 
   }
 }
 
-template <int NG, bool PF = false>
+template <int NP, int NG, bool PF = false>
 __device__ __forceinline__ void reduce_pair(const GTabs &g, const GRedSys &S, int u, int tid, float *part_hi,
                                             float *part_lo, int bar) {
   if (S.fp64)
-    reduce_pair_t<NG, true, PF>(g, S, u, tid, part_hi, part_lo, bar);
+    reduce_pair_t<NP, NG, true, PF>(g, S, u, tid, part_hi, part_lo, bar);
   else
-    reduce_pair_t<NG, false, PF>(g, S, u, tid, part_hi, part_lo, bar);
+    reduce_pair_t<NP, NG, false, PF>(g, S, u, tid, part_hi, part_lo, bar);
 }
 
-// A system with at most kRedFewPairs upper pairs has them summed in kRedGroupsFew parts, others in kRedGroups: a
+// A system with no more upper pairs than the GPU has SMs has them summed in kRedGroupsFew parts, others in kRedGroups: a
 // part's list is walked in batches of dependent loads, so in a launch of few pairs, which are those of small
 // cells and so have long lists, the length of a part sets the time (the 8-atom cell: 36 pairs of 864 bricks,
 // 42 us in 4 parts, 23.5 in 16).  Where the pairs fill the GPU the smaller CTAs are the faster (512-atom Si with its long
 // lists in 16 parts: 0.11 ms slower).  The rule looks at the system only, so its blocks do not depend on what
-// shares the launch.
-constexpr int kRedGroupsFew = 16, kRedFewPairs = 152;
+// shares the launch; a served job is summed in the same parts.
+constexpr int kRedGroupsFew = 16;
 template <int NG>
 __global__ void __launch_bounds__(NG * kRedLanes, 1024 / (NG * kRedLanes))
     k_h_reduce(const __grid_constant__ GTabs g, const __grid_constant__ GRed R) {
@@ -1752,7 +1759,7 @@ __global__ void __launch_bounds__(NG * kRedLanes, 1024 / (NG * kRedLanes))
     else
       hi = mid - 1;
   }
-  reduce_pair<NG, true>(g, R.sys[lo], (int)(gu - R.start[lo]), threadIdx.x, part_hi, part_lo, 0);
+  reduce_pair<NG, NG, true>(g, R.sys[lo], (int)(gu - R.start[lo]), threadIdx.x, part_hi, part_lo, 0);
 }
 
 // ------------------------------------------------------------------------------ batched preparation
@@ -2240,7 +2247,7 @@ struct GJob {
   GPrepSys prep;
   GTileSys tile;
   GRedSys red;
-  int npairs, nupper, fixed, pad;
+  int npairs, nupper, fixed, few;   // few: H reduction in kRedGroupsFew parts
   long long nbricks;
   long long n_prep, n_tile, n_red;  // items of each kind (plus one scales item)
   long long item0, nitems;          // first item and item count of the job
@@ -2518,7 +2525,7 @@ __global__ void __launch_bounds__(kT, 1)
         brick_body<FORCE, DZP>(g, S, b, do_rho, do_h, split3, dsmem, zero, tmem, sh, smem, cx);
         tc_fence_before();
       }
-    } else {  // H reduction: two upper pairs, one per 256 threads (named barriers 2, 3), in four parts
+    } else {  // H reduction: two upper pairs, one per 256 threads (named barriers 2, 3)
       bool go = true;
       if (t == 0 && ld_acquire_s32(&JS.bricks) < J.nbricks) {
         flush();
@@ -2527,10 +2534,12 @@ __global__ void __launch_bounds__(kT, 1)
       __syncthreads();
       if (go && !*(volatile unsigned *)err) {
         const int sg = t / kRedThreads, u = (int)((li - r0) * kServeRedPairs) + sg;
-        float *part = reinterpret_cast<float *>(smem) + sg * 2 * (kRedGroups - 1) * kRedE * kRedLanes;
-        if (u < J.nupper)
-          reduce_pair<kRedGroups>(g, J.red, u, t % kRedThreads, part, part + (kRedGroups - 1) * kRedE * kRedLanes,
-                                  2 + sg);
+        constexpr int kPart = (kRedGroupsFew - 1) * kRedE * kRedLanes;
+        float *part = reinterpret_cast<float *>(smem) + sg * 2 * kPart;
+        if (u < J.nupper && J.few)
+          reduce_pair<kRedGroupsFew, kRedGroups>(g, J.red, u, t % kRedThreads, part, part + kPart, 2 + sg);
+        else if (u < J.nupper)
+          reduce_pair<kRedGroups, kRedGroups>(g, J.red, u, t % kRedThreads, part, part + kPart, 2 + sg);
       }
     }
     if (!cx.ok) atomicOr(err, GINT_ERRBIT_TIMEOUT);  // the next claim sees it: every CTA leaves
@@ -3042,7 +3051,7 @@ static int run_group(const gint_task *tk, int n, int split3, cudaStream_t st, cu
       rs.species = h->species_dev;
       rs.H = T.H_blocks;
       rs.fp64 = h->reduce_fp64 ? 1 : 0;
-      const int nu = h->reduce_R ? h->r_nupper : h->nupper, k = nu <= kRedFewPairs ? 0 : 1;
+      const int nu = h->reduce_R ? h->r_nupper : h->nupper, k = nu <= h->num_sms ? 0 : 1;
       if (h->reduce_R) {  // the same tiles keyed by (I, J, R): H(R) blocks
         rs.hu_pair = h->r_hu_key;
         rs.hu_off = h->r_hu_off;
@@ -3299,6 +3308,7 @@ extern "C" int gint_server_submit(gint_server *v, const gint_task *T, void *stre
   if (loc) fill_red_gamma(J.red, *T);
   J.npairs = dens ? h->npairs : 0;
   J.nupper = loc ? h->nupper : 0;
+  J.few = h->nupper <= h->num_sms ? 1 : 0;
   J.fixed = (v->forces && v->split3) ? 1 : 0;
   J.nbricks = h->geom.nbricks;
   const long long span = std::max(std::max(h->nblock, h->geom.ngrid), 3LL * h->geom.natoms);

@@ -132,3 +132,24 @@ def test_idle_exit_relaunch_and_busy(mods):
     q.stop()
     q.close()
     c["g"].close()
+
+
+@pytest.mark.parametrize("mode", ["double-float", "fp64"])
+def test_served_blocks_are_summed_as_batched_ones(mods, mode):
+    """Pair sums of few long lists (16 parts) and of many (4): the served job's H against the batched call's, to the
+    float32 rounding of a few tile elements at most (see above) and mostly bit for bit, as the tiles and parts are the
+    same; other parts would leave almost no equal bits."""
+    torch, G = mods
+    lib = inputs.serving_library()
+    q = G.DeviceQueue(G.F16X3, forces=True, idle_s=0.2)
+    for cells, grid in (((1, 1, 1), (48, 48, 48)), ((2, 2, 2), (96, 96, 96))):
+        c = _case(G, torch, inputs.on_species(inputs.si_workload(cells, grid, seed=3, disp_sigma=0.05).system, lib), 11)
+        c["g"].set_reduction(mode)
+        _, H, _ = _reference(G, torch, c)
+        o = _outputs(torch, c)
+        _wait(q, [q.submit(G.Task(c["g"], c["D"], c["V"], rho=o[0], H=o[1], F=o[2]))])
+        Hq = o[1].cpu().numpy()
+        assert (H == Hq).mean() > 0.9, (cells, (H == Hq).mean())
+        assert np.abs(H - Hq).max() <= 1e-6 * np.abs(H).max()
+    q.stop()
+    q.close()
