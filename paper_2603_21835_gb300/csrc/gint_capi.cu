@@ -50,7 +50,7 @@ void free_all(gint_handle *h) {
   dfree(h->tab64); dfree(h->otab64); dfree(h->otab64q); dfree(h->tab32); dfree(h->tab32i); dfree(h->dtab32); dfree(h->dtab32i);
   dfree(h->pos_dev); dfree(h->species_dev);
   dfree(h->pair_row_dev); dfree(h->pair_col_dev); dfree(h->pair_off_dev); dfree(h->pair_T_dev); dfree(h->pair_I_dev);
-  dfree(h->n_at); dfree(h->n_ent); dfree(h->n_orb); dfree(h->frac_dev); dfree(h->b_list);
+  dfree(h->n_at); dfree(h->n_ent); dfree(h->n_orb); dfree(h->frac_dev);
   dfree(h->fx_eD); dfree(h->atom_off_dev);
   dfree(h->b_at_off); dfree(h->b_ent_off); dfree(h->b_pair_off); dfree(h->scan_out);
   dfree(h->s_atom); dfree(h->s_col); dfree(h->s_ent); dfree(h->e_shift); dfree(h->b_pair);
@@ -421,7 +421,7 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
   // neighbour structure
   const size_t nb = (size_t)g.nbricks;
   TRY(dalloc(&h->n_at, nb)); TRY(dalloc(&h->n_ent, nb)); TRY(dalloc(&h->n_orb, nb));
-  TRY(dalloc(&h->frac_dev, 3 * (size_t)d->natoms)); TRY(dalloc(&h->b_list, nb * (kNbrListBytes / sizeof(int4))));
+  TRY(dalloc(&h->frac_dev, 3 * (size_t)d->natoms));
   TRY(dalloc(&h->b_at_off, nb + 1)); TRY(dalloc(&h->b_ent_off, nb + 1)); TRY(dalloc(&h->b_pair_off, nb + 1));
   TRY(dalloc(&h->scan_out, 8));
   TRY(dalloc(&h->red, 1024));
@@ -558,7 +558,7 @@ int gint_memory(const gint_handle *h, long long *device_bytes) {
                 2 * h->notab64 * (long long)sizeof(double);  // tables
   b += na * (3 * (long long)sizeof(double) + 4) + (na + 1 + 2 * h->norb) * 4;                // atoms
   b += (na + 1) * 4 + np * 4 + (np + 1) * L + 2 * np * 4;                                  // pair set
-  b += nb * (3 * 4 + kNbrListBytes) + (nb + 1) * 3 * L + 8 * L + na * 3 * 4;                // brick counts and lists
+  b += nb * 3 * 4 + (nb + 1) * 3 * L + 8 * L + na * 3 * 4;                // brick counts and lists
   b += h->cap_slots * 8 + (h->cap_slots + 1) * L + h->cap_ent * 3 * (long long)sizeof(double) +
        h->cap_pairtab * 4;                                                                  // neighbours
   b += 1024 * (long long)sizeof(double) + 16 * (long long)sizeof(double) + 16 + h->nblock * 4 + 16;  // workspace

@@ -50,7 +50,6 @@ struct gint_handle {
   // neighbour structure
   int *n_at = nullptr, *n_ent = nullptr, *n_orb = nullptr;
   float *frac_dev = nullptr;  // fractional coordinates of the atoms (float32 screen of the neighbour kernels)
-  int4 *b_list = nullptr;     // first entries of each brick (counting pass -> filling pass)
   long long *b_at_off = nullptr, *b_ent_off = nullptr, *b_pair_off = nullptr;
   long long *scan_out = nullptr;
   int *s_atom = nullptr, *s_col = nullptr;
@@ -165,7 +164,7 @@ struct gint_handle {
 };
 
 // gint_nbr.cu
-constexpr long long kNbrListBytes = 64 * 16;  // of b_list per brick
+constexpr long long kNbrListBytes = 64 * 16;  // per brick: its first entries, counting pass -> filling pass (in hs)
 int gint_build_neighbours(gint_handle *h, cudaStream_t st);
 // gint_capi.cu
 int gint_reserve_nbr(gint_handle *h);
@@ -187,6 +186,7 @@ int gint_tc_vlocal(gint_handle *h, int precision, const double *V, double *H, cu
 int gint_tc_batch(const gint_task *tasks, int n, int precision, cudaStream_t st, cudaEvent_t ev0,
                   cudaEvent_t ev1);
 int gint_tc_check_capacity(const gint_handle *h);
+int gint_tc_reserve_hs(gint_handle *h, long long bytes);
 int gint_tc_prepare(gint_handle *h, cudaStream_t st);  // layouts and scratch of the tensor-core path (after neighbours)
 void gint_tc_free(gint_handle *h);
 // gint_hr.cu

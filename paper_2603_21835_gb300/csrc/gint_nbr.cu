@@ -612,9 +612,13 @@ int gint_build_neighbours(gint_handle *h, cudaStream_t st) {
   const long long nb = g.nbricks;
   const unsigned nblk = (unsigned)((nb + kNbrWarps - 1) / kNbrWarps);
   const GBrickGeo G = brick_geo(g);
+  // the lists lie in the tiles' scratch buffer, whose contents no call keeps (a buffer of their own was 1 KB a brick)
+  const int hrc = gint_tc_reserve_hs(h, nb * kNbrListBytes);
+  if (hrc) return hrc;
+  int4 *const b_list = reinterpret_cast<int4 *>(h->hs);
   k_frac<<<(unsigned)((g.natoms + 127) / 128), 128, 0, st>>>(g, h->pos_dev, h->frac_dev);
   k_brick_count<<<nblk, 32 * kNbrWarps, 0, st>>>(g, G, h->pos_dev, h->frac_dev, h->species_dev, h->unfold ? 1 : 0, h->n_at,
-                                                 h->n_ent, h->n_orb, h->b_list);
+                                                 h->n_ent, h->n_orb, b_list);
   NBR_CHECK(cudaGetLastError());
   k_brick_scan<<<1, 1024, 0, st>>>(nb, h->n_at, h->n_ent, h->n_orb, h->b_at_off, h->b_ent_off, h->b_pair_off,
                                    h->scan_out);
@@ -635,7 +639,7 @@ int gint_build_neighbours(gint_handle *h, cudaStream_t st) {
   if (rc) return rc;
   NBR_CHECK(cudaMemsetAsync(h->err_word, 0, sizeof(unsigned), st));
   k_brick_fill<<<nblk, 32 * kNbrWarps, 0, st>>>(g, G, h->pos_dev, h->frac_dev, h->species_dev, h->unfold ? 1 : 0, h->b_at_off,
-                                                h->b_ent_off, h->b_list, h->s_atom, h->s_col, h->s_ent, h->e_shift,
+                                                h->b_ent_off, b_list, h->s_atom, h->s_col, h->s_ent, h->e_shift,
                                                 h->err_word);
   NBR_CHECK(cudaGetLastError());
   // sentinel: s_ent[nslots] = nent

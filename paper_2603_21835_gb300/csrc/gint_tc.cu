@@ -2829,7 +2829,7 @@ static int tc_allocate(gint_handle *h) {
     cudaGetLastError();
     return GINT_ENOMEM;
   }
-  h->tc_bytes = 4 * (long long)tbytes + 512 + 8 * sizeof(float) + (long long)lay + 4 * sizeof(long long) +
+  h->tc_bytes += 4 * (long long)tbytes + 512 + 8 * sizeof(float) + (long long)lay + 4 * sizeof(long long) +
                 (h->npairs + 1 + 2 * h->nupper + 2 + 4 * nb + 2) * (long long)sizeof(long long) +
                 (h->nupper + h->npairs) * (long long)sizeof(int);
   TC_CHECK(cudaMemset(h->zero_dev, 0, 512));
@@ -2840,13 +2840,13 @@ static int tc_allocate(gint_handle *h) {
   return GINT_OK;
 }
 
-// A buffer of at least n elements of T: kept when it is large enough, otherwise replaced (exactly n the first
-// time, an eighth more after that if memory allows, so that moving atoms do not reallocate at every step).
+// A buffer of at least n elements of T: kept when it is large enough, otherwise replaced (by exactly n, or an eighth
+// more if memory allows and `grow`, so that moving atoms do not reallocate at every step).
 template <typename T>
-static int tc_reserve(gint_handle *h, T *&p, long long &cap, long long n) {
+static int tc_reserve(gint_handle *h, T *&p, long long &cap, long long n, bool grow) {
   n = std::max(n, 1LL);
   if (p && n <= cap) return GINT_OK;
-  long long want = p ? n + n / 8 : n;
+  long long want = grow ? n + n / 8 : n;
   dfree(p);
   h->tc_bytes -= cap * (long long)sizeof(T);
   cap = 0;
@@ -2860,6 +2860,27 @@ static int tc_reserve(gint_handle *h, T *&p, long long &cap, long long n) {
   h->tc_bytes += cap * (long long)sizeof(T);
   return GINT_OK;
 }
+
+// The same for a buffer that is wanted larger but may stay: false, and the buffer kept, without the memory.
+template <typename T>
+static bool tc_enlarge(gint_handle *h, T *&p, long long &cap, long long n, bool grow) {
+  if (n <= cap) return true;
+  for (long long want : {grow ? n + n / 8 : n, n}) {
+    T *q = nullptr;
+    if (cudaMalloc(&q, want * sizeof(T)) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    dfree(p);
+    h->tc_bytes += (want - cap) * (long long)sizeof(T);
+    p = q;
+    cap = want;
+    return true;
+  }
+  return false;
+}
+
+int gint_tc_reserve_hs(gint_handle *h, long long bytes) { return tc_reserve(h, h->hs, h->cap_hs, (bytes + 3) / 4, false); }
 
 // Layouts of the tensor-core path for the current neighbour lists: scratch ranges, contribution lists and plan
 // records.  Synchronous on st.
@@ -2885,7 +2906,11 @@ static int tc_layouts(gint_handle *h, cudaStream_t st) {
   h->max_brick_porb = (int)tot[3];
   int rc;
   h->fx_batch = 0;
-  if ((rc = tc_reserve(h, h->plan, h->cap_plan, tot[1])) || (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2]))) return rc;
+  const bool grow = h->plan != nullptr;  // not the first geometry
+  const long long hs_min = std::max(tot[0], nb * kNbrListBytes / 4);  // (the next geometry's brick lists too)
+  if ((rc = tc_reserve(h, h->plan, h->cap_plan, tot[1], grow)) ||
+      (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2], grow)) || (rc = tc_reserve(h, h->hs, h->cap_hs, hs_min, grow)))
+    return rc;
   // the scratch tiles' buffer also serves the float64 passes: enlarged (small systems) to hold a brick per SM for
   // them, to no more than twice the tiles and 96 MB (a server keeps many small handles), if memory allows.  A batch
   // of fewer than 64 bricks would leave the chip to launch tails; the CUDA-core kernels are then as fast.  (After the
@@ -2895,10 +2920,9 @@ static int tc_layouts(gint_handle *h, cudaStream_t st) {
     const long long room = (2 * tot[0] * 4 + (96LL << 20) - fx0) / fx1;
     const int want = (int)std::min<long long>({(long long)h->num_sms, nb, std::max(room, 0LL)});
     if (want >= std::min<long long>(nb, 64) && want > 0 &&
-        tc_reserve(h, h->hs, h->cap_hs, std::max(tot[0], (gint_fx_bytes(h, want) + 3) / 4)) == GINT_OK)
+        tc_enlarge(h, h->hs, h->cap_hs, (gint_fx_bytes(h, want) + 3) / 4, grow))
       h->fx_batch = want;
   }
-  if ((rc = tc_reserve(h, h->hs, h->cap_hs, tot[0]))) return rc;
   if ((size_t)nu * sizeof(int) <= kLaySmem) {
     if ((rc = set_smem(k_lay_fill<true>, kLaySmem))) return rc;
     k_lay_fill<true><<<(unsigned)nr, 32, nu * sizeof(int), st>>>(g, h->nbr(), nb, h->pair_u, nu, per, h->lay_cnt,

@@ -60,6 +60,7 @@ void fake_plan_error(int on) { g_err_plans = on; }
 void fake_limit(size_t bytes) { g_limit = bytes; }  // device memory
 size_t fake_live() { return g_live; }
 void fake_list_entries(long long n) { g_tot[2] = n; }
+void fake_tiles(long long n) { g_tot[0] = n; }  // float32 elements
 
 // what nvcc's host code calls
 void **__cudaRegisterFatBinary(void *) {

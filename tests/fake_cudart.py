@@ -36,4 +36,5 @@ def load(tmpdir):
     lib.fake_live.restype = ctypes.c_size_t
     lib.fake_limit.argtypes = [ctypes.c_size_t]
     lib.fake_list_entries.argtypes = [ctypes.c_longlong]
+    lib.fake_tiles.argtypes = [ctypes.c_longlong]
     return G, lib

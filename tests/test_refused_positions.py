@@ -114,6 +114,41 @@ def test_scratch_of_the_float64_passes_takes_no_memory_that_others_need(fake):
     assert lib.fake_live() == before
 
 
+def test_no_buffer_for_the_brick_lists_alone(fake):
+    """The counting pass's lists (1 KB a brick) lie in the scratch buffer: a handle holds what gint_memory says, and less
+    than lists and scratch tiles together."""
+    G, lib = fake
+    lib.fake_refuse(0)
+    lib.fake_plan_error(0)
+    w = inputs.si_workload((1, 1, 1), (64, 64, 64), seed=0)
+    bricks = 16 * 16 * 8
+    before = lib.fake_live()
+    lib.fake_tiles(bricks * 200)  # 800 bytes a brick of tiles
+    lib.fake_limit(2 ** 63)
+    g = G.Gint(w.system)
+    try:
+        live = lib.fake_live() - before
+        assert abs(live - g.memory()) <= 0.01 * live
+        # without the float64 scratch: the first limit that admits the handle
+        g.close()
+        lib.fake_limit(before + live - 1)
+        g = G.Gint(w.system)
+        small = lib.fake_live() - before
+        assert abs(small - g.memory()) <= 0.01 * small
+        for _ in range(2):  # kept, not grown, by a rebuild of the same size
+            g.set_positions(torch.from_numpy(w.system.pos.copy()))
+            assert lib.fake_live() - before == small
+        rest = small - bricks * 1024
+        g.close()
+        lib.fake_tiles(bricks * 1024 // 4)  # tiles of the lists' size
+        g = G.Gint(w.system)
+        assert lib.fake_live() - before - rest == bricks * 1024
+    finally:
+        g.close()
+        lib.fake_limit(2 ** 63)
+        lib.fake_tiles(1000)
+
+
 @pytest.mark.gpu
 def test_refused_and_recovered_on_the_gpu():
     from paper_2603_21835_gb300 import gint as G
