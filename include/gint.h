@@ -101,6 +101,13 @@ typedef struct gint_handle gint_handle;
  * GINT_ECAPACITY if a brick exceeds the kernels' limits.  *out is NULL on failure. */
 int gint_create(const gint_desc *desc, gint_handle **out);
 
+/* gint_create with flags.  GINT_NO_FP64_SCRATCH: the handle does not enlarge its scratch for the float64
+ * passes on the tensor cores (at most as much again as its local-H tiles and 96 MB), which then run on the
+ * CUDA cores, four times slower; for handles that serve the tensor-core precisions only (a pool of
+ * replicas counted against a memory budget). */
+#define GINT_NO_FP64_SCRATCH 1u
+int gint_create_flags(const gint_desc *desc, unsigned flags, gint_handle **out);
+
 /* Frees the handle and all its device memory.  NULL is accepted. */
 int gint_destroy(gint_handle *h);
 

@@ -170,7 +170,7 @@ int gint_reserve_nbr(gint_handle *h) {
 namespace {
 
 // The handle's set-up; `unfold` gives every (atom, image) entry of a brick a slot of its own.
-int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
+int create_impl(const gint_desc *d, bool unfold, unsigned flags, gint_handle **out) {
   if (!out) return GINT_EINVAL;
   *out = nullptr;
   int v = validate(d);
@@ -178,6 +178,7 @@ int create_impl(const gint_desc *d, bool unfold, gint_handle **out) {
   gint_handle *h = new (std::nothrow) gint_handle();
   if (!h) return GINT_ENOMEM;
   h->unfold = unfold;
+  h->fx_off = (flags & GINT_NO_FP64_SCRATCH) != 0;
   std::memset(static_cast<void *>(&h->geom), 0, sizeof(GGeom));  // batched launches compare GTabs bytes
   // host copy of the descriptor's species (an unfolded twin is built from it on demand)
   {
@@ -455,7 +456,7 @@ int make_twin(gint_handle *h) {
   d.n3 = h->geom.n3;
   d.skin = h->d_skin;
   gint_handle *t = nullptr;
-  int rc = create_impl(&d, true, &t);
+  int rc = create_impl(&d, true, GINT_NO_FP64_SCRATCH, &t);
   if (rc) return rc;
   if (h->pos_host != h->d_pos0) {
     rc = gint_set_positions(t, h->pos_dev, h->own_stream);
@@ -491,7 +492,12 @@ int hr_handle(gint_handle *h, gint_handle **t) {
 
 extern "C" {
 
-int gint_create(const gint_desc *d, gint_handle **out) { return create_impl(d, false, out); }
+int gint_create(const gint_desc *d, gint_handle **out) { return create_impl(d, false, 0u, out); }
+
+int gint_create_flags(const gint_desc *d, unsigned flags, gint_handle **out) {
+  if (flags & ~GINT_NO_FP64_SCRATCH) return GINT_EINVAL;
+  return create_impl(d, false, flags, out);
+}
 
 int gint_destroy(gint_handle *h) {
   if (!h) return GINT_OK;

@@ -108,6 +108,7 @@ struct gint_handle {
   long long cap_hs = 0, cap_src = 0, cap_plan = 0;
   // float64 passes on digit products (gint_fx.cu): scratch in hs, for fx_batch bricks at a time (0: not available)
   int fx_batch = 0;
+  bool fx_off = false;                            // GINT_NO_FP64_SCRATCH (and unfolded twins, which no float64 call reaches)
   int *fx_eD = nullptr, *atom_off_dev = nullptr;  // [2][norb] exponents of D's rows; first orbital of each atom
   signed char fx_q[GINT_MAX_SPECIES][GINT_MAX_ORB_ATOM] = {};  // exponent of each orbital's largest radial value
   double *otab64q = nullptr;                      // otab64, each radial times 2^-fx_q

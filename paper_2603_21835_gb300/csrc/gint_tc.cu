@@ -2912,11 +2912,11 @@ static int tc_layouts(gint_handle *h, cudaStream_t st) {
       (rc = tc_reserve(h, h->hu_src, h->cap_src, tot[2], grow)) || (rc = tc_reserve(h, h->hs, h->cap_hs, hs_min, grow)))
     return rc;
   // the scratch tiles' buffer also serves the float64 passes: enlarged (small systems) to hold a brick per SM for
-  // them, to no more than twice the tiles and 96 MB (a server keeps many small handles), if memory allows.  A batch
+  // them, to no more than twice the tiles and 96 MB, if memory allows and the handle's creator has not declined it.  A batch
   // of fewer than 64 bricks would leave the chip to launch tails; the CUDA-core kernels are then as fast.  (After the
   // buffers that every pass needs, so that it never takes their memory.)
   const long long fx0 = gint_fx_bytes(h, 0), fx1 = gint_fx_bytes(h, 1) - fx0;
-  if (fx1 > 0) {
+  if (fx1 > 0 && !h->fx_off) {
     const long long room = (2 * tot[0] * 4 + (96LL << 20) - fx0) / fx1;
     const int want = (int)std::min<long long>({(long long)h->num_sms, nb, std::max(room, 0LL)});
     if (want >= std::min<long long>(nb, 64) && want > 0 &&

@@ -56,6 +56,7 @@ _vp, _ll, _i, _d = ctypes.c_void_p, ctypes.c_longlong, ctypes.c_int, ctypes.c_do
 _lib.gint_strerror.restype = ctypes.c_char_p
 _lib.gint_strerror.argtypes = [_i]
 _lib.gint_create.argtypes = [ctypes.POINTER(_Desc), ctypes.POINTER(_vp)]
+_lib.gint_create_flags.argtypes = [ctypes.POINTER(_Desc), ctypes.c_uint, ctypes.POINTER(_vp)]
 _lib.gint_destroy.argtypes = [_vp]
 _lib.gint_layout.argtypes = [_vp, ctypes.POINTER(_i), ctypes.POINTER(_i), ctypes.POINTER(_ll)]
 _lib.gint_pairs.argtypes = [_vp, _vp, _vp]
@@ -107,7 +108,7 @@ C_ABI_SYMBOLS = ("gint_create", "gint_destroy", "gint_layout", "gint_pairs", "gi
                  "gint_set_projectors", "gint_psibeta_layout", "gint_psibeta", "gint_cn_create", "gint_cn_destroy",
                  "gint_cn_step", "gint_dm_build", "gint_dm_build_f16x3", "gint_cn_info", "gint_edm",
                  "gint_brick_lists", "gint_orbitals", "gint_server_create", "gint_server_submit", "gint_server_test",
-                 "gint_server_stats", "gint_server_stop", "gint_server_destroy")
+                 "gint_server_stats", "gint_server_stop", "gint_server_destroy", "gint_create_flags")
 
 
 class CrankNicolson:
@@ -299,9 +300,12 @@ def _species_array(species_list):
 
 
 class Gint:
-    """One geometry (cell, atoms, species radial tables, grid) resident on the current GPU."""
+    """One geometry (cell, atoms, species radial tables, grid) resident on the current GPU.
 
-    def __init__(self, system, skin: float = 0.0):
+    fp64_scratch=False: no scratch for the float64 passes on the tensor cores, which then run on the CUDA cores
+    (handles that serve the mixed precisions only: 80 MB less for the 8-atom Si cell)."""
+
+    def __init__(self, system, skin: float = 0.0, fp64_scratch: bool = True):
         sp_arr, rad_keep = _species_array(system.sp)
         pos = np.ascontiguousarray(system.pos, dtype=np.float64)
         spc = np.ascontiguousarray(system.species, dtype=np.int32)
@@ -312,7 +316,10 @@ class Gint:
         d.n1, d.n2, d.n3 = (int(x) for x in system.grid)
         d.skin = float(skin)
         h = ctypes.c_void_p()
-        _check(_lib.gint_create(ctypes.byref(d), ctypes.byref(h)), "gint_create")
+        if fp64_scratch:
+            _check(_lib.gint_create(ctypes.byref(d), ctypes.byref(h)), "gint_create")
+        else:
+            _check(_lib.gint_create_flags(ctypes.byref(d), 1, ctypes.byref(h)), "gint_create_flags")
         self._h = h
         self.grid = tuple(int(x) for x in system.grid)
         self.ngrid = int(np.prod(self.grid))

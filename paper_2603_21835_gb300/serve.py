@@ -48,7 +48,7 @@ class Replica:
 
     def __init__(self, session: "Session", index: int, device: torch.device):
         self.session, self.index = session, index
-        self.g = G.Gint(session.system)
+        self.g = G.Gint(session.system, fp64_scratch=session.server.fp64_scratch)
         s = session
         self.D = torch.empty(s.nblock, dtype=torch.float64, device=device)
         self.V = torch.empty(s.ngrid, dtype=torch.float64, device=device)
@@ -74,7 +74,7 @@ class Session:
     def __init__(self, server: "Server", key: int, system):
         self.server, self.key, self.system = server, key, system
         self.replicas: Dict[int, Replica] = {}
-        g = G.Gint(system)
+        g = G.Gint(system, fp64_scratch=server.fp64_scratch)
         self.nblock, self.ngrid, self.natoms, self.norb = g.nblock, g.ngrid, g.natoms, g.norb
         self.pair_IJ, self.pair_off, self.atom_off = g.pair_IJ, g.pair_off, g.atom_off
         self.W = g.stats()["W"]
@@ -147,15 +147,18 @@ def _pinned(x) -> torch.Tensor:
 # Server
 # ----------------------------------------------------------------------------------------------
 class Server:
-    """Continuous-batching gint server on one GPU (see the module docstring)."""
+    """Continuous-batching gint server on one GPU (see the module docstring).  fp64_scratch=False: replicas without the
+    scratch of the float64 passes, which no job uses, so that more of them fit the budget."""
 
     def __init__(self, species: Sequence, budget_bytes: int, precision: int = G.F16X3, replicas: int = 1,
-                 device: Optional[torch.device] = None, idle_s: float = 0.2, poll_s: float = 5e-5):
+                 device: Optional[torch.device] = None, idle_s: float = 0.2, poll_s: float = 5e-5,
+                 fp64_scratch: bool = True):
         self.species = list(species)
         self.precision = int(precision)
         self.replicas = max(1, int(replicas))
         self.device = torch.device(device if device is not None else "cuda")
         self.poll_s = poll_s
+        self.fp64_scratch = bool(fp64_scratch)
         self.budget = Budget(budget_bytes)
         self._sessions: Dict[int, Session] = {}
         self._queue: Deque[_Request] = collections.deque()  # guarded by _cv

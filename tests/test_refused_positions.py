@@ -149,6 +149,26 @@ def test_no_buffer_for_the_brick_lists_alone(fake):
         lib.fake_tiles(1000)
 
 
+def test_handles_without_the_float64_scratch(fake):
+    """fp64_scratch=False holds the tiles only; the float64 passes run on the CUDA cores, now and after set_positions."""
+    G, lib = fake
+    lib.fake_refuse(0)
+    lib.fake_plan_error(0)
+    w = inputs.si_workload((1, 1, 1), (16, 16, 16), seed=0)
+    before = lib.fake_live()
+    full = G.Gint(w.system)
+    n_full = lib.fake_live() - before
+    lean = G.Gint(w.system, fp64_scratch=False)
+    n_lean = lib.fake_live() - before - n_full
+    assert full.memory() - lean.memory() == n_full - n_lean > 0
+    assert b"k_fx_eval" in _rho64(G, lib, full) and b"k_simt_rho" in _rho64(G, lib, lean)
+    lean.set_positions(torch.from_numpy(w.system.pos.copy()))
+    assert b"k_simt_rho" in _rho64(G, lib, lean) and lib.fake_live() - before - n_full == n_lean
+    assert lib.gint_create_flags(None, 2, None) == -1
+    full.close()
+    lean.close()
+
+
 @pytest.mark.gpu
 def test_refused_and_recovered_on_the_gpu():
     from paper_2603_21835_gb300 import gint as G
