@@ -248,10 +248,21 @@ def run_reference(args):
 
 # ------------------------------------------------------------------------------ our arm
 # kernels of ours per step (density + local-H passes; memsets are not kernels):
-#   fp64: k_simt_rho, k_simt_vlocal;  fp32: k_to_f32, k_simt_rho, k_simt_vlocal;
+#   fp64: see fp64_path;  fp32: k_to_f32, k_simt_rho, k_simt_vlocal;
 #   f16x3 / f16x1: k_prep, k_build_tiles, k_tc_fused (both passes), k_h_reduce
 KERNEL_LAUNCHES = {"fp64": None, "fp32": 3, "f16x3": 4, "f16x1": 4}
 TENSOR_PRECISIONS = ("f16x3", "f16x1")
+
+
+def fp64_path(batch, bricks):
+    """What the float64 density and local-H passes launch: digits of D and two kernels a batch of bricks and pass and
+    the mirror (batch: gint_fp64_batch), or one CUDA-core kernel each (batch 0)."""
+    if batch:
+        return {"launches": 3 + 4 * -(-bricks // batch), "bound": "tensor",
+                "kernels": "k_fx_eval, k_fx_mma (float64 orbitals, exact digit products)",
+                "rho": "k_fx_eval + k_fx_mma (density)", "h": "k_fx_eval + k_fx_mma (local H)"}
+    return {"launches": 2, "bound": "alu", "kernels": "k_simt_rho, k_simt_vlocal (float64 CUDA cores)",
+            "rho": "k_simt_rho", "h": "k_simt_vlocal"}
 
 
 def run_serving(args, prec, dev):
@@ -636,6 +647,7 @@ def main():
     # the float64 GPU path on the same workload and inputs (the comparator of the
     # mixed-precision path), timed the same way: density + local-H passes, L2 flushed
     fp64_gpu = None
+    path64 = fp64_path(g.fp64_batch(), g.stats()["nbricks"])
     if args.precision != "fp64" and args.fp64_steps > 0:
         g.rho(Db, G.FP64, out=rho)
         g.vlocal(V, G.FP64, out=H)
@@ -653,7 +665,7 @@ def main():
         ms64 = max_over_ranks(statistics.mean(t64), world, dev)
         v64 = world * 2.0 * W / (ms64 * 1e-3) / 1e9
         fp64_gpu = {"value": v64, "unit": UNIT, "ms_per_step": ms64, "steps": args.fp64_steps,
-                    "kernels": "k_fx_eval, k_fx_mma (float64 orbitals, exact digit products)",
+                    "kernels": path64["kernels"],
                     "mixed_over_fp64": value / v64}
 
     # roofline of the dominant kernel (per-launch mean over the timed region, CUDA events on its stream)
@@ -666,14 +678,16 @@ def main():
     else:
         mr = statistics.mean(a.elapsed_time(b) for a, b in evr)
         mh = statistics.mean(a.elapsed_time(b) for a, b in evh)
-        k64 = args.precision == "fp64"  # orbital evaluation and digit products per batch of bricks
-        dom, tdom = (("k_fx_eval + k_fx_mma (density)" if k64 else "k_simt_rho", mr) if mr >= mh else
-                     ("k_fx_eval + k_fx_mma (local H)" if k64 else "k_simt_vlocal", mh))
+        names = path64 if args.precision == "fp64" else fp64_path(0, 0)  # (float32: the CUDA-core kernels)
+        dom, tdom = (names["rho"], mr) if mr >= mh else (names["h"], mh)
         flops = 2.0 * W  # one pass per launch, 2 flops per ordered orbital pair per grid point
     if tensor:
         peak = peaks.get("bf16_tflops")
         bound, punit = "tensor", "TFLOP/s"
         pdesc = f"f16 dense = {peak_kind} bf16 burst (nominal f16 and bf16 dense rates are equal)"
+    elif args.precision == "fp64" and path64["bound"] == "alu":
+        peak = FP64_NOMINAL_TFLOPS
+        bound, punit, pdesc = "alu", "TFLOP/s", "fp64 nominal 1.25 TFLOP/s (GB300)"
     elif args.precision == "fp64":
         peak = peaks.get("bf16_tflops") / 36
         bound, punit, pdesc = "tensor", "TFLOP/s", f"{peak_kind} bf16 burst / 36 float16 digit products"
@@ -741,10 +755,8 @@ def main():
         cn = run_cn(g.norb, 128 if g.norb < 2048 else 1024, 3 if g.norb < 2048 else 2, stream)
 
     launches = KERNEL_LAUNCHES.get(args.precision)
-    if args.precision == "fp64":  # digits of D, two kernels a batch of bricks and pass (one brick per SM), the mirror
-        n1, n2, n3 = w.system.grid
-        bricks = -(-n1 // 4) * -(-n2 // 4) * -(-n3 // 8)
-        launches = 3 + 4 * -(-bricks // torch.cuda.get_device_properties(dev).multi_processor_count)
+    if args.precision == "fp64":
+        launches = path64["launches"]
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": max(3, args.warmup), "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",

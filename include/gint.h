@@ -154,6 +154,11 @@ int gint_orbitals(gint_handle *h, int precision, long long npts, const double *p
  * output).  The footprint that a serving loop counts against its HBM budget. */
 int gint_memory(const gint_handle *h, long long *device_bytes);
 
+/* Diagnostic: how many bricks a launch of the float64 passes on the tensor cores takes at the current
+ * geometry (host output); 0: the float64 passes run on the CUDA cores (no scratch, or bricks of more than
+ * 512 padded orbital columns). */
+int gint_fp64_batch(const gint_handle *h, int *bricks);
+
 /* Replaces the atom positions from a DEVICE array [natoms][3] and rebuilds the neighbour
  * lists on the device (the BigGrid neighbour relation of paper Sec. 3.3.1 and Fig. 2, renewed as
  * the ions move in the Ehrenfest dynamics of Sec. 2).  The pair set stays fixed: GINT_ESKIN if a

@@ -574,6 +574,12 @@ int gint_memory(const gint_handle *h, long long *device_bytes) {
   return GINT_OK;
 }
 
+int gint_fp64_batch(const gint_handle *h, int *bricks) {
+  if (!h || !bricks) return GINT_EINVAL;
+  *bricks = h->fx_batch;
+  return GINT_OK;
+}
+
 static int rebuild_geometry(gint_handle *h, const double *pos_dev, cudaStream_t st) {
   if (cudaMemcpyAsync(h->pos_dev, pos_dev, 3 * sizeof(double) * h->geom.natoms, cudaMemcpyDeviceToDevice, st) !=
       cudaSuccess)

@@ -76,6 +76,7 @@ _lib.gint_grid_dot_noalloc.argtypes = [_vp, _vp, _ll, _d, _vp, _vp]
 _lib.gint_run_batch.argtypes = [ctypes.POINTER(_Task), _i, _i, _vp]
 _lib.gint_run_batch_timed.argtypes = [ctypes.POINTER(_Task), _i, _i, _vp, _vp, _vp]
 _lib.gint_memory.argtypes = [_vp, ctypes.POINTER(_ll)]
+_lib.gint_fp64_batch.argtypes = [_vp, ctypes.POINTER(_i)]
 _lib.gint_set_reduction.argtypes = [_vp, _i]
 _lib.gint_layout_R.argtypes = [_vp, ctypes.POINTER(_i), ctypes.POINTER(_ll), ctypes.POINTER(ctypes.POINTER(_i)),
                                ctypes.POINTER(ctypes.POINTER(_ll))]
@@ -108,7 +109,8 @@ C_ABI_SYMBOLS = ("gint_create", "gint_destroy", "gint_layout", "gint_pairs", "gi
                  "gint_set_projectors", "gint_psibeta_layout", "gint_psibeta", "gint_cn_create", "gint_cn_destroy",
                  "gint_cn_step", "gint_dm_build", "gint_dm_build_f16x3", "gint_cn_info", "gint_edm",
                  "gint_brick_lists", "gint_orbitals", "gint_server_create", "gint_server_submit", "gint_server_test",
-                 "gint_server_stats", "gint_server_stop", "gint_server_destroy", "gint_create_flags")
+                 "gint_server_stats", "gint_server_stop", "gint_server_destroy", "gint_create_flags",
+                 "gint_fp64_batch")
 
 
 class CrankNicolson:
@@ -375,6 +377,12 @@ class Gint:
         """Device bytes held by the handle (tables, neighbour lists, workspace)."""
         b = _ll()
         _check(_lib.gint_memory(self._h, ctypes.byref(b)), "gint_memory")
+        return b.value
+
+    def fp64_batch(self) -> int:
+        """Bricks per launch of the float64 passes on the tensor cores; 0: they run on the CUDA cores."""
+        b = _i()
+        _check(_lib.gint_fp64_batch(self._h, ctypes.byref(b)), "gint_fp64_batch")
         return b.value
 
     def close(self):

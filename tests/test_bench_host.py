@@ -37,3 +37,10 @@ def test_peaks_and_profile_lookup():
     traffic, src = bench.profiled_traffic("si64_g96", "f16x3")
     if traffic is not None:  # None once the kernel source has changed since the counters were taken
         assert traffic > 0 and src.startswith("profiles" + os.sep)
+
+
+def test_float64_launches_follow_the_batch():
+    assert bench.fp64_path(152, 864)["launches"] == 3 + 4 * 6
+    assert bench.fp64_path(64, 64)["launches"] == 7 and bench.fp64_path(64, 65)["launches"] == 11
+    cuda = bench.fp64_path(0, 864)
+    assert cuda["launches"] == 2 and cuda["bound"] == "alu" and "k_fx" not in str(cuda)

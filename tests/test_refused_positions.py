@@ -162,6 +162,8 @@ def test_handles_without_the_float64_scratch(fake):
     n_lean = lib.fake_live() - before - n_full
     assert full.memory() - lean.memory() == n_full - n_lean > 0
     assert b"k_fx_eval" in _rho64(G, lib, full) and b"k_simt_rho" in _rho64(G, lib, lean)
+    assert _rho64(G, lib, full).count(b"k_fx_eval") == -(-full.stats()["nbricks"] // full.fp64_batch())
+    assert lean.fp64_batch() == 0
     lean.set_positions(torch.from_numpy(w.system.pos.copy()))
     assert b"k_simt_rho" in _rho64(G, lib, lean) and lib.fake_live() - before - n_full == n_lean
     assert lib.gint_create_flags(None, 2, None) == -1
