@@ -277,8 +277,9 @@ int gint_psibeta(gint_handle *h, const double *A, double *out, void *stream);
  * allocation.
  * gint_cn_info: the LAPACK-style info of the last factorisation (0: success; i > 0: the pivot d_i of
  * L D L^T is zero or not finite, or for gint_edm not positive);
- * synchronous; returns GINT_ETIMEDOUT (once) when a bounded wait of the tensor-core build gave up.  The
- * D of that call is then undefined; and since a CTA whose final completion wait also gave up releases
+ * synchronous; returns GINT_ETIMEDOUT (once) when a bounded wait (2 s) of a tensor-core product gave up, in
+ * any of gint_cn_step, gint_dm_build, gint_dm_build_f16x3 and gint_edm: it is the only sign of it, and the
+ * results of the calls since the last gint_cn_info are then undefined; and since a CTA whose final completion wait also gave up releases
  * its tensor memory with MMAs possibly still in flight, destroy the context after GINT_ETIMEDOUT rather
  * than reuse it. */
 typedef struct gint_cn gint_cn;

@@ -208,8 +208,9 @@ __device__ __forceinline__ void dm_tile(long long p, int T, int &I, int &J) {
     J = J0 + y;
   }
 }
-// (double)x for a normal x or zero (smaller values count as zero) in integer arithmetic: a conversion takes the SM's
-// float64 pipe 16 clocks a warp.
+// (double)x for a normal x or zero in integer arithmetic: a conversion takes the SM's float64 pipe 16 clocks a warp.
+// Sums, compensations and cross terms are never denormal: products of float16 values are multiples of 2^-48, and
+// float32 sums and differences of such multiples are again (their roundings are to coarser ones).
 __device__ __forceinline__ double widen(float x) {
   const uint32_t b = __float_as_uint(x), m = b & 0x7fffffu, e = (b >> 23) & 0xffu;
   return e ? __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | (m >> 3)), (int)(m << 29)) : 0.0;

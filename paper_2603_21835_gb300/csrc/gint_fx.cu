@@ -4,8 +4,8 @@
 // The contraction of a brick (128 points, NP orbitals) takes 128 NP^2 multiply-adds; at the CUDA cores' 2 float64
 // ones per clock and SM that is nine tenths of a pass (8-atom Si, 864 bricks: density 2.2 ms, local H 1.8 ms, forces
 // 4.3 ms).  Here the CUDA cores evaluate the orbitals only, and the contractions run as 36 float16 digit products:
-// 0.51, 0.59 and 0.97 ms.  Left are the evaluations, bound by the float64 pipe (16 cycles a warp instruction and SM),
-// and the scratch round trip through L2.  Per 152 bricks: k_fx_eval 51 (density) and 63 us (local H), k_fx_mma 28 to
+// 0.52, 0.60 and 0.98 ms.  Left are the evaluations, bound by the float64 pipe (16 cycles a warp instruction and SM),
+// and the scratch round trip through L2.  Per 152 bricks: k_fx_eval 52 (density) and 63 us (local H), k_fx_mma 28 to
 // 36 us, k_fx_grad 76 us.  Errors against extended precision on that system (Frobenius norm, mean of five geometries),
 // CUDA cores -> here: rho 6.9e-16 -> 6.1e-16, H 1.7e-15 -> 9.1e-16, F 2.0e-15 -> 1.9e-15.
 //

@@ -12,16 +12,17 @@
 // warp-wide float64 instruction occupies the SM's pipe for 16 clocks, and the kernel's time is the number of
 // those instructions.  So what does not depend on the pair is formed once per call (k_pb_phase: quadrature
 // weight times projector radial times the phase e^{-i A.x} of the point relative to tau_I; e^{-i A.tau_I}
-// multiplies the sums at the end), the orbital tables hold the knot differences, dr f' and the Y_lm
+// multiplies the sums at the end), the orbital tables hold the interpolant's polynomial coefficients times the Y_lm
 // constants, and points outside an image's support cost the distance test only.  A warp takes 2 neighbouring rays
 // times 16 neighbouring radial nodes at a time, a compact patch that is mostly all inside or all outside
 // (32 rays of one radius, a band around the whole sphere, are rarely either), and 81 such ray pairs fill whole
 // warps where 162 rays leave the last of six with two.  k_psibeta: a CTA of 3 warps (four share an SM: one's
 // set-up and sums overlap the others' points; one CTA of 9 warps took 5.33 ms where this takes 4.77) works on a
 // pair and a group of its ray pairs; k_pb_sum adds the groups' sums in order (no atomics).
-// Per point and image inside the support 121 float64 instructions, outside a float32 test for the patch.
-// Bound: the float64 pipe (0.8 of its cycles active).  64-atom Si, 1,856 pairs x 22,680 points: 22.9 ms
-// (one CTA a pair and one thread a ray, every point evaluated in full) -> 4.61 ms.
+// Inside the support 151 float64 additions, multiplications and fused ones are executed per point (12.7 of the 42.1
+// million points below), outside a float32 test for the patch.
+// Bound: the float64 pipe (0.88 of its cycles active).  64-atom Si, 1,856 pairs x 22,680 points: 22.9 ms
+// (one CTA a pair and one thread a ray, every point evaluated in full) -> 4.62 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>

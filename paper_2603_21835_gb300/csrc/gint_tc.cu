@@ -1600,7 +1600,7 @@ struct GRed {
 // as double-float pairs (two-sum: error-free additions into a hi + lo pair of float32, relative error
 // about n^2 2^-48 for n bricks, far below the float32 rounding of the tiles themselves) and combined
 // in float64; H_JI = H_IJ^T (per R: H_JI(-R) = H_IJ(R)^T, also for I == J, R != 0).  A thread
-// sums kRedE elements of the block (stride kRedLanes) over one of kRedGroups contiguous parts of
+// sums kRedE elements of the block (stride kRedLanes) over one of kRedGroups (or kRedGroupsFew) contiguous parts of
 // the pair's brick list, kRedB bricks' loads in flight; the parts'
 // sums are then combined in part order (the result does not depend on scheduling).  A float64 sum
 // of every tile value would cost more than the brick pass itself on this GPU (float64 runs at about

@@ -141,7 +141,7 @@ class CrankNicolson:
     def density_matrix(self, psi: torch.Tensor, f: torch.Tensor, out: Optional[torch.Tensor] = None,
                        stream=None, precision: str = "fp64") -> torch.Tensor:
         """Re(psi^T diag(f) conj(psi)) as [n, n] float64 (rows of psi are the states); precision "fp64"
-        (complex float64 GEMM) or "f16x3" (tensor cores, float16 three-term split)."""
+        (float64 from exact digit products) or "f16x3" (tensor cores, float16 three-term split)."""
         if out is None:
             out = torch.empty((self.n, self.n), dtype=torch.float64, device=psi.device)
         fn = {"fp64": _lib.gint_dm_build, "f16x3": _lib.gint_dm_build_f16x3}[precision]
@@ -160,6 +160,8 @@ class CrankNicolson:
         return out
 
     def info(self) -> int:
+        """Info of the last factorisation (0: success); raises if a product's bounded wait gave up since the last call,
+        which nothing else reports."""
         i = _i()
         _check(_lib.gint_cn_info(self._c, ctypes.byref(i)), "gint_cn_info")
         return i.value
