@@ -197,8 +197,8 @@ __device__ __forceinline__ void put(double *t, int i, double2 x) {
 // The exponent of |d|^(-1/2) for a pivot d, from 1 / d.  The update's contraction runs over pivots: W = L D has
 // their scale in full and L has none, so that a row's largest element may hide the others' low bits (sg's digits are
 // relative to it).  W |d|^(-1/2) against L |d|^(1/2), rounded to powers of two, are of the size of a Cholesky factor's rows: below the
-// square root of the matrix diagonal, whatever the pivots.  (Graded bases, norms over 10^8: 3e-11 in the solution
-// without it, 2e-15 as in plain float64 with it and the scaled basis of gint_cn.cu.)
+// square root of the matrix diagonal, whatever the pivots.  (Pivots of 1e-8 to 1e-12 under a unit diagonal, n = 160:
+// residual over |X| 4e-14 to 5e-12 without it, 4e-16 to 1e-15 with it, as float64 elimination leaves.)
 __device__ __forceinline__ int pivot_balance(double dinv) {
   const int e = (__double2hiint(dinv) >> 20) & 0x7ff;
   return e == 0 || e == 0x7ff ? 0 : (e - 1023) >> 1;
